@@ -792,7 +792,7 @@ def run_learned(args):
                                       EM_BATCH_TRAFFIC_PER_IMAGE[bps] * n if bps in EM_BATCH_TRAFFIC_PER_IMAGE
                                       else None)},
         "tuning": tuning,
-        "net_roofline": {"kernels": "k_pix + 4 x k_gemm (forward)", "bound": "tensor",
+        "net_roofline": {"kernels": "k_pix + 4 x k_conv3 (forward)", "bound": "tensor",
                          "achieved": round(net_tflops, 3), "peak": bf16_peak, "unit": "TFLOP/s",
                          "frac": round(net_tflops / bf16_peak, 5), "ms": round(net_ms, 5),
                          "flops_per_launch": net_flops,

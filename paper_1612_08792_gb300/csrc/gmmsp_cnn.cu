@@ -12,14 +12,16 @@
 //           MMAs with the accumulators in TMEM, the average pooling in shared
 //           memory.  Reads the CIELAB planes once and writes c0 (and, when
 //           training, x0, h1 and h2 for the backward pass).
-//   k_gemm  implicit-GEMM convolution in three modes: forward (rows =
-//           positions, columns = output channels, K = taps x 32), data
-//           gradient (rows = positions, columns = input channels, K = taps x
-//           output channels, the ReLU mask of the layer input applied in the
-//           epilogue) and weight gradient (rows = taps x 32 + 1, the extra
-//           row of ones giving the bias gradient; columns = output channels;
-//           K = positions, split over blocks and reduced in a fixed order).
-//   k_pool_bwd, k_loss, k_wgrad_reduce, k_adam, k_targets, k_init_from_net.
+//   k_conv3 3 x 3 convolution of the cell grid, forward and data gradient: one
+//           tile of 128 zero-bordered positions and its halo per step, the
+//           taps addressed by shifting the matrix descriptor's start, all 18
+//           MMAs issued at once.
+//   k_wgrad3 weight and bias gradient of a 3 x 3 layer from the same tiles
+//           (one accumulator per tap in tensor memory, kept over the tiles).
+//   k_pix_bwd the backward pass of the pixel level fused: pooling and ReLU
+//           gradient, data gradient of the second 1 x 1 layer, both weight
+//           gradients.
+//   k_loss, k_grad_reduce, k_adam, k_targets, k_init_from_net.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -46,9 +48,7 @@ namespace cnn {
 constexpr int kC = 32;                     // channels of every hidden layer
 constexpr int kOut = GMMSP_NET_CHANNELS;   // output channels of the last layer (16)
 constexpr int kUsed = GMMSP_NET_OUTPUTS;   // outputs used per superpixel (10)
-constexpr int kStageK = 32;                // K per shared-memory stage (two K = 16 MMAs)
 constexpr uint32_t kWaitTries = 1u << 22;  // bound on every mbarrier wait
-constexpr int kChunk = 2048;               // positions per weight-gradient block
 constexpr int kLossBlocks = 128;
 
 constexpr float kInScale = 0.02f;    // L, a, b -> about [-1, 1] (L shifted by 50)
@@ -60,6 +60,7 @@ struct ParamLayout {
   int w[6], b[6], taps[6], cout[6];
   int total;
 };
+inline int pix_params(const ParamLayout& p) { return p.w[2]; }  // of the two 1 x 1 layers, at the front
 inline ParamLayout param_layout() {
   ParamLayout p{};
   const int taps[6] = {1, 1, 9, 9, 9, 9};
@@ -77,28 +78,6 @@ inline ParamLayout param_layout() {
   return p;
 }
 
-enum Mode : int { FWD = 0, DGRAD = 1, WGRAD = 2 };
-
-// One convolution over a batch of B images of H x W positions (NHWC).
-struct Layer {
-  int B, H, W;
-  int taps;                   // 1 or 9 (3 x 3, padding 1)
-  int cout;                   // 32 or 16
-  int relu;                   // forward: ReLU after the bias
-  const __nv_bfloat16* x;     // layer input [B H W][32]
-  const __nv_bfloat16* w;     // weights [cout][taps 32]
-  const float* bias;          // [cout]
-  __nv_bfloat16* y;           // forward output, BF16 [B H W][cout] ...
-  float* y32;                 // ... or FP32 (the last layer)
-  const __nv_bfloat16* gy;    // gradient of the layer output (pre-activation) [B H W][cout]
-  const __nv_bfloat16* mask;  // data gradient: zero where mask <= 0 (or null)
-  __nv_bfloat16* gx;          // data gradient output [B H W][32]
-  float* wpart;               // weight-gradient partials [splits][taps 32 + 1][cout]
-};
-
-__device__ __forceinline__ int tap_dy(int t, int taps) { return taps == 1 ? 0 : t / 3 - 1; }
-__device__ __forceinline__ int tap_dx(int t, int taps) { return taps == 1 ? 0 : t % 3 - 1; }
-
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&v);
@@ -106,183 +85,197 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
-// 8 consecutive K-elements (k a multiple of 8) of the A row of position
-// (img, y, x), forward and data-gradient modes.
-template <int MODE>
-__device__ __forceinline__ uint4 a_vec8(const Layer& L, bool row_ok, int img, int y, int x, int k, int kdim) {
-  const uint4 z = make_uint4(0, 0, 0, 0);
-  if (!row_ok || k >= kdim) return z;
-  if (MODE == FWD) {
-    const int t = k >> 5, c = k & 31;
-    const int yy = y + tap_dy(t, L.taps), xx = x + tap_dx(t, L.taps);
-    if (yy < 0 || yy >= L.H || xx < 0 || xx >= L.W) return z;
-    return __ldg(reinterpret_cast<const uint4*>(L.x + (((long long)img * L.H + yy) * L.W + xx) * kC + c));
-  } else {
-    // gx[p] = sum_t W_t^T gy[p - d_t]
-    const int t = k / L.cout, co = k - t * L.cout;
-    const int yy = y - tap_dy(t, L.taps), xx = x - tap_dx(t, L.taps);
-    if (yy < 0 || yy >= L.H || xx < 0 || xx >= L.W) return z;
-    return __ldg(reinterpret_cast<const uint4*>(L.gy + (((long long)img * L.H + yy) * L.W + xx) * L.cout + co));
+// ------------------------------------------------- 3 x 3 layers: tiles
+// The cell grid of an image is cut into strips of at most kStripMax columns
+// (one strip up to nx = 126).  Within a strip the positions are numbered with
+// a zero border column on either side, q = y PW + x', PW = TW + 2, x' = 0 and
+// PW - 1 being the neighbouring columns (zero outside the image).  A tile is
+// 128 consecutive numbers q; its inputs are the 130 + 2 PW numbers
+// q0 - PW - 1 .. q0 + 127 + PW + 1 (rows above and below the image zero), and
+// tap (dy, dx) of row q is the input at q + dy PW + dx.
+//
+// In shared memory the inputs lie as channel groups of 8 (16 bytes), position
+// after position: group g of input i at g GS + 16 i.  Eight consecutive
+// positions of a group are then one 128-byte core matrix wherever they start,
+// so a tap is the same tile read from another start address: every input is
+// loaded once instead of nine times, and the 18 MMAs of a tile are issued
+// together (the gather per tap that this replaced read each activation nine
+// times from L2 and paid one MMA round trip per tap).  The same bytes serve as
+// a K-major operand (rows = positions: 8-row groups 128 bytes apart, K groups
+// GS apart) and as an MN-major one (K = positions).
+constexpr int kStripMax = 126;
+constexpr int kWLd = 528;                     // bytes between (tap, input group) slices of the staged weights
+constexpr int kWBytes = 36 * kWLd;            // 9 taps x 4 groups x 32 output channels x 16 bytes, padded
+constexpr int kRowTile = 128 * 16 + 32;       // a group of a 128-position tile without halo (bank offset 32)
+
+struct Grid3 {
+  int B, H, W;         // images and their cell grids
+  int strips, TW, PW;  // strips per image, their columns, the bordered row length
+  int tps;             // tiles per strip
+  int tiles;           // B strips tps
+  int NP, GS;          // inputs of a tile; bytes per channel group of them
+  unsigned rPW;        // floor(2^32 / PW) + 1: q / PW = umulhi(q, rPW) for q PW < 2^32, which holds here
+                       // (PW <= 128, and H PW <= 3 * the image's < 2^31 / 9 cells for narrower strips)
+};
+inline Grid3 grid3_of(int B, int H, int W) {
+  Grid3 g{};
+  g.B = B;
+  g.H = H;
+  g.W = W;
+  g.strips = (W + kStripMax - 1) / kStripMax;
+  g.TW = (W + g.strips - 1) / g.strips;
+  g.PW = g.TW + 2;
+  g.rPW = unsigned((1ull << 32) / unsigned(g.PW)) + 1u;
+  g.tps = (H * g.PW + 127) / 128;
+  g.tiles = B * g.strips * g.tps;
+  g.NP = 130 + 2 * g.PW;
+  g.GS = (g.NP * 16 + 127) / 128 * 128 + 32;  // 32 mod 128: the four groups of a position fall into other banks
+  return g;
+}
+
+struct Tile3 {
+  int img, c0, q0;
+};
+__device__ __forceinline__ Tile3 tile3_at(const Grid3& g, int tile) {
+  const int s = tile / g.tps;
+  return {s / g.strips, (s % g.strips) * g.TW, (tile - s * g.tps) * 128};
+}
+
+// Row of position q of a tile's strip in the [B H W] arrays, or -1 where q is
+// no output (border column, below the image, past the strip or the image).
+__device__ __forceinline__ int row3(const Grid3& g, const Tile3& t, int q) {
+  const int y = int(__umulhi(unsigned(q), g.rPW)), x = q - y * g.PW, col = t.c0 + x - 1;
+  return (y < g.H && x >= 1 && x <= g.TW && col < g.W) ? (t.img * g.H + y) * g.W + col : -1;
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The tile's inputs with their halo, G channel groups per position.
+template <int G>
+__device__ __forceinline__ void load_halo(const Grid3& g, const Tile3& t, const __nv_bfloat16* __restrict__ x,
+                                          uint32_t dst) {
+  for (int i = threadIdx.x; i < g.NP * G; i += 128) {
+    const int p = i / G, gr = i - p * G;
+    const int q = t.q0 + p + g.PW - 1;  // t.q0 - (PW + 1) + p + 2 PW, not negative
+    const int y = int(__umulhi(unsigned(q), g.rPW)) - 2, col = t.c0 + q - (y + 2) * g.PW - 1;
+    const bool ok = unsigned(y) < unsigned(g.H) && unsigned(col) < unsigned(g.W);
+    const int r = ok ? (t.img * g.H + y) * g.W + col : 0;
+    cp_async16(dst + gr * g.GS + p * 16, x + (long long)r * (8 * G) + gr * 8, ok);
   }
 }
 
-// Implicit GEMM D[rows x N] = A[rows x K] B[N x K]^T: one 128-row tile per
-// block of 128 threads, FP32 accumulator in TMEM (32 columns), K in stages of
-// 32 gathered into shared memory (K-major, no swizzle).  Weight-gradient
-// blocks (blockIdx.y) cover the positions [y chunk, (y + 1) chunk).
-template <int MODE, int N>
-__global__ void __launch_bounds__(128) k_gemm(Layer L, int rows, int kdim, int chunk, int* err) {
-  __shared__ __align__(1024) unsigned char sA[128 * kStageK * 2];
-  __shared__ __align__(1024) unsigned char sB[N * kStageK * 2];
+// The staged weights of a 3 x 3 layer: slices (tap, group of 8 input channels),
+// output channel co of slice s at s kWLd + 16 co.  K-major for the forward
+// pass (rows = output channels), MN-major for the data gradient (rows = input
+// channels, K = output channels).  Kept in global memory in this form beside
+// the plain BF16 parameters (store_bf16), so that staging is a linear copy.
+__device__ __forceinline__ void load_weights3(const unsigned char* __restrict__ w, uint32_t dst) {
+#pragma unroll
+  for (int i = threadIdx.x; i < kWBytes / 16; i += 128) cp_async16(dst + i * 16, w + i * 16, true);
+}
+
+// BF16 copies of parameter i: the flat one and, for the 3 x 3 layers, the
+// staged one.
+struct BfParams {
+  __nv_bfloat16* flat;
+  unsigned char* staged;  // kWBytes per 3 x 3 layer
+  int w[4], n[4];         // offset and number of each 3 x 3 layer's weights
+};
+__device__ __forceinline__ void store_bf16(const BfParams& p, int i, float v) {
+  const __nv_bfloat16 h = __float2bfloat16(v);
+  p.flat[i] = h;
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const int j = i - p.w[l];
+    if (j >= 0 && j < p.n[l]) {
+      const int co = j / 288, r = j - co * 288;
+      reinterpret_cast<__nv_bfloat16*>(p.staged + l * kWBytes + (r >> 3) * kWLd)[co * 8 + (r & 7)] = h;
+    }
+  }
+}
+
+struct Conv3 {
+  Grid3 g;
+  const __nv_bfloat16* a;     // forward: layer input [B H W][32]; data gradient: gradient of the output [B H W][cout]
+  const unsigned char* w;     // staged weights
+  const float* bias;          // forward: [cout]
+  __nv_bfloat16* y;           // output [B H W][32] BF16 (forward: ReLU(. + bias); data gradient: masked), or ...
+  float* y32;                 // ... FP32 [B H W][cout] without ReLU (the last layer's forward)
+  const __nv_bfloat16* mask;  // data gradient: zero where mask <= 0 (or null)
+};
+
+// 3 x 3 convolution, one tile per step: forward (A = the input, K = (tap,
+// input channel)) or data gradient (A = the output's gradient with GC groups
+// of 8 channels, K = (tap, output channel), taps mirrored).  K runs in the
+// same order of 16-wide MMAs as a tap-by-tap GEMM would, so the FP32 sums are
+// the same.
+//
+// Bound by latency: a tile is one load round trip, 18 MMAs, one epilogue.
+// 31.8 KB of shared memory at nx = 32 leave 6 blocks per SM to overlap them,
+// and a block takes further tiles with its weights staged once.  Measured
+// per 32-channel layer at 481x321, v = 15 (nx = 32), ncu, cold cache: 13.9 us
+// on 256 images (30.3 us for the tap-by-tap gather), 6.1 us on 32 (15.2 us);
+// index divisions by the row length in place of the multiplications cost
+// 29.7 and 10.2 us.
+template <bool DGRAD, int GC, int N>
+__global__ void __launch_bounds__(128, 6) k_conv3(Conv3 c, int* err) {
+  extern __shared__ __align__(128) unsigned char smem3[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_sh;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int r = blockIdx.x * 128 + tid;  // this thread's A row
-  int k_begin = 0, k_end = kdim;
-  if (MODE == WGRAD) {
-    k_begin = blockIdx.y * chunk;
-    k_end = min(k_begin + chunk, kdim);
-  }
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const uint32_t sW = tc::smem_u32(smem3), sX = sW + kWBytes;
   if (warp == 0) {
     tc::tmem_alloc(&tmem_sh, 32);
     tc::tmem_relinquish();
   }
   if (tid == 0) tc::mbar_init(&mbar, 1);
-  // forward / data gradient: the row is a position
-  int img = 0, y = 0, x = 0;
-  const bool row_ok = r < rows;
-  if (MODE != WGRAD && row_ok) {
-    const int hw = L.H * L.W;
-    img = r / hw;
-    const int rem = r - img * hw;
-    y = rem / L.W;
-    x = rem - y * L.W;
-  }
-  // weight gradient: the row is (tap, input channel) or the bias row; the
-  // stage's positions are walked incrementally from k_begin
-  const int wt = r / kC, wc = r - (r / kC) * kC;
-  int pimg = 0, py = 0, px = 0;
-  if (MODE == WGRAD && k_begin < k_end) {
-    const int hw = L.H * L.W;
-    pimg = k_begin / hw;
-    const int rem = k_begin - pimg * hw;
-    py = rem / L.W;
-    px = rem - py * L.W;
-  }
+  load_weights3(c.w, sW);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_sh;
-  constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N);
+  constexpr uint32_t idesc = tc::idesc_bf16_f32(128, N) | (DGRAD ? tc::kTransB : 0u);
   bool ok = true;
   uint32_t phase = 0;
-  for (int k0 = k_begin; k0 < k_end && ok; k0 += kStageK) {
-    if (MODE != WGRAD) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint4 v = a_vec8<MODE>(L, row_ok, img, y, x, k0 + 8 * j, k_end);
-        *reinterpret_cast<uint4*>(sA + tc::tile_offset(tid, 8 * j, kStageK)) = v;
-      }
-      if (tid < N) {
-        if (MODE == FWD) {
-          // B row = output channel tid: 32 contiguous weights (K is a multiple of 32)
-          const uint4* src = reinterpret_cast<const uint4*>(L.w + (long long)tid * L.taps * kC + k0);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint4 v = tid < L.cout ? __ldg(src + j) : make_uint4(0, 0, 0, 0);
-            *reinterpret_cast<uint4*>(sB + tc::tile_offset(tid, 8 * j, kStageK)) = v;
-          }
-        } else {
-          // B row = input channel tid; column k = (tap, output channel)
-          uint32_t u[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            float e[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int k = k0 + 2 * j + h;
-              e[h] = 0.f;
-              if (k < k_end) {
-                const int t = k / L.cout, co = k - t * L.cout;
-                e[h] = __bfloat162float(L.w[(long long)co * L.taps * kC + t * kC + tid]);
-              }
-            }
-            u[j] = pack2(e[0], e[1]);
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            *reinterpret_cast<uint4*>(sB + tc::tile_offset(tid, 8 * j, kStageK)) =
-                make_uint4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
-        }
-      }
-    } else {
-      const int dy = tap_dy(wt, L.taps), dx = tap_dx(wt, L.taps);
-      const bool is_w = wt < L.taps, is_b = r == L.taps * kC;
-      const bool has_b = tid < N && tid < L.cout;
-      float ea[32], eb[32];
-      int qi = pimg, qy = py, qx = px;
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        ea[j] = 0.f;
-        eb[j] = 0.f;
-        if (k0 + j < k_end) {
-          if (is_b) {
-            ea[j] = 1.f;
-          } else if (is_w) {
-            const int yy = qy + dy, xx = qx + dx;
-            if (yy >= 0 && yy < L.H && xx >= 0 && xx < L.W)
-              ea[j] = __bfloat162float(L.x[(((long long)qi * L.H + yy) * L.W + xx) * kC + wc]);
-          }
-          if (has_b) eb[j] = __bfloat162float(L.gy[(long long)(k0 + j) * L.cout + tid]);
-        }
-        if (++qx == L.W) {
-          qx = 0;
-          if (++qy == L.H) {
-            qy = 0;
-            ++qi;
-          }
-        }
-      }
-      pimg = qi;
-      py = qy;
-      px = qx;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        *reinterpret_cast<uint4*>(sA + tc::tile_offset(tid, 8 * j, kStageK)) =
-            make_uint4(pack2(ea[8 * j], ea[8 * j + 1]), pack2(ea[8 * j + 2], ea[8 * j + 3]),
-                       pack2(ea[8 * j + 4], ea[8 * j + 5]), pack2(ea[8 * j + 6], ea[8 * j + 7]));
-        if (tid < N)
-          *reinterpret_cast<uint4*>(sB + tc::tile_offset(tid, 8 * j, kStageK)) =
-              make_uint4(pack2(eb[8 * j], eb[8 * j + 1]), pack2(eb[8 * j + 2], eb[8 * j + 3]),
-                         pack2(eb[8 * j + 4], eb[8 * j + 5]), pack2(eb[8 * j + 6], eb[8 * j + 7]));
-      }
-    }
+  for (int tile = blockIdx.x; tile < c.g.tiles; tile += gridDim.x) {
+    const Tile3 t = tile3_at(c.g, tile);
+    load_halo<GC>(c.g, t, c.a, sX);
+    cp_async_wait_all();
     tc::fence_async_smem();
+    tc::fence_before_sync();  // the previous tile's accumulator has been read
     __syncthreads();
     if (tid == 0) {
       tc::fence_after_sync();
-      const uint32_t a0 = tc::smem_u32(sA), b0 = tc::smem_u32(sB);
+      // descriptor start addresses count 16 bytes: one input position per unit
+      uint64_t ad[GC / 2];
 #pragma unroll
-      for (int kk = 0; kk < kStageK / 16; ++kk) {
-        const uint64_t ad = tc::smem_desc(a0 + kk * 256, 128, (kStageK / 8) * 128);
-        const uint64_t bd = tc::smem_desc(b0 + kk * 256, 128, (kStageK / 8) * 128);
-        tc::mma_bf16(tmem, ad, bd, idesc, (k0 > k_begin || kk > 0) ? 1u : 0u);
+      for (int kk = 0; kk < GC / 2; ++kk) ad[kk] = tc::smem_desc(sX + 2 * kk * c.g.GS, c.g.GS, 128) + (c.g.PW + 1);
+      const uint64_t bd = DGRAD ? tc::smem_desc(sW, 128, kWLd) : tc::smem_desc(sW, kWLd, 128);
+#pragma unroll
+      for (int tap = 0; tap < 9; ++tap) {
+        const int d = (tap / 3 - 1) * c.g.PW + (tap % 3 - 1);
+#pragma unroll
+        for (int kk = 0; kk < GC / 2; ++kk)
+          tc::mma_bf16(tmem, ad[kk] + (DGRAD ? -d : d), bd + (tap * 4 * kWLd + (DGRAD ? kk * 256 : 2 * kk * kWLd)) / 16,
+                       idesc, (tap > 0 || kk > 0) ? 1u : 0u);
       }
       tc::mma_commit(&mbar);
     }
-    // The stage buffers are refilled next: wait until the MMAs have read them.
+    const int row = row3(c.g, t, t.q0 + tid);
+    uint4 m[4] = {};
+    if (DGRAD && c.mask && row >= 0) {
+      const uint4* ms = reinterpret_cast<const uint4*>(c.mask + (long long)row * kC);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) m[j] = __ldg(ms + j);
+    }
     const bool w = tc::mbar_wait(&mbar, phase & 1u, kWaitTries);
     ok = __syncthreads_and(w) != 0;
-    if (ok) ++phase;
-  }
-  tc::fence_after_sync();
-  const int row = blockIdx.x * 128 + warp * 32 + lane;
-  if (!ok) {
-    // give the MMAs in flight one more bounded chance to land before TMEM is freed
-    tc::mbar_wait(&mbar, phase & 1u, kWaitTries);
-    if (tid == 0) atomicExch(err, 1);
-  } else if (k_begin < k_end) {
-    // Epilogue: warp w holds TMEM lanes (rows) 32 w .. 32 w + 31.
+    if (!ok) break;
+    ++phase;
+    tc::fence_after_sync();
     float acc[N];
 #pragma unroll
     for (int c0 = 0; c0 < N; c0 += 16) {
@@ -291,60 +284,166 @@ __global__ void __launch_bounds__(128) k_gemm(Layer L, int rows, int kdim, int c
 #pragma unroll
       for (int i = 0; i < 16; ++i) acc[c0 + i] = v[i];
     }
-    if (row < rows) {
-      if (MODE == FWD) {
-        if (L.y32) {
+    if (row < 0) continue;
+    if (!DGRAD && c.y32) {
 #pragma unroll
-          for (int c = 0; c < N; ++c) L.y32[(long long)row * N + c] = acc[c] + __ldg(L.bias + c);
-        } else {
-          uint32_t u[N / 2];
-#pragma unroll
-          for (int c = 0; c < N; c += 2) {
-            float a = acc[c] + __ldg(L.bias + c), b = acc[c + 1] + __ldg(L.bias + c + 1);
-            if (L.relu) {
-              a = fmaxf(a, 0.f);
-              b = fmaxf(b, 0.f);
-            }
-            u[c / 2] = pack2(a, b);
-          }
-          uint4* dst = reinterpret_cast<uint4*>(L.y + (long long)row * N);
-#pragma unroll
-          for (int j = 0; j < N / 8; ++j) dst[j] = make_uint4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
-        }
-      } else if (MODE == DGRAD) {
-        uint4 m[4] = {};
-        if (L.mask) {
-          const uint4* ms = reinterpret_cast<const uint4*>(L.mask + (long long)row * kC);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) m[j] = ms[j];
-        }
-        const uint32_t* mw = reinterpret_cast<const uint32_t*>(m);
-        uint32_t u[16];
-#pragma unroll
-        for (int c = 0; c < 32; c += 2) {
-          float a = acc[c], b = acc[c + 1];
-          if (L.mask) {
-            if (!(bf_lo(mw[c / 2]) > 0.f)) a = 0.f;
-            if (!(bf_hi(mw[c / 2]) > 0.f)) b = 0.f;
-          }
-          u[c / 2] = pack2(a, b);
-        }
-        uint4* dst = reinterpret_cast<uint4*>(L.gx + (long long)row * kC);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) dst[j] = make_uint4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
-      } else {
-        float* out = L.wpart + ((long long)blockIdx.y * rows + row) * N;
-#pragma unroll
-        for (int c = 0; c < N; ++c) out[c] = acc[c];
-      }
+      for (int i = 0; i < N; i += 4)
+        *reinterpret_cast<float4*>(c.y32 + (long long)row * N + i) =
+            make_float4(acc[i] + __ldg(c.bias + i), acc[i + 1] + __ldg(c.bias + i + 1),
+                        acc[i + 2] + __ldg(c.bias + i + 2), acc[i + 3] + __ldg(c.bias + i + 3));
+      continue;
     }
-  } else if (MODE == WGRAD && row < rows) {
-    float* out = L.wpart + ((long long)blockIdx.y * rows + row) * N;
-    for (int c = 0; c < N; ++c) out[c] = 0.f;
+    const uint32_t* mw = reinterpret_cast<const uint32_t*>(m);
+    uint32_t u[N / 2];
+#pragma unroll
+    for (int i = 0; i < N; i += 2) {
+      float a = acc[i], b = acc[i + 1];
+      if (!DGRAD) {
+        a = fmaxf(a + __ldg(c.bias + i), 0.f);
+        b = fmaxf(b + __ldg(c.bias + i + 1), 0.f);
+      } else if (c.mask) {
+        if (!(bf_lo(mw[i / 2]) > 0.f)) a = 0.f;
+        if (!(bf_hi(mw[i / 2]) > 0.f)) b = 0.f;
+      }
+      u[i / 2] = pack2(a, b);
+    }
+    uint4* dst = reinterpret_cast<uint4*>(c.y + (long long)row * N);
+#pragma unroll
+    for (int j = 0; j < N / 8; ++j) dst[j] = make_uint4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
+  }
+  if (!ok) {
+    // give the MMAs in flight one more bounded chance to land before TMEM is freed
+    tc::mbar_wait(&mbar, phase & 1u, kWaitTries);
+    if (tid == 0) atomicExch(err, 1);
   }
   tc::fence_before_sync();
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 32);
+}
+
+// 128 zero-bordered positions of [B H W][8 G] without halo, zero where the
+// position is no output: a contraction over positions must not see the border.
+template <int G>
+__device__ __forceinline__ void load_rows3(const Grid3& g, const Tile3& t, const __nv_bfloat16* __restrict__ x,
+                                           uint32_t dst) {
+  for (int i = threadIdx.x; i < 128 * G; i += 128) {
+    const int p = i / G, gr = i - p * G;
+    const int r = row3(g, t, t.q0 + p);
+    cp_async16(dst + gr * kRowTile + p * 16, x + (long long)max(r, 0) * (8 * G) + gr * 8, r >= 0);
+  }
+}
+
+// `bytes` of BF16 ones: as the channel group behind an input's four they make
+// the bias gradient column 32 of the weight gradient's product (N = 48; the
+// columns of the group after that hold any bits and are not read).
+__device__ __forceinline__ void fill_ones(unsigned char* p, int bytes) {
+  for (int i = threadIdx.x * 16; i < bytes; i += 128 * 16)
+    *reinterpret_cast<uint4*>(p + i) = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
+}
+
+// The MMAs read 128 rows of an MN-major operand of 16 or 32: rows past the
+// channel count come from the shared memory behind it (any bits: they only
+// enter accumulator rows that nothing reads), which must exist.
+constexpr int kMnSpan = 16 * kRowTile;
+
+// First accumulator column of a tap: 32 each, the centre's last, followed by
+// the bias column.
+__device__ __forceinline__ int wgrad3_col(int tap) { return tap < 4 ? tap * 32 : (tap > 4 ? (tap - 1) * 32 : 256); }
+
+struct Wgrad3 {
+  Grid3 g;
+  const __nv_bfloat16* x[4];   // each layer's input [B H W][32]
+  const __nv_bfloat16* gy[4];  // gradient of its output before the activation [B H W][32] (the last layer: [16])
+  int off[4];                  // its place in a block's sums
+  float* part;                 // sums of block b at part + b stride: per layer [cout][288], then [cout] of the bias
+  long long stride;
+};
+
+// Weight and bias gradients of the 3 x 3 layers (blockIdx.y the layer):
+// D_tap[co][cin] += sum over the tile's positions of gy[q][co] x[q + tap][cin],
+// both operands MN-major (K = positions), the accumulators and the bias column
+// in tensor memory over all tiles of the block, written once at the end.  One
+// block per SM (512 TMEM columns), so the four layers share one launch of at
+// most one block per SM: a quarter of the partial sums of a launch per layer.
+// Bound by latency; it replaces a GEMM whose operands
+// were gathered two bytes at a time and which ran few blocks of 64 serial
+// steps (1.0-1.2 ms per layer at 32 images of 481x321, v = 15, against 26.5 us
+// for the four layers).
+template <int GC>
+__device__ __forceinline__ void wgrad3_layer(const Wgrad3& c, int layer, int* err) {
+  extern __shared__ __align__(128) unsigned char smem3[];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tmem_sh;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const uint32_t sG = tc::smem_u32(smem3), sX = sG + GC * kRowTile;
+  if (warp == 0) {
+    tc::tmem_alloc(&tmem_sh, 512);
+    tc::tmem_relinquish();
+  }
+  if (tid == 0) tc::mbar_init(&mbar, 1);
+  fill_ones(smem3 + GC * kRowTile + 4 * c.g.GS, c.g.GS);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = tmem_sh;
+  constexpr uint32_t id32 = tc::idesc_bf16_f32(128, 32) | tc::kTransA | tc::kTransB;
+  constexpr uint32_t id48 = tc::idesc_bf16_f32(128, 48) | tc::kTransA | tc::kTransB;
+  bool ok = true;
+  uint32_t phase = 0;
+  for (int tile = blockIdx.x; tile < c.g.tiles; tile += gridDim.x) {
+    const Tile3 t = tile3_at(c.g, tile);
+    load_rows3<GC>(c.g, t, c.gy[layer], sG);
+    load_halo<4>(c.g, t, c.x[layer], sX);
+    cp_async_wait_all();
+    tc::fence_async_smem();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after_sync();
+      const bool first = tile == int(blockIdx.x);
+      const uint64_t a0 = tc::smem_desc(sG, 128, kRowTile), b0 = tc::smem_desc(sX, 128, c.g.GS) + (c.g.PW + 1);
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint64_t ad = a0 + kk * 16;
+        const uint32_t acc = first && kk == 0 ? 0u : 1u;
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+          const int d = (tap / 3 - 1) * c.g.PW + (tap % 3 - 1);
+          tc::mma_bf16(tmem + wgrad3_col(tap), ad, b0 + (d + kk * 16), tap == 4 ? id48 : id32, acc);
+        }
+      }
+      tc::mma_commit(&mbar);
+    }
+    const bool w = tc::mbar_wait(&mbar, phase & 1u, kWaitTries);  // the tiles are refilled next
+    ok = __syncthreads_and(w) != 0;
+    if (!ok) break;
+    ++phase;
+  }
+  tc::fence_after_sync();
+  if (!ok) {
+    tc::mbar_wait(&mbar, phase & 1u, kWaitTries);
+    if (tid == 0) atomicExch(err, 1);
+  } else if (warp == 0) {  // accumulator row = output channel = lane
+    float* out = c.part + blockIdx.x * c.stride + c.off[layer];
+    for (int c0 = 0; c0 <= 288; c0 += 16) {
+      float v[16];
+      tc::tmem_ld16(tmem + uint32_t(c0), v);
+      if (tid >= 8 * GC) continue;
+      if (c0 == 288) {
+        out[8 * GC * 288 + tid] = v[0];
+      } else {
+        const int j = c0 >> 5, tap = j < 4 ? j : (j < 8 ? j + 1 : 4);
+        float4* o = reinterpret_cast<float4*>(out + tid * 288 + tap * 32 + (c0 & 16));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+__global__ void __launch_bounds__(128) k_wgrad3(Wgrad3 c, int* err) {
+  if (blockIdx.y == 3) wgrad3_layer<2>(c, 3, err);
+  else wgrad3_layer<4>(c, blockIdx.y, err);
 }
 
 // ------------------------------------------------------------------ k_pix
@@ -365,7 +464,8 @@ struct PixArgs {
   const __nv_bfloat16* w2;
   const float* b2;
   __nv_bfloat16* c0;            // [cells][32]
-  __nv_bfloat16 *x0, *h1, *h2;  // training: [blocks 128][32], or null
+  __nv_bfloat16 *x0, *h1;       // training: [blocks 128][32]
+  uint32_t* h2;                 // training: bit c of row r set where h2 > 0
   int* err;
 };
 
@@ -393,6 +493,8 @@ static_assert(128 * kPoolLd * 4 <= kPixSmem, "pooling buffer");
 // conversion kernels' own table code, so that both give the same bits).
 __global__ void k_srgb_table(float* lin) { build_srgb_table(lin); }
 
+// TRAIN: x0, h1 and the signs of h2 are kept for the backward pass.
+template <bool TRAIN>
 __global__ void __launch_bounds__(128, kPixMinBlocks) k_pix(PixArgs a) {
   __shared__ __align__(1024) unsigned char smem[kPixSmem];
   __shared__ __align__(8) uint64_t mbar;
@@ -522,7 +624,7 @@ __global__ void __launch_bounds__(128, kPixMinBlocks) k_pix(PixArgs a) {
   for (int j = 0; j < 4; ++j) {
     const uint4 v4 = make_uint4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
     *reinterpret_cast<uint4*>(sA + tc::tile_offset(row_in, 8 * j, kC)) = v4;
-    if (a.x0) reinterpret_cast<uint4*>(a.x0 + ((long long)blockIdx.x * 128 + row_in) * kC)[j] = v4;
+    if (TRAIN) reinterpret_cast<uint4*>(a.x0 + ((long long)blockIdx.x * 128 + row_in) * kC)[j] = v4;
   }
   tc::fence_async_smem();
   tc::fence_before_sync();
@@ -561,12 +663,18 @@ __global__ void __launch_bounds__(128, kPixMinBlocks) k_pix(PixArgs a) {
       const float e1 = valid ? fmaxf(acc[2 * i + 1] + __ldg(bias + 2 * i + 1), 0.f) : 0.f;
       u[i] = pack2(e0, e1);
     }
-    __nv_bfloat16* store = layer == 0 ? a.h1 : a.h2;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
+      if (layer == 1) break;
       const uint4 v4 = make_uint4(u[4 * j], u[4 * j + 1], u[4 * j + 2], u[4 * j + 3]);
-      if (layer == 0) *reinterpret_cast<uint4*>(sA + tc::tile_offset(tid, 8 * j, kC)) = v4;
-      if (store) reinterpret_cast<uint4*>(store + ((long long)blockIdx.x * 128 + tid) * kC)[j] = v4;
+      *reinterpret_cast<uint4*>(sA + tc::tile_offset(tid, 8 * j, kC)) = v4;
+      if (TRAIN) reinterpret_cast<uint4*>(a.h1 + ((long long)blockIdx.x * 128 + tid) * kC)[j] = v4;
+    }
+    if (TRAIN && layer == 1) {  // the backward pass needs only where h2 > 0
+      uint32_t m = 0;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) m |= (bf_lo(u[i]) > 0.f ? 1u : 0u) << (2 * i) | (bf_hi(u[i]) > 0.f ? 1u : 0u) << (2 * i + 1);
+      a.h2[(long long)blockIdx.x * 128 + tid] = m;
     }
     if (layer == 0) {
       tc::fence_async_smem();
@@ -607,27 +715,184 @@ __global__ void __launch_bounds__(128, kPixMinBlocks) k_pix(PixArgs a) {
   if (warp == 0) tc::tmem_dealloc(tmem, 32);
 }
 
-// ------------------------------------------------------------ elementwise
-// Gradient of the pre-activation of h2 from the gradient of c0 (average
-// pooling, then the ReLU of h2): g[row] = g_c0[cell(row)] / f^2 where h2 > 0,
-// for the pooled channels (channels kStartCh.. are the start pixel's inputs).
-__global__ void k_pool_bwd(const __nv_bfloat16* __restrict__ gc0, const __nv_bfloat16* __restrict__ h2,
-                           long long nrows, int cpb, int ff, long long cells, __nv_bfloat16* __restrict__ g) {
-  const float inv = 1.f / float(ff);
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nrows * kC;
-       i += (long long)gridDim.x * blockDim.x) {
-    const long long row = i >> 5;
-    const int ch = int(i & 31);
-    const long long blk = row >> 7;
-    const int lc = int(row & 127) / ff;
-    const long long cell = blk * cpb + lc;
-    float v = 0.f;
-    if (lc < cpb && cell < cells && ch < kStartCh && __bfloat162float(h2[i]) > 0.f)
-      v = __bfloat162float(gc0[cell * kC + ch]) * inv;
-    g[i] = __float2bfloat16(v);
+// --------------------------------------------------------------- k_pix_bwd
+struct PixBwd {
+  const __nv_bfloat16* gc0;           // gradient of c0 [cells][32]
+  const __nv_bfloat16 *x0, *h1;       // saved by k_pix: [blocks 128][32]
+  const uint32_t* h2;                 // saved by k_pix: bit c of row r set where h2 > 0
+  const __nv_bfloat16* w2;            // [32][32]
+  int blocks, cells, cpb, ff;         // row blocks of k_pix, superpixels, cells per block, patches per cell
+  unsigned rff;                       // floor(2^32 / ff) + 1: p / ff = umulhi(p, rff) for a row p < 128 (ff > 1)
+  float* part;                        // block b's sums at part + b stride: W1, b1, W2, b2 as in the parameters
+  long long stride;
+};
+constexpr int kPixTile = 4 * kRowTile;  // 128 rows x 32 channels
+// g2, g1, h1 and its ones, x0 and its ones, W2
+constexpr int kPixBwdH1 = 2 * kPixTile, kPixBwdX0 = kPixBwdH1 + kPixTile + kRowTile,
+              kPixBwdW = kPixBwdX0 + kPixTile + kRowTile;
+constexpr int kPixBwdCols = 128;        // accumulators: W2 and b2 48, W1 and b1 48, data gradient 32
+constexpr int kPixBwdPerSm = 4;         // resident blocks: 4 x 128 TMEM columns, and no fifth by shared memory
+constexpr int kPixBwdSmem = 46 * 1024;
+static_assert(kPixBwdW + 4 * kWLd <= kPixBwdSmem && kPixTile + kMnSpan <= kPixBwdSmem, "shared memory");
+static_assert(kPixBwdX0 + 6 * kRowTile <= kPixBwdSmem, "shared memory");
+
+// Backward pass of the pixel level over the 128-row blocks of k_pix:
+//   g2 = gradient of c0 / f^2 where h2 > 0 (average pooling, ReLU; channels
+//        kStartCh.. of c0 are inputs), BF16
+//   W2 += g2^T h1, b2 += g2^T 1, g1 = (g2 W2 where h1 > 0), BF16
+//   W1 += g1^T x0, b1 += g1^T 1
+// with g2 and g1 in shared memory only.  A tile of rows lies as in the 3 x 3
+// layers (groups of 8 channels, 16 bytes per row), so that g2 is the K-major
+// operand of the data gradient and the MN-major one of the weight gradient.
+// The weight gradients stay in tensor memory over the block's tiles.
+// Bound by the latency of a tile's steps (load, MMA, mask, MMA) at four blocks
+// per SM (128 TMEM columns, 46 KB each); the loads of the next tile are in
+// flight, in registers, during the MMAs of this one.  At 32 images of
+// 481x321, v = 15: 29 us (48 us without loading ahead), 74 MB read, in place
+// of a pooling pass (59 us), a data gradient and two weight-gradient GEMMs
+// (2.5 ms) that read g2 and g1 four times from memory.
+__global__ void __launch_bounds__(128, kPixBwdPerSm) k_pix_bwd(PixBwd a, int* err) {
+  extern __shared__ __align__(128) unsigned char smem3[];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tmem_sh;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  unsigned char *pG2 = smem3, *pG1 = smem3 + kPixTile, *pH1 = smem3 + kPixBwdH1, *pX0 = smem3 + kPixBwdX0;
+  const uint32_t sG2 = tc::smem_u32(pG2), sG1 = sG2 + kPixTile, sH1 = sG2 + kPixBwdH1, sX0 = sG2 + kPixBwdX0,
+                 sW = sG2 + kPixBwdW;
+  if (warp == 0) {
+    tc::tmem_alloc(&tmem_sh, kPixBwdCols);
+    tc::tmem_relinquish();
   }
+  if (tid == 0) tc::mbar_init(&mbar, 1);
+  fill_ones(pH1 + kPixTile, kRowTile);
+  fill_ones(pX0 + kPixTile, kRowTile);
+  cp_async16(sW + (tid & 3) * kWLd + (tid >> 2) * 16, a.w2 + (tid >> 2) * kC + (tid & 3) * 8, true);
+  cp_async_wait_all();
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tW2 = tmem_sh, tW1 = tW2 + 48, tD = tW2 + 96;
+  constexpr uint32_t idD = tc::idesc_bf16_f32(128, 32) | tc::kTransB;
+  constexpr uint32_t id48 = tc::idesc_bf16_f32(128, 48) | tc::kTransA | tc::kTransB;
+  const float inv = 1.f / float(a.ff);
+  bool ok = true;
+  uint32_t phase = 0;
+  // a tile's loads, held in registers from the previous tile's MMAs on
+  uint4 xv[4], hv[4], gv[4];
+  uint32_t h2[4];
+  auto load = [&](int b) {
+    const long long r0 = (long long)b * 128;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = tid + 128 * j, p = i >> 2, gr = i & 3;
+      const int lc = a.ff == 1 ? p : int(__umulhi(unsigned(p), a.rff)), cell = b * a.cpb + lc;
+      const bool in = lc < a.cpb && cell < a.cells;
+      hv[j] = __ldg(reinterpret_cast<const uint4*>(a.h1 + r0 * kC) + i);
+      xv[j] = __ldg(reinterpret_cast<const uint4*>(a.x0 + r0 * kC) + i);
+      h2[j] = in ? __ldg(a.h2 + r0 + p) : 0u;
+      gv[j] = in ? __ldg(reinterpret_cast<const uint4*>(a.gc0 + (long long)cell * kC + gr * 8)) : make_uint4(0, 0, 0, 0);
+    }
+  };
+  load(blockIdx.x);  // blockIdx.x < a.blocks
+  for (int b = blockIdx.x; b < a.blocks; b += gridDim.x) {
+    const uint32_t acc0 = b == int(blockIdx.x) ? 0u : 1u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = tid + 128 * j, p = i >> 2, gr = i & 3;
+      *reinterpret_cast<uint4*>(pH1 + gr * kRowTile + p * 16) = hv[j];
+      *reinterpret_cast<uint4*>(pX0 + gr * kRowTile + p * 16) = xv[j];
+      uint32_t m = h2[j] >> (gr * 8);
+      if (gr == 3) m &= (1u << (kStartCh - 24)) - 1u;  // channels kStartCh.. are inputs
+      const uint32_t* gw = reinterpret_cast<const uint32_t*>(&gv[j]);
+      uint32_t u[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        u[k] = pack2((m >> (2 * k)) & 1u ? bf_lo(gw[k]) * inv : 0.f, (m >> (2 * k + 1)) & 1u ? bf_hi(gw[k]) * inv : 0.f);
+      *reinterpret_cast<uint4*>(pG2 + gr * kRowTile + p * 16) = make_uint4(u[0], u[1], u[2], u[3]);
+    }
+    if (b + int(gridDim.x) < a.blocks) load(b + gridDim.x);
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after_sync();
+#pragma unroll
+      for (int kk = 0; kk < 2; ++kk)
+        tc::mma_bf16(tD, tc::smem_desc(sG2 + 2 * kk * kRowTile, kRowTile, 128), tc::smem_desc(sW + kk * 256, 128, kWLd),
+                     idD, kk);
+      tc::mma_commit(&mbar);
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint64_t ad = tc::smem_desc(sG2 + kk * 256, 128, kRowTile);
+        tc::mma_bf16(tW2, ad, tc::smem_desc(sH1 + kk * 256, 128, kRowTile), id48, kk ? 1u : acc0);
+      }
+    }
+    bool w = tc::mbar_wait(&mbar, phase & 1u, kWaitTries);
+    ok = __syncthreads_and(w) != 0;
+    if (!ok) break;
+    ++phase;
+    tc::fence_after_sync();
+    // g1 of row tid: the data gradient where h1 > 0
+    float d[32];
+#pragma unroll
+    for (int c0 = 0; c0 < 32; c0 += 16) {
+      float v[16];
+      tc::tmem_ld16(tD + (uint32_t(warp * 32) << 16) + uint32_t(c0), v);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) d[c0 + i] = v[i];
+    }
+#pragma unroll
+    for (int gr = 0; gr < 4; ++gr) {
+      const uint4 m = *reinterpret_cast<const uint4*>(pH1 + gr * kRowTile + tid * 16);
+      const uint32_t* mw = reinterpret_cast<const uint32_t*>(&m);
+      uint32_t u[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        u[k] = pack2(bf_lo(mw[k]) > 0.f ? d[gr * 8 + 2 * k] : 0.f, bf_hi(mw[k]) > 0.f ? d[gr * 8 + 2 * k + 1] : 0.f);
+      *reinterpret_cast<uint4*>(pG1 + gr * kRowTile + tid * 16) = make_uint4(u[0], u[1], u[2], u[3]);
+    }
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after_sync();
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint64_t ad = tc::smem_desc(sG1 + kk * 256, 128, kRowTile);
+        tc::mma_bf16(tW1, ad, tc::smem_desc(sX0 + kk * 256, 128, kRowTile), id48, kk ? 1u : acc0);
+      }
+      tc::mma_commit(&mbar);
+    }
+    w = tc::mbar_wait(&mbar, phase & 1u, kWaitTries);  // the tiles are refilled next
+    ok = __syncthreads_and(w) != 0;
+    if (!ok) break;
+    ++phase;
+  }
+  tc::fence_after_sync();
+  if (!ok) {
+    tc::mbar_wait(&mbar, phase & 1u, kWaitTries);
+    if (tid == 0) atomicExch(err, 1);
+  } else if (warp == 0) {  // accumulator row = output channel = lane
+    float* out = a.part + blockIdx.x * a.stride;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      float* o = out + l * (kC * kC + kC);
+      for (int c0 = 0; c0 < 32; c0 += 16) {
+        float v[16];
+        tc::tmem_ld16((l ? tW2 : tW1) + uint32_t(c0), v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          reinterpret_cast<float4*>(o + tid * kC + c0)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+      }
+      float v[16];
+      tc::tmem_ld16((l ? tW2 : tW1) + 32u, v);
+      o[kC * kC + tid] = v[0];
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc(tW2, kPixBwdCols);
 }
 
+// ------------------------------------------------------------ elementwise
 // Mean squared error over the used outputs: gradient (BF16) into g, per-block
 // sums of squares (FP64) into lpart.
 __global__ void __launch_bounds__(256) k_loss(const float* __restrict__ out, const float* __restrict__ target,
@@ -657,22 +922,42 @@ __global__ void __launch_bounds__(256) k_loss(const float* __restrict__ out, con
   if (threadIdx.x == 0) lpart[blockIdx.x] = red[0];
 }
 
-// Sum of the weight-gradient partials over the splits (fixed order): row
-// t 32 + c -> gw[cout][t 32 + c], the last row -> gb[cout].
-__global__ void k_wgrad_reduce(const float* __restrict__ part, int splits, int rows, int cout,
-                               float* __restrict__ gw, float* __restrict__ gb) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows * cout; i += gridDim.x * blockDim.x) {
-    const int r = i / cout, c = i - r * cout;
-    float s = 0.f;
-    for (int sp = 0; sp < splits; ++sp) s += part[((long long)sp * rows + r) * cout + c];
-    if (r == rows - 1) gb[c] = s;
-    else gw[(long long)c * (rows - 1) + r] = s;
+// Sum of the blocks' weight-gradient partials (rows in parameter order; a
+// fixed order: G interleaved sums, then those in turn).  A block of 256
+// threads takes 256 / G parameters, thread (g, l) rows g, g + G, ...
+template <int G>
+__device__ __forceinline__ void reduce_rows(const float* __restrict__ p, int rows, int stride, int i0,
+                                            float* __restrict__ out) {
+  constexpr int L = 256 / G;
+  __shared__ float red[G][L + 1];
+  const int l = threadIdx.x % L, g = threadIdx.x / L, i = i0 + l;
+  float s = 0.f;
+  if (i < stride) {
+#pragma unroll 4
+    for (int r = g; r < rows; r += G) s += __ldg(p + (long long)r * stride + i);
   }
+  red[g][l] = s;
+  __syncthreads();
+  if (g == 0 && i < stride) {
+#pragma unroll
+    for (int k = 1; k < G; ++k) s += red[k][l];
+    out[i] = s;
+  }
+}
+// The first `split` parameters (the pixel level's) over n0 rows of p0: up to
+// 608 of them, whose chain of loads sets the time, so 32 sums per parameter;
+// the others over n1 <= 38 rows of p1, 8 sums per parameter.
+__global__ void __launch_bounds__(256) k_grad_reduce(const float* __restrict__ p0, int n0, int split,
+                                                     const float* __restrict__ p1, int n1, int total,
+                                                     float* __restrict__ grad) {
+  const int first = (split + 7) / 8;
+  if (int(blockIdx.x) < first) reduce_rows<32>(p0, n0, split, blockIdx.x * 8, grad);
+  else reduce_rows<8>(p1, n1, total - split, (blockIdx.x - first) * 32, grad + split);
 }
 
 // Adam (Kingma and Ba, 2015) on the FP32 master weights; refreshes the BF16 copy.
 __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, __nv_bfloat16* __restrict__ wb, int n, float lr, float b1,
+                       const float* __restrict__ g, BfParams wb, int n, float lr, float b1,
                        float b2, float eps, float c1, float c2) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -682,13 +967,13 @@ __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __re
     v[i] = vi;
     const float wi = w[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
     w[i] = wi;
-    wb[i] = __float2bfloat16(wi);
+    store_bf16(wb, i, wi);
   }
 }
 
-__global__ void k_to_bf16(const float* __restrict__ a, __nv_bfloat16* __restrict__ b, int n) {
+__global__ void k_to_bf16(const float* __restrict__ a, BfParams b, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    b[i] = __float2bfloat16(a[i]);
+    store_bf16(b, i, a[i]);
 }
 
 // Targets from fitted parameters of B images of geometry g (theta and the
@@ -832,18 +1117,22 @@ struct gmmsp_net_s {
   void* pslab = nullptr;  // parameters, Adam state, gradients, error word
   float *w32 = nullptr, *m = nullptr, *vv = nullptr, *grad = nullptr;
   __nv_bfloat16* wbf = nullptr;
+  unsigned char* wst = nullptr;  // the 3 x 3 layers' weights as the kernels stage them
   int* err = nullptr;
   float* srgb = nullptr;  // the converting mode's sRGB table
   long long adam_t = 0;
+  int sms = 152;          // SMs of the device
   // workspace (grown on demand, never during stream capture)
   void* wslab = nullptr;
   long long cap_cells = 0;
   bool cap_train = false;
   long long generation = 0;
   __nv_bfloat16* c[4] = {};
-  __nv_bfloat16 *x0 = nullptr, *h1 = nullptr, *h2 = nullptr, *gp0 = nullptr, *gp1 = nullptr, *gout = nullptr;
-  __nv_bfloat16* gc[2] = {};
-  float *out = nullptr, *wpart = nullptr;
+  __nv_bfloat16 *x0 = nullptr, *h1 = nullptr, *gout = nullptr;
+  uint32_t* h2 = nullptr;
+  __nv_bfloat16* gc[4] = {};
+  float *out = nullptr;
+  float *wpart0 = nullptr, *wpart1 = nullptr;  // weight-gradient partials per block: layers 0-1, layers 2-5
   double* lpart = nullptr;
   long long last_cells = 0;  // superpixels of the last forward pass
   std::string msg;
@@ -865,6 +1154,15 @@ gmmsp_status nfail(gmmsp_net n, gmmsp_status s, const std::string& m) {
       return nfail((n), e_ == cudaErrorMemoryAllocation ? GMMSP_E_NOMEM : GMMSP_E_CUDA, \
                    std::string(#call) + ": " + cudaGetErrorString(e_));                \
   } while (0)
+
+BfParams bf_params(gmmsp_net n) {
+  BfParams p{n->wbf, n->wst, {}, {}};
+  for (int l = 0; l < 4; ++l) {
+    p.w[l] = n->pl.w[l + 2];
+    p.n[l] = n->pl.cout[l + 2] * 288;
+  }
+  return p;
+}
 
 long long nblocks_of(gmmsp_net n, long long cells) { return (cells + n->cpb - 1) / n->cpb; }
 
@@ -891,21 +1189,18 @@ gmmsp_status reserve(gmmsp_net n, long long cells, bool train) {
   if (cudaStreamIsCapturing(n->stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone)
     return nfail(n, GMMSP_E_STATE, "network workspace must be reserved before stream capture");
   const long long nrows = nblocks_of(n, cells) * 128;
-  const long long splits_pix = (nrows + kChunk - 1) / kChunk;
-  const long long splits_cell = (cells + kChunk - 1) / kChunk;
-  const size_t wpart = size_t(std::max(splits_pix * (kC + 1), splits_cell * (9 * kC + 1))) * kC * sizeof(float);
   const size_t act = up256(size_t(cells) * kC * 2);
   const size_t pix = up256(size_t(nrows) * kC * 2);
   size_t off = 0;
   const size_t o_c = off;   off += 4 * act;
   const size_t o_out = off; off += up256(size_t(cells) * kOut * sizeof(float));
-  size_t o_x0 = 0, o_gp0 = 0, o_gout = 0, o_gc = 0, o_wp = 0, o_lp = 0;
+  size_t o_x0 = 0, o_gout = 0, o_gc = 0, o_wp0 = 0, o_wp1 = 0, o_lp = 0;
   if (train) {
-    o_x0 = off;   off += 3 * pix;  // x0, h1, h2
-    o_gp0 = off;  off += 2 * pix;  // gp0, gp1
+    o_x0 = off;   off += 2 * pix + up256(size_t(nrows) * 4);  // x0, h1, the bits of h2
     o_gout = off; off += up256(size_t(cells) * kOut * 2);
-    o_gc = off;   off += 2 * act;
-    o_wp = off;   off += up256(wpart);
+    o_gc = off;   off += 4 * act;
+    o_wp0 = off;  off += up256(size_t(n->sms) * kPixBwdPerSm * pix_params(n->pl) * sizeof(float));
+    o_wp1 = off;  off += up256(size_t(std::max(1, n->sms / 4)) * (n->pl.total - pix_params(n->pl)) * sizeof(float));
     o_lp = off;   off += up256(kLossBlocks * sizeof(double));
   }
   if (n->wslab) {
@@ -925,17 +1220,17 @@ gmmsp_status reserve(gmmsp_net n, long long cells, bool train) {
   if (train) {
     n->x0 = reinterpret_cast<__nv_bfloat16*>(b + o_x0);
     n->h1 = reinterpret_cast<__nv_bfloat16*>(b + o_x0 + pix);
-    n->h2 = reinterpret_cast<__nv_bfloat16*>(b + o_x0 + 2 * pix);
-    n->gp0 = reinterpret_cast<__nv_bfloat16*>(b + o_gp0);
-    n->gp1 = reinterpret_cast<__nv_bfloat16*>(b + o_gp0 + pix);
+    n->h2 = reinterpret_cast<uint32_t*>(b + o_x0 + 2 * pix);
     n->gout = reinterpret_cast<__nv_bfloat16*>(b + o_gout);
-    n->gc[0] = reinterpret_cast<__nv_bfloat16*>(b + o_gc);
-    n->gc[1] = reinterpret_cast<__nv_bfloat16*>(b + o_gc + act);
-    n->wpart = reinterpret_cast<float*>(b + o_wp);
+    for (int i = 0; i < 4; ++i) n->gc[i] = reinterpret_cast<__nv_bfloat16*>(b + o_gc + i * act);
+    n->wpart0 = reinterpret_cast<float*>(b + o_wp0);
+    n->wpart1 = reinterpret_cast<float*>(b + o_wp1);
     n->lpart = reinterpret_cast<double*>(b + o_lp);
   } else {
-    n->x0 = n->h1 = n->h2 = n->gp0 = n->gp1 = n->gout = n->gc[0] = n->gc[1] = nullptr;
-    n->wpart = nullptr;
+    n->x0 = n->h1 = n->gout = nullptr;
+    for (auto& p : n->gc) p = nullptr;
+    n->h2 = nullptr;
+    n->wpart0 = n->wpart1 = nullptr;
     n->lpart = nullptr;
   }
   n->cap_cells = cells;
@@ -943,17 +1238,16 @@ gmmsp_status reserve(gmmsp_net n, long long cells, bool train) {
   return GMMSP_OK;
 }
 
-Layer cell_layer(gmmsp_net n, int B, const Geom& g, int l) {
-  Layer L{};
-  L.B = B;
-  L.H = g.ny;
-  L.W = g.nx;
-  L.taps = n->pl.taps[l];
-  L.cout = n->pl.cout[l];
-  L.relu = l < 5;
-  L.w = n->wbf + n->pl.w[l];
-  L.bias = n->w32 + n->pl.b[l];
-  return L;
+// One tile per step on as many blocks as are resident at once (shared memory
+// and the 512 TMEM columns: 16 blocks of 32), so that each stages the weights
+// once.
+template <bool DGRAD, int GC, int N>
+cudaError_t launch_conv3(gmmsp_net n, const Conv3& c, cudaStream_t s) {
+  const int smem = kWBytes + GC * c.g.GS;
+  const int per = std::max(1, std::min(16, 228 * 1024 / (smem + 2048)));
+  const unsigned blocks = unsigned(std::min(c.g.tiles, n->sms * per));
+  k_conv3<DGRAD, GC, N><<<blocks, 128, smem, s>>>(c, n->err);
+  return cudaGetLastError();
 }
 
 // Forward pass; out receives [B K][16] FP32.  Training also stores x0, h1, h2.
@@ -981,41 +1275,24 @@ gmmsp_status enqueue_forward(gmmsp_net n, const float* lab, int B, const Geom& g
   a.h1 = train ? n->h1 : nullptr;
   a.h2 = train ? n->h2 : nullptr;
   a.err = n->err;
-  k_pix<<<unsigned(nblocks_of(n, cells)), 128, 0, s>>>(a);
+  const unsigned pblocks = unsigned(nblocks_of(n, cells));
+  if (train) k_pix<true><<<pblocks, 128, 0, s>>>(a);
+  else k_pix<false><<<pblocks, 128, 0, s>>>(a);
   GN_CHECK(n, cudaGetLastError());
-  const int rows = int(cells);
-  const unsigned tiles = unsigned((rows + 127) / 128);
+  Conv3 c{};
+  c.g = grid3_of(B, g.ny, g.nx);
   for (int l = 2; l < 6; ++l) {
-    Layer L = cell_layer(n, B, g, l);
-    L.x = n->c[l - 2];
-    const int kdim = L.taps * kC;
+    c.a = n->c[l - 2];
+    c.w = n->wst + (l - 2) * kWBytes;
+    c.bias = n->w32 + n->pl.b[l];
     if (l < 5) {
-      L.y = n->c[l - 1];
-      k_gemm<FWD, 32><<<tiles, 128, 0, s>>>(L, rows, kdim, 0, n->err);
+      c.y = n->c[l - 1];
+      GN_CHECK(n, (launch_conv3<false, 4, 32>(n, c, s)));
     } else {
-      L.y32 = out;
-      k_gemm<FWD, 16><<<tiles, 128, 0, s>>>(L, rows, kdim, 0, n->err);
+      c.y32 = out;
+      GN_CHECK(n, (launch_conv3<false, 4, 16>(n, c, s)));
     }
-    GN_CHECK(n, cudaGetLastError());
   }
-  return GMMSP_OK;
-}
-
-// Weight and bias gradient of layer l from its input L.x and the gradient
-// L.gy of its pre-activation output, over `positions` positions.
-gmmsp_status enqueue_wgrad(gmmsp_net n, Layer L, int l, int positions, cudaStream_t s) {
-  const int rows = L.taps * kC + 1;
-  const unsigned tiles = unsigned((rows + 127) / 128);
-  const unsigned splits = unsigned((positions + kChunk - 1) / kChunk);
-  L.wpart = n->wpart;
-  if (L.cout == kC)
-    k_gemm<WGRAD, 32><<<dim3(tiles, splits), 128, 0, s>>>(L, rows, positions, kChunk, n->err);
-  else
-    k_gemm<WGRAD, 16><<<dim3(tiles, splits), 128, 0, s>>>(L, rows, positions, kChunk, n->err);
-  GN_CHECK(n, cudaGetLastError());
-  k_wgrad_reduce<<<grid_for(rows * L.cout, 256), 256, 0, s>>>(n->wpart, int(splits), rows, L.cout,
-                                                               n->grad + n->pl.w[l], n->grad + n->pl.b[l]);
-  GN_CHECK(n, cudaGetLastError());
   return GMMSP_OK;
 }
 
@@ -1025,47 +1302,54 @@ gmmsp_status enqueue_grad(gmmsp_net n, const float* lab, int B, const Geom& g, c
   gmmsp_status st = enqueue_forward(n, lab, B, g, n->out, true, s);
   if (st != GMMSP_OK) return st;
   const long long cells = (long long)B * g.K;
-  const int rows = int(cells);
-  const unsigned tiles = unsigned((rows + 127) / 128);
   k_loss<<<kLossBlocks, 256, 0, s>>>(n->out, target, cells, n->gout, n->lpart);
   GN_CHECK(n, cudaGetLastError());
   // the 3 x 3 layers, last to first
+  const int np0 = pix_params(n->pl), np1 = n->pl.total - np0;
+  const Grid3 g3 = grid3_of(B, g.ny, g.nx);
   const __nv_bfloat16* gy = n->gout;
+  Wgrad3 w{};
+  w.g = g3;
+  w.part = n->wpart1;
+  w.stride = np1;
   for (int l = 5; l >= 2; --l) {
-    Layer L = cell_layer(n, B, g, l);
-    L.x = n->c[l - 2];
-    L.gy = gy;
-    st = enqueue_wgrad(n, L, l, rows, s);
-    if (st != GMMSP_OK) return st;
-    L.gx = n->gc[l & 1];
-    L.mask = l > 2 ? n->c[l - 2] : nullptr;  // c0 is a pooled value with no ReLU of its own
-    k_gemm<DGRAD, 32><<<tiles, 128, 0, s>>>(L, rows, L.taps * L.cout, 0, n->err);
-    GN_CHECK(n, cudaGetLastError());
-    gy = L.gx;
+    w.x[l - 2] = n->c[l - 2];
+    w.gy[l - 2] = gy;
+    w.off[l - 2] = n->pl.w[l] - np0;
+    Conv3 c{};
+    c.g = g3;
+    c.a = gy;
+    c.w = n->wst + (l - 2) * kWBytes;
+    c.y = n->gc[l - 2];
+    c.mask = l > 2 ? n->c[l - 2] : nullptr;  // c0 is a pooled value with no ReLU of its own
+    if (l == 5) GN_CHECK(n, (launch_conv3<true, 2, 32>(n, c, s)));
+    else GN_CHECK(n, (launch_conv3<true, 4, 32>(n, c, s)));
+    gy = c.y;
   }
-  // pooling and the ReLU of h2, then the two 1 x 1 layers over the patch rows
-  const long long nrows = nblocks_of(n, cells) * 128;
-  k_pool_bwd<<<grid_for(nrows * kC, 256), 256, 0, s>>>(gy, n->h2, nrows, n->cpb, n->f * n->f, cells, n->gp0);
+  const unsigned wblocks = unsigned(std::min(g3.tiles, std::max(1, n->sms / 4)));
+  k_wgrad3<<<dim3(wblocks, 4), 128, std::max(kMnSpan, 4 * kRowTile + 6 * g3.GS), s>>>(w, n->err);
   GN_CHECK(n, cudaGetLastError());
-  Layer L2{};
-  L2.B = 1; L2.H = 1; L2.W = int(nrows);
-  L2.taps = 1; L2.cout = kC;
-  L2.w = n->wbf + n->pl.w[1];
-  L2.x = n->h1;
-  L2.gy = n->gp0;
-  st = enqueue_wgrad(n, L2, 1, int(nrows), s);
-  if (st != GMMSP_OK) return st;
-  L2.gx = n->gp1;
-  L2.mask = n->h1;
-  k_gemm<DGRAD, 32><<<unsigned(nrows / 128), 128, 0, s>>>(L2, int(nrows), kC, 0, n->err);
+  // the pixel level, then the sums over the blocks
+  PixBwd p{};
+  p.gc0 = gy;
+  p.x0 = n->x0;
+  p.h1 = n->h1;
+  p.h2 = n->h2;
+  p.w2 = n->wbf + n->pl.w[1];
+  p.blocks = int(nblocks_of(n, cells));
+  p.cells = int(cells);
+  p.cpb = n->cpb;
+  p.ff = n->f * n->f;
+  p.rff = unsigned((1ull << 32) / unsigned(p.ff)) + 1u;
+  p.part = n->wpart0;
+  p.stride = np0;
+  const unsigned pblocks = unsigned(std::min(p.blocks, n->sms * kPixBwdPerSm));
+  k_pix_bwd<<<pblocks, 128, kPixBwdSmem, s>>>(p, n->err);
   GN_CHECK(n, cudaGetLastError());
-  Layer L1 = L2;
-  L1.w = n->wbf + n->pl.w[0];
-  L1.x = n->x0;
-  L1.gy = n->gp1;
-  L1.gx = nullptr;
-  L1.mask = nullptr;
-  return enqueue_wgrad(n, L1, 0, int(nrows), s);
+  k_grad_reduce<<<unsigned((np0 + 7) / 8 + (np1 + 31) / 32), 256, 0, s>>>(n->wpart0, int(pblocks), np0, n->wpart1,
+                                                                 int(wblocks), n->pl.total, n->grad);
+  GN_CHECK(n, cudaGetLastError());
+  return GMMSP_OK;
 }
 
 gmmsp_status check_err(gmmsp_net n) {
@@ -1153,6 +1437,13 @@ gmmsp_status gmmsp_net_create(gmmsp_net* out, int spacing, void* stream) {
   n->cpb = 128 / (n->f * n->f);
   n->stream = static_cast<cudaStream_t>(stream);
   n->pl = param_layout();
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    delete n;
+    return GMMSP_E_CUDA;
+  }
   const size_t np = size_t(n->pl.total);
   size_t off = 0;
   const size_t o_w = off; off += up256(np * 4);
@@ -1160,6 +1451,7 @@ gmmsp_status gmmsp_net_create(gmmsp_net* out, int spacing, void* stream) {
   const size_t o_v = off; off += up256(np * 4);
   const size_t o_g = off; off += up256(np * 4);
   const size_t o_b = off; off += up256(np * 2);
+  const size_t o_s = off; off += up256(4 * kWBytes);
   const size_t o_e = off; off += 256;
   const size_t o_t = off; off += 256 * 4;
   const char* inj = getenv("GMMSP_FAIL_ALLOC");
@@ -1175,6 +1467,7 @@ gmmsp_status gmmsp_net_create(gmmsp_net* out, int spacing, void* stream) {
   n->vv = reinterpret_cast<float*>(b + o_v);
   n->grad = reinterpret_cast<float*>(b + o_g);
   n->wbf = reinterpret_cast<__nv_bfloat16*>(b + o_b);
+  n->wst = reinterpret_cast<unsigned char*>(b + o_s);
   n->err = reinterpret_cast<int*>(b + o_e);
   n->srgb = reinterpret_cast<float*>(b + o_t);
   e = cudaMemsetAsync(n->pslab, 0, off, n->stream);
@@ -1201,7 +1494,7 @@ gmmsp_status gmmsp_net_set_weights(gmmsp_net n, const float* host, long long cou
   GN_CHECK(n, cudaMemcpyAsync(n->w32, host, bytes, cudaMemcpyHostToDevice, n->stream));
   GN_CHECK(n, cudaMemsetAsync(n->m, 0, bytes, n->stream));
   GN_CHECK(n, cudaMemsetAsync(n->vv, 0, bytes, n->stream));
-  k_to_bf16<<<grid_for(count, 256), 256, 0, n->stream>>>(n->w32, n->wbf, int(count));
+  k_to_bf16<<<grid_for(count, 256), 256, 0, n->stream>>>(n->w32, bf_params(n), int(count));
   GN_CHECK(n, cudaGetLastError());
   GN_CHECK(n, cudaStreamSynchronize(n->stream));
   n->adam_t = 0;
@@ -1279,7 +1572,7 @@ gmmsp_status gmmsp_net_adam(gmmsp_net n, float lr, float beta1, float beta2, flo
   const float c1 = float(1.0 / (1.0 - pow(double(beta1), double(n->adam_t))));
   const float c2 = float(1.0 / (1.0 - pow(double(beta2), double(n->adam_t))));
   const int np = n->pl.total;
-  k_adam<<<grid_for(np, 256), 256, 0, n->stream>>>(n->w32, n->m, n->vv, n->grad, n->wbf, np, lr, beta1, beta2,
+  k_adam<<<grid_for(np, 256), 256, 0, n->stream>>>(n->w32, n->m, n->vv, n->grad, bf_params(n), np, lr, beta1, beta2,
                                                    eps, c1, c2);
   GN_CHECK(n, cudaGetLastError());
   return GMMSP_OK;

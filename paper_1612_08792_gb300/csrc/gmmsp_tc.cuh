@@ -37,7 +37,11 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
 
 // Instruction descriptor for kind::f16: FP32 accumulator (bits 4-5 = 1),
 // BF16 A and B (bits 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0),
-// N >> 3 in bits 17-22, M >> 4 in bits 24-28.
+// N >> 3 in bits 17-22, M >> 4 in bits 24-28.  Or'ed with kTransA / kTransB
+// an operand is MN-major: its core matrices hold 8 K rows of 8 consecutive
+// M (N) elements, the descriptor's leading byte offset steps along K (to the
+// next 8 rows) and its stride byte offset along M (N).
+constexpr uint32_t kTransA = 1u << 15, kTransB = 1u << 16;
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(N >> 3) << 17) | (uint32_t(M >> 4) << 24);
 }
