@@ -78,7 +78,7 @@ __device__ __forceinline__ void stage_params(const Geom& g, const Cell& c, const
 // E part for one pixel: the posteriors of its candidates (Eq. Rik) into
 // R[0..8] (zero for slots off the grid) and ln-sum-exp in log2 units into ll.
 template <bool FULL, int CM, bool DIAG = false>
-__device__ __forceinline__ void e_pixel(const float4* sp, unsigned mask, float fx, float fy, float4 z,
+__device__ __forceinline__ void e_pixel(const float4* sp, unsigned mask, const Pix2& z,
                                         float (&R)[kSlots],
                                         float& ll) {
   float m = -INFINITY;
@@ -86,7 +86,7 @@ __device__ __forceinline__ void e_pixel(const float4* sp, unsigned mask, float f
   for (int s = 0; s < kSlots; ++s) {
     R[s] = 0.f;
     if (FULL || ((mask >> s) & 1u)) {
-      R[s] = log2_density<CM, DIAG>(sp + 4 * s, fx, fy, z);
+      R[s] = log2_density<CM, DIAG>(sp + 4 * s, z);
       m = fmaxf(m, R[s]);
     }
   }
@@ -121,19 +121,38 @@ __device__ __forceinline__ void e_pixel(const float4* sp, unsigned mask, float f
 // lanes of each slot, then the WPC warps, are added through shared memory and
 // written once per cell as FP32 (no global atomics).
 //
-// Layout of the batch in shared memory: arrays of kBatchLd floats, one per
-// slot (posteriors), colour channel and coordinate, the pixel of E lane i at
-// 12 (i mod 3) + i / 3.  The pixels of one M phase are then consecutive and
-// 16-byte aligned, and an M lane reads four of its pixels per load: 18 loads
-// per batch instead of 33, about 45 wavefronts instead of 88.  Its pixels
-// keep their order, so the sums keep their bits.
+// Layout of the batch in shared memory: arrays of kBatchLd entries, one per
+// slot (posteriors), of (x, y) pairs, of (L, a) pairs and of b, the pixel of E
+// lane i at 12 (i mod 3) + i / 3.  The pixels of one M phase are then
+// consecutive and 16-byte aligned, and an M lane reads four of its pixels with
+// six loads: 18 loads per batch instead of 33, about 45 wavefronts instead of
+// 88.  Its pixels keep their order, so the sums keep their bits.
+//
+// The pass is bound by instruction issue (84 % of the cycles before the
+// following): the statistics of x and y, and of L and a, run as packed FP32
+// pairs, which takes 18 instructions per (pixel, slot) instead of 25, each
+// component rounded as before.
 constexpr int kBatchLd = 36;
-constexpr int kBatchRows = kSlots + 5;  // R[0..8], L, a, b, x, y
+constexpr int kBatchXY = kSlots * kBatchLd, kBatchLa = kBatchXY + 2 * kBatchLd, kBatchB = kBatchLa + 2 * kBatchLd,
+              kBatchFloats = kBatchB + kBatchLd;
+
+// The statistics of one slot over one lane's pixels.
+struct Acc {
+  float w = 0.f, b = 0.f, xy = 0.f, La = 0.f, Lb = 0.f, ab = 0.f, bb = 0.f;  // W, S1 b, S2 xy La Lb ab bb
+  f2 Sxy = 0, SLa = 0;  // S1 (x, y), (L, a)
+  f2 Qxy = 0, QLa = 0;  // S2 (xx, yy), (LL, aa)
+  __device__ __forceinline__ void store(float* o) const {  // in the order of the partials
+    o[0] = w;
+    o[1] = lo_f2(Sxy); o[2] = hi_f2(Sxy); o[3] = lo_f2(SLa); o[4] = hi_f2(SLa); o[5] = b;
+    o[6] = lo_f2(Qxy); o[7] = xy; o[8] = hi_f2(Qxy);
+    o[9] = lo_f2(QLa); o[10] = La; o[11] = Lb; o[12] = hi_f2(QLa); o[13] = ab; o[14] = bb;
+  }
+};
 
 template <int WPC>
 struct EmSmem {
   float4 sp[kEmWarps / WPC][kSlots * 4];            // candidate parameters per cell
-  float px[kEmWarps][kBatchRows * kBatchLd];        // the 32 pixels in flight: posteriors, colour, position
+  float px[kEmWarps][kBatchFloats];                 // the 32 pixels in flight: posteriors, colour, position
   float part[kEmWarps][kSlots * kStats + 1 + 3];    // per-warp sums (row 135: log-likelihood)
   float red[kEmWarps][27][kStats + 2];              // per-lane sums before the 3-lane add (odd row
                                                     // stride: the 27 lanes' stores hit 27 banks)
@@ -145,47 +164,55 @@ constexpr int em_smem_bytes() { return int(sizeof(EmSmem<WPC>)); }
 template <bool FULL, bool SHIFT, int WPC, class Src, int CM, bool DIAG = false>
 __device__ __forceinline__ void em_cell_warp(const Src& lab, const Geom& g, const Cell& c,
                                              EmSmem<WPC>& sm, int slot, int warp, int lane, int wic,
-                                             float (&acc)[kStats], float& ll) {
+                                             Acc& acc, float& ll) {
   const int npx = c.cw * c.ch;
   const float inv_cw = 1.f / float(c.cw);
   const float4* sp = sm.sp[slot];
   float* pw = sm.px[warp];
-  float* pe = pw + 12 * (lane % 3) + lane / 3;  // this lane's pixel in the arrays
+  const int pi = 12 * (lane % 3) + lane / 3;  // this lane's pixel in the arrays
+  float* pe = pw + pi;
   // M-part role of this lane: slot ms, pixel phase ph (lanes 27-31 idle there)
   const int ms = lane % 9, ph = lane / 9;
   const bool m_on = lane < 27 && (FULL || ((c.mask >> ms) & 1u));
-  float cx = 0.f, cy = 0.f, mL = 0.f, ma = 0.f, mb = 0.f;
+  f2 cxy, mLa = 0;
+  float mb = 0.f;
   {
     const float4 p0 = sp[4 * ms], p1 = sp[4 * ms + 1];
     // SHIFT: d_x = rx - mu_x (the staged mean, relative to this cell's origin);
     // raw moments: x relative to the candidate's cell origin, rx + (1 - ms % 3) v
-    cx = SHIFT ? -p0.x : float((1 - ms % 3) * g.v);
-    cy = SHIFT ? -p0.y : float((1 - ms / 3) * g.v);
-    if (SHIFT) { mL = p0.z; ma = p0.w; mb = p1.x; }
+    cxy = SHIFT ? pack_f2(-p0.x, -p0.y) : pack_f2(float((1 - ms % 3) * g.v), float((1 - ms / 3) * g.v));
+    if (SHIFT) {
+      mLa = pack_f2(p0.z, p0.w);
+      mb = p1.x;
+    }
   }
   auto locate = [&](int p, int& rx, int& ry) {
     ry = __float2int_rz((float(p) + 0.5f) * inv_cw);  // exact floor(p / cw)
     rx = p - ry * c.cw;
   };
   // the statistics of one (pixel, slot ms) pair with posterior r into acc
-  auto add_stats = [&](float r, float dx, float dy, float dL, float da, float db) {
-    const float rxd = r * dx, ryd = r * dy, rL = r * dL;
-    acc[0] += r;
-    acc[1] += rxd; acc[2] += ryd; acc[3] += rL;
-    acc[6] = fmaf(rxd, dx, acc[6]);
-    acc[7] = fmaf(rxd, dy, acc[7]);
-    acc[8] = fmaf(ryd, dy, acc[8]);
-    acc[9] = fmaf(rL, dL, acc[9]);
-    if constexpr (CM != kColourGray) {
-      const float ra = r * da, rb = r * db;
-      acc[4] += ra; acc[5] += rb;
+  auto add_stats = [&](float r, f2 xy, f2 La, float b) {
+    const f2 rr = pack_f2(r, r), d = add_f2(xy, cxy), rd = mul_f2(rr, d);
+    acc.w += r;
+    acc.Sxy = add_f2(acc.Sxy, rd);
+    acc.Qxy = fma_f2(rd, d, acc.Qxy);
+    acc.xy = fmaf(lo_f2(rd), hi_f2(d), acc.xy);
+    if constexpr (CM == kColourGray) {
+      const float dL = lo_f2(La) - lo_f2(mLa), rL = r * dL;
+      acc.SLa = pack_f2(lo_f2(acc.SLa) + rL, 0.f);
+      acc.QLa = pack_f2(fmaf(rL, dL, lo_f2(acc.QLa)), 0.f);
+    } else {
+      const f2 c = sub_f2(La, mLa), rc = mul_f2(rr, c);
+      const float db = b - mb, rb = r * db;
+      acc.SLa = add_f2(acc.SLa, rc);
+      acc.b += rb;
+      acc.QLa = fma_f2(rc, c, acc.QLa);
       if constexpr (CM == kColourFull) {
-        acc[10] = fmaf(rL, da, acc[10]);
-        acc[11] = fmaf(rL, db, acc[11]);
+        acc.La = fmaf(lo_f2(rc), hi_f2(c), acc.La);
+        acc.Lb = fmaf(lo_f2(rc), db, acc.Lb);
       }
-      acc[12] = fmaf(ra, da, acc[12]);
-      acc[13] = fmaf(ra, db, acc[13]);
-      acc[14] = fmaf(rb, db, acc[14]);
+      acc.ab = fmaf(hi_f2(rc), db, acc.ab);
+      acc.bb = fmaf(rb, db, acc.bb);
     }
   };
   // A cell of 32 b + 1 pixels (v = 15: 225) would end in a batch of one
@@ -201,7 +228,7 @@ __device__ __forceinline__ void em_cell_warp(const Src& lab, const Geom& g, cons
     locate(npx_b, rx, ry);
     const float4 z = load_pixel<CM>(lab, g, c.x0 + rx, c.y0 + ry);
     const bool on = lane < kSlots && (FULL || ((c.mask >> lane) & 1u));
-    const float q = on ? log2_density<CM, DIAG>(sp + 4 * (lane < kSlots ? lane : 0), float(rx), float(ry), z)
+    const float q = on ? log2_density<CM, DIAG>(sp + 4 * (lane < kSlots ? lane : 0), pix2(float(rx), float(ry), z))
                        : -INFINITY;
     float m = q;
 #pragma unroll
@@ -213,7 +240,7 @@ __device__ __forceinline__ void em_cell_warp(const Src& lab, const Geom& g, cons
     if (lane == 0) ll += m + lg2_approx(sum);
     if (on && m_on) {
       const float r = e * rcp_approx(sum);
-      add_stats(r, float(rx) + cx, float(ry) + cy, z.x - mL, z.y - ma, z.z - mb);
+      add_stats(r, pack_f2(float(rx), float(ry)), pack_f2(z.x, z.y), z.z);
     }
   }
   // The colour of this lane's next pixel is loaded one batch ahead.
@@ -235,7 +262,7 @@ __device__ __forceinline__ void em_cell_warp(const Src& lab, const Geom& g, cons
     int rx = 0, ry = 0;
     if (p < npx_b) {
       locate(p, rx, ry);
-      e_pixel<FULL, CM, DIAG>(sp, c.mask, float(rx), float(ry), z, R, ll);
+      e_pixel<FULL, CM, DIAG>(sp, c.mask, pix2(float(rx), float(ry), z), R, ll);
     } else {  // no pixel: adds r = 0 times finite values, which changes no sum
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) R[s] = 0.f;
@@ -243,29 +270,24 @@ __device__ __forceinline__ void em_cell_warp(const Src& lab, const Geom& g, cons
     }
 #pragma unroll
     for (int s = 0; s < kSlots; ++s) pe[s * kBatchLd] = R[s];
-    pe[kSlots * kBatchLd] = z.x;
-    if constexpr (CM != kColourGray) {
-      pe[(kSlots + 1) * kBatchLd] = z.y;
-      pe[(kSlots + 2) * kBatchLd] = z.z;
-    }
-    pe[(kSlots + 3) * kBatchLd] = float(rx);
-    pe[(kSlots + 4) * kBatchLd] = float(ry);
+    *reinterpret_cast<float2*>(pe + kBatchXY + pi) = make_float2(float(rx), float(ry));
+    *reinterpret_cast<float2*>(pe + kBatchLa + pi) = make_float2(z.x, z.y);
+    if constexpr (CM != kColourGray) pe[kBatchB] = z.z;
     __syncwarp();
     if (m_on) {
       // four pixels of this lane's phase (4 j .. 4 j + 3 of it)
       auto quad = [&](int j, int n) {
         const float* q = pw + 12 * ph + 4 * j;
-        auto ld = [&](int row) { return *reinterpret_cast<const float4*>(q + row * kBatchLd); };
-        const float4 r = ld(ms), x = ld(kSlots + 3), y = ld(kSlots + 4), L = ld(kSlots);
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-        if constexpr (CM != kColourGray) {
-          a = ld(kSlots + 1);
-          b = ld(kSlots + 2);
-        }
-        add_stats(r.x, x.x + cx, y.x + cy, L.x - mL, a.x - ma, b.x - mb);
-        add_stats(r.y, x.y + cx, y.y + cy, L.y - mL, a.y - ma, b.y - mb);
-        if (n > 2) add_stats(r.z, x.z + cx, y.z + cy, L.z - mL, a.z - ma, b.z - mb);
-        if (n > 3) add_stats(r.w, x.w + cx, y.w + cy, L.w - mL, a.w - ma, b.w - mb);
+        const float4 r = *reinterpret_cast<const float4*>(q + ms * kBatchLd);
+        const ulonglong2* xy = reinterpret_cast<const ulonglong2*>(pw + kBatchXY + 2 * (12 * ph + 4 * j));
+        const ulonglong2* La = reinterpret_cast<const ulonglong2*>(pw + kBatchLa + 2 * (12 * ph + 4 * j));
+        const ulonglong2 xy0 = xy[0], xy1 = xy[1], La0 = La[0], La1 = La[1];
+        float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (CM != kColourGray) b = *reinterpret_cast<const float4*>(q + kBatchB);
+        add_stats(r.x, xy0.x, La0.x, b.x);
+        add_stats(r.y, xy0.y, La0.y, b.y);
+        if (n > 2) add_stats(r.z, xy1.x, La1.x, b.z);
+        if (n > 3) add_stats(r.w, xy1.y, La1.y, b.w);
       };
       const int np = npx_b - base;  // pixels of the batch (or more)
       quad(0, 4);
@@ -290,9 +312,7 @@ __device__ __forceinline__ void em_cell_block(const Src& lab, const Geom& g, con
   }
   if (WPC == 1) __syncwarp(); else __syncthreads();
 
-  float acc[kStats];
-#pragma unroll
-  for (int j = 0; j < kStats; ++j) acc[j] = 0.f;
+  Acc acc;
   float ll = 0.f;
   if (active) {
     if (c.mask == 0x1ffu)
@@ -303,10 +323,7 @@ __device__ __forceinline__ void em_cell_block(const Src& lab, const Geom& g, con
   // Per-warp totals: add the three lanes of each slot, and the lanes' log-likelihoods.
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
-  if (lane < 27) {
-#pragma unroll
-    for (int j = 0; j < kStats; ++j) sm.red[warp][lane][j] = acc[j];
-  }
+  if (lane < 27) acc.store(sm.red[warp][lane]);
   __syncwarp();
   for (int o = lane; o < kSlots * kStats; o += 32) {
     const int s = o / kStats, j = o - s * kStats;
@@ -451,7 +468,7 @@ __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
     locate(npx, rx, ry);
     const float4 z = load_pixel<CM>(lab, g, c.x0 + rx, c.y0 + ry);
     const bool on = lane < kSlots && (FULL || ((c.mask >> lane) & 1u));
-    const float q = on ? log2_density<CM>(sp + 4 * (lane < kSlots ? lane : 0), float(rx), float(ry), z)
+    const float q = on ? log2_density<CM>(sp + 4 * (lane < kSlots ? lane : 0), pix2(float(rx), float(ry), z))
                        : -INFINITY;
     float m = q;
 #pragma unroll
@@ -500,6 +517,9 @@ __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
       }
       locate(p0 + 32 * j, rx[j], ry[j]);
     }
+    Pix2 zp[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) zp[j] = pix2(float(rx[j]), float(ry[j]), z[j]);
     float e[J][kSlots];
     float m[J];
     int best[J];
@@ -513,7 +533,7 @@ __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
       if (FULL || ((c.mask >> s) & 1u)) {
 #pragma unroll
         for (int j = 0; j < J; ++j) {
-          e[j][s] = log2_density<CM>(sp + 4 * s, float(rx[j]), float(ry[j]), z[j]);
+          e[j][s] = log2_density<CM>(sp + 4 * s, zp[j]);
           if (e[j][s] > m[j]) { m[j] = e[j][s]; best[j] = s; }
         }
       } else {
@@ -1028,8 +1048,10 @@ __device__ __forceinline__ void finalize_l16_body(const Geom& g, const float* __
   if (l == 14)
     out = -0.5f * (Num<double>::log2_(dpos(ds) ? ds : 1.0) + Num<double>::log2_(dpos(dc) ? dc : 1.0)) -
           float(Num<double>::kHalfD_Log2_2Pi);
+  // packed positions of the lanes' values (lane 15: mu_b again)
+  const float mb = __shfl_sync(kFull, out, 4, 16);
   if (live && pd) {
-    G[l] = out;
+    G[nib(0x5FBADE987C643210ull, l)] = l == 15 ? mb : out;
     // theta: [0..4] mu, [5..7] Sigma_s, [8..13] Sigma_c (= M in order)
     if (l < 14) theta[(long long)kk * kTheta + l] = (l < 5) ? mu_l : X[21 + (l - 5)];
   }

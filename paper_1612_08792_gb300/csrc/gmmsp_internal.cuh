@@ -58,13 +58,15 @@ enum : int { ST_W = 0, ST_S1 = 1, ST_S2S = 6, ST_S2C = 9 };
 // Packed FP32 E-step parameters of superpixel k (64 bytes, 16-byte aligned):
 //   [0..4]   mu (x - k_x v, y - k_y v, L, a, b): the spatial mean relative
 //            to the first pixel of the superpixel's own cell
-//   [5..7]   spatial quadratic form coefficients (xx, 2xy, yy) of
-//            -(1/2) log2(e) Sigma_s^{-1}
-//   [8..13]  colour coefficients (LL, aa, bb, 2La, 2Lb, 2ab) of
-//            -(1/2) log2(e) Sigma_c^{-1}
-//   [14]     log2 of the Gaussian normaliser (2 pi)^{-5/2} det(Sigma)^{-1/2}
-//   [15]     unused
-// so log2 p(z; theta_k) = gp[14] + the two quadratic forms in d = z - mu.
+//   [5]      mu_b again, so that (b, b) is a pair
+//   [6, 7, 12]              xx, yy, 2xy of the spatial quadratic form
+//                           -(1/2) log2(e) Sigma_s^{-1}
+//   [8, 9, 14, 13, 10, 11]  LL, aa, bb, 2La, 2Lb, 2ab of the colour form
+//                           -(1/2) log2(e) Sigma_c^{-1}
+//   [15]     log2 of the Gaussian normaliser (2 pi)^{-5/2} det(Sigma)^{-1/2}
+// so log2 p(z; theta_k) = gp[15] + the two quadratic forms in d = z - mu.
+// The order pairs what the kernels take two at a time as packed FP32:
+// (x, y), (L, a), (b, b), (xx, yy), (LL, aa), (2Lb, 2ab).
 //
 // Master FP64 parameters (128 bytes): [0..4] mu, [5..7] Sigma_s (xx, xy, yy),
 // [8..13] Sigma_c (LL, La, Lb, aa, ab, bb), [14..15] unused.

@@ -216,10 +216,10 @@ __device__ bool pack_gp(const T* mu, const T* cs, const T* cc_in, T ox, T oy, fl
     const T hs = T(-0.5) * M::kLog2e * M::rcp(ds);
     const T hc = T(-0.5) * M::kLog2e * M::rcp(cc_in[0]);
     o[0] = make_float4(to_f32(mu[0] - ox), to_f32(mu[1] - oy), to_f32(mu[2]), 0.f);
-    o[1] = make_float4(0.f, to_f32(hs * cs[2]), to_f32(T(-2) * hs * cs[1]), to_f32(hs * cs[0]));
+    o[1] = make_float4(0.f, 0.f, to_f32(hs * cs[2]), to_f32(hs * cs[0]));
     o[2] = make_float4(to_f32(hc), 0.f, 0.f, 0.f);
     const float lnorm = -0.5f * (M::log2_(ds) + M::log2_(cc_in[0])) - float(M::kHalf3_Log2_2Pi);
-    o[3] = make_float4(0.f, 0.f, lnorm, 0.f);
+    o[3] = make_float4(to_f32(T(-2) * hs * cs[1]), 0.f, 0.f, lnorm);
     return true;
   }
   const bool split = cm == kColourSplit;
@@ -236,10 +236,11 @@ __device__ bool pack_gp(const T* mu, const T* cs, const T* cc_in, T ox, T oy, fl
   const T hs = T(-0.5) * M::kLog2e * M::rcp(ds);   // -(1/2) log2(e) / det
   const T hc = T(-0.5) * M::kLog2e * M::rcp(dc);
   o[0] = make_float4(to_f32(mu[0] - ox), to_f32(mu[1] - oy), to_f32(mu[2]), to_f32(mu[3]));
-  o[1] = make_float4(to_f32(mu[4]), to_f32(hs * cs[2]), to_f32(T(-2) * hs * cs[1]), to_f32(hs * cs[0]));
-  o[2] = make_float4(to_f32(hc * c00), to_f32(hc * c11), to_f32(hc * c22), to_f32(T(2) * hc * c01));
+  const float mb = to_f32(mu[4]);
+  o[1] = make_float4(mb, mb, to_f32(hs * cs[2]), to_f32(hs * cs[0]));
+  o[2] = make_float4(to_f32(hc * c00), to_f32(hc * c11), to_f32(T(2) * hc * c02), to_f32(T(2) * hc * c12));
   const float lnorm = -0.5f * (M::log2_(ds) + M::log2_(dc)) - float(M::kHalfD_Log2_2Pi);
-  o[3] = make_float4(to_f32(T(2) * hc * c02), to_f32(T(2) * hc * c12), lnorm, 0.f);
+  o[3] = make_float4(to_f32(T(-2) * hs * cs[1]), to_f32(T(2) * hc * c01), to_f32(hc * c22), lnorm);
   return true;
 }
 
