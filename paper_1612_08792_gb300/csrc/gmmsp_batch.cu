@@ -35,7 +35,6 @@ struct gmmsp_batch_s {
   int blocks_per_sm = 4;           // persistent grid of the E + M pass (autotuned)
   int first_bps = 0;               // the first E + M pass (diagonal blocks); 0: as blocks_per_sm
   double first_ms[2] = {0.0, 0.0}; // autotuned first-pass times at 6 and 7 blocks per SM
-  int label_blocks_per_sm = 4;     // persistent grid of the label pass (its occupancy)
   bool fin16 = false;              // finalize with 16 lanes per superpixel (autotuned)
   double fin_ms[2] = {0.0, 0.0};   // autotuned finalize times: 16 lanes, one thread per superpixel
   std::vector<BatchImage> host;    // the table as last uploaded
@@ -167,10 +166,8 @@ gmmsp_status enqueue_batch(gmmsp_batch b, int iters, bool want_ll) {
                                              b->p.eps_s, b->p.eps_c, b->counters, b->p.precision,
                                              use_fin16(b) ? 0 : fblocks, s));
   }
-  const long long lneed = (b->total_cells + 3) / 4;
-  const int lb = int(std::min<long long>(lneed, (long long)b->sm_count * b->label_blocks_per_sm));
   GB_CHECK(b, gmmsp::launch_label_pass_batch(b->table, n, b->total_cells, b->lab, b->gp,
-                                              want_ll ? b->cell_ll : nullptr, lb, b->p.colour_model, s));
+                                              want_ll ? b->cell_ll : nullptr, b->p.colour_model, s));
   if (want_ll) GB_CHECK(b, gmmsp::launch_ll_per_image(b->table, n, b->cell_ll, b->img_ll, s));
   return GMMSP_OK;
 }
@@ -260,7 +257,6 @@ gmmsp_status gmmsp_batch_create(gmmsp_batch* out, int n, const int* widths, cons
     return GMMSP_E_CUDA;
   }
   b->sm_count = prop.multiProcessorCount;
-  b->label_blocks_per_sm = std::max(1, gmmsp::label_pass_batch_occupancy());
   const size_t pbytes = size_t(cells) * gmmsp::kPartStride * sizeof(float);
   size_t off = 0;
   const size_t o_lab = off;   off += up256(3 * size_t(pix) * sizeof(float));

@@ -26,6 +26,17 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
+// The largest of three (NaNs are passed over, as by fmaxf).
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float y;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+// ... and of nine (four instructions).
+__device__ __forceinline__ float max9(const float (&e)[9]) {
+  return max3(max3(e[0], e[1], e[2]), max3(e[3], e[4], e[5]), max3(e[6], e[7], e[8]));
+}
+
 struct Cell {
   int cx, cy;      // cell coordinates
   int x0, y0;      // first pixel
@@ -59,6 +70,49 @@ __device__ __forceinline__ float4 load_pixel(const Src& s, const Geom& g, int x,
     return make_float4(0.f, 0.f, 0.f, 0.f);
   return load_z<CM>(s, x, y);
 }
+
+// One lane's walk over a cell's pixels p, p + step, ... (p = y cw + x, row
+// after row): the position as floats (exact small integers) and the pixel's
+// offset, advanced by additions -- no division, conversion or address
+// product per pixel.
+template <class Src>
+struct Walk {
+  typedef typename Src::Off Off;
+  float fx, fy;      // position in the cell
+  Off at;            // offset of the pixel
+  float cw, dx, dy;  // the cell's width; step = dy cw + dx
+  Off inc, wrap;
+  __device__ __forceinline__ void start(const Src& s, const Cell& c, int p, int step) {
+    const int y = __float2int_rz((float(p) + 0.5f) * (1.f / float(c.cw)));  // exact floor(p / cw)
+    const int x = p - y * c.cw;
+    const int q = __float2int_rz((float(step) + 0.5f) * (1.f / float(c.cw))), r = step - q * c.cw;
+    fx = float(x);
+    fy = float(y);
+    cw = float(c.cw);
+    dx = float(r);
+    dy = float(q);
+    at = s.at(c.x0 + x, c.y0 + y);
+    inc = q * s.row() + r * Src::kStep;
+    wrap = s.row() - c.cw * Src::kStep;
+  }
+  __device__ __forceinline__ void next() {
+    fx += dx;
+    fy += dy;
+    at += inc;
+    if (fx >= cw) {
+      fx -= cw;
+      fy += 1.f;
+      at += wrap;
+    }
+  }
+  template <int CM>
+  __device__ __forceinline__ float4 load(const Src& s, const Geom& g, const Cell& c) const {
+    if (!(GMMSP_IN_BOUNDS(c.x0 + int(fx), g.W, BND_PIXEL_X) && GMMSP_IN_BOUNDS(c.y0 + int(fy), g.H, BND_PIXEL_Y)))
+      return make_float4(0.f, 0.f, 0.f, 0.f);
+    if constexpr (CM == kColourGray) return make_float4(s.load_l_at(at), 0.f, 0.f, 0.f);
+    else return s.load_at(at);
+  }
+};
 
 // Two FP32 values in a register pair, and the packed arithmetic on them (one
 // instruction for both, each rounded as the scalar operation).

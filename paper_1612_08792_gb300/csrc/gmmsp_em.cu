@@ -87,21 +87,44 @@ __device__ __forceinline__ void e_pixel(const float4* sp, unsigned mask, const P
     R[s] = 0.f;
     if (FULL || ((mask >> s) & 1u)) {
       R[s] = log2_density<CM, DIAG>(sp + 4 * s, z);
-      m = fmaxf(m, R[s]);
+      if (!FULL) m = fmaxf(m, R[s]);
     }
   }
   float sum = 0.f;
+  if (FULL) {
+    m = fmaxf(m, max9(R));
+    const f2 mm = pack_f2(m, m);
 #pragma unroll
-  for (int s = 0; s < kSlots; ++s) {
-    if (FULL || ((mask >> s) & 1u)) {
-      R[s] = ex2_approx(R[s] - m);
+    for (int s = 0; s + 1 < kSlots; s += 2) {
+      const f2 t = sub_f2(pack_f2(R[s], R[s + 1]), mm);
+      R[s] = lo_f2(t);
+      R[s + 1] = hi_f2(t);
+    }
+    R[kSlots - 1] -= m;
+#pragma unroll
+    for (int s = 0; s < kSlots; ++s) {
+      R[s] = ex2_approx(R[s]);
       sum += R[s];
+    }
+  } else {
+#pragma unroll
+    for (int s = 0; s < kSlots; ++s) {
+      if ((mask >> s) & 1u) {
+        R[s] = ex2_approx(R[s] - m);
+        sum += R[s];
+      }
     }
   }
   const float inv = rcp_approx(sum);
   ll += m + lg2_approx(sum);
+  const f2 ii = pack_f2(inv, inv);
 #pragma unroll
-  for (int s = 0; s < kSlots; ++s) R[s] *= inv;
+  for (int s = 0; s + 1 < kSlots; s += 2) {
+    const f2 t = mul_f2(pack_f2(R[s], R[s + 1]), ii);
+    R[s] = lo_f2(t);
+    R[s + 1] = hi_f2(t);
+  }
+  R[kSlots - 1] *= inv;
 }
 
 // Fused E-step + M-step partial sums, stored as PT = float.  SHIFT: mixed
@@ -245,24 +268,20 @@ __device__ __forceinline__ void em_cell_warp(const Src& lab, const Geom& g, cons
   }
   // The colour of this lane's next pixel is loaded one batch ahead.
   float4 zn = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (wic * 32 + lane < npx_b) {
-    int rx0, ry0;
-    locate(wic * 32 + lane, rx0, ry0);
-    zn = load_pixel<CM>(lab, g, c.x0 + rx0, c.y0 + ry0);
-  }
+  Walk<Src> wk;
+  wk.start(lab, c, wic * 32 + lane, 32 * WPC);
+  if (wic * 32 + lane < npx_b) zn = wk.template load<CM>(lab, g, c);
   for (int base = wic * 32; base < npx_b; base += 32 * WPC) {
     const int p = base + lane;
     float R[kSlots];
     float4 z = zn;
+    const float fx = wk.fx, fy = wk.fy;
     if (p + 32 * WPC < npx_b) {
-      int rx1, ry1;
-      locate(p + 32 * WPC, rx1, ry1);
-      zn = load_pixel<CM>(lab, g, c.x0 + rx1, c.y0 + ry1);
+      wk.next();
+      zn = wk.template load<CM>(lab, g, c);
     }
-    int rx = 0, ry = 0;
     if (p < npx_b) {
-      locate(p, rx, ry);
-      e_pixel<FULL, CM, DIAG>(sp, c.mask, pix2(float(rx), float(ry), z), R, ll);
+      e_pixel<FULL, CM, DIAG>(sp, c.mask, pix2(fx, fy, z), R, ll);
     } else {  // no pixel: adds r = 0 times finite values, which changes no sum
 #pragma unroll
       for (int s = 0; s < kSlots; ++s) R[s] = 0.f;
@@ -270,7 +289,7 @@ __device__ __forceinline__ void em_cell_warp(const Src& lab, const Geom& g, cons
     }
 #pragma unroll
     for (int s = 0; s < kSlots; ++s) pe[s * kBatchLd] = R[s];
-    *reinterpret_cast<float2*>(pe + kBatchXY + pi) = make_float2(float(rx), float(ry));
+    *reinterpret_cast<float2*>(pe + kBatchXY + pi) = make_float2(fx, fy);
     *reinterpret_cast<float2*>(pe + kBatchLa + pi) = make_float2(z.x, z.y);
     if constexpr (CM != kColourGray) pe[kBatchB] = z.z;
     __syncwarp();
@@ -325,21 +344,30 @@ __device__ __forceinline__ void em_cell_block(const Src& lab, const Geom& g, con
   for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
   if (lane < 27) acc.store(sm.red[warp][lane]);
   __syncwarp();
-  for (int o = lane; o < kSlots * kStats; o += 32) {
+  const auto slot_sum = [&](int o) {
     const int s = o / kStats, j = o - s * kStats;
-    sm.part[warp][o] = sm.red[warp][s][j] + sm.red[warp][s + 9][j] + sm.red[warp][s + 18][j];
-  }
-  if (lane == 0) sm.part[warp][kSlots * kStats] = ll;
-  if (WPC == 1) __syncwarp(); else __syncthreads();
-  // Cell totals (sum over the WPC warps of the cell), written as PT.
-  if (active && GMMSP_IN_BOUNDS(cell, g.ncells, BND_PARTIAL_W)) {
-    PT* out = partials + (long long)cell * kPartStride;
-    const int w0 = slot * WPC;
-    for (int o = t; o < kPartStride; o += 32 * WPC) {
-      float v = sm.part[w0][o];
+    return sm.red[warp][s][j] + sm.red[warp][s + 9][j] + sm.red[warp][s + 18][j];
+  };
+  if constexpr (WPC == 1) {  // the warp's sums are the cell's
+    if (active && GMMSP_IN_BOUNDS(cell, g.ncells, BND_PARTIAL_W)) {
+      PT* out = partials + (long long)cell * kPartStride;
+      for (int o = lane; o < kSlots * kStats; o += 32) out[o] = PT(slot_sum(o));
+      if (lane == 0) out[kSlots * kStats] = SHIFT ? PT(ll) : PT(ll) * PT(0.69314718055994530942);
+    }
+  } else {
+    for (int o = lane; o < kSlots * kStats; o += 32) sm.part[warp][o] = slot_sum(o);
+    if (lane == 0) sm.part[warp][kSlots * kStats] = ll;
+    __syncthreads();
+    // Cell totals (sum over the WPC warps of the cell), written as PT.
+    if (active && GMMSP_IN_BOUNDS(cell, g.ncells, BND_PARTIAL_W)) {
+      PT* out = partials + (long long)cell * kPartStride;
+      const int w0 = slot * WPC;
+      for (int o = t; o < kPartStride; o += 32 * WPC) {
+        float v = sm.part[w0][o];
 #pragma unroll
-      for (int w = 1; w < WPC; ++w) v += sm.part[w0 + w][o];
-      out[o] = (o < kSlots * kStats || SHIFT) ? PT(v) : PT(v) * PT(0.69314718055994530942);
+        for (int w = 1; w < WPC; ++w) v += sm.part[w0 + w][o];
+        out[o] = (o < kSlots * kStats || SHIFT) ? PT(v) : PT(v) * PT(0.69314718055994530942);
+      }
     }
   }
   if (WPC == 1) __syncwarp(); else __syncthreads();  // the slot's buffers are reused next
@@ -373,7 +401,7 @@ __global__ void __launch_bounds__(kEmWarps * 32) k_em_pass(Src lab, Geom g, cons
 // 24% to 40% on large images (the split and grayscale kernels are faster
 // uncapped).
 template <typename PT, bool SHIFT, int WPC, class Src, int CM>
-__global__ void __launch_bounds__(kEmWarps * 32, 7) k_em_pass_capped(Src lab, Geom g, const float* __restrict__ gp,
+__global__ void __launch_bounds__(kEmWarps * 32, 6) k_em_pass_capped(Src lab, Geom g, const float* __restrict__ gp,
                                                                      PT* __restrict__ partials) {
   em_pass_body<PT, SHIFT, WPC, Src, CM>(lab, g, gp, partials);
 }
@@ -448,9 +476,8 @@ __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
                                                   const Cell& c, const float4* sp, int lane,
                                                   int32_t* __restrict__ labels, float& ll) {
   const int npx_all = c.cw * c.ch;
-  const float inv_cw = 1.f / float(c.cw);
   auto locate = [&](int p, int& rx, int& ry) {
-    ry = __float2int_rz((float(p) + 0.5f) * inv_cw);  // exact floor(p / cw)
+    ry = __float2int_rz((float(p) + 0.5f) * (1.f / float(c.cw)));  // exact floor(p / cw)
     rx = p - ry * c.cw;
   };
   // start at the cell's first candidate, so that the label is one of the
@@ -489,71 +516,72 @@ __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
       if (GMMSP_IN_BOUNDS(at, (long long)g.W * g.H, BND_LABEL) && GMMSP_IN_BOUNDS(kl, g.K, BND_LABEL_K)) labels[at] = kl;
     }
   }
+  // the walk over this lane's pixels lane, lane + 32, ...: position, offset and
+  // colour of the pixels of the next step, loaded ahead
+  Walk<Src> wk;
+  wk.start(lab, c, lane, 32);
   float4 zn[kLabelPPL];
-#pragma unroll
-  for (int j = 0; j < kLabelPPL; ++j) {
+  float xn[kLabelPPL], yn[kLabelPPL];
+  typename Src::Off an[kLabelPPL];
+  auto ahead = [&](int j, int p) {
     zn[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    const int p = lane + 32 * j;
-    if (p < npx) {
-      int rx, ry;
-      locate(p, rx, ry);
-      zn[j] = load_pixel<CM>(lab, g, c.x0 + rx, c.y0 + ry);
-    }
-  }
-  // One step: J pixels per lane (p0, p0 + 32, ...), the colours of the next
-  // step's pixels loaded ahead into zn.
+    if (p < npx) zn[j] = wk.template load<CM>(lab, g, c);
+    xn[j] = wk.fx;
+    yn[j] = wk.fy;
+    an[j] = wk.at;
+    if (p + 32 < npx) wk.next();
+  };
+#pragma unroll
+  for (int j = 0; j < kLabelPPL; ++j) ahead(j, lane + 32 * j);
+  const int k00 = (c.cy - 1) * g.nx + c.cx - 1;
+  // One step: J pixels per lane (p0, p0 + 32, ...).
   auto step = [&](auto jt, int p0) {
     constexpr int J = decltype(jt)::value;
-    float4 z[J];
-    int rx[J], ry[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      z[j] = zn[j];
-      const int pn = p0 + 32 * (j + kLabelPPL);
-      if (pn < npx) {
-        int x1, y1;
-        locate(pn, x1, y1);
-        zn[j] = load_pixel<CM>(lab, g, c.x0 + x1, c.y0 + y1);
-      }
-      locate(p0 + 32 * j, rx[j], ry[j]);
-    }
     Pix2 zp[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) zp[j] = pix2(float(rx[j]), float(ry[j]), z[j]);
-    float e[J][kSlots];
-    float m[J];
-    int best[J];
+    float fx[J], fy[J];
+    typename Src::Off at[J];
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-      m[j] = -INFINITY;
-      best[j] = first;
+      zp[j] = pix2(xn[j], yn[j], zn[j]);
+      fx[j] = xn[j];
+      fy[j] = yn[j];
+      at[j] = an[j];
+      ahead(j, p0 + 32 * (j + kLabelPPL));
     }
+    float e[J][kSlots];
 #pragma unroll
     for (int s = 0; s < kSlots; ++s) {
       if (FULL || ((c.mask >> s) & 1u)) {
 #pragma unroll
-        for (int j = 0; j < J; ++j) {
-          e[j][s] = log2_density<CM>(sp + 4 * s, zp[j]);
-          if (e[j][s] > m[j]) { m[j] = e[j][s]; best[j] = s; }
-        }
+        for (int j = 0; j < J; ++j) e[j][s] = log2_density<CM>(sp + 4 * s, zp[j]);
       } else {
 #pragma unroll
-        for (int j = 0; j < J; ++j) e[j][s] = 0.f;
+        for (int j = 0; j < J; ++j) e[j][s] = -INFINITY;
       }
     }
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       if (p0 + 32 * j >= npx) continue;
+      // argmax: the smallest slot that reaches the maximum (the first candidate
+      // when none is above -infinity or comparable)
+      const float m = max9(e[j]);
+      int best = first;
+#pragma unroll
+      for (int s = kSlots - 1; s >= 0; --s)
+        if (e[j][s] == m) best = s;
+      if (!(m > -INFINITY)) best = first;
       if (LL) {
         float sum = 0.f;
 #pragma unroll
         for (int s = 0; s < kSlots; ++s)
-          if (FULL || ((c.mask >> s) & 1u)) sum += ex2_approx(e[j][s] - m[j]);
-        ll += m[j] + lg2_approx(sum);
+          if (FULL || ((c.mask >> s) & 1u)) sum += ex2_approx(e[j][s] - m);
+        ll += m + lg2_approx(sum);
       }
-      const long long at = (long long)(c.y0 + ry[j]) * g.W + (c.x0 + rx[j]);
-      const int kl = (c.cy - 1 + best[j] / 3) * g.nx + (c.cx - 1 + best[j] % 3);
-      if (GMMSP_IN_BOUNDS(at, (long long)g.W * g.H, BND_LABEL) && GMMSP_IN_BOUNDS(kl, g.K, BND_LABEL_K)) labels[at] = kl;
+      const int row = best / 3, kl = k00 + row * g.nx + (best - 3 * row);
+      const long long i = std::is_same<Src, LabPlanar>::value
+                              ? (long long)at[j]  // the offset of a planar image's pixel is its index
+                              : (long long)(c.y0 + int(fy[j])) * g.W + (c.x0 + int(fx[j]));
+      if (GMMSP_IN_BOUNDS(i, (long long)g.W * g.H, BND_LABEL) && GMMSP_IN_BOUNDS(kl, g.K, BND_LABEL_K)) labels[i] = kl;
     }
   };
   // kLabelPPL pixels per lane while more than 32 remain, then one
@@ -599,6 +627,8 @@ __global__ void __launch_bounds__(kEmWarps * 32) k_label_pass(Src lab, Geom g, c
   label_cell_warp<Src, CM>(lab, g, gp, labels, cell_ll, cell, sp_all[warp], lane);
 }
 
+// One cell per warp over a grid sized to the work (a persistent loop over the
+// cells costs registers: 60 bytes of spill under the same bound).
 template <int CM>
 __global__ void __launch_bounds__(kEmWarps * 32, 5) k_label_pass_batch(const BatchImage* __restrict__ imgs, int n,
                                                                     int total_cells,
@@ -607,17 +637,15 @@ __global__ void __launch_bounds__(kEmWarps * 32, 5) k_label_pass_batch(const Bat
                                                                     double* __restrict__ cell_ll) {
   __shared__ float4 sp_all[kEmWarps][kSlots * 4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int cell = blockIdx.x * kEmWarps + warp; cell < total_cells; cell += gridDim.x * kEmWarps) {
-    const int ii = find_image(imgs, n, cell, 0);
-    if (!GMMSP_IN_BOUNDS(ii, n, BND_IMAGE)) continue;
-    const BatchImage& im = imgs[ii];
-    if (!GMMSP_IN_BOUNDS(cell - im.cell_off, im.g.ncells, BND_ITEM)) continue;
-    const LabPlanar src{lab + 3 * im.pix_off, (long long)im.g.W * im.g.H, im.g.W};
-    label_cell_warp<LabPlanar, CM>(src, im.g, gp + (long long)im.k_off * kGP, im.labels,
-                                   cell_ll ? cell_ll + im.cell_off : nullptr, cell - im.cell_off, sp_all[warp],
-                                   lane);
-    __syncwarp();
-  }
+  const int cell = blockIdx.x * kEmWarps + warp;
+  if (cell >= total_cells) return;
+  const int ii = find_image(imgs, n, cell, 0);
+  if (!GMMSP_IN_BOUNDS(ii, n, BND_IMAGE)) return;
+  const BatchImage& im = imgs[ii];
+  if (!GMMSP_IN_BOUNDS(cell - im.cell_off, im.g.ncells, BND_ITEM)) return;
+  const LabPlanar src{lab + 3 * im.pix_off, (long long)im.g.W * im.g.H, im.g.W};
+  label_cell_warp<LabPlanar, CM>(src, im.g, gp + (long long)im.k_off * kGP, im.labels,
+                                 cell_ll ? cell_ll + im.cell_off : nullptr, cell - im.cell_off, sp_all[warp], lane);
 }
 
 // ---------------------------------------------------------------- finalize
@@ -1301,27 +1329,18 @@ cudaError_t launch_finalize_batch(const BatchImage* imgs, int n, int total_k, co
   return cudaGetLastError();
 }
 
-int label_pass_batch_occupancy() {
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_label_pass_batch<kColourFull>, kEmWarps * 32, 0) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return 4;
-  }
-  return nb;
-}
-
 cudaError_t launch_label_pass_batch(const BatchImage* imgs, int n, int total_cells, const float* lab,
-                                    const float* gp, double* cell_ll, int blocks, int cm, cudaStream_t s) {
+                                    const float* gp, double* cell_ll, int cm, cudaStream_t s) {
+  const int nb = (total_cells + kEmWarps - 1) / kEmWarps;
   switch (cm) {
     case kColourFull:
-      k_label_pass_batch<kColourFull><<<blocks, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
+      k_label_pass_batch<kColourFull><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
       break;
     case kColourSplit:
-      k_label_pass_batch<kColourSplit><<<blocks, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
+      k_label_pass_batch<kColourSplit><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
       break;
     case kColourGray:
-      k_label_pass_batch<kColourGray><<<blocks, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
+      k_label_pass_batch<kColourGray><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
       break;
     default: return cudaErrorInvalidValue;
   }

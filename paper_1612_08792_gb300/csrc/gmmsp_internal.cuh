@@ -100,6 +100,17 @@ struct LabPlanar {  // the context's image: three float32 planes L, a, b of W H 
     return make_float4(__ldg(p + i), __ldg(p + plane + i), __ldg(p + 2 * plane + i), 0.f);
   }
   __device__ __forceinline__ float load_l(int x, int y) const { return __ldg(p + (long long)y * W + x); }
+  // offset of pixel (x, y) (W H < 2^31), the step to the next row, a load from an offset
+  typedef int Off;
+  static constexpr int kStep = 1;
+  __device__ __forceinline__ Off row() const { return W; }
+  __device__ __forceinline__ Off at(int x, int y) const { return y * W + x; }
+  __device__ __forceinline__ float load_l_at(Off i) const { return __ldg(p + i); }
+  __device__ __forceinline__ float4 load_at(Off i) const {
+    const int n = int(plane);
+    const float* q = p + i;
+    return make_float4(__ldg(q), __ldg(q + n), __ldg(q + n + (long long)n), 0.f);
+  }
 };
 struct LabPitched {  // a caller's image: rows of (L, a, b) float32, row pitch in bytes
   const char* p;
@@ -110,6 +121,15 @@ struct LabPitched {  // a caller's image: rows of (L, a, b) float32, row pitch i
   }
   __device__ __forceinline__ float load_l(int x, int y) const {
     return __ldg(reinterpret_cast<const float*>(p + (long long)y * pitch) + 3LL * x);
+  }
+  typedef long long Off;
+  static constexpr int kStep = 12;
+  __device__ __forceinline__ Off row() const { return pitch; }
+  __device__ __forceinline__ Off at(int x, int y) const { return (long long)y * pitch + 12LL * x; }
+  __device__ __forceinline__ float load_l_at(Off i) const { return __ldg(reinterpret_cast<const float*>(p + i)); }
+  __device__ __forceinline__ float4 load_at(Off i) const {
+    const float* q = reinterpret_cast<const float*>(p + i);
+    return make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), 0.f);
   }
 };
 
@@ -266,9 +286,7 @@ cudaError_t launch_finalize_batch(const BatchImage* imgs, int n, int total_k, co
                                   unsigned long long* counters, int precision, int blocks,
                                   cudaStream_t s);
 cudaError_t launch_label_pass_batch(const BatchImage* imgs, int n, int total_cells, const float* lab,
-                                    const float* gp, double* cell_ll, int blocks, int cm, cudaStream_t s);
-// Resident 128-thread blocks per SM of the batch label pass.
-int label_pass_batch_occupancy();
+                                    const float* gp, double* cell_ll, int cm, cudaStream_t s);
 // ll_out[i] = sum of image i's per-cell log-likelihoods (fixed order).
 cudaError_t launch_ll_per_image(const BatchImage* imgs, int n, const double* cell_ll, double* ll_out,
                                 cudaStream_t s);
