@@ -33,7 +33,8 @@ typedef struct {
 /* labels_dev: W H int32 superpixel labels in [0, K); gt_dev: W H int32
  * ground-truth segment ids in [0, G) (both device memory, row-major, owned by
  * the caller).  K G must not exceed 2^31 (a dense K x G overlap table is
- * counted on the device).  Allocates its scratch, works on `stream`
+ * counted on the device).  Takes its scratch from a bounded pool
+ * (gmmsp_release_scratch), works on `stream`
  * (cudaStream_t, NULL = legacy default) and synchronises.  Returns
  * GMMSP_E_INVALID for bad arguments or for a label or id out of range (found
  * on the device), GMMSP_E_NOMEM / GMMSP_E_CUDA on CUDA failures. */
@@ -41,8 +42,8 @@ gmmsp_status gmmsp_segmentation_metrics(const int32_t *labels_dev, const int32_t
                                         int G, int radius, double eps, gmmsp_seg_metrics *out_host,
                                         void *stream);
 
-/* The same for n images in one call (four kernel launches for all of them,
- * one allocation, one synchronisation): image i is labels_dev[i], gt_dev[i]
+/* The same for n images in one call (two kernel launches for all of them,
+ * one synchronisation): image i is labels_dev[i], gt_dev[i]
  * of W[i] x H[i] pixels with K[i] superpixels and G[i] segments, and its
  * metrics go to out_host[i] (n entries).  Returns GMMSP_E_INVALID for bad
  * arguments, or when a label or id of any image is out of range (out_host is

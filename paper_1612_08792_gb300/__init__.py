@@ -25,7 +25,7 @@ __all__ = [
     "gmmsp_default_params", "gmmsp_init", "gmmsp_reinit", "gmmsp_em_iters", "gmmsp_labels",
     "gmmsp_segment", "gmmsp_get_lab", "gmmsp_get_grid", "gmmsp_get_params", "gmmsp_set_params", "gmmsp_get_stats",
     "gmmsp_profile_kernel", "gmmsp_probe_peaks", "gmmsp_probe_fp64_helpers", "gmmsp_set_timing", "gmmsp_get_timing", "gmmsp_set_launch", "gmmsp_get_launch",
-    "gmmsp_autotune", "gmmsp_segment_lab_noalloc", "gmmsp_last_error", "SuperpixelsBatch", "gmmsp_bounds_status",
+    "gmmsp_autotune", "gmmsp_segment_lab_noalloc", "gmmsp_last_error", "SuperpixelsBatch", "gmmsp_bounds_status", "gmmsp_release_scratch",
     "gmmsp_batch_create", "gmmsp_batch_segment", "gmmsp_batch_get_params", "gmmsp_batch_autotune",
     "gmmsp_batch_set_launch", "gmmsp_batch_set_tuning", "gmmsp_batch_info", "gmmsp_batch_destroy", "gmmsp_status_string", "gmmsp_destroy",
     "gmmsp_batch_get_tuning", "gmmsp_batch_set_first_pass", "gmmsp_batch_get_first_pass",
@@ -116,6 +116,7 @@ def load_library(path: str | None = None):
             "gmmsp_status_string": (ctypes.c_char_p, [I]),
             "gmmsp_destroy": (None, [P]),
             "gmmsp_bounds_status": (I, [pint, ctypes.POINTER(ctypes.c_ulonglong)]),
+            "gmmsp_release_scratch": (I, []),
         }
         for name, (res, args) in sig.items():
             f = getattr(lib, name)
@@ -138,6 +139,13 @@ def gmmsp_bounds_status():
     if st != 0:
         raise GmmspError(st, "bounds status")
     return bool(checked.value), bounds_decode(code.value)
+
+
+def gmmsp_release_scratch() -> None:
+    """Gives back the device scratch kept between calls without a context (at most 256 MiB per device)."""
+    st = load_library().gmmsp_release_scratch()
+    if st != 0:
+        raise GmmspError(st, "release scratch")
 
 
 def bounds_decode(code: int):

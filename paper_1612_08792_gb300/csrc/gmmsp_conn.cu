@@ -717,10 +717,15 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   o[O_TILE] = off; off += up(size_t(ntiles + 1) * 4);
   void* slab = nullptr;
   cudaError_t e = cudaSuccess;
-  if (cache && cache->bytes >= off) {
+  CallScratch scratch;  // without a context's cache
+  if (!cache) {
+    e = scratch.alloc(off, s);
+    if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GMMSP_E_NOMEM : GMMSP_E_CUDA;
+    slab = scratch.ptr;
+  } else if (cache->bytes >= off) {
     slab = cache->ptr;
   } else {
-    if (cache && cache->ptr) {
+    if (cache->ptr) {
       cudaStreamSynchronize(s);
       cudaFree(cache->ptr);
       cache->ptr = nullptr;
@@ -731,10 +736,8 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
       cudaGetLastError();
       return e == cudaErrorMemoryAllocation ? GMMSP_E_NOMEM : GMMSP_E_CUDA;
     }
-    if (cache) {
-      cache->ptr = slab;
-      cache->bytes = off;
-    }
+    cache->ptr = slab;
+    cache->bytes = off;
   }
   char* b = static_cast<char*>(slab);
   auto ia = [&](int j) { return reinterpret_cast<int*>(b + o[j]); };
@@ -797,7 +800,6 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
     if ((e = cudaMemcpyAsync(&herr, S.err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
     e = cudaStreamSynchronize(s);
   } while (false);
-  if (!cache) cudaFree(slab);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GMMSP_E_NOMEM : GMMSP_E_CUDA;
   if (herr) return GMMSP_E_TIMEOUT;
   if (stats) {

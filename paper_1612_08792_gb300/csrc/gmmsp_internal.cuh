@@ -295,6 +295,18 @@ cudaError_t launch_ll_per_image(const BatchImage* imgs, int n, const double* cel
 
 #include "../../include/gmmsp_conn.h"
 namespace gmmsp {
+// Device scratch of one call, from a bounded pool (gmmsp_scratch.cu); freed in
+// stream order when it goes out of scope.
+struct CallScratch {
+  void* ptr = nullptr;
+  cudaStream_t stream = nullptr;
+  bool pooled = false;
+  CallScratch() = default;
+  CallScratch(const CallScratch&) = delete;
+  CallScratch& operator=(const CallScratch&) = delete;
+  ~CallScratch();
+  cudaError_t alloc(size_t bytes, cudaStream_t s);
+};
 // Device scratch a context keeps between post-processing calls (grown on demand).
 struct ConnScratch {
   void* ptr = nullptr;
