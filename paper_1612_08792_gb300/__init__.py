@@ -415,7 +415,8 @@ def _ptr_array(tensors):
     one already (callers that keep their arrays skip rebuilding them on every call)."""
     if isinstance(tensors, ctypes.Array):
         return tensors
-    return (ctypes.c_void_p * len(tensors))(*[_dptr(t) for t in tensors])
+    ptrs = np.array([_dptr(t) for t in tensors], dtype=np.uint64)
+    return (ctypes.c_void_p * len(tensors)).from_buffer(ptrs)
 
 
 def gmmsp_batch_segment(b, images, pitches, iters, labels, want_loglik=False):
@@ -670,6 +671,10 @@ class gmmsp_seg_metrics(ctypes.Structure):
                 ("ue_sum", ctypes.c_longlong), ("asa_sum", ctypes.c_longlong)]
 
 
+# gmmsp_seg_metrics as a numpy record
+_METRICS_DTYPE = np.dtype([(k, np.float64 if t is ctypes.c_double else np.int64) for k, t in gmmsp_seg_metrics._fields_])
+
+
 def gmmsp_segmentation_metrics(labels, gt, K: int, G: int, radius: int = 2, eps: float = 0.05, stream=None):
     """BR, UE (Eq. ue) and ASA (Eq. asa) of an (H, W) int32 CUDA label map against an
     (H, W) int32 CUDA ground truth with ids in [0, G); synchronises."""
@@ -705,21 +710,26 @@ def gmmsp_segmentation_metrics_many(labels, gts, Ks, Gs, radius: int = 2, eps: f
         f._sig = True
     if len(gts) != n or n < 1:
         raise ValueError("one ground truth per label map")
-    Ks = [int(Ks)] * n if isinstance(Ks, int) else [int(k) for k in Ks]
-    Gs = [int(Gs)] * n if isinstance(Gs, int) else [int(g) for g in Gs]
-    for l, g in zip(labels, gts):
-        if tuple(g.shape) != tuple(l.shape) or not l.is_contiguous() or not g.is_contiguous():
-            raise ValueError("labels and gt must be contiguous (H, W) maps of one size")
-    Ws = np.array([int(l.shape[1]) for l in labels], dtype=np.int32)
-    Hs = np.array([int(l.shape[0]) for l in labels], dtype=np.int32)
-    Ka, Ga = np.array(Ks, dtype=np.int32), np.array(Gs, dtype=np.int32)
-    out = (gmmsp_seg_metrics * n)()
+    Ka = np.full(n, Ks, dtype=np.int32) if isinstance(Ks, int) else np.array([int(k) for k in Ks], dtype=np.int32)
+    Ga = np.full(n, Gs, dtype=np.int32) if isinstance(Gs, int) else np.array([int(g) for g in Gs], dtype=np.int32)
+    # one C-level pass per property: a Python loop over the maps costs as much as the kernels
+    shapes = [l.shape for l in labels]
+    if ([g.shape for g in gts] != shapes or not all(t.is_contiguous() for t in labels)
+            or not all(t.is_contiguous() for t in gts)):
+        raise ValueError("labels and gt must be contiguous (H, W) maps of one size")
+    if shapes.count(shapes[0]) == n:
+        Hs, Ws = (np.full(n, d, dtype=np.int32) for d in shapes[0])
+    else:
+        Hs, Ws = (np.array([s[i] for s in shapes], dtype=np.int32) for i in (0, 1))
+    out = np.empty(n, dtype=_METRICS_DTYPE)
     st = f(n, _ptr_array(labels), _ptr_array(gts), Ws.ctypes.data_as(ctypes.c_void_p),
            Hs.ctypes.data_as(ctypes.c_void_p), Ka.ctypes.data_as(ctypes.c_void_p), Ga.ctypes.data_as(ctypes.c_void_p),
-           int(radius), float(eps), out, _stream_handle(stream))
+           int(radius), float(eps), ctypes.cast(out.ctypes.data, ctypes.POINTER(gmmsp_seg_metrics)),
+           _stream_handle(stream))
     if st != 0:
         raise GmmspError(st, "segmentation metrics failed (bad arguments or ids out of range)")
-    return [{k: getattr(o, k) for k, _ in gmmsp_seg_metrics._fields_} for o in out]
+    names = _METRICS_DTYPE.names
+    return [dict(zip(names, row)) for row in out.tolist()]
 
 
 class gmmsp_conn_stats(ctypes.Structure):

@@ -228,11 +228,17 @@ gmmsp_status enqueue_labels(gmmsp_ctx c, int32_t* labels, double* llk_out) {
   return GMMSP_OK;
 }
 
-// Synchronises and turns device-side findings into a status.
-gmmsp_status sync_and_check(gmmsp_ctx c) {
+// The first n log-likelihoods of llk to the host, and device-side findings as
+// a status: the counters lie directly before llk, so one copy and one
+// synchronisation bring both.
+gmmsp_status read_back(gmmsp_ctx c, int n, double* loglik_host) {
+  static_assert(sizeof(unsigned long long) == sizeof(double) && gmmsp::CNT_N % 2 == 0, "layout");
+  double buf[gmmsp::CNT_N + kLlkCap];
+  GM_CHECK(c, cudaMemcpyAsync(buf, c->counters, sizeof(double) * (gmmsp::CNT_N + n), cudaMemcpyDeviceToHost, c->stream));
   GM_CHECK(c, cudaStreamSynchronize(c->stream));
   unsigned long long cnt[gmmsp::CNT_N];
-  GM_CHECK(c, cudaMemcpy(cnt, c->counters, sizeof(cnt), cudaMemcpyDeviceToHost));
+  memcpy(cnt, buf, sizeof(cnt));
+  memcpy(loglik_host, buf + gmmsp::CNT_N, sizeof(double) * n);
   if (cnt[gmmsp::CNT_NONFINITE])
     return fail(c, GMMSP_E_NUMERIC, std::to_string(cnt[gmmsp::CNT_NONFINITE]) +
                                         " non-finite input values");
@@ -319,10 +325,10 @@ gmmsp_status gmmsp_init(gmmsp_ctx* out, const void* image_dev, int width, int he
   const size_t o_gp = off;       off += align_up(size_t(g.K) * gmmsp::kGP * sizeof(float));
   const size_t o_part = off;     off += align_up(partial_bytes(g, p->precision));
   const size_t o_cll = off;      off += align_up(size_t(g.ncells) * sizeof(double));
-  const size_t o_llk = off;      off += align_up(kLlkCap * sizeof(double));
+  const size_t o_cnt = off;      off += sizeof(unsigned long long) * gmmsp::CNT_N;  // directly before llk:
+  const size_t o_llk = off;      off += align_up(kLlkCap * sizeof(double));         // read back in one copy
   const size_t o_ws = off;       off += align_up(gmmsp::finalize_workspace_doubles(g) * sizeof(double));
   const size_t o_ticket = off;   off += align_up(sizeof(unsigned));
-  const size_t o_cnt = off;      off += align_up(sizeof(unsigned long long) * gmmsp::CNT_N);
   const size_t o_bad = off;      off += align_up(sizeof(int));
   cudaError_t e = inject_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc(&c->slab, off);
   if (e != cudaSuccess) {
@@ -380,9 +386,7 @@ gmmsp_status gmmsp_em_iters(gmmsp_ctx c, int iters, double* loglik_host) {
     st = enqueue_em(c, n, 0, loglik_host != nullptr);
     if (st != GMMSP_OK) return st;
     if (loglik_host) {
-      GM_CHECK(c, cudaMemcpyAsync(loglik_host + done, c->llk, sizeof(double) * n, cudaMemcpyDeviceToHost,
-                                  c->stream));
-      st = sync_and_check(c);
+      st = read_back(c, n, loglik_host + done);
       if (st != GMMSP_OK) return st;
     }
   }
@@ -398,10 +402,7 @@ gmmsp_status gmmsp_labels(gmmsp_ctx c, int32_t* labels_dev, double* loglik_host)
   GM_MARK(c);
   st = enqueue_labels(c, labels_dev, loglik_host ? c->llk : nullptr);
   if (st != GMMSP_OK) return st;
-  if (loglik_host) {
-    GM_CHECK(c, cudaMemcpyAsync(loglik_host, c->llk, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    return sync_and_check(c);
-  }
+  if (loglik_host) return read_back(c, 1, loglik_host);
   return GMMSP_OK;
 }
 
@@ -455,11 +456,7 @@ gmmsp_status gmmsp_segment(gmmsp_ctx c, const void* image_dev, int pitch_bytes, 
     }
     GM_CHECK(c, cudaGraphLaunch(gr.exec, c->stream));
   }
-  if (loglik_host) {
-    GM_CHECK(c, cudaMemcpyAsync(loglik_host, c->llk, sizeof(double) * (iters + 1), cudaMemcpyDeviceToHost,
-                                c->stream));
-    return sync_and_check(c);
-  }
+  if (loglik_host) return read_back(c, iters + 1, loglik_host);
   return GMMSP_OK;
 }
 

@@ -267,9 +267,9 @@ gmmsp_status gmmsp_batch_create(gmmsp_batch* out, int n, const int* widths, cons
   const size_t o_gp = off;    off += up256(size_t(ks) * gmmsp::kGP * sizeof(float));
   const size_t o_part = off;  off += up256(pbytes);
   const size_t o_cll = off;   off += up256(size_t(cells) * sizeof(double));
-  const size_t o_ill = off;   off += up256(size_t(n) * sizeof(double));
+  const size_t o_cnt = off;   off += sizeof(unsigned long long) * gmmsp::CNT_N;  // directly before img_ll:
+  const size_t o_ill = off;   off += up256(size_t(n) * sizeof(double));           // read back in one copy
   const size_t o_tab = off;   off += up256(size_t(n) * sizeof(BatchImage));
-  const size_t o_cnt = off;   off += up256(sizeof(unsigned long long) * gmmsp::CNT_N);
   const char* inj = getenv("GMMSP_FAIL_ALLOC");
   cudaError_t e = (inj && inj[0] == '1') ? cudaErrorMemoryAllocation : cudaMalloc(&b->slab, off);
   if (e != cudaSuccess) {
@@ -362,11 +362,13 @@ gmmsp_status gmmsp_batch_segment(gmmsp_batch b, const void* const* images_dev, c
     GB_CHECK(b, cudaGraphLaunch(b->exec, b->stream));
   }
   if (want_ll) {
-    GB_CHECK(b, cudaMemcpyAsync(loglik_host, b->img_ll, sizeof(double) * b->n, cudaMemcpyDeviceToHost,
-                                b->stream));
+    // the counters lie directly before the log-likelihoods: one copy
+    std::vector<double> buf(gmmsp::CNT_N + size_t(b->n));
+    GB_CHECK(b, cudaMemcpyAsync(buf.data(), b->counters, sizeof(double) * buf.size(), cudaMemcpyDeviceToHost, b->stream));
     GB_CHECK(b, cudaStreamSynchronize(b->stream));
     unsigned long long cnt[gmmsp::CNT_N];
-    GB_CHECK(b, cudaMemcpy(cnt, b->counters, sizeof(cnt), cudaMemcpyDeviceToHost));
+    memcpy(cnt, buf.data(), sizeof(cnt));
+    memcpy(loglik_host, buf.data() + gmmsp::CNT_N, sizeof(double) * b->n);
     if (cnt[gmmsp::CNT_NONFINITE]) return bfail(b, GMMSP_E_NUMERIC, "non-finite input values");
   }
   return GMMSP_OK;

@@ -1135,6 +1135,7 @@ struct gmmsp_net_s {
   float *wpart0 = nullptr, *wpart1 = nullptr;  // weight-gradient partials per block: layers 0-1, layers 2-5
   double* lpart = nullptr;
   long long last_cells = 0;  // superpixels of the last forward pass
+  std::vector<char> back;    // host side of grad_to_host
   std::string msg;
 };
 
@@ -1194,14 +1195,13 @@ gmmsp_status reserve(gmmsp_net n, long long cells, bool train) {
   size_t off = 0;
   const size_t o_c = off;   off += 4 * act;
   const size_t o_out = off; off += up256(size_t(cells) * kOut * sizeof(float));
-  size_t o_x0 = 0, o_gout = 0, o_gc = 0, o_wp0 = 0, o_wp1 = 0, o_lp = 0;
+  size_t o_x0 = 0, o_gout = 0, o_gc = 0, o_wp0 = 0, o_wp1 = 0;
   if (train) {
     o_x0 = off;   off += 2 * pix + up256(size_t(nrows) * 4);  // x0, h1, the bits of h2
     o_gout = off; off += up256(size_t(cells) * kOut * 2);
     o_gc = off;   off += 4 * act;
     o_wp0 = off;  off += up256(size_t(n->sms) * kPixBwdPerSm * pix_params(n->pl) * sizeof(float));
     o_wp1 = off;  off += up256(size_t(std::max(1, n->sms / 4)) * (n->pl.total - pix_params(n->pl)) * sizeof(float));
-    o_lp = off;   off += up256(kLossBlocks * sizeof(double));
   }
   if (n->wslab) {
     GN_CHECK(n, cudaStreamSynchronize(n->stream));
@@ -1225,13 +1225,11 @@ gmmsp_status reserve(gmmsp_net n, long long cells, bool train) {
     for (int i = 0; i < 4; ++i) n->gc[i] = reinterpret_cast<__nv_bfloat16*>(b + o_gc + i * act);
     n->wpart0 = reinterpret_cast<float*>(b + o_wp0);
     n->wpart1 = reinterpret_cast<float*>(b + o_wp1);
-    n->lpart = reinterpret_cast<double*>(b + o_lp);
   } else {
     n->x0 = n->h1 = n->gout = nullptr;
     for (auto& p : n->gc) p = nullptr;
     n->h2 = nullptr;
     n->wpart0 = n->wpart1 = nullptr;
-    n->lpart = nullptr;
   }
   n->cap_cells = cells;
   n->cap_train = train;
@@ -1360,14 +1358,26 @@ gmmsp_status check_err(gmmsp_net n) {
   return GMMSP_OK;
 }
 
-gmmsp_status loss_to_host(gmmsp_net n, long long cells, double* loss_host) {
-  double lp[kLossBlocks];
-  GN_CHECK(n, cudaMemcpyAsync(lp, n->lpart, sizeof(lp), cudaMemcpyDeviceToHost, n->stream));
-  const gmmsp_status st = check_err(n);
-  if (st != GMMSP_OK) return st;
-  double s = 0.0;
-  for (int i = 0; i < kLossBlocks; ++i) s += lp[i];
-  *loss_host = s / double(cells * kUsed);
+// The gradient and / or the loss of the last backward pass to the host, and
+// the error word: one copy of the memory that holds them side by side.
+gmmsp_status grad_to_host(gmmsp_net n, long long cells, float* grad_host, double* loss_host) {
+  const char* from = grad_host ? reinterpret_cast<const char*>(n->grad) : reinterpret_cast<const char*>(n->lpart);
+  const size_t bytes = size_t(reinterpret_cast<const char*>(n->err + 1) - from);
+  n->back.resize(bytes);
+  GN_CHECK(n, cudaMemcpyAsync(n->back.data(), from, bytes, cudaMemcpyDeviceToHost, n->stream));
+  GN_CHECK(n, cudaStreamSynchronize(n->stream));
+  auto at = [&](const void* dev) { return n->back.data() + (static_cast<const char*>(dev) - from); };
+  int e = 0;
+  memcpy(&e, at(n->err), sizeof(int));
+  if (grad_host) memcpy(grad_host, at(n->grad), size_t(n->pl.total) * 4);
+  if (e) return nfail(n, GMMSP_E_TIMEOUT, "a tensor-core kernel gave up waiting on its MMA barrier");
+  if (loss_host) {
+    double lp[kLossBlocks];
+    memcpy(lp, at(n->lpart), sizeof(lp));
+    double s = 0.0;
+    for (int i = 0; i < kLossBlocks; ++i) s += lp[i];
+    *loss_host = s / double(cells * kUsed);
+  }
   return GMMSP_OK;
 }
 
@@ -1449,10 +1459,12 @@ gmmsp_status gmmsp_net_create(gmmsp_net* out, int spacing, void* stream) {
   const size_t o_w = off; off += up256(np * 4);
   const size_t o_m = off; off += up256(np * 4);
   const size_t o_v = off; off += up256(np * 4);
+  // gradient, loss sums and error word side by side: read back in one copy
   const size_t o_g = off; off += up256(np * 4);
+  const size_t o_l = off; off += kLossBlocks * sizeof(double);
+  const size_t o_e = off; off += 256;
   const size_t o_b = off; off += up256(np * 2);
   const size_t o_s = off; off += up256(4 * kWBytes);
-  const size_t o_e = off; off += 256;
   const size_t o_t = off; off += 256 * 4;
   const char* inj = getenv("GMMSP_FAIL_ALLOC");
   cudaError_t e = (inj && inj[0] == '1') ? cudaErrorMemoryAllocation : cudaMalloc(&n->pslab, off);
@@ -1468,6 +1480,7 @@ gmmsp_status gmmsp_net_create(gmmsp_net* out, int spacing, void* stream) {
   n->grad = reinterpret_cast<float*>(b + o_g);
   n->wbf = reinterpret_cast<__nv_bfloat16*>(b + o_b);
   n->wst = reinterpret_cast<unsigned char*>(b + o_s);
+  n->lpart = reinterpret_cast<double*>(b + o_l);
   n->err = reinterpret_cast<int*>(b + o_e);
   n->srgb = reinterpret_cast<float*>(b + o_t);
   e = cudaMemsetAsync(n->pslab, 0, off, n->stream);
@@ -1557,11 +1570,7 @@ gmmsp_status gmmsp_net_grad(gmmsp_net n, const float* lab_dev, int B, int W, int
   if (st != GMMSP_OK) return st;
   st = enqueue_grad(n, lab_dev, B, g, target_dev, n->stream);
   if (st != GMMSP_OK) return st;
-  if (grad_host)
-    GN_CHECK(n, cudaMemcpyAsync(grad_host, n->grad, size_t(n->pl.total) * 4, cudaMemcpyDeviceToHost, n->stream));
-  if (loss_host) return loss_to_host(n, cells, loss_host);
-  if (grad_host) return check_err(n);
-  return GMMSP_OK;
+  return grad_host || loss_host ? grad_to_host(n, cells, grad_host, loss_host) : GMMSP_OK;
 }
 
 gmmsp_status gmmsp_net_adam(gmmsp_net n, float lr, float beta1, float beta2, float eps) {
@@ -1587,7 +1596,7 @@ gmmsp_status gmmsp_net_train_step(gmmsp_net n, const float* lab_dev, int B, int 
   if (st != GMMSP_OK || !loss_host) return st;
   Geom g;
   net_geom(n, W, H, &g);
-  return loss_to_host(n, (long long)B * g.K, loss_host);
+  return grad_to_host(n, (long long)B * g.K, nullptr, loss_host);
 }
 
 gmmsp_status gmmsp_net_get_activation(gmmsp_net n, int layer, float* host, long long count) {
