@@ -24,27 +24,30 @@
 // about 1.6 M entries for 256 images of 481x321, a few MB each, which the
 // L2 keeps while the merge reads them at random.
 //
-// Kernels (all images of a call at once; pixel loops take blockIdx.y as the
+// Kernels (all images of a call at once; pixel kernels take blockIdx.y as the
 // image, tile loops cover all pixels of the call):
-//   k_cc_init / _union / _flatten   union-find labelling, parent = root pixel
-//   k_root_count / _scan / _assign  compact index per root (tile counts, scan)
+//   k_cc_tile                       union-find labelling of 32 x 32 tiles in
+//                                   shared memory, parent = the tile's root
+//   k_cc_border                     unions across the tiles' borders
+//   k_cc_flatten / k_root_scan / k_root_assign  parent = root pixel, compact
+//                                   index per root (tile counts, scan)
 //   k_comp_map                      parent := compact index; sizes and
 //                                   fixed-point colour sums (atomics)
 //   k_comp_flags                    small flag, mean colour, group state per component
-//   k_edges (x2)                    small-small clusters and adjacency counts;
-//                                   adjacency lists (of the small components)
-//   k_scan_tiles / _tile_sums / _add  offsets (twice)
+//   k_scan_* (twice)                offsets of the adjacency lists and of the clusters
+//   k_edges                         small-small clusters and adjacency lists
 //   k_cluster_count / _fill         member lists as (size << 32 | c) keys
 //   k_cluster_merge                 one thread per cluster of <= kThreadCluster
-//   k_cluster_merge_warp            one warp per larger cluster (keys sorted
-//                                   in shared memory, adjacency over the lanes)
-//   k_relabel                       label of the group founder
+//                                   members, one warp per larger cluster (keys
+//                                   sorted in shared memory, adjacency over the lanes)
+//   k_group_label / k_relabel       label of the group founder
 // One allocation (kept by a context between calls) and one synchronisation
 // per call.  Every loop over a parent chain or a retry is bounded; running
 // out sets the error word (reported as GMMSP_E_TIMEOUT).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <algorithm>
 #include <vector>
@@ -64,6 +67,12 @@ constexpr int kHugeCluster = 32;       // warp clusters above this size are star
 constexpr int kWarpSortMax = 1024;     // members a warp sorts in shared memory
 constexpr int kScanTile = 4096;        // elements per block of the tile kernels (1024 threads x 4)
 constexpr int kMergeWarps = 4;
+constexpr int kCcTile = 32;            // side of the tiles labelled in shared memory
+constexpr int kCcWarps = 4;            // tiles per block
+constexpr int kCcAhead = 8;            // rows of labels in flight
+constexpr int kChunk = 128;            // pixels a warp walks down at once: four per lane
+constexpr int kChunkRows = 32;         // at most; fewer where the call has few pixels
+constexpr long long kOneBlockScan = 1 << 18;  // pixels up to which one block scans (64 steps at most)
 
 // One image of a call: pixels [off, off + W H) of the call's arrays.
 struct Img {
@@ -85,11 +94,11 @@ struct Scratch {
   int32_t* clabel;            // its label
   int* small;                 // 1 for a small component
   int* cpar;                  // cluster union-find over small components
-  int* deg;                   // adjacency count, then fill cursor
-  int* aoff;                  // (ncomp + 1) adjacency offsets
+  int* deg;                   // entries of its adjacency list
+  unsigned* aoff;             // (ncomp + 1) offsets of the lists, each with room for the component's perimeter
   int* adj;                   // adjacency lists (compact indices of neighbouring components)
-  int* cl_count;              // members of the cluster it roots, then fill cursor
-  int* cl_off;                // (ncomp + 1) member offsets
+  int* cl_count;              // members of the cluster it roots, counted down as they are filled in
+  unsigned* cl_off;           // (ncomp + 1) member offsets
   unsigned long long* cl_key; // members as (size << 32 | c), grouped by cluster
   int* big;                   // roots of clusters above kThreadCluster members: those above
                               // kHugeCluster from the front, the others from the back
@@ -180,76 +189,115 @@ __device__ __forceinline__ bool small_size(long long s, int K, long long N) { re
   const int ncomp_ = *S.ncomp; \
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncomp_; c += gridDim.x * blockDim.x)
 
-// Warp-uniform pixel loop (32 consecutive pixels per warp and step, every
-// lane taking part in the shuffles; `valid` marks the pixels of the image).
-#define FOR_PIXEL_WARPS(im, i, valid)                                                          \
-  const Img im = imgs[blockIdx.y];                                                             \
-  const long long im##_N = (long long)im.W * im.H;                                             \
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i - (threadIdx.x & 31) < im##_N; \
-       i += (long long)gridDim.x * blockDim.x)                                                 \
-    if (const bool valid = i < im##_N; true)
-
-// Every pixel starts under the first pixel of its run: the pixels of one
-// label that follow each other in a row within the warp's 32 (a ballot).  No
-// union runs yet, so these plain stores race with nothing.
-__global__ void k_cc_init(const Img* __restrict__ imgs, int* __restrict__ p) {
-  const int lane = threadIdx.x & 31;
-  FOR_PIXEL_WARPS(im, i, valid) {
-    const int x = valid ? int(i % im.W) : 0;
-    const int32_t l = valid ? im.labels[i] : 0;
-    const int32_t lprev = __shfl_up_sync(0xffffffffu, l, 1);
-    const bool head = !valid || lane == 0 || x == 0 || lprev != l;
-    const unsigned heads = __ballot_sync(0xffffffffu, head);
-    const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-    if (valid) p[im.off + i] = int(im.off + i - (lane - start));
+// Labels one 32 x 32 tile per warp in shared memory: every pixel starts under
+// the first pixel of its row's run of one label (a ballot), and one union per
+// pair of vertically adjacent runs (at the leftmost pixel of their overlap)
+// links the rows as the warp walks down.  Local indices order like pixels, so
+// a tile's root is the smallest pixel of its piece of the component.  Then
+// parent = the root's pixel.  Only the tiles' borders are left to global
+// unions: 6 % of the pixels (labelling all of them in global memory took
+// 195 + 703 us on 256 images of 481x321).
+__global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict__ imgs, int* __restrict__ p,
+                                                          int* err) {
+  __shared__ int sp[kCcWarps][kCcTile * kCcTile];
+  const Img im = imgs[blockIdx.y];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int tx = (im.W + kCcTile - 1) / kCcTile;
+  const long long tiles = (long long)tx * ((im.H + kCcTile - 1) / kCcTile);
+  int* q = sp[warp];
+  for (long long t = (long long)blockIdx.x * kCcWarps + warp; t < tiles; t += (long long)gridDim.x * kCcWarps) {
+    const int ty = int(t / tx), x0 = int(t - (long long)ty * tx) * kCcTile, y0 = ty * kCcTile;
+    const int rows = min(kCcTile, im.H - y0);
+    const bool in = x0 + lane < im.W;
+    const long long g0 = (long long)y0 * im.W + x0;
+    const int32_t* L = im.labels + g0 + lane;
+    int32_t next[kCcAhead], up = 0;  // the labels of the next rows, loaded ahead
+#pragma unroll
+    for (int j = 0; j < kCcAhead; ++j) next[j] = in && j < rows ? L[(long long)j * im.W] : 0;
+    for (int r0 = 0; r0 < rows; r0 += kCcAhead) {
+#pragma unroll
+      for (int j = 0; j < kCcAhead; ++j) {
+        const int r = r0 + j;
+        if (r >= rows) continue;
+        const int32_t l = next[j];
+        if (in && r + kCcAhead < rows) next[j] = L[(long long)(r + kCcAhead) * im.W];
+        const int32_t lprev = __shfl_up_sync(0xffffffffu, l, 1), uprev = __shfl_up_sync(0xffffffffu, up, 1);
+        const bool left_same = in && lane > 0 && lprev == l;
+        const unsigned heads = __ballot_sync(0xffffffffu, !left_same);
+        q[r * 32 + lane] = r * 32 + 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+        __syncwarp();
+        if (in && r > 0 && l == up && !(left_same && uprev == l)) unite(q, r * 32 + lane, (r - 1) * 32 + lane, err);
+        __syncwarp();
+        up = l;
+      }
+    }
+    for (int r = 0; r < rows; ++r) {
+      const int root = find_root(q, r * 32 + lane, err);
+      if (in) p[im.off + g0 + (long long)r * im.W + lane] = int(im.off + g0 + (long long)(root >> 5) * im.W + (root & 31));
+    }
+    __syncwarp();  // the tile's array is refilled
   }
 }
 
-// The unions the runs leave: a run that begins at a warp's first lane with the
-// same label to its left, and one vertical union per pair of vertically
-// adjacent runs (at the leftmost pixel of their overlap).
-__global__ void k_cc_union(const Img* __restrict__ imgs, int* p, int* err) {
-  FOR_PIXELS(im, i) {
-    const int y = int(i / im.W), x = int(i - (long long)y * im.W);
-    const long long g = im.off + i;
-    const int32_t l = im.labels[i];
-    const bool left_same = x > 0 && im.labels[i - 1] == l;
-    if (left_same && (threadIdx.x & 31) == 0) unite(p, int(g), int(g - 1), err);
-    if (y + 1 < im.H && l == im.labels[i + im.W] && !(left_same && im.labels[i - 1 + im.W] == l))
-      unite(p, int(g), int(g + im.W), err);
+// The unions across the tiles' borders: pixels x = 32 k with their left
+// neighbour, pixels y = 32 k with the one above.  A pair that the previous one
+// along the border already joined (both pairs of one label, inside the same
+// two tiles) is skipped.
+__global__ void k_cc_border(const Img* __restrict__ imgs, int* p, int* err) {
+  const Img im = imgs[blockIdx.y];
+  const int nx = (im.W - 1) / kCcTile, ny = (im.H - 1) / kCcTile;
+  const long long vertical = (long long)nx * im.H, total = vertical + (long long)ny * im.W;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    int x, y;
+    long long other, back;  // offsets of the pixel across the border, of the previous pixel along it
+    bool first;             // of its tile's side
+    if (i < vertical) {
+      const int k = int(i / im.H);
+      y = int(i - (long long)k * im.H);
+      x = (k + 1) * kCcTile;
+      other = -1;
+      back = -(long long)im.W;
+      first = y % kCcTile == 0;
+    } else {
+      const long long j = i - vertical;
+      const int k = int(j / im.W);
+      x = int(j - (long long)k * im.W);
+      y = (k + 1) * kCcTile;
+      other = -(long long)im.W;
+      back = -1;
+      first = x % kCcTile == 0;
+    }
+    const long long g = (long long)y * im.W + x;
+    const int32_t l = im.labels[g];
+    if (im.labels[g + other] != l) continue;
+    if (!first && im.labels[g + back] == l && im.labels[g + back + other] == l) continue;
+    unite(p, int(im.off + g), int(im.off + g + other), err);
   }
 }
 
-// After the unions: every pixel points at its root.  The walks only read, so
-// the one store per pixel (its root) cannot be overwritten by another
-// thread's walk (a halving store here could leave a non-root behind).
-__global__ void k_cc_flatten(const Img* __restrict__ imgs, int* p, int* err) {
-  FOR_PIXELS(im, i) p[im.off + i] = find_root(p, int(im.off + i), err);
-}
-
-// Exclusive scan of one int per thread over the block; total = the block sum.
-__device__ __forceinline__ int block_exclusive_scan(int v, int* warp_sums, int& total) {
+// Exclusive scan of one value per thread over the block; total = the block sum.
+__device__ __forceinline__ unsigned block_exclusive_scan(unsigned v, unsigned* warp_sums, unsigned& total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x = v;
+  unsigned x = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
   if (lane == 31) warp_sums[warp] = x;
   __syncthreads();
   if (warp == 0) {
-    int w = lane < int(blockDim.x >> 5) ? warp_sums[lane] : 0;
+    unsigned w = lane < int(blockDim.x >> 5) ? warp_sums[lane] : 0u;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, w, o);
+      const unsigned y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
     warp_sums[lane] = w;  // inclusive prefix of the warp totals
   }
   __syncthreads();
   total = warp_sums[(blockDim.x >> 5) - 1];
-  const int before = warp ? warp_sums[warp - 1] : 0;
+  const unsigned before = warp ? warp_sums[warp - 1] : 0u;
   __syncthreads();  // warp_sums is reused by the next call
   return before + x - v;
 }
@@ -264,32 +312,48 @@ __device__ __forceinline__ int image_of(const Img* __restrict__ imgs, int n, lon
   return lo;
 }
 
-// Compact indices of the components in the order of their roots (smallest
-// pixels): a count per tile of kScanTile pixels, a scan of the counts, the
-// assignment.  No counter that every block updates.
-__global__ void __launch_bounds__(1024) k_root_count(long long T, Scratch S) {
-  __shared__ int warp_sums[32];
+// After the unions: every pixel points at its root, and the roots are counted
+// per tile of kScanTile pixels.  The walks only read, so the one store per
+// pixel (its root) cannot be overwritten by another thread's walk (a halving
+// store here could leave a non-root behind).  The compact indices of the
+// components are in the order of their roots (smallest pixels): these counts,
+// a scan of them, the assignment; no counter that every block updates.
+__global__ void __launch_bounds__(1024) k_cc_flatten(long long T, Scratch S) {
+  __shared__ unsigned warp_sums[32];
   const long long g0 = (long long)blockIdx.x * kScanTile + 4LL * threadIdx.x;
   int c = 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) c += (g0 + j < T && S.parent[g0 + j] == int(g0 + j));
-  int total;
-  block_exclusive_scan(c, warp_sums, total);
-  if (threadIdx.x == 0) S.tile_sum[blockIdx.x] = total;
+  if (g0 + 3 < T) {
+    int4 q = *reinterpret_cast<const int4*>(S.parent + g0);
+    c = (q.x == int(g0)) + (q.y == int(g0 + 1)) + (q.z == int(g0 + 2)) + (q.w == int(g0 + 3));
+    q.x = find_root(S.parent, q.x, S.err);
+    q.y = find_root(S.parent, q.y, S.err);
+    q.z = find_root(S.parent, q.z, S.err);
+    q.w = find_root(S.parent, q.w, S.err);
+    *reinterpret_cast<int4*>(S.parent + g0) = q;
+  } else {
+    for (int j = 0; j < 4 && g0 + j < T; ++j) {
+      const int q = S.parent[g0 + j];
+      c += q == int(g0 + j);
+      S.parent[g0 + j] = find_root(S.parent, q, S.err);
+    }
+  }
+  unsigned total;
+  block_exclusive_scan(unsigned(c), warp_sums, total);
+  if (threadIdx.x == 0) S.tile_sum[blockIdx.x] = int(total);
 }
 
 // Exclusive scan of the ntiles tile counts in place (one block); the total
 // is the component count.
 __global__ void __launch_bounds__(1024) k_root_scan(int ntiles, Scratch S) {
-  __shared__ int warp_sums[32];
+  __shared__ unsigned warp_sums[32];
   int carry = 0;
   for (int c = 0; c < ntiles; c += 1024) {
     const int i = c + threadIdx.x;
     const int v = i < ntiles ? S.tile_sum[i] : 0;
-    int total;
-    const int ex = block_exclusive_scan(v, warp_sums, total);
-    if (i < ntiles) S.tile_sum[i] = carry + ex;
-    carry += total;
+    unsigned total;
+    const unsigned ex = block_exclusive_scan(unsigned(v), warp_sums, total);
+    if (i < ntiles) S.tile_sum[i] = carry + int(ex);
+    carry += int(total);
   }
   if (threadIdx.x == 0) {
     *S.ncomp = carry;
@@ -298,7 +362,7 @@ __global__ void __launch_bounds__(1024) k_root_scan(int ntiles, Scratch S) {
 }
 
 __global__ void __launch_bounds__(1024) k_root_assign(const Img* __restrict__ imgs, int n, long long T, Scratch S) {
-  __shared__ int warp_sums[32];
+  __shared__ unsigned warp_sums[32];
   const long long g0 = (long long)blockIdx.x * kScanTile + 4LL * threadIdx.x;
   bool f[4];
   int cnt = 0;
@@ -307,61 +371,94 @@ __global__ void __launch_bounds__(1024) k_root_assign(const Img* __restrict__ im
     f[j] = g0 + j < T && S.parent[g0 + j] == int(g0 + j);
     cnt += f[j];
   }
-  int total;
-  int c = S.tile_sum[blockIdx.x] + block_exclusive_scan(cnt, warp_sums, total);
+  unsigned total;
+  int c = S.tile_sum[blockIdx.x] + int(block_exclusive_scan(unsigned(cnt), warp_sums, total));
+  // the tile's first image once per warp; a pixel's image from there on
+  int i = 0;
+  if (cnt) i = image_of(imgs, n, (long long)blockIdx.x * kScanTile);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     if (!f[j]) continue;
     const long long g = g0 + j;
-    const int i = image_of(imgs, n, g);
+    while (i + 1 < n && imgs[i + 1].off <= g) ++i;
     S.cidr[g] = c;
     S.cimg[c] = i;
     S.clabel[c] = imgs[i].labels[g - imgs[i].off];
+    S.size[c] = 0;
+    S.deg[c] = 0;
+    S.cl_count[c] = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) S.csum[3LL * c + k] = 0;
     ++c;
   }
 }
 
 // parent := compact index of the pixel's component; component sizes and
-// fixed-point colour sums.  A warp takes 32 consecutive pixels; the lanes of
-// a run of equal components (a row segment of one component) add their
-// values to the run's first lane (a segmented reduction by shuffles), which
-// alone updates the sums: one set of atomics per run instead of per pixel.
-__global__ void k_comp_map(const Img* __restrict__ imgs, Scratch S) {
+// fixed-point colour sums.  A warp walks a chunk of 128 pixels down 32 rows,
+// four pixels per lane; a lane adds its pixels of one component in registers,
+// going back and forth along its four pixels, and updates the component's sums
+// when it changes: about one set of atomics per eight pixels.  (A warp-wide
+// segmented reduction of 64-bit values per row run took 373 us on 256 images
+// of 481x321.)
+__global__ void __launch_bounds__(128) k_comp_map(const Img* __restrict__ imgs, Scratch S, int chunk_rows) {
   const Img im = imgs[blockIdx.y];
   const long long N = (long long)im.W * im.H;
   const int lane = threadIdx.x & 31;
-  const long long step = (long long)gridDim.x * blockDim.x;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i - lane < N; i += step) {
-    const bool valid = i < N;  // warp-uniform loop: every lane takes part in the shuffles
-    int c = -1 - lane;         // distinct for invalid lanes: they form runs of their own
-    long long v[4] = {0, 0, 0, 0};
-    if (valid) {
-      const long long g = im.off + i;
-      c = S.cidr[S.parent[g]];
-      S.parent[g] = c;
-      v[0] = 1;
+  const int cx = (im.W + kChunk - 1) / kChunk;
+  const long long chunks = (long long)cx * ((im.H + chunk_rows - 1) / chunk_rows);
+  for (long long t = (long long)blockIdx.x * 4 + (threadIdx.x >> 5); t < chunks; t += (long long)gridDim.x * 4) {
+    const int cy = int(t / cx), x = int(t - (long long)cy * cx) * kChunk + 4 * lane, y0 = cy * chunk_rows;
+    const int n = min(4, im.W - x), rows = min(chunk_rows, im.H - y0);
+    if (n <= 0) continue;
+    int root = -1, c = 0, cnt = 0;
+    long long s0 = 0, s1 = 0, s2 = 0;
+    auto flush = [&] {
+      if (!cnt) return;
+      atomicAdd(S.size + c, cnt);
+      unsigned long long* o = reinterpret_cast<unsigned long long*>(S.csum + 3LL * c);
+      atomicAdd(o, (unsigned long long)s0);
+      atomicAdd(o + 1, (unsigned long long)s1);
+      atomicAdd(o + 2, (unsigned long long)s2);
+    };
+    int* P = S.parent + im.off + (long long)y0 * im.W + x;
+    const float* Z = im.lab + (long long)y0 * im.W + x;
+    for (int r = 0; r < rows; ++r, P += im.W, Z += im.W) {
+      int q[4], cq[4];
+      float z[3][4];
 #pragma unroll
-      for (int k = 0; k < 3; ++k)  // z 2^20 is exact in FP32 (a power-of-two scaling): round(2^20 z)
-        v[1 + k] = __float2ll_rn(im.lab[k * N + i] * float(1 << kFixedShift));
-    }
-    const int cprev = __shfl_up_sync(0xffffffffu, c, 1);
-    const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || cprev != c);
-    const int start = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));  // first lane of my run
-    const int run_end = (heads & (0xfffffffeu << lane)) ? __ffs(heads & (0xfffffffeu << lane)) - 1 : 32;
+      for (int j = 0; j < 4; ++j) {
+        q[j] = -1;
+        if (j < n) {
+          q[j] = P[j];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
+          for (int k = 0; k < 3; ++k) z[k][j] = __ldg(Z + k * N + j);
+        }
+      }
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const long long w = __shfl_down_sync(0xffffffffu, v[k], o);
-        if (lane + o < run_end) v[k] += w;
+      for (int j = 0; j < 4; ++j) cq[j] = j < n ? S.cidr[q[j]] : 0;
+      auto add = [&](int j) {
+        if (j >= n) return;
+        if (q[j] != root) {
+          flush();
+          root = q[j];
+          c = cq[j];
+          cnt = 0;
+          s0 = s1 = s2 = 0;
+        }
+        P[j] = c;
+        ++cnt;
+        // z 2^20 is exact in FP32 (a power-of-two scaling): round(2^20 z)
+        s0 += __float2ll_rn(z[0][j] * float(1 << kFixedShift));
+        s1 += __float2ll_rn(z[1][j] * float(1 << kFixedShift));
+        s2 += __float2ll_rn(z[2][j] * float(1 << kFixedShift));
+      };
+      if (r & 1) {
+        add(3); add(2); add(1); add(0);
+      } else {
+        add(0); add(1); add(2); add(3);
       }
     }
-    if (valid && lane == start) {
-      atomicAdd(S.size + c, int(v[0]));
-#pragma unroll
-      for (int k = 0; k < 3; ++k)
-        atomicAdd(reinterpret_cast<unsigned long long*>(S.csum + 3LL * c + k), (unsigned long long)v[1 + k]);
-    }
+    flush();
   }
 }
 
@@ -391,93 +488,183 @@ __global__ void __launch_bounds__(256) k_comp_flags(const Img* __restrict__ imgs
   }
 }
 
-// Walks the 4-neighbour edges between different components; `mode` 0 unites
-// small-small pairs into clusters and counts each small side's adjacency, 1
-// fills the adjacency lists.  An edge whose pair of components the previous
-// edge along the same line already gave (the pixel to the left for a vertical
-// edge, the pixel above for a horizontal one) is skipped: the lists are
-// neighbour sets, and most repeats go.
-__global__ void k_edges(const Img* __restrict__ imgs, Scratch S, int mode) {
-  FOR_PIXELS(im, i) {
-    const int y = int(i / im.W), x = int(i - (long long)y * im.W);
-    const long long g = im.off + i;
-    const int ci = S.parent[g];
-#pragma unroll
-    for (int d = 0; d < 2; ++d) {
-      long long j, back;  // back: the same edge one pixel earlier along the line, or -1
-      if (d == 0) {
-        if (x + 1 >= im.W) continue;
-        j = g + 1;
-        back = y > 0 ? g - im.W : -1;
-      } else {
-        if (y + 1 >= im.H) continue;
-        j = g + im.W;
-        back = x > 0 ? g - 1 : -1;
-      }
-      const int cj = S.parent[j];
-      if (ci == cj) continue;
-      if (back >= 0 && S.parent[back] == ci && S.parent[back + (j - g)] == cj) continue;
-      const int si = S.small[ci], sj = S.small[cj];
-      if (mode == 0) {
-        if (si && sj) unite(S.cpar, ci, cj, S.err);
-        if (si) atomicAdd(S.deg + ci, 1);
-        if (sj) atomicAdd(S.deg + cj, 1);
-      } else {
-        if (si) S.adj[S.aoff[ci] + atomicAdd(S.deg + ci, 1)] = cj;
-        if (sj) S.adj[S.aoff[cj] + atomicAdd(S.deg + cj, 1)] = ci;
-      }
-    }
-  }
+// One edge between different components i and j: small ones that touch join a
+// cluster, and each small side's list gets the other.  A list has room for its
+// component's whole perimeter (2 size + 2 edges at most for a 4-connected set
+// of pixels), so it is filled in the pass that finds the edges.
+__device__ __forceinline__ void add_neighbour(const Scratch& S, int i, int j) {
+  const unsigned at = S.aoff[i] + unsigned(atomicAdd(S.deg + i, 1));  // < 4 T < 2^32
+  if (at < S.aoff[i + 1]) S.adj[at] = j;
+  else atomicExch(S.err, 1);
+}
+__device__ __forceinline__ void add_edge(const Scratch& S, int i, int j) {
+  const int si = S.small[i], sj = S.small[j];
+  if (si) add_neighbour(S, i, j);
+  if (sj) add_neighbour(S, j, i);
+  if (si && sj) unite(S.cpar, i, j, S.err);
 }
 
-// Exclusive prefix sum of the first n = *np ints of `in` into out[0..n]
-// (out[n] = the total), in three kernels: tile scans (kScanTile elements per
-// block), a scan of the tile sums (one block), the tile offsets added.  The
-// grids cover the largest possible n; blocks past n return at once.
-__global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restrict__ in, const int* __restrict__ np,
-                                                     int* __restrict__ out, int* __restrict__ tile_sum) {
-  __shared__ int warp_sums[32];
-  const int n = *np;
+// Walks the 4-neighbour edges between different components (the edge to the
+// right and the edge below of every pixel).  An edge whose pair of components
+// the previous edge along the same line already gave (the row above for the
+// edge to the right, the pixel to the left for the edge below) is skipped: the
+// lists are neighbour sets, and most repeats go.  A warp walks a chunk of 128
+// pixels down 32 rows, four pixels per lane with the rows above and below in
+// registers, so an index is loaded once; the edges found go through a queue in
+// shared memory and are worked on 32 at a time, so that their chains of random
+// accesses overlap (worked on where they were found: 684 us on 256 images of
+// 481x321; one pixel per thread, in a counting and a filling pass: 2 x 390).
+__global__ void __launch_bounds__(128, 8) k_edges(const Img* __restrict__ imgs, Scratch S, int chunk_rows) {
+  const Img im = imgs[blockIdx.y];
+  const int lane = threadIdx.x & 31;
+  __shared__ int2 queue[4][32 + 8 * 32];
+  int2* Q = queue[threadIdx.x >> 5];
+  int queued = 0;  // below 32 between rows; a row adds at most 8 per lane
+  auto push = [&](bool has, int i, int j) {
+    const unsigned m = __ballot_sync(0xffffffffu, has);
+    if (has) Q[queued + __popc(m & ((1u << lane) - 1u))] = make_int2(i, j);
+    queued += __popc(m);
+  };
+  auto work = [&](int at_least) {
+    __syncwarp();
+    while (queued >= at_least && queued > 0) {
+      const int k = min(32, queued);
+      queued -= k;
+      if (lane < k) {
+        const int2 e = Q[queued + lane];
+        add_edge(S, e.x, e.y);
+      }
+      __syncwarp();
+    }
+  };
+  const int cx = (im.W + kChunk - 1) / kChunk;
+  const long long chunks = (long long)cx * ((im.H + chunk_rows - 1) / chunk_rows);
+  for (long long t = (long long)blockIdx.x * 4 + (threadIdx.x >> 5); t < chunks; t += (long long)gridDim.x * 4) {
+    const int cy = int(t / cx), x = int(t - (long long)cy * cx) * kChunk + 4 * lane, y0 = cy * chunk_rows;
+    const int n = max(0, min(4, im.W - x)), rows = min(chunk_rows, im.H - y0);
+    const bool left = x > 0 && x < im.W, right = x + 4 < im.W;  // pixel x - 1, x + 4 exists
+    // the pixel beside the warp's first / last lane
+    const int beside = lane == 0 ? -1 : 4;
+    const bool e_in = (lane == 0 && left) || (lane == 31 && right);
+    const int* P = S.parent + im.off + (long long)y0 * im.W + x;
+    int up[4], v[4], dn[4], ue = -1, e = -1, de = -1;
+    auto row = [&](const int* q, bool ok, int (&d)[4], int& de_) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) d[j] = ok && j < n ? q[j] : -1;
+      de_ = ok && e_in ? q[beside] : -1;
+    };
+    row(P - im.W, y0 > 0, up, ue);
+    row(P, true, v, e);
+    for (int r = 0; r < rows; ++r, P += im.W) {
+      row(P + im.W, y0 + r + 1 < im.H, dn, de);
+      // neighbours across the lanes: left of pixel 0 (this row, the row below), right of pixel 3 (this row, above)
+      const int lv = __shfl_up_sync(0xffffffffu, v[3], 1), ld = __shfl_up_sync(0xffffffffu, dn[3], 1);
+      const int rv = __shfl_down_sync(0xffffffffu, v[0], 1), ru = __shfl_down_sync(0xffffffffu, up[0], 1);
+      const int l_v = lane == 0 ? e : lv, l_d = lane == 0 ? de : ld, r_v = lane == 31 ? e : rv, r_u = lane == 31 ? ue : ru;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int ci = v[j];
+        const bool has_r = j < n && (j < 3 ? j + 1 < n : right);
+        const int cr = j < 3 ? v[j < 3 ? j + 1 : 3] : r_v, cru = j < 3 ? up[j < 3 ? j + 1 : 3] : r_u;
+        push(has_r && cr != ci && !(up[j] == ci && cru == cr), ci, cr);
+        const int cd = dn[j];
+        const bool has_l = j > 0 || left;
+        const int cl = j > 0 ? v[j > 0 ? j - 1 : 0] : l_v, cld = j > 0 ? dn[j > 0 ? j - 1 : 0] : l_d;
+        push(j < n && cd >= 0 && cd != ci && !(has_l && cl == ci && cld == cd), ci, cd);
+      }
+      work(32);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        up[j] = v[j];
+        v[j] = dn[j];
+      }
+      ue = e;
+      e = de;
+    }
+  }
+  work(1);
+}
+
+// What the scans add up: the room of a component's adjacency list (the
+// perimeter of a small component, at most 2 size + 2 edges), or the members of
+// the cluster it roots.
+enum ScanOf : int { kScanLists = 0, kScanClusters = 1 };
+template <int OF>
+__device__ __forceinline__ unsigned scan_value(const Scratch& S, int c) {
+  if (OF == kScanClusters) return unsigned(S.cl_count[c]);
+  return S.small[c] ? 2u * unsigned(S.size[c]) + 2u : 0u;
+}
+
+// Exclusive prefix sum over the n = *S.ncomp components into out[0..n] (out[n]
+// = the total), in three kernels: tile scans (kScanTile elements per block), a
+// scan of the tile sums (one block), the tile offsets added.  The grids cover
+// the largest possible n; blocks past n return at once.  Few pixels: one block
+// does it alone (k_scan_one).
+template <int OF>
+__global__ void __launch_bounds__(1024) k_scan_tiles(Scratch S, unsigned* __restrict__ out) {
+  __shared__ unsigned warp_sums[32];
+  const int n = *S.ncomp;
   const long long base = (long long)blockIdx.x * kScanTile;
   if (base >= n) return;
   const long long i0 = base + 4LL * threadIdx.x;
-  int v[4];
+  unsigned v[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) v[j] = (i0 + j < n) ? in[i0 + j] : 0;
-  const int t = v[0] + v[1] + v[2] + v[3];
-  int total;
-  int run = block_exclusive_scan(t, warp_sums, total);
+  for (int j = 0; j < 4; ++j) v[j] = (i0 + j < n) ? scan_value<OF>(S, int(i0 + j)) : 0u;
+  const unsigned t = v[0] + v[1] + v[2] + v[3];
+  unsigned total;
+  unsigned run = block_exclusive_scan(t, warp_sums, total);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     if (i0 + j < n) out[i0 + j] = run;
     run += v[j];
   }
-  if (threadIdx.x == 0) tile_sum[blockIdx.x] = total;
+  if (threadIdx.x == 0) S.tile_sum[blockIdx.x] = int(total);
 }
 
-__global__ void __launch_bounds__(1024) k_scan_tile_sums(int* __restrict__ tile_sum, const int* __restrict__ np,
-                                                         int* __restrict__ out) {
-  __shared__ int warp_sums[32];
-  const int n = *np;
-  const int ntiles = (n + kScanTile - 1) / kScanTile;
-  int carry = 0;
-  for (int c = 0; c < ntiles; c += 1024) {
-    const int i = c + threadIdx.x;
-    const int v = i < ntiles ? tile_sum[i] : 0;
-    int total;
-    const int ex = block_exclusive_scan(v, warp_sums, total);
-    if (i < ntiles) tile_sum[i] = carry + ex;
+template <int OF>
+__global__ void __launch_bounds__(1024) k_scan_one(Scratch S, unsigned* __restrict__ out) {
+  __shared__ unsigned warp_sums[32];
+  const int n = *S.ncomp;
+  unsigned carry = 0;
+  for (int base = 0; base < n; base += kScanTile) {
+    const int i0 = base + 4 * threadIdx.x;
+    unsigned v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = (i0 + j < n) ? scan_value<OF>(S, i0 + j) : 0u;
+    const unsigned t = v[0] + v[1] + v[2] + v[3];
+    unsigned total;
+    unsigned run = carry + block_exclusive_scan(t, warp_sums, total);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (i0 + j < n) out[i0 + j] = run;
+      run += v[j];
+    }
     carry += total;
   }
   if (threadIdx.x == 0) out[n] = carry;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_add(int* __restrict__ out, const int* __restrict__ tile_sum,
-                                                   const int* __restrict__ np) {
-  const int n = *np;
+__global__ void __launch_bounds__(1024) k_scan_tile_sums(Scratch S, unsigned* __restrict__ out) {
+  __shared__ unsigned warp_sums[32];
+  const int n = *S.ncomp;
+  const int ntiles = (n + kScanTile - 1) / kScanTile;
+  unsigned carry = 0;
+  for (int c = 0; c < ntiles; c += 1024) {
+    const int i = c + threadIdx.x;
+    const unsigned v = i < ntiles ? unsigned(S.tile_sum[i]) : 0u;
+    unsigned total;
+    const unsigned ex = block_exclusive_scan(v, warp_sums, total);
+    if (i < ntiles) S.tile_sum[i] = int(carry + ex);
+    carry += total;
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
+__global__ void __launch_bounds__(1024) k_scan_add(Scratch S, unsigned* __restrict__ out) {
+  const int n = *S.ncomp;
   const long long base = (long long)blockIdx.x * kScanTile;
   if (base >= n || blockIdx.x == 0) return;
-  const int add = tile_sum[blockIdx.x];
+  const unsigned add = unsigned(S.tile_sum[blockIdx.x]);
   const long long i0 = base + 4LL * threadIdx.x;
 #pragma unroll
   for (int j = 0; j < 4; ++j)
@@ -493,26 +680,31 @@ __global__ void k_cluster_count(Scratch S) {
 }
 
 // Members of each cluster as sort keys (size << 32 | c): contiguous per
-// cluster, so that the sort reads and writes no scattered data.
+// cluster, so that the sort reads and writes no scattered data.  The clusters
+// for a warp (above kThreadCluster members) go to its list.
 __global__ void k_cluster_fill(Scratch S) {
   FOR_COMPONENTS(c) {
     if (!S.small[c]) continue;
     const int r = find_root(S.cpar, c, S.err);
-    S.cl_key[S.cl_off[r] + atomicAdd(S.cl_count + r, 1)] =
+    if (r == c) {
+      const int n = int(S.cl_off[c + 1] - S.cl_off[c]);
+      if (n > kHugeCluster) S.big[atomicAdd(S.nbig, 1)] = c;
+      else if (n > kThreadCluster) S.big[*S.ncomp - 1 - atomicAdd(S.nbig + 1, 1)] = c;
+    }
+    S.cl_key[S.cl_off[r] + unsigned(atomicSub(S.cl_count + r, 1) - 1)] =
         ((unsigned long long)(unsigned)S.size[c] << 32) | unsigned(c);
   }
 }
 
 // Squared distance of the mean colours of components a and b, in a fixed
 // order without contractions.
+__device__ __forceinline__ double dist2_of(double a0, double a1, double a2, double b0, double b1, double b2) {
+  const double t0 = __dsub_rn(a0, b0), t1 = __dsub_rn(a1, b1), t2 = __dsub_rn(a2, b2);
+  return __dadd_rn(__dadd_rn(__dmul_rn(t0, t0), __dmul_rn(t1, t1)), __dmul_rn(t2, t2));
+}
 __device__ __forceinline__ double dist2(const double* mean, int a, int b) {
-  double d = 0.0;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const double t = __dsub_rn(mean[3LL * a + k], mean[3LL * b + k]);
-    d = __dadd_rn(d, __dmul_rn(t, t));
-  }
-  return d;
+  return dist2_of(mean[3LL * a], mean[3LL * a + 1], mean[3LL * a + 2], mean[3LL * b], mean[3LL * b + 1],
+                  mean[3LL * b + 2]);
 }
 
 // Merge of small component r (still its group's founder, still small) into
@@ -543,18 +735,14 @@ __device__ __forceinline__ void sort_keys(unsigned long long* key, int n) {
 }
 
 // One thread per cluster of at most kThreadCluster members: the sequential
-// rule over the members in (size, index) order.  Larger clusters go to the
-// list of the warp kernel.
-__global__ void k_cluster_merge(const Img* __restrict__ imgs, Scratch S) {
+// rule over the members in (size, index) order.
+__device__ __forceinline__ unsigned merge_small_clusters(const Img* __restrict__ imgs, Scratch& S, int first, int step) {
   unsigned merged = 0;
-  FOR_COMPONENTS(c) {
+  const int ncomp = *S.ncomp;
+  for (int c = first; c < ncomp; c += step) {
     if (!S.small[c] || S.cpar[c] != c) continue;  // not a cluster root
-    const int n = S.cl_off[c + 1] - S.cl_off[c];
-    if (n > kThreadCluster) {
-      if (n > kHugeCluster) S.big[atomicAdd(S.nbig, 1)] = c;
-      else S.big[*S.ncomp - 1 - atomicAdd(S.nbig + 1, 1)] = c;
-      continue;
-    }
+    const int n = int(S.cl_off[c + 1] - S.cl_off[c]);
+    if (n > kThreadCluster) continue;
     const Img im = imgs[S.cimg[c]];
     const long long N = (long long)im.W * im.H;
     unsigned long long* key = S.cl_key + S.cl_off[c];
@@ -566,7 +754,8 @@ __global__ void k_cluster_merge(const Img* __restrict__ imgs, Scratch S) {
       double bd = 0.0;
       int hops = 0;
       for (int m = r; m >= 0 && hops < kMaxHops; m = S.next[m], ++hops) {
-        for (int q = S.aoff[m]; q < S.aoff[m + 1]; ++q) {
+        const unsigned q0 = S.aoff[m], q1 = q0 + unsigned(S.deg[m]);
+        for (unsigned q = q0; q < q1; ++q) {
           const int g = find_group(S.gpar, S.adj[q], S.err);
           if (g == r) continue;
           const double d = dist2(S.mean, r, g);
@@ -582,102 +771,179 @@ __global__ void k_cluster_merge(const Img* __restrict__ imgs, Scratch S) {
       ++merged;
     }
   }
-  merged = __reduce_add_sync(0xffffffffu, merged);
-  if ((threadIdx.x & 31) == 0 && merged) atomicAdd(S.cnt + 1, (unsigned long long)merged);
+  return merged;
 }
 
-// One warp per cluster above kThreadCluster members, the clusters above
-// kHugeCluster members first (the longest serial chains start earliest).
-// The keys are sorted in
-// shared memory (bitonic; clusters above kWarpSortMax members are sorted in
-// place by one lane), then the members are taken in order as above, with the
-// adjacency entries of each member's group spread over the lanes and the
-// nearest group found by a warp reduction on (distance, group index) -- the
-// same minimum the sequential scan finds.  __syncwarp orders lane 0's merge
-// writes before the next member's reads.
-__global__ void __launch_bounds__(kMergeWarps * 32) k_cluster_merge_warp(const Img* __restrict__ imgs, Scratch S) {
-  __shared__ unsigned long long sk[kMergeWarps][kWarpSortMax];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nhuge = S.nbig[0], nbig = S.nbig[0] + S.nbig[1], ncomp = *S.ncomp;
+// The nearest group over the lanes: the smallest distance (doubles >= 0 order
+// like their bits), then the smallest group index; 0x7fffffff where no lane
+// has one.
+__device__ __forceinline__ int warp_nearest(double bd, int best) {
+  const unsigned hi = unsigned(__double2hiint(bd)), lo = unsigned(__double2loint(bd));
+  const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : ~0u);
+  return __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? best : 0x7fffffff);
+}
+
+// A member's data that no merge changes, fetched ahead of its turn: its list's
+// place, its first 32 neighbours (one per lane), and the mean colours.
+struct Member {
+  int r = -1;
+  unsigned q0 = 0, deg = 0;
+  int adj = -1;
+  double mr[3], ma[3];
+  __device__ __forceinline__ void list(const Scratch& S, int r_) {
+    r = r_;
+    q0 = S.aoff[r];
+    deg = unsigned(S.deg[r]);
+  }
+  __device__ __forceinline__ void neighbours(const Scratch& S, int lane) { adj = unsigned(lane) < deg ? S.adj[q0 + lane] : -1; }
+  __device__ __forceinline__ void means(const Scratch& S) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      mr[k] = S.mean[3LL * r + k];
+      ma[k] = adj >= 0 ? S.mean[3LL * adj + k] : 0.0;
+    }
+  }
+};
+
+// One warp per cluster above kThreadCluster members (list entry b).  The keys
+// are sorted in shared memory (bitonic; clusters above kWarpSortMax members
+// are sorted in place by one lane), then the members are taken in order as
+// above, with the adjacency entries of each member's group spread over the
+// lanes.  The chain over the members of the largest cluster sets the time, so
+// what no merge changes is fetched one to three members ahead.  __syncwarp
+// orders lane 0's merge writes before the next member's reads.
+__device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, Scratch& S, int c,
+                                                  unsigned long long* sk, int lane) {
   unsigned merged = 0;
-  for (int b = blockIdx.x * kMergeWarps + warp; b < nbig; b += gridDim.x * kMergeWarps) {
-    const int c = b < nhuge ? S.big[b] : S.big[ncomp - 1 - (b - nhuge)];
-    const Img im = imgs[S.cimg[c]];
-    const long long N = (long long)im.W * im.H;
-    unsigned long long* gkey = S.cl_key + S.cl_off[c];
-    const int n = S.cl_off[c + 1] - S.cl_off[c];
-    const unsigned long long* key = sk[warp];
-    if (n <= kWarpSortMax) {
-      int P = 32;
-      while (P < n) P <<= 1;
-      unsigned long long* k = sk[warp];
-      for (int i = lane; i < P; i += 32) k[i] = i < n ? gkey[i] : ~0ull;
-      __syncwarp();
-      for (int w = 2; w <= P; w <<= 1)
-        for (int j = w >> 1; j > 0; j >>= 1) {
-          for (int i = lane; i < P; i += 32) {
-            const int l = i ^ j;
-            if (l > i) {
-              const unsigned long long x = k[i], y = k[l];
-              if ((x > y) == ((i & w) == 0)) {
-                k[i] = y;
-                k[l] = x;
-              }
+  const Img im = imgs[S.cimg[c]];
+  const long long N = (long long)im.W * im.H;
+  unsigned long long* gkey = S.cl_key + S.cl_off[c];
+  const int n = int(S.cl_off[c + 1] - S.cl_off[c]);
+  const unsigned long long* key = sk;
+  if (n <= kWarpSortMax) {
+    int P = 32;
+    while (P < n) P <<= 1;
+    for (int i = lane; i < P; i += 32) sk[i] = i < n ? gkey[i] : ~0ull;
+    __syncwarp();
+    for (int w = 2; w <= P; w <<= 1)
+      for (int j = w >> 1; j > 0; j >>= 1) {
+        for (int i = lane; i < P; i += 32) {
+          const int l = i ^ j;
+          if (l > i) {
+            const unsigned long long x = sk[i], y = sk[l];
+            if ((x > y) == ((i & w) == 0)) {
+              sk[i] = y;
+              sk[l] = x;
             }
           }
-          __syncwarp();
         }
-    } else {
-      if (lane == 0) {
-        if (n > kMaxCluster) atomicExch(S.err, 1);
-        else sort_keys(gkey, n);
+        __syncwarp();
       }
-      __syncwarp();
-      if (n > kMaxCluster) continue;
-      key = gkey;
+  } else {
+    if (lane == 0) {
+      if (n > kMaxCluster) atomicExch(S.err, 1);
+      else sort_keys(gkey, n);
     }
-    for (int a = 0; a < n; ++a) {
-      const int r = int(unsigned(key[a]));
-      if (S.gpar[r] != r || !small_size(S.gsize[r], im.K, N)) continue;  // warp-uniform
-      int best = 0x7fffffff;
-      double bd = INFINITY;
-      int hops = 0;
-      for (int m = r; m >= 0 && hops < kMaxHops; m = S.next[m], ++hops) {
-        const int q1 = S.aoff[m + 1];
-        for (int q = S.aoff[m] + lane; q < q1; q += 32) {
-          const int g = find_group(S.gpar, S.adj[q], S.err);
-          if (g == r) continue;
-          const double d = dist2(S.mean, r, g);
-          if (d < bd || (d == bd && g < best)) {
-            best = g;
-            bd = d;
-          }
-        }
-      }
-      if (hops >= kMaxHops && lane == 0) atomicExch(S.err, 1);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double d2 = __shfl_xor_sync(0xffffffffu, bd, o);
-        const int g2 = __shfl_xor_sync(0xffffffffu, best, o);
-        if (d2 < bd || (d2 == bd && g2 < best)) {
-          bd = d2;
-          best = g2;
-        }
-      }
-      if (best != 0x7fffffff && lane == 0) {
-        merge_into(S, r, best);
-        ++merged;
-      }
-      __syncwarp();
+    __syncwarp();
+    if (n > kMaxCluster) return 0;
+    key = gkey;
+  }
+  const auto member = [&](int a) { return int(unsigned(key[a])); };
+  Member m0, m1, m2;  // this member, the next, the one after
+  m0.list(S, member(0));
+  m0.neighbours(S, lane);
+  m0.means(S);
+  if (n > 1) {
+    m1.list(S, member(1));
+    m1.neighbours(S, lane);
+  }
+  if (n > 2) m2.list(S, member(2));
+  for (int a = 0; a < n; ++a) {
+    const Member me = m0;
+    if (a + 1 < n) {
+      m0 = m1;
+      m0.means(S);
     }
-    __syncwarp();  // sk[warp] is refilled by the next cluster
+    if (a + 2 < n) {
+      m1 = m2;
+      m1.neighbours(S, lane);
+    }
+    if (a + 3 < n) m2.list(S, member(a + 3));
+    const int r = me.r;
+    if (S.gpar[r] != r || !small_size(S.gsize[r], im.K, N)) continue;  // warp-uniform
+    int best = 0x7fffffff;
+    double bd = INFINITY;
+    auto consider = [&](int g, double x, double y, double z) {
+      if (g == r) return;
+      const double d = dist2_of(me.mr[0], me.mr[1], me.mr[2], x, y, z);
+      if (d < bd || (d == bd && g < best)) {
+        best = g;
+        bd = d;
+      }
+    };
+    if (me.adj >= 0) {
+      const int g = find_group(S.gpar, me.adj, S.err);
+      if (g == me.adj) consider(g, me.ma[0], me.ma[1], me.ma[2]);
+      else consider(g, S.mean[3LL * g], S.mean[3LL * g + 1], S.mean[3LL * g + 2]);
+    }
+    int hops = 0;
+    for (int m = r; m >= 0 && hops < kMaxHops; m = S.next[m], ++hops) {
+      const unsigned q0 = m == r ? me.q0 : S.aoff[m], q1 = q0 + (m == r ? me.deg : unsigned(S.deg[m]));
+      for (unsigned q = q0 + lane + (m == r ? 32u : 0u); q < q1; q += 32) {
+        const int g = find_group(S.gpar, S.adj[q], S.err);
+        consider(g, S.mean[3LL * g], S.mean[3LL * g + 1], S.mean[3LL * g + 2]);
+      }
+    }
+    if (hops >= kMaxHops && lane == 0) atomicExch(S.err, 1);
+    best = warp_nearest(bd, best);
+    if (best != 0x7fffffff && lane == 0) {
+      merge_into(S, r, best);
+      ++merged;
+    }
+    __syncwarp();
+  }
+  __syncwarp();  // sk is refilled by the next cluster
+  return merged;
+}
+
+// All clusters in one launch: the first `warp_blocks` blocks take the list of
+// the larger ones, a warp each, those above kHugeCluster members first (the
+// longest serial chains start earliest); the other blocks take the clusters of
+// one or two members, a thread each, beside them.
+__global__ void __launch_bounds__(kMergeWarps * 32) k_cluster_merge(const Img* __restrict__ imgs, Scratch S,
+                                                                   int warp_blocks) {
+  __shared__ unsigned long long sk[kMergeWarps][kWarpSortMax];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  unsigned merged = 0;
+  if (int(blockIdx.x) < warp_blocks) {
+    const int nhuge = S.nbig[0], nbig = S.nbig[0] + S.nbig[1], ncomp = *S.ncomp;
+    for (int b = blockIdx.x * kMergeWarps + warp; b < nbig; b += warp_blocks * kMergeWarps)
+      merged += merge_cluster(imgs, S, b < nhuge ? S.big[b] : S.big[ncomp - 1 - (b - nhuge)], sk[warp], lane);
+  } else {
+    const int blocks = int(gridDim.x) - warp_blocks;
+    merged = merge_small_clusters(imgs, S, (int(blockIdx.x) - warp_blocks) * int(blockDim.x) + int(threadIdx.x),
+                                  blocks * int(blockDim.x));
   }
   merged = __reduce_add_sync(0xffffffffu, merged);
   if (lane == 0 && merged) atomicAdd(S.cnt + 1, (unsigned long long)merged);
 }
 
+// The label of every merged component's group founder, in the place of its own
+// (a component that is its own group keeps its label).
+__global__ void k_group_label(Scratch S) {
+  FOR_COMPONENTS(c) {
+    const int g = S.gpar[c];
+    if (g != c) S.next[c] = S.clabel[find_root(S.gpar, g, S.err)];  // the member lists are done with
+  }
+}
+
+// Pixels of merged components only: the others have their label already.
 __global__ void k_relabel(const Img* __restrict__ imgs, Scratch S) {
-  FOR_PIXELS(im, i) im.labels[i] = S.clabel[find_root(S.gpar, S.parent[im.off + i], S.err)];
+  FOR_PIXELS(im, i) {
+    const int c = S.parent[im.off + i];
+    if (S.gpar[c] != c) im.labels[i] = S.next[c];
+  }
 }
 
 }  // namespace conn
@@ -709,10 +975,10 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   for (int j = 0; j < kIntArrays; ++j) { o[j] = off; off += nI; }
   o[O_AOFF] = off; off += nI1;
   o[O_CLOFF] = off; off += nI1;
-  o[O_ADJ] = off; off += up(size_t(T) * 16);   // <= 2 edges per pixel, 2 entries per edge
+  o[O_ADJ] = off; off += up(size_t(T) * 16);   // 2 size + 2 <= 4 size entries per small component
   o[O_CSUM] = off; off += up(size_t(T) * 24);
   o[O_TABLE] = off; off += up(sizeof(Img) * n);
-  o[O_CNT] = off; off += 256;
+  o[O_CNT] = off; off += 256;                  // behind the table: uploaded (as zeros) with it
   o[O_KEY] = off; off += up(size_t(T) * 8);
   o[O_TILE] = off; off += up(size_t(ntiles + 1) * 4);
   void* slab = nullptr;
@@ -746,8 +1012,8 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   S.clabel = reinterpret_cast<int32_t*>(ia(A_CLABEL)); S.small = ia(A_SMALL); S.cpar = ia(A_CPAR);
   S.deg = ia(A_DEG); S.cl_count = ia(A_CLCOUNT); S.big = ia(A_BIG); S.gpar = ia(A_GPAR); S.gsize = ia(A_GSIZE);
   S.next = ia(A_NEXT); S.tail = ia(A_TAIL);
-  S.aoff = ia(O_AOFF);
-  S.cl_off = ia(O_CLOFF);
+  S.aoff = reinterpret_cast<unsigned*>(ia(O_AOFF));
+  S.cl_off = reinterpret_cast<unsigned*>(ia(O_CLOFF));
   S.adj = ia(O_ADJ);
   S.csum = reinterpret_cast<long long*>(b + o[O_CSUM]);
   S.mean = reinterpret_cast<double*>(b + o[O_CSUM]);
@@ -763,42 +1029,61 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   const dim3 gp{static_cast<unsigned>(per), static_cast<unsigned>(n)};
   const int gs = 152 * 8;
   const unsigned nt = unsigned(ntiles);
+  const bool one = T <= kOneBlockScan;
+  // chunks and tiles of an image, four per block, at least enough blocks to fill the machine across the images
+  const auto blocks_of = [&](int w, int h) {
+    long long most = 1;
+    for (int i = 0; i < n; ++i)
+      most = std::max(most, ((W[i] + w - 1LL) / w) * ((H[i] + h - 1LL) / h));
+    return dim3(unsigned(std::max<long long>(1, std::min<long long>((most + 3) / 4, (152LL * 64 + n - 1) / n))), unsigned(n));
+  };
+  // rows a warp walks: 32, fewer where that would leave most of the machine idle (the walk over a chunk is serial)
+  long long chunk_cols = 0;
+  for (int i = 0; i < n; ++i) chunk_cols += (W[i] + kChunk - 1LL) / kChunk * H[i];
+  int rows = kChunkRows;
+  while (rows > 4 && chunk_cols / rows < 152LL * 32) rows /= 2;
+  const dim3 gt = blocks_of(kCcTile, kCcTile), gc = blocks_of(kChunk, rows);
+  const int warp_blocks = int(std::max<long long>(1, std::min<long long>(152 * 7, (T + 4095) / 4096 * 4)));
+  const int thread_blocks = int(std::max<long long>(1, std::min<long long>(152 * 7, (T + 1023) / 1024)));
+  std::vector<char> up_host(o[O_CNT] + 256 - o[O_TABLE], 0);
+  memcpy(up_host.data(), host.data(), sizeof(Img) * n);
+  char back[256] = {};
   unsigned long long hc[3] = {};
   int herr = 0;
   do {
-    if ((e = cudaMemcpyAsync(table, host.data(), sizeof(Img) * n, cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(S.size, 0, nI, s)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(S.csum, 0, up(size_t(T) * 24), s)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(S.deg, 0, nI, s)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(S.cl_count, 0, nI, s)) != cudaSuccess) break;
-    if ((e = cudaMemsetAsync(S.cnt, 0, 256, s)) != cudaSuccess) break;
-    k_cc_init<<<gp, 256, 0, s>>>(table, S.parent);
-    k_cc_union<<<gp, 256, 0, s>>>(table, S.parent, S.err);
-    k_cc_flatten<<<gp, 256, 0, s>>>(table, S.parent, S.err);
-    k_root_count<<<nt, 1024, 0, s>>>(T, S);
+    if ((e = cudaMemcpyAsync(table, up_host.data(), up_host.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
+    k_cc_tile<<<gt, kCcWarps * 32, 0, s>>>(table, S.parent, S.err);
+    k_cc_border<<<gp, 256, 0, s>>>(table, S.parent, S.err);
+    k_cc_flatten<<<nt, 1024, 0, s>>>(T, S);
     k_root_scan<<<1, 1024, 0, s>>>(int(ntiles), S);
     k_root_assign<<<nt, 1024, 0, s>>>(table, n, T, S);
-    k_comp_map<<<gp, 256, 0, s>>>(table, S);
+    k_comp_map<<<gc, 128, 0, s>>>(table, S, rows);
     k_comp_flags<<<gs, 256, 0, s>>>(table, S);
-    k_edges<<<gp, 256, 0, s>>>(table, S, 0);
-    k_scan_tiles<<<nt, 1024, 0, s>>>(S.deg, S.ncomp, S.aoff, S.tile_sum);
-    k_scan_tile_sums<<<1, 1024, 0, s>>>(S.tile_sum, S.ncomp, S.aoff);
-    k_scan_add<<<nt, 1024, 0, s>>>(S.aoff, S.tile_sum, S.ncomp);
-    if ((e = cudaMemsetAsync(S.deg, 0, nI, s)) != cudaSuccess) break;
-    k_edges<<<gp, 256, 0, s>>>(table, S, 1);
+    if (one) {
+      k_scan_one<kScanLists><<<1, 1024, 0, s>>>(S, S.aoff);
+    } else {
+      k_scan_tiles<kScanLists><<<nt, 1024, 0, s>>>(S, S.aoff);
+      k_scan_tile_sums<<<1, 1024, 0, s>>>(S, S.aoff);
+      k_scan_add<<<nt, 1024, 0, s>>>(S, S.aoff);
+    }
+    k_edges<<<gc, 128, 0, s>>>(table, S, rows);
     k_cluster_count<<<gs, 256, 0, s>>>(S);
-    k_scan_tiles<<<nt, 1024, 0, s>>>(S.cl_count, S.ncomp, S.cl_off, S.tile_sum);
-    k_scan_tile_sums<<<1, 1024, 0, s>>>(S.tile_sum, S.ncomp, S.cl_off);
-    k_scan_add<<<nt, 1024, 0, s>>>(S.cl_off, S.tile_sum, S.ncomp);
-    if ((e = cudaMemsetAsync(S.cl_count, 0, nI, s)) != cudaSuccess) break;
+    if (one) {
+      k_scan_one<kScanClusters><<<1, 1024, 0, s>>>(S, S.cl_off);
+    } else {
+      k_scan_tiles<kScanClusters><<<nt, 1024, 0, s>>>(S, S.cl_off);
+      k_scan_tile_sums<<<1, 1024, 0, s>>>(S, S.cl_off);
+      k_scan_add<<<nt, 1024, 0, s>>>(S, S.cl_off);
+    }
     k_cluster_fill<<<gs, 256, 0, s>>>(S);
-    k_cluster_merge<<<gs, 256, 0, s>>>(table, S);
-    k_cluster_merge_warp<<<152 * 16, kMergeWarps * 32, 0, s>>>(table, S);
+    k_cluster_merge<<<warp_blocks + thread_blocks, kMergeWarps * 32, 0, s>>>(table, S, warp_blocks);
+    k_group_label<<<gs, 256, 0, s>>>(S);
     k_relabel<<<gp, 256, 0, s>>>(table, S);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
-    if ((e = cudaMemcpyAsync(hc, S.cnt, sizeof(hc), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
-    if ((e = cudaMemcpyAsync(&herr, S.err, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
+    if ((e = cudaMemcpyAsync(back, S.cnt, sizeof(back), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
     e = cudaStreamSynchronize(s);
+    memcpy(hc, back, sizeof(hc));
+    memcpy(&herr, back + 128, sizeof(herr));
   } while (false);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? GMMSP_E_NOMEM : GMMSP_E_CUDA;
   if (herr) return GMMSP_E_TIMEOUT;
