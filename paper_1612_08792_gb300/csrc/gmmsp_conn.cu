@@ -38,8 +38,8 @@
 //   k_edges                         small-small clusters and adjacency lists
 //   k_cluster_count / _fill         member lists as (size << 32 | c) keys
 //   k_cluster_merge                 one thread per cluster of <= kThreadCluster
-//                                   members, one warp per larger cluster (keys
-//                                   sorted in shared memory, adjacency over the lanes)
+//                                   members, one warp per larger cluster (adjacency
+//                                   over the lanes)
 //   k_group_label / k_relabel       label of the group founder
 // One allocation (kept by a context between calls) and one synchronisation
 // per call.  Every loop over a parent chain or a retry is bounded; running
@@ -61,10 +61,9 @@ namespace conn {
 
 constexpr int kMaxHops = 1 << 24;      // bound on any parent-chain walk or union retry
 constexpr int kFixedShift = 20;        // colour sums in units of 2^-20
-constexpr int kMaxCluster = 1 << 16;   // bound on the members a cluster sorted in global memory may have
+constexpr int kMaxCluster = 1 << 16;   // bound on the members of a cluster
 constexpr int kThreadCluster = 2;      // clusters up to this size: one thread; larger: one warp
 constexpr int kHugeCluster = 32;       // warp clusters above this size are started first
-constexpr int kWarpSortMax = 1024;     // members a warp sorts in shared memory
 constexpr int kScanTile = 4096;        // elements per block of the tile kernels (1024 threads x 4)
 constexpr int kMergeWarps = 4;
 constexpr int kCcTile = 32;            // side of the tiles labelled in shared memory
@@ -90,6 +89,7 @@ struct Scratch {
   int* size;                  // pixel count
   long long* csum;            // 3 fixed-point colour sums, then (k_comp_flags) ...
   double* mean;               // ... the 3 mean colours csum / size, in the same memory
+  float4* mean32;             // the means in FP32 and the largest of their magnitudes
   int* cimg;                  // image
   int32_t* clabel;            // its label
   int* small;                 // 1 for a small component
@@ -177,43 +177,40 @@ __device__ __forceinline__ void unite(int* p, int a, int b, int* err) {
 
 __device__ __forceinline__ bool small_size(long long s, int K, long long N) { return 4LL * K * s < N; }
 
-// Per-image pixel loops: blockIdx.y is the image, x strides over its pixels.
-#define FOR_PIXELS(im, i)                                                                    \
-  const Img im = imgs[blockIdx.y];                                                           \
-  const long long im##_N = (long long)im.W * im.H;                                           \
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < im##_N;           \
-       i += (long long)gridDim.x * blockDim.x)
-
 // Per-component loops over c < *S.ncomp.
 #define FOR_COMPONENTS(c)      \
   const int ncomp_ = *S.ncomp; \
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncomp_; c += gridDim.x * blockDim.x)
 
-// Labels one 32 x 32 tile per warp in shared memory: every pixel starts under
+// Labels one tile of 32 x 32 pixels (x tile_rows where the call has few pixels:
+// a tile is a serial walk) per warp in shared memory: every pixel starts under
 // the first pixel of its row's run of one label (a ballot), and one union per
 // pair of vertically adjacent runs (at the leftmost pixel of their overlap)
-// links the rows as the warp walks down.  Local indices order like pixels, so
+// is queued and then done 32 at a time.  Local indices order like pixels, so
 // a tile's root is the smallest pixel of its piece of the component.  Then
 // parent = the root's pixel.  Only the tiles' borders are left to global
 // unions: 6 % of the pixels (labelling all of them in global memory took
 // 195 + 703 us on 256 images of 481x321).
 __global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict__ imgs, int* __restrict__ p,
-                                                          int* err) {
+                                                          int* err, int tile_rows) {
   __shared__ int sp[kCcWarps][kCcTile * kCcTile];
+  __shared__ uint16_t queue[kCcWarps][kCcTile * kCcTile], first[kCcWarps][kCcTile * kCcTile];
   const Img im = imgs[blockIdx.y];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tx = (im.W + kCcTile - 1) / kCcTile;
-  const long long tiles = (long long)tx * ((im.H + kCcTile - 1) / kCcTile);
+  const long long tiles = (long long)tx * ((im.H + tile_rows - 1) / tile_rows);
   int* q = sp[warp];
+  uint16_t *Q = queue[warp], *F = first[warp];  // the unions; the runs' first pixels
   for (long long t = (long long)blockIdx.x * kCcWarps + warp; t < tiles; t += (long long)gridDim.x * kCcWarps) {
-    const int ty = int(t / tx), x0 = int(t - (long long)ty * tx) * kCcTile, y0 = ty * kCcTile;
-    const int rows = min(kCcTile, im.H - y0);
+    const int ty = int(t / tx), x0 = int(t - (long long)ty * tx) * kCcTile, y0 = ty * tile_rows;
+    const int rows = min(tile_rows, im.H - y0);
     const bool in = x0 + lane < im.W;
     const long long g0 = (long long)y0 * im.W + x0;
     const int32_t* L = im.labels + g0 + lane;
     int32_t next[kCcAhead], up = 0;  // the labels of the next rows, loaded ahead
 #pragma unroll
     for (int j = 0; j < kCcAhead; ++j) next[j] = in && j < rows ? L[(long long)j * im.W] : 0;
+    int queued = 0, runs = 0;
     for (int r0 = 0; r0 < rows; r0 += kCcAhead) {
 #pragma unroll
       for (int j = 0; j < kCcAhead; ++j) {
@@ -225,27 +222,39 @@ __global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict
         const bool left_same = in && lane > 0 && lprev == l;
         const unsigned heads = __ballot_sync(0xffffffffu, !left_same);
         q[r * 32 + lane] = r * 32 + 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-        __syncwarp();
-        if (in && r > 0 && l == up && !(left_same && uprev == l)) unite(q, r * 32 + lane, (r - 1) * 32 + lane, err);
-        __syncwarp();
+        const bool join = in && r > 0 && l == up && !(left_same && uprev == l);
+        const unsigned joins = __ballot_sync(0xffffffffu, join);
+        if (join) Q[queued + __popc(joins & ((1u << lane) - 1u))] = uint16_t(r * 32 + lane);
+        queued += __popc(joins);
+        if (!left_same) F[runs + __popc(heads & ((1u << lane) - 1u))] = uint16_t(r * 32 + lane);
+        runs += __popc(heads);
         up = l;
       }
     }
-    for (int r = 0; r < rows; ++r) {
-      const int root = find_root(q, r * 32 + lane, err);
-      if (in) p[im.off + g0 + (long long)r * im.W + lane] = int(im.off + g0 + (long long)(root >> 5) * im.W + (root & 31));
+    __syncwarp();
+    for (int i = lane; i < queued; i += 32) unite(q, Q[i], Q[i] - 32, err);
+    __syncwarp();
+    // the runs' roots, from the top, each kept for the runs below (their chains
+    // are then two or three links long); then every pixel has its run's
+    for (int i = lane; i < runs; i += 32) q[F[i]] = find_root(q, F[i], err);
+    __syncwarp();
+    int* P = p + im.off + g0 + lane;
+    const int at0 = int(im.off + g0);
+    for (int r = 0; r < rows; ++r, P += im.W) {
+      const int root = q[q[r * 32 + lane]];
+      if (in) *P = at0 + (root >> 5) * im.W + (root & 31);  // pixel numbers of a call stay below 2^30
     }
     __syncwarp();  // the tile's array is refilled
   }
 }
 
 // The unions across the tiles' borders: pixels x = 32 k with their left
-// neighbour, pixels y = 32 k with the one above.  A pair that the previous one
+// neighbour, pixels y = tile_rows k with the one above.  A pair that the previous one
 // along the border already joined (both pairs of one label, inside the same
 // two tiles) is skipped.
-__global__ void k_cc_border(const Img* __restrict__ imgs, int* p, int* err) {
+__global__ void k_cc_border(const Img* __restrict__ imgs, int* p, int* err, int tile_rows) {
   const Img im = imgs[blockIdx.y];
-  const int nx = (im.W - 1) / kCcTile, ny = (im.H - 1) / kCcTile;
+  const int nx = (im.W - 1) / kCcTile, ny = (im.H - 1) / tile_rows;
   const long long vertical = (long long)nx * im.H, total = vertical + (long long)ny * im.W;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
     int x, y;
@@ -257,12 +266,12 @@ __global__ void k_cc_border(const Img* __restrict__ imgs, int* p, int* err) {
       x = (k + 1) * kCcTile;
       other = -1;
       back = -(long long)im.W;
-      first = y % kCcTile == 0;
+      first = y % tile_rows == 0;
     } else {
       const long long j = i - vertical;
       const int k = int(j / im.W);
       x = int(j - (long long)k * im.W);
-      y = (k + 1) * kCcTile;
+      y = (k + 1) * tile_rows;
       other = -(long long)im.W;
       back = -1;
       first = x % kCcTile == 0;
@@ -363,7 +372,9 @@ __global__ void __launch_bounds__(1024) k_root_scan(int ntiles, Scratch S) {
 
 __global__ void __launch_bounds__(1024) k_root_assign(const Img* __restrict__ imgs, int n, long long T, Scratch S) {
   __shared__ unsigned warp_sums[32];
-  const long long g0 = (long long)blockIdx.x * kScanTile + 4LL * threadIdx.x;
+  __shared__ uint16_t root[kScanTile];  // the tile's roots in order, so that a thread takes one
+  __shared__ int first_image;
+  const long long base = (long long)blockIdx.x * kScanTile, g0 = base + 4LL * threadIdx.x;
   bool f[4];
   int cnt = 0;
 #pragma unroll
@@ -371,15 +382,18 @@ __global__ void __launch_bounds__(1024) k_root_assign(const Img* __restrict__ im
     f[j] = g0 + j < T && S.parent[g0 + j] == int(g0 + j);
     cnt += f[j];
   }
+  if (threadIdx.x == 0) first_image = image_of(imgs, n, base);
   unsigned total;
-  int c = S.tile_sum[blockIdx.x] + int(block_exclusive_scan(unsigned(cnt), warp_sums, total));
-  // the tile's first image once per warp; a pixel's image from there on
-  int i = 0;
-  if (cnt) i = image_of(imgs, n, (long long)blockIdx.x * kScanTile);
+  unsigned at = block_exclusive_scan(unsigned(cnt), warp_sums, total);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (!f[j]) continue;
-    const long long g = g0 + j;
+  for (int j = 0; j < 4; ++j)
+    if (f[j]) root[at++] = uint16_t(4 * threadIdx.x + j);
+  __syncthreads();
+  const int c0 = S.tile_sum[blockIdx.x];
+  for (unsigned k = threadIdx.x; k < total; k += 1024) {
+    const long long g = base + root[k];
+    const int c = c0 + int(k);
+    int i = first_image;
     while (i + 1 < n && imgs[i + 1].off <= g) ++i;
     S.cidr[g] = c;
     S.cimg[c] = i;
@@ -388,8 +402,7 @@ __global__ void __launch_bounds__(1024) k_root_assign(const Img* __restrict__ im
     S.deg[c] = 0;
     S.cl_count[c] = 0;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) S.csum[3LL * c + k] = 0;
-    ++c;
+    for (int q = 0; q < 3; ++q) S.csum[3LL * c + q] = 0;
   }
 }
 
@@ -422,20 +435,29 @@ __global__ void __launch_bounds__(128) k_comp_map(const Img* __restrict__ imgs, 
     };
     int* P = S.parent + im.off + (long long)y0 * im.W + x;
     const float* Z = im.lab + (long long)y0 * im.W + x;
+    int qn[4] = {};
+    float zn[3][4] = {};  // the next row's
+    auto ahead = [&](const int* p, const float* z) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (j < n) {
+          qn[j] = p[j];
+#pragma unroll
+          for (int k = 0; k < 3; ++k) zn[k][j] = __ldg(z + k * N + j);
+        }
+    };
+    ahead(P, Z);
     for (int r = 0; r < rows; ++r, P += im.W, Z += im.W) {
       int q[4], cq[4];
       float z[3][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        q[j] = -1;
-        if (j < n) {
-          q[j] = P[j];
+        q[j] = qn[j];
+        cq[j] = j < n ? S.cidr[q[j]] : 0;
 #pragma unroll
-          for (int k = 0; k < 3; ++k) z[k][j] = __ldg(Z + k * N + j);
-        }
+        for (int k = 0; k < 3; ++k) z[k][j] = zn[k][j];
       }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) cq[j] = j < n ? S.cidr[q[j]] : 0;
+      if (r + 1 < rows) ahead(P + im.W, Z + im.W);
       auto add = [&](int j) {
         if (j >= n) return;
         if (q[j] != root) {
@@ -475,8 +497,11 @@ __global__ void __launch_bounds__(256) k_comp_flags(const Img* __restrict__ imgs
       const int sz = S.size[c];
       sm = small_size(sz, im.K, (long long)im.W * im.H);
       S.small[c] = sm ? 1 : 0;
+      double m[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) S.mean[3LL * c + k] = double(S.csum[3LL * c + k]) / double(sz);
+      for (int k = 0; k < 3; ++k) S.mean[3LL * c + k] = m[k] = double(S.csum[3LL * c + k]) / double(sz);
+      const float x = float(m[0]), y = float(m[1]), z = float(m[2]);
+      S.mean32[c] = make_float4(x, y, z, fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z))));
       S.gpar[c] = c;
       S.gsize[c] = sz;
       S.cpar[c] = c;
@@ -682,17 +707,29 @@ __global__ void k_cluster_count(Scratch S) {
 // Members of each cluster as sort keys (size << 32 | c): contiguous per
 // cluster, so that the sort reads and writes no scattered data.  The clusters
 // for a warp (above kThreadCluster members) go to its list.
-__global__ void k_cluster_fill(Scratch S) {
-  FOR_COMPONENTS(c) {
-    if (!S.small[c]) continue;
-    const int r = find_root(S.cpar, c, S.err);
-    if (r == c) {
-      const int n = int(S.cl_off[c + 1] - S.cl_off[c]);
-      if (n > kHugeCluster) S.big[atomicAdd(S.nbig, 1)] = c;
-      else if (n > kThreadCluster) S.big[*S.ncomp - 1 - atomicAdd(S.nbig + 1, 1)] = c;
+__global__ void __launch_bounds__(256) k_cluster_fill(Scratch S) {
+  const int ncomp = *S.ncomp;
+  __shared__ int n_of[2], at_of[2];  // huge and other clusters of this step: their number, their place in the list
+  for (int base = blockIdx.x * 256; base < ncomp; base += gridDim.x * 256) {
+    const int c = base + threadIdx.x;
+    if (threadIdx.x < 2) n_of[threadIdx.x] = 0;
+    __syncthreads();
+    int kind = -1, at = 0;
+    if (c < ncomp && S.small[c]) {
+      const int r = find_root(S.cpar, c, S.err);
+      const unsigned off = S.cl_off[r];
+      if (r == c) {
+        const int n = int(S.cl_off[c + 1] - off);
+        kind = n > kHugeCluster ? 0 : (n > kThreadCluster ? 1 : -1);
+        if (kind >= 0) at = atomicAdd(&n_of[kind], 1);
+      }
+      S.cl_key[off + unsigned(atomicSub(S.cl_count + r, 1) - 1)] = ((unsigned long long)(unsigned)S.size[c] << 32) | unsigned(c);
     }
-    S.cl_key[S.cl_off[r] + unsigned(atomicSub(S.cl_count + r, 1) - 1)] =
-        ((unsigned long long)(unsigned)S.size[c] << 32) | unsigned(c);
+    __syncthreads();
+    if (threadIdx.x < 2 && n_of[threadIdx.x]) at_of[threadIdx.x] = atomicAdd(S.nbig + threadIdx.x, n_of[threadIdx.x]);
+    __syncthreads();
+    if (kind == 0) S.big[at_of[0] + at] = c;
+    if (kind == 1) S.big[ncomp - 1 - (at_of[1] + at)] = c;
   }
 }
 
@@ -705,6 +742,19 @@ __device__ __forceinline__ double dist2_of(double a0, double a1, double a2, doub
 __device__ __forceinline__ double dist2(const double* mean, int a, int b) {
   return dist2_of(mean[3LL * a], mean[3LL * a + 1], mean[3LL * a + 2], mean[3LL * b], mean[3LL * b + 1],
                   mean[3LL * b + 2]);
+}
+
+// The same distance in FP32, and how far it may be from the FP64 one: with the
+// means within 2^-24 M of theirs (M the largest magnitude), each difference is
+// off by at most 2^-22 M, its square by 2^-20 M^2, and the rounding of the
+// squares and sums (of at most 12 M^2) adds less than 2.3 2^-20 M^2: below
+// 5.5 2^-20 M^2 in all, taken as 2^-17 M^2.  FP64 runs at 1/64 of the FP32
+// rate here, so a nearest group is found in FP32 and FP64 decides only between
+// those that the bound cannot tell apart.
+__device__ __forceinline__ float dist2_32(float4 a, float4 b, float& off) {
+  const float t0 = a.x - b.x, t1 = a.y - b.y, t2 = a.z - b.z, m = fmaxf(a.w, b.w);
+  off = m * m * 0x1p-17f;
+  return t0 * t0 + t1 * t1 + t2 * t2;
 }
 
 // Merge of small component r (still its group's founder, still small) into
@@ -750,23 +800,50 @@ __device__ __forceinline__ unsigned merge_small_clusters(const Img* __restrict__
     for (int a = 0; a < n; ++a) {
       const int r = int(unsigned(key[a]));
       if (S.gpar[r] != r || !small_size(S.gsize[r], im.K, N)) continue;
+      const float4 mr = S.mean32[r];
       int best = -1;
-      double bd = 0.0;
+      float low = 0.f, high = INFINITY;  // the nearest one's distance lies in [low, high]
+      bool close = false;                // another group may be as near
       int hops = 0;
       for (int m = r; m >= 0 && hops < kMaxHops; m = S.next[m], ++hops) {
         const unsigned q0 = S.aoff[m], q1 = q0 + unsigned(S.deg[m]);
         for (unsigned q = q0; q < q1; ++q) {
           const int g = find_group(S.gpar, S.adj[q], S.err);
-          if (g == r) continue;
-          const double d = dist2(S.mean, r, g);
-          if (best < 0 || d < bd || (d == bd && g < best)) {
+          if (g == r || g == best) continue;
+          float off;
+          const float d = dist2_32(mr, S.mean32[g], off);
+          if (best < 0 || d + off < low) {  // certainly nearer
             best = g;
-            bd = d;
+            low = d - off;
+            high = d + off;
+            close = false;
+          } else if (d - off <= high) {     // not certainly farther
+            close = true;
+            low = fminf(low, d - off);
+            high = fminf(high, d + off);
           }
         }
       }
       if (hops >= kMaxHops) atomicExch(S.err, 1);
       if (best < 0) continue;
+      if (close) {
+        best = -1;
+        double bd = 0.0;
+        for (int m = r, h = 0; m >= 0 && h < kMaxHops; m = S.next[m], ++h) {
+          const unsigned q0 = S.aoff[m], q1 = q0 + unsigned(S.deg[m]);
+          for (unsigned q = q0; q < q1; ++q) {
+            const int g = find_group(S.gpar, S.adj[q], S.err);
+            if (g == r) continue;
+            float off;
+            if (dist2_32(mr, S.mean32[g], off) - off > high) continue;  // certainly not the nearest
+            const double d = dist2(S.mean, r, g);
+            if (best < 0 || d < bd || (d == bd && g < best)) {
+              best = g;
+              bd = d;
+            }
+          }
+        }
+      }
       merge_into(S, r, best);
       ++merged;
     }
@@ -790,7 +867,7 @@ struct Member {
   int r = -1;
   unsigned q0 = 0, deg = 0;
   int adj = -1;
-  double mr[3], ma[3];
+  float4 mr, ma;
   __device__ __forceinline__ void list(const Scratch& S, int r_) {
     r = r_;
     q0 = S.aoff[r];
@@ -798,58 +875,46 @@ struct Member {
   }
   __device__ __forceinline__ void neighbours(const Scratch& S, int lane) { adj = unsigned(lane) < deg ? S.adj[q0 + lane] : -1; }
   __device__ __forceinline__ void means(const Scratch& S) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      mr[k] = S.mean[3LL * r + k];
-      ma[k] = adj >= 0 ? S.mean[3LL * adj + k] : 0.0;
-    }
+    mr = S.mean32[r];
+    ma = adj >= 0 ? S.mean32[adj] : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 };
 
-// One warp per cluster above kThreadCluster members (list entry b).  The keys
-// are sorted in shared memory (bitonic; clusters above kWarpSortMax members
-// are sorted in place by one lane), then the members are taken in order as
-// above, with the adjacency entries of each member's group spread over the
-// lanes.  The chain over the members of the largest cluster sets the time, so
-// what no merge changes is fetched one to three members ahead.  __syncwarp
-// orders lane 0's merge writes before the next member's reads.
-__device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, Scratch& S, int c,
-                                                  unsigned long long* sk, int lane) {
+// One warp per cluster above kThreadCluster members.  The members are ordered
+// by counting the smaller keys of each (keys are distinct), up to 32 through
+// the lanes, more through memory; then they are taken in order as above, with
+// the adjacency entries of each member's group spread over the lanes.  The
+// chain over the members of the largest cluster sets the time, so what no
+// merge changes is fetched one to three members ahead.  __syncwarp orders lane
+// 0's merge writes before the next member's reads.
+__device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, Scratch& S, int c, int* order,
+                                                  int lane) {
   unsigned merged = 0;
   const Img im = imgs[S.cimg[c]];
   const long long N = (long long)im.W * im.H;
-  unsigned long long* gkey = S.cl_key + S.cl_off[c];
+  const unsigned long long* key = S.cl_key + S.cl_off[c];
   const int n = int(S.cl_off[c + 1] - S.cl_off[c]);
-  const unsigned long long* key = sk;
-  if (n <= kWarpSortMax) {
-    int P = 32;
-    while (P < n) P <<= 1;
-    for (int i = lane; i < P; i += 32) sk[i] = i < n ? gkey[i] : ~0ull;
-    __syncwarp();
-    for (int w = 2; w <= P; w <<= 1)
-      for (int j = w >> 1; j > 0; j >>= 1) {
-        for (int i = lane; i < P; i += 32) {
-          const int l = i ^ j;
-          if (l > i) {
-            const unsigned long long x = sk[i], y = sk[l];
-            if ((x > y) == ((i & w) == 0)) {
-              sk[i] = y;
-              sk[l] = x;
-            }
-          }
-        }
-        __syncwarp();
-      }
-  } else {
-    if (lane == 0) {
-      if (n > kMaxCluster) atomicExch(S.err, 1);
-      else sort_keys(gkey, n);
-    }
-    __syncwarp();
-    if (n > kMaxCluster) return 0;
-    key = gkey;
+  if (n > kMaxCluster) {
+    if (lane == 0) atomicExch(S.err, 1);
+    return 0;
   }
-  const auto member = [&](int a) { return int(unsigned(key[a])); };
+  if (n <= 32) {
+    const unsigned long long k = lane < n ? key[lane] : ~0ull;
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += __shfl_sync(0xffffffffu, k, j) < k;
+    if (lane < n) order[rank] = int(unsigned(k));
+  } else {
+    order = S.cidr + S.cl_off[c];  // the roots' indices are not needed any more
+    for (int i = lane; i < n; i += 32) {
+      const unsigned long long k = key[i];
+      int rank = 0;
+#pragma unroll 4
+      for (int j = 0; j < n; ++j) rank += __ldg(key + j) < k;
+      order[rank] = int(unsigned(k));
+    }
+  }
+  __syncwarp();
+  const auto member = [&](int a) { return order[a]; };
   Member m0, m1, m2;  // this member, the next, the one after
   m0.list(S, member(0));
   m0.neighbours(S, lane);
@@ -872,38 +937,74 @@ __device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, 
     if (a + 3 < n) m2.list(S, member(a + 3));
     const int r = me.r;
     if (S.gpar[r] != r || !small_size(S.gsize[r], im.K, N)) continue;  // warp-uniform
+    // this lane's neighbour groups: one that is nearest in FP32, and whether
+    // another may be as near
     int best = 0x7fffffff;
-    double bd = INFINITY;
-    auto consider = [&](int g, double x, double y, double z) {
-      if (g == r) return;
-      const double d = dist2_of(me.mr[0], me.mr[1], me.mr[2], x, y, z);
-      if (d < bd || (d == bd && g < best)) {
+    float low = INFINITY, high = INFINITY;
+    bool close = false;
+    auto consider = [&](int g, float4 mg) {
+      if (g == r || g == best) return;
+      float off;
+      const float d = dist2_32(me.mr, mg, off);
+      if (best == 0x7fffffff || d + off < low) {
         best = g;
-        bd = d;
+        low = d - off;
+        high = d + off;
+        close = false;
+      } else if (d - off <= high) {
+        close = true;
+        low = fminf(low, d - off);
+        high = fminf(high, d + off);
       }
     };
     if (me.adj >= 0) {
       const int g = find_group(S.gpar, me.adj, S.err);
-      if (g == me.adj) consider(g, me.ma[0], me.ma[1], me.ma[2]);
-      else consider(g, S.mean[3LL * g], S.mean[3LL * g + 1], S.mean[3LL * g + 2]);
+      consider(g, g == me.adj ? me.ma : S.mean32[g]);
     }
     int hops = 0;
     for (int m = r; m >= 0 && hops < kMaxHops; m = S.next[m], ++hops) {
       const unsigned q0 = m == r ? me.q0 : S.aoff[m], q1 = q0 + (m == r ? me.deg : unsigned(S.deg[m]));
       for (unsigned q = q0 + lane + (m == r ? 32u : 0u); q < q1; q += 32) {
         const int g = find_group(S.gpar, S.adj[q], S.err);
-        consider(g, S.mean[3LL * g], S.mean[3LL * g + 1], S.mean[3LL * g + 2]);
+        consider(g, S.mean32[g]);
       }
     }
     if (hops >= kMaxHops && lane == 0) atomicExch(S.err, 1);
-    best = warp_nearest(bd, best);
+    // the smallest upper bound over the lanes: what lies above it is out
+    const unsigned hb = __reduce_min_sync(0xffffffffu, high >= 0.f ? __float_as_uint(high) : 0u);
+    const float hmin = __uint_as_float(hb);
+    const bool in = best != 0x7fffffff && low <= hmin;
+    const unsigned lanes = __ballot_sync(0xffffffffu, in);
+    if (lanes == 0u) continue;  // no neighbour
+    const int first = __shfl_sync(0xffffffffu, best, __ffs(lanes) - 1);
+    if (__any_sync(0xffffffffu, in && (close || best != first))) {  // FP64 decides
+      best = 0x7fffffff;
+      double bd = INFINITY;
+      for (int m = r, h = 0; m >= 0 && h < kMaxHops; m = S.next[m], ++h) {
+        const unsigned q0 = S.aoff[m], q1 = q0 + unsigned(S.deg[m]);
+        for (unsigned q = q0 + lane; q < q1; q += 32) {
+          const int g = find_group(S.gpar, S.adj[q], S.err);
+          if (g == r) continue;
+          float off;
+          if (dist2_32(me.mr, S.mean32[g], off) - off > hmin) continue;
+          const double d = dist2(S.mean, r, g);
+          if (d < bd || (d == bd && g < best)) {
+            best = g;
+            bd = d;
+          }
+        }
+      }
+      best = warp_nearest(bd, best);
+    } else {
+      best = first;
+    }
     if (best != 0x7fffffff && lane == 0) {
       merge_into(S, r, best);
       ++merged;
     }
     __syncwarp();
   }
-  __syncwarp();  // sk is refilled by the next cluster
+  __syncwarp();  // `order` is refilled by the next cluster
   return merged;
 }
 
@@ -911,15 +1012,15 @@ __device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, 
 // the larger ones, a warp each, those above kHugeCluster members first (the
 // longest serial chains start earliest); the other blocks take the clusters of
 // one or two members, a thread each, beside them.
-__global__ void __launch_bounds__(kMergeWarps * 32) k_cluster_merge(const Img* __restrict__ imgs, Scratch S,
-                                                                   int warp_blocks) {
-  __shared__ unsigned long long sk[kMergeWarps][kWarpSortMax];
+__global__ void __launch_bounds__(kMergeWarps * 32, 8) k_cluster_merge(const Img* __restrict__ imgs, Scratch S,
+                                                                      int warp_blocks) {
+  __shared__ int order[kMergeWarps][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   unsigned merged = 0;
   if (int(blockIdx.x) < warp_blocks) {
     const int nhuge = S.nbig[0], nbig = S.nbig[0] + S.nbig[1], ncomp = *S.ncomp;
     for (int b = blockIdx.x * kMergeWarps + warp; b < nbig; b += warp_blocks * kMergeWarps)
-      merged += merge_cluster(imgs, S, b < nhuge ? S.big[b] : S.big[ncomp - 1 - (b - nhuge)], sk[warp], lane);
+      merged += merge_cluster(imgs, S, b < nhuge ? S.big[b] : S.big[ncomp - 1 - (b - nhuge)], order[warp], lane);
   } else {
     const int blocks = int(gridDim.x) - warp_blocks;
     merged = merge_small_clusters(imgs, S, (int(blockIdx.x) - warp_blocks) * int(blockDim.x) + int(threadIdx.x),
@@ -938,11 +1039,34 @@ __global__ void k_group_label(Scratch S) {
   }
 }
 
-// Pixels of merged components only: the others have their label already.
-__global__ void k_relabel(const Img* __restrict__ imgs, Scratch S) {
-  FOR_PIXELS(im, i) {
-    const int c = S.parent[im.off + i];
-    if (S.gpar[c] != c) im.labels[i] = S.next[c];
+// Pixels of merged components only: the others have their label already.  A
+// thread takes four consecutive pixels of the call.
+__global__ void __launch_bounds__(256) k_relabel(const Img* __restrict__ imgs, int n, long long T, Scratch S) {
+  __shared__ int first_image;
+  const long long base = 4LL * blockIdx.x * 256, g0 = base + 4 * threadIdx.x;
+  if (threadIdx.x == 0) first_image = image_of(imgs, n, base);
+  __syncthreads();
+  int c[4];
+  if (g0 + 3 < T) {
+    const int4 q = *reinterpret_cast<const int4*>(S.parent + g0);
+    c[0] = q.x;
+    c[1] = q.y;
+    c[2] = q.z;
+    c[3] = q.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c[j] = g0 + j < T ? S.parent[g0 + j] : -1;
+  }
+  int gp[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) gp[j] = c[j] >= 0 ? __ldg(S.gpar + c[j]) : -1;
+  int i = first_image;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (gp[j] == c[j]) continue;
+    const long long g = g0 + j;
+    while (i + 1 < n && imgs[i + 1].off <= g) ++i;
+    imgs[i].labels[g - imgs[i].off] = S.next[c[j]];
   }
 }
 
@@ -969,7 +1093,7 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   const long long ntiles = std::max<long long>(1, (T + kScanTile - 1) / kScanTile);
   enum { A_PARENT, A_CIDR, A_SIZE, A_CIMG, A_CLABEL, A_SMALL, A_CPAR, A_DEG, A_CLCOUNT, A_BIG, A_GPAR, A_GSIZE,
          A_NEXT, A_TAIL, kIntArrays };
-  enum { O_AOFF = kIntArrays, O_CLOFF, O_ADJ, O_CSUM, O_TABLE, O_CNT, O_KEY, O_TILE, kRegions };
+  enum { O_AOFF = kIntArrays, O_CLOFF, O_ADJ, O_CSUM, O_MEAN32, O_TABLE, O_CNT, O_KEY, O_TILE, kRegions };
   size_t o[kRegions];
   size_t off = 0;
   for (int j = 0; j < kIntArrays; ++j) { o[j] = off; off += nI; }
@@ -977,6 +1101,7 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   o[O_CLOFF] = off; off += nI1;
   o[O_ADJ] = off; off += up(size_t(T) * 16);   // 2 size + 2 <= 4 size entries per small component
   o[O_CSUM] = off; off += up(size_t(T) * 24);
+  o[O_MEAN32] = off; off += up(size_t(T) * 16);
   o[O_TABLE] = off; off += up(sizeof(Img) * n);
   o[O_CNT] = off; off += 256;                  // behind the table: uploaded (as zeros) with it
   o[O_KEY] = off; off += up(size_t(T) * 8);
@@ -1017,6 +1142,7 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   S.adj = ia(O_ADJ);
   S.csum = reinterpret_cast<long long*>(b + o[O_CSUM]);
   S.mean = reinterpret_cast<double*>(b + o[O_CSUM]);
+  S.mean32 = reinterpret_cast<float4*>(b + o[O_MEAN32]);
   Img* table = reinterpret_cast<Img*>(b + o[O_TABLE]);
   S.cnt = reinterpret_cast<unsigned long long*>(b + o[O_CNT]);
   S.ncomp = reinterpret_cast<int*>(b + o[O_CNT] + 64);
@@ -1042,9 +1168,11 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   for (int i = 0; i < n; ++i) chunk_cols += (W[i] + kChunk - 1LL) / kChunk * H[i];
   int rows = kChunkRows;
   while (rows > 4 && chunk_cols / rows < 152LL * 32) rows /= 2;
-  const dim3 gt = blocks_of(kCcTile, kCcTile), gc = blocks_of(kChunk, rows);
-  const int warp_blocks = int(std::max<long long>(1, std::min<long long>(152 * 7, (T + 4095) / 4096 * 4)));
-  const int thread_blocks = int(std::max<long long>(1, std::min<long long>(152 * 7, (T + 1023) / 1024)));
+  const int tile_rows = rows < kChunkRows ? 8 : kCcTile;
+  const dim3 gt = blocks_of(kCcTile, tile_rows), gc = blocks_of(kChunk, rows);
+  // merging: half of the resident blocks for either kind of cluster
+  const int warp_blocks = int(std::max<long long>(1, std::min<long long>(152 * 4, (T + 1023) / 1024)));
+  const int thread_blocks = int(std::max<long long>(1, std::min<long long>(152 * 4, (T + 1023) / 1024)));
   std::vector<char> up_host(o[O_CNT] + 256 - o[O_TABLE], 0);
   memcpy(up_host.data(), host.data(), sizeof(Img) * n);
   char back[256] = {};
@@ -1052,8 +1180,8 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   int herr = 0;
   do {
     if ((e = cudaMemcpyAsync(table, up_host.data(), up_host.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
-    k_cc_tile<<<gt, kCcWarps * 32, 0, s>>>(table, S.parent, S.err);
-    k_cc_border<<<gp, 256, 0, s>>>(table, S.parent, S.err);
+    k_cc_tile<<<gt, kCcWarps * 32, 0, s>>>(table, S.parent, S.err, tile_rows);
+    k_cc_border<<<gp, 256, 0, s>>>(table, S.parent, S.err, tile_rows);
     k_cc_flatten<<<nt, 1024, 0, s>>>(T, S);
     k_root_scan<<<1, 1024, 0, s>>>(int(ntiles), S);
     k_root_assign<<<nt, 1024, 0, s>>>(table, n, T, S);
@@ -1078,7 +1206,7 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
     k_cluster_fill<<<gs, 256, 0, s>>>(S);
     k_cluster_merge<<<warp_blocks + thread_blocks, kMergeWarps * 32, 0, s>>>(table, S, warp_blocks);
     k_group_label<<<gs, 256, 0, s>>>(S);
-    k_relabel<<<gp, 256, 0, s>>>(table, S);
+    k_relabel<<<unsigned((T + 1023) / 1024), 256, 0, s>>>(table, n, T, S);
     if ((e = cudaGetLastError()) != cudaSuccess) break;
     if ((e = cudaMemcpyAsync(back, S.cnt, sizeof(back), cudaMemcpyDeviceToHost, s)) != cudaSuccess) break;
     e = cudaStreamSynchronize(s);

@@ -65,3 +65,17 @@ def test_large_call_uses_the_multi_block_scans():
     L[pts[:, 0], pts[:, 1]] = rng.integers(2, 9, len(pts))
     lab = rng.normal(40, 20, (H, W, 3)).astype(np.float32)
     run(gm, [(L, lab, K)])
+
+
+@pytest.mark.parametrize("spread", [0.0, 1e-4, 1e-2, 1.0])
+def test_near_ties_are_decided_in_fp64(spread):
+    """Islands of 1 to 40 members whose neighbours' colours differ by nothing, by less than FP32 can tell, or by
+    little: the nearest group and the tie rule are the oracle's."""
+    import paper_1612_08792_gb300 as gm
+    rng = np.random.default_rng(int(spread * 1e6) + 1)
+    H, W, K = 60, 90, 12
+    L = (np.arange(W)[None, :] // 15 + 6 * (np.arange(H)[:, None] // 20)).astype(np.int32)
+    m = rng.random((H, W)) < 0.25
+    L[m] = rng.integers(20, 24, m.sum())
+    lab = (np.array([60.0, -35.0, 80.0]) + spread * rng.normal(0, 1, (H, W, 3))).astype(np.float32)
+    run(gm, [(L, lab, K)])
