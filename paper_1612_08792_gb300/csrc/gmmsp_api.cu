@@ -5,7 +5,7 @@
 //   lab       3 W H float         CIELAB image as planes L, a, b
 //   theta     K x 16 double       master parameters (mu, Sigma_s, Sigma_c)
 //   gp        K x 16 float        packed E-step coefficients
-//   partials  ncells x 136        per-cell FP32 partial sums
+//   partials  ncells x 144        per-cell FP32 partial sums (16 floats per slot)
 //   cell_ll   ncells double       per-cell log-likelihood of the label pass
 //   llk       kLlkCap double      L(theta_t) per E-step
 //   ws        finalize workspace; ticket; counters; bad flag

@@ -444,7 +444,9 @@ gmmsp_status gmmsp_batch_first_pass_partials(gmmsp_batch b, const void* const* i
   if (!b || (!partials_host && !n_floats) || blocks_per_sm < 1 || blocks_per_sm > 16 || diagonal < 0 ||
       diagonal > 1)
     return GMMSP_E_INVALID;
-  const long long nf = (long long)b->total_cells * gmmsp::kPartStride;
+  // a cell's row: 9 slots x 15 statistics, then its log-likelihood
+  constexpr int kRow = gmmsp::kSlots * gmmsp::kStats + 1;
+  const long long nf = (long long)b->total_cells * kRow;
   if (n_floats) *n_floats = nf;
   if (!partials_host) return GMMSP_OK;
   if (b->state == GMMSP_E_CUDA || b->state == GMMSP_E_NOMEM) return GMMSP_E_STATE;
@@ -456,9 +458,16 @@ gmmsp_status gmmsp_batch_first_pass_partials(gmmsp_batch b, const void* const* i
   GB_CHECK(b, gmmsp::launch_em_pass_batch(b->table, b->n, b->total_cells, b->lab, b->gp, b->partials,
                                           b->p.precision, em_blocks(b, blocks_per_sm), blocks_per_sm,
                                           b->p.colour_model, b->stream, diagonal != 0));
-  GB_CHECK(b, cudaMemcpyAsync(partials_host, b->partials, size_t(nf) * sizeof(float), cudaMemcpyDeviceToHost,
-                              b->stream));
+  std::vector<float> rows(size_t(b->total_cells) * gmmsp::kPartStride);
+  GB_CHECK(b, cudaMemcpyAsync(rows.data(), b->partials, rows.size() * sizeof(float), cudaMemcpyDeviceToHost, b->stream));
   GB_CHECK(b, cudaStreamSynchronize(b->stream));
+  for (int c = 0; c < b->total_cells; ++c) {
+    const float* from = rows.data() + size_t(c) * gmmsp::kPartStride;
+    float* to = partials_host + size_t(c) * kRow;
+    for (int s = 0; s < gmmsp::kSlots; ++s)
+      memcpy(to + s * gmmsp::kStats, from + s * gmmsp::kSlotLd, gmmsp::kStats * sizeof(float));
+    to[kRow - 1] = from[gmmsp::kPartLl];
+  }
   return GMMSP_OK;
 }
 

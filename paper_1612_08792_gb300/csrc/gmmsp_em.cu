@@ -176,7 +176,7 @@ template <int WPC>
 struct EmSmem {
   float4 sp[kEmWarps / WPC][kSlots * 4];            // candidate parameters per cell
   float px[kEmWarps][kBatchFloats];                 // the 32 pixels in flight: posteriors, colour, position
-  float part[kEmWarps][kSlots * kStats + 1 + 3];    // per-warp sums (row 135: log-likelihood)
+  float part[kEmWarps][kPartStride];                // per-warp sums, as the partials lie
   float red[kEmWarps][27][kStats + 2];              // per-lane sums before the 3-lane add (odd row
                                                     // stride: the 27 lanes' stores hit 27 banks)
 };
@@ -344,19 +344,21 @@ __device__ __forceinline__ void em_cell_block(const Src& lab, const Geom& g, con
   for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
   if (lane < 27) acc.store(sm.red[warp][lane]);
   __syncwarp();
-  const auto slot_sum = [&](int o) {
-    const int s = o / kStats, j = o - s * kStats;
-    return sm.red[warp][s][j] + sm.red[warp][s + 9][j] + sm.red[warp][s + 18][j];
+  const auto slot_sum = [&](int o) {  // entry o of the cell's partials
+    const int s = o / kSlotLd, j = o % kSlotLd;
+    if (j < kStats) return sm.red[warp][s][j] + sm.red[warp][s + 9][j] + sm.red[warp][s + 18][j];
+    return o == kPartLl ? ll : 0.f;
   };
   if constexpr (WPC == 1) {  // the warp's sums are the cell's
     if (active && GMMSP_IN_BOUNDS(cell, g.ncells, BND_PARTIAL_W)) {
       PT* out = partials + (long long)cell * kPartStride;
-      for (int o = lane; o < kSlots * kStats; o += 32) out[o] = PT(slot_sum(o));
-      if (lane == 0) out[kSlots * kStats] = SHIFT ? PT(ll) : PT(ll) * PT(0.69314718055994530942);
+      for (int o = lane; o < kPartStride; o += 32) {
+        const float v = slot_sum(o);
+        out[o] = (o != kPartLl || SHIFT) ? PT(v) : PT(v) * PT(0.69314718055994530942);
+      }
     }
   } else {
-    for (int o = lane; o < kSlots * kStats; o += 32) sm.part[warp][o] = slot_sum(o);
-    if (lane == 0) sm.part[warp][kSlots * kStats] = ll;
+    for (int o = lane; o < kPartStride; o += 32) sm.part[warp][o] = slot_sum(o);
     __syncthreads();
     // Cell totals (sum over the WPC warps of the cell), written as PT.
     if (active && GMMSP_IN_BOUNDS(cell, g.ncells, BND_PARTIAL_W)) {
@@ -366,7 +368,7 @@ __device__ __forceinline__ void em_cell_block(const Src& lab, const Geom& g, con
         float v = sm.part[w0][o];
 #pragma unroll
         for (int w = 1; w < WPC; ++w) v += sm.part[w0 + w][o];
-        out[o] = (o < kSlots * kStats || SHIFT) ? PT(v) : PT(v) * PT(0.69314718055994530942);
+        out[o] = (o != kPartLl || SHIFT) ? PT(v) : PT(v) * PT(0.69314718055994530942);
       }
     }
   }
@@ -737,11 +739,17 @@ __device__ __forceinline__ void finalize_k(const Geom& g, const PT* __restrict__
       const int cx = kx + dx;
       if (cx < 0 || cx >= g.ncx) continue;
       if (!GMMSP_IN_BOUNDS(cy * g.ncx + cx, g.ncells, BND_PARTIAL_R)) continue;
-      const PT* P = partials + (long long)(cy * g.ncx + cx) * kPartStride + ((1 - dy) * 3 + (1 - dx)) * kStats;
+      const float4* P = reinterpret_cast<const float4*>(partials + (long long)(cy * g.ncx + cx) * kPartStride) +
+                        ((1 - dy) * 3 + (1 - dx)) * (kSlotLd / 4);
+      float4 p4[kSlotLd / 4];
+#pragma unroll
+      for (int j = 0; j < kSlotLd / 4; ++j) p4[j] = P[j];
+      const float p[kSlotLd] = {p4[0].x, p4[0].y, p4[0].z, p4[0].w, p4[1].x, p4[1].y, p4[1].z, p4[1].w,
+                                p4[2].x, p4[2].y, p4[2].z, p4[2].w, p4[3].x, p4[3].y, p4[3].z, p4[3].w};
 #pragma unroll
       for (int j = 0; j < kStats; ++j) {
-        if (SHIFT) two_sum_acc(hi[j], lo[j], P[j]);
-        else S[j] += T(P[j]);
+        if (SHIFT) two_sum_acc(hi[j], lo[j], p[j]);
+        else S[j] += T(p[j]);
       }
     }
   }
@@ -826,7 +834,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(Geom g, const PT* __re
   pdl_wait();
   pdl_trigger();
   if (llk_out)
-    block_ll_sum<PT, kFinThreads, SHIFT>(partials + kSlots * kStats, kPartStride, g.ncells, blk, ticket, llk_out);
+    block_ll_sum<PT, kFinThreads, SHIFT>(partials + kPartLl, kPartStride, g.ncells, blk, ticket, llk_out);
 
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned dead = 0, rs = 0, rc = 0;
@@ -934,7 +942,7 @@ __device__ __forceinline__ void finalize_l16_body(const Geom& g, const float* __
                         GMMSP_IN_BOUNDS(cy * g.ncx + cx, g.ncells, BND_PARTIAL_R);
         v[(dy + 1) * 3 + (dx + 1)] =
             in ? __ldg(partials + (long long)(cy * g.ncx + cx) * kPartStride +
-                       ((1 - dy) * 3 + (1 - dx)) * kStats + l)
+                       ((1 - dy) * 3 + (1 - dx)) * kSlotLd + l)
                : 0.f;
       }
     float hi = 0.f, lo = 0.f;
@@ -1106,7 +1114,7 @@ __global__ void __launch_bounds__(kFin16Threads) k_finalize_l16(Geom g, const fl
   pdl_wait();
   pdl_trigger();
   if (llk_out)
-    block_ll_sum<float, kFin16Threads, true>(partials + kSlots * kStats, kPartStride, g.ncells, blk, ticket,
+    block_ll_sum<float, kFin16Threads, true>(partials + kPartLl, kPartStride, g.ncells, blk, ticket,
                                         llk_out);
   const int q = threadIdx.x >> 4;
   const int k = blockIdx.x * (kFin16Threads / 16) + q;

@@ -48,7 +48,12 @@ struct NvtxRange {
 
 constexpr int kSlots = 9;          // |K_i| <= 9
 constexpr int kStats = 15;         // W, S1[5], S2s[3], S2c[6]
-constexpr int kPartStride = kSlots * kStats + 1;  // + per-cell log-likelihood = 136
+// Partial sums of a cell: 16 floats per slot (64 bytes, aligned, so that the
+// finalize reads a slot's 15 statistics with four 16-byte loads), the cell's
+// log-likelihood in the 16th of slot 0.
+constexpr int kSlotLd = 16;
+constexpr int kPartStride = kSlots * kSlotLd;
+constexpr int kPartLl = kStats;
 constexpr int kGP = 16;            // floats of packed E-step parameters per superpixel
 constexpr int kTheta = 16;         // doubles of master parameters per superpixel
 
