@@ -73,6 +73,7 @@ struct gmmsp_ctx_s {
   int* bad = nullptr;
   int wpc = 1;                    // warps per cell of the E+M pass (launch shape)
   gmmsp::ConnScratch conn;        // post-processing scratch, kept between calls
+  bool diag = true;               // theta as a start left it: covariance blocks diagonal
   bool timing = false;            // record events between the kernels (gmmsp_set_timing)
   std::vector<cudaEvent_t> tev;   // timing events, created on demand
   int tev_used = 0;               // events recorded by the last enqueued sequence
@@ -198,6 +199,7 @@ gmmsp_status enqueue_prepare(gmmsp_ctx c, const void* image, int pitch) {
   else
     GM_CHECK(c, gmmsp::launch_lab32(static_cast<const float*>(image), pitch, g, c->lab, c->counters,
                                     c->stream));
+  c->diag = true;
   GM_CHECK(c, gmmsp::launch_init_theta(gmmsp::LabPlanar{c->lab, (long long)g.W * g.H, g.W}, g, c->p.lambda_c, c->theta, c->gp, c->stream));
   GM_MARK(c);
   return GMMSP_OK;
@@ -207,7 +209,8 @@ gmmsp_status enqueue_prepare(gmmsp_ctx c, const void* image, int pitch) {
 gmmsp_status enqueue_em(gmmsp_ctx c, int iters, int t0, bool want_ll) {
   for (int t = 0; t < iters; ++t) {
     GM_CHECK(c, gmmsp::launch_em_pass(gmmsp::LabPlanar{c->lab, (long long)c->g.W * c->g.H, c->g.W}, c->g, c->gp, c->partials, c->p.precision, c->wpc,
-                                      c->stream));
+                                      c->stream, c->diag));
+    c->diag = false;
     double* llk_out = want_ll ? c->llk + ((t0 + t) % kLlkCap) : nullptr;
     GM_MARK(c);
     GM_CHECK(c, gmmsp::launch_finalize(c->g, c->partials, c->theta, c->gp, c->p.eps_s, c->p.eps_c,
@@ -455,6 +458,7 @@ gmmsp_status gmmsp_segment(gmmsp_ctx c, const void* image_dev, int pitch_bytes, 
       gr.want_ll = want_ll;
     }
     GM_CHECK(c, cudaGraphLaunch(gr.exec, c->stream));
+    c->diag = iters == 0;  // a replay enqueues nothing itself
   }
   if (loglik_host) return read_back(c, iters + 1, loglik_host);
   return GMMSP_OK;
@@ -515,6 +519,7 @@ gmmsp_status gmmsp_set_params(gmmsp_ctx c, const double* mu_host, const double* 
     memcpy(t + 5, cov_s_host + 3 * size_t(k), 3 * sizeof(double));
     memcpy(t + 8, cov_c_host + 6 * size_t(k), 6 * sizeof(double));
   }
+  c->diag = false;
   GM_CHECK(c, cudaMemsetAsync(c->bad, 0, sizeof(int), c->stream));
   GM_CHECK(c, cudaMemcpyAsync(c->theta, th.data(), th.size() * sizeof(double), cudaMemcpyHostToDevice,
                               c->stream));
@@ -548,6 +553,7 @@ gmmsp_status gmmsp_set_init(gmmsp_ctx c, const float* dmu_dev, const float* loge
   if (c->g.cm == gmmsp::kColourGray) return fail(c, GMMSP_E_INVALID, "theta_0 arrays need a colour model with a, b");
   GM_CHECK(c, gmmsp::launch_init_from_outputs(dmu_dev, 5, logeig_dev, 5, c->lab, 1, c->g, c->p.lambda_c, c->p.eps_s,
                                               c->p.eps_c, c->theta, c->gp, c->counters, c->stream));
+  c->diag = true;
   return GMMSP_OK;
 }
 
@@ -568,6 +574,7 @@ gmmsp_status gmmsp_init_from_net(gmmsp_ctx c, gmmsp_net n) {
   }
   GM_CHECK(c, gmmsp::net_enqueue_init(n, c->lab, nullptr, 1, c->g, c->p.lambda_c, c->p.eps_s, c->p.eps_c, c->theta, c->gp,
                                       c->counters, c->stream));
+  c->diag = true;
   return GMMSP_OK;
 }
 

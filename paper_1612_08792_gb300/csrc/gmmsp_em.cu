@@ -375,7 +375,7 @@ __device__ __forceinline__ void em_cell_block(const Src& lab, const Geom& g, con
   if (WPC == 1) __syncwarp(); else __syncthreads();  // the slot's buffers are reused next
 }
 
-template <typename PT, bool SHIFT, int WPC, class Src, int CM>
+template <typename PT, bool SHIFT, int WPC, class Src, int CM, bool DIAG>
 __device__ __forceinline__ void em_pass_body(const Src& lab, const Geom& g, const float* __restrict__ gp,
                                              PT* __restrict__ partials) {
   constexpr int kCellsPerBlock = kEmWarps / WPC;
@@ -389,23 +389,25 @@ __device__ __forceinline__ void em_pass_body(const Src& lab, const Geom& g, cons
   const bool active = cell < g.ncells;  // inactive threads still reach every barrier
   pdl_wait();  // gp and the image are written by the preceding kernels
   pdl_trigger();
-  em_cell_block<PT, SHIFT, WPC, Src, CM>(lab, g, gp, partials, cell, active, sm, warp, lane, slot, wic, t);
+  em_cell_block<PT, SHIFT, WPC, Src, CM, DIAG>(lab, g, gp, partials, cell, active, sm, warp, lane, slot, wic, t);
 }
 
-template <typename PT, bool SHIFT, int WPC, class Src, int CM>
+template <typename PT, bool SHIFT, int WPC, class Src, int CM, bool DIAG>
 __global__ void __launch_bounds__(kEmWarps * 32) k_em_pass(Src lab, Geom g, const float* __restrict__ gp,
                                                            PT* __restrict__ partials) {
-  em_pass_body<PT, SHIFT, WPC, Src, CM>(lab, g, gp, partials);
+  em_pass_body<PT, SHIFT, WPC, Src, CM, DIAG>(lab, g, gp, partials);
 }
 
-// The same, registers capped for 7 blocks per SM (72): the launch for one
-// warp per cell in the full colour model, where it raised the occupancy from
-// 24% to 40% on large images (the split and grayscale kernels are faster
-// uncapped).
-template <typename PT, bool SHIFT, int WPC, class Src, int CM>
-__global__ void __launch_bounds__(kEmWarps * 32, 6) k_em_pass_capped(Src lab, Geom g, const float* __restrict__ gp,
-                                                                     PT* __restrict__ partials) {
-  em_pass_body<PT, SHIFT, WPC, Src, CM>(lab, g, gp, partials);
+// The same, registers capped for MINB blocks per SM, in the full colour model
+// (the split and grayscale kernels are faster uncapped).  One warp per cell: 6
+// (3840x2160, v = 20: 189 us, 203 us at 7).  Four warps per cell: 7, which
+// puts the 1107 cells of a 481x321 image at v = 12 into little more than one
+// wave of 1064 blocks (10 iterations and labels 162 us, 175 uncapped at 5
+// blocks, 166 at 8).  Two warps per cell run uncapped.
+template <typename PT, bool SHIFT, int WPC, class Src, int CM, bool DIAG, int MINB>
+__global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_capped(Src lab, Geom g, const float* __restrict__ gp,
+                                                                        PT* __restrict__ partials) {
+  em_pass_body<PT, SHIFT, WPC, Src, CM, DIAG>(lab, g, gp, partials);
 }
 
 // ---------------------------------------------------------------- batches
@@ -466,10 +468,15 @@ __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_batch_flat(cons
 
 // Label pass: argmax posterior per pixel (ties to the smaller k, i.e. the
 // smaller slot) and the per-cell log-likelihood.
-// Each lane takes kLabelPPL pixels per step (p, p + 32, ...), so that every
+// Each lane takes kLabelPixels pixels per step (p, p + 32, ...), so that every
 // candidate's parameters, read from shared memory once, serve all of them;
 // the colours of the next step are loaded one step ahead.
-constexpr int kLabelPPL = 2;
+// Grayscale: one pixel per lane, whose kernel then fits 8 blocks on an SM
+// (64 images of 640x480: conversion, start and labels 0.208 ms against 0.218;
+// the split model is slower that way, 0.247 against 0.236 on 96 of 481x321,
+// the full model the same).
+template <int CM>
+constexpr int kLabelPixels = CM == kColourGray ? 1 : 2;
 
 // LL = false: argmax only (no log-sum-exp), for callers that want no
 // log-likelihood.
@@ -477,6 +484,7 @@ template <bool FULL, bool LL, class Src, int CM>
 __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
                                                   const Cell& c, const float4* sp, int lane,
                                                   int32_t* __restrict__ labels, float& ll) {
+  constexpr int kLabelPPL = kLabelPixels<CM>;
   const int npx_all = c.cw * c.ch;
   auto locate = [&](int p, int& rx, int& ry) {
     ry = __float2int_rz((float(p) + 0.5f) * (1.f / float(c.cw)));  // exact floor(p / cw)
@@ -588,8 +596,8 @@ __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
   };
   // kLabelPPL pixels per lane while more than 32 remain, then one
   int p0 = lane;
-  for (; p0 - lane + 32 < npx; p0 += 32 * kLabelPPL) step(std::integral_constant<int, kLabelPPL>{}, p0);
-  if (p0 - lane < npx) step(std::integral_constant<int, 1>{}, p0);
+  for (; p0 - lane + 32 * (kLabelPPL - 1) < npx; p0 += 32 * kLabelPPL) step(std::integral_constant<int, kLabelPPL>{}, p0);
+  if (kLabelPPL > 1 && p0 - lane < npx) step(std::integral_constant<int, 1>{}, p0);
 }
 
 // One cell of the label pass, run by one warp.
@@ -632,7 +640,7 @@ __global__ void __launch_bounds__(kEmWarps * 32) k_label_pass(Src lab, Geom g, c
 // One cell per warp over a grid sized to the work (a persistent loop over the
 // cells costs registers: 60 bytes of spill under the same bound).
 template <int CM>
-__global__ void __launch_bounds__(kEmWarps * 32, 5) k_label_pass_batch(const BatchImage* __restrict__ imgs, int n,
+__global__ void __launch_bounds__(kEmWarps * 32, CM == kColourGray ? 8 : 5) k_label_pass_batch(const BatchImage* __restrict__ imgs, int n,
                                                                     int total_cells,
                                                                     const float* __restrict__ lab,
                                                                     const float* __restrict__ gp,
@@ -1172,14 +1180,15 @@ size_t finalize_workspace_doubles(const Geom& g) {
   return (b16 > size_t(ll_blocks(g)) ? b16 : size_t(ll_blocks(g))) + 1;
 }
 
-template <typename PT, bool SHIFT, int WPC, class Src, int CM>
+template <typename PT, bool SHIFT, int WPC, class Src, int CM, bool DIAG>
 static cudaError_t em_pass_impl(Src lab, const Geom& g, const float* gp, PT* partials,
                                 cudaStream_t s) {
   constexpr int smem = em_smem_bytes<WPC>();
   static_assert(smem <= 227 * 1024, "shared memory");
   const auto kernel = [] {
-    if constexpr (WPC == 1 && CM == kColourFull) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM>;
-    else return k_em_pass<PT, SHIFT, WPC, Src, CM>;
+    if constexpr (WPC == 1 && CM == kColourFull) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 6>;
+    else if constexpr (WPC == 4 && CM == kColourFull) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 7>;
+    else return k_em_pass<PT, SHIFT, WPC, Src, CM, DIAG>;
   }();
   static bool attr_set = false;  // per process; the attribute is per function
   if (!attr_set && smem > 48 * 1024) {
@@ -1192,13 +1201,13 @@ static cudaError_t em_pass_impl(Src lab, const Geom& g, const float* gp, PT* par
   return launch_pdl(kernel, dim3(blocks), dim3(kEmWarps * 32), smem, s, lab, g, gp, partials);
 }
 
-template <typename PT, bool SHIFT, class Src, int CM>
+template <typename PT, bool SHIFT, class Src, int CM, bool DIAG = false>
 static cudaError_t em_pass_wpc(Src lab, const Geom& g, const float* gp, PT* partials, int wpc,
                                cudaStream_t s) {
   switch (wpc) {
-    case 2: return em_pass_impl<PT, SHIFT, 2, Src, CM>(lab, g, gp, partials, s);
-    case 4: return em_pass_impl<PT, SHIFT, 4, Src, CM>(lab, g, gp, partials, s);
-    default: return em_pass_impl<PT, SHIFT, 1, Src, CM>(lab, g, gp, partials, s);
+    case 2: return em_pass_impl<PT, SHIFT, 2, Src, CM, DIAG>(lab, g, gp, partials, s);
+    case 4: return em_pass_impl<PT, SHIFT, 4, Src, CM, DIAG>(lab, g, gp, partials, s);
+    default: return em_pass_impl<PT, SHIFT, 1, Src, CM, DIAG>(lab, g, gp, partials, s);
   }
 }
 
@@ -1206,7 +1215,7 @@ static cudaError_t em_pass_wpc(Src lab, const Geom& g, const float* gp, PT* part
 // only (the entry points check it).
 template <class Src>
 cudaError_t launch_em_pass(Src lab, const Geom& g, const float* gp, void* partials, int precision,
-                           int wpc, cudaStream_t s) {
+                           int wpc, cudaStream_t s, bool diag) {
   float* part = static_cast<float*>(partials);
   if (precision == 1) return em_pass_wpc<float, false, Src, kColourFull>(lab, g, gp, part, wpc, s);
   if constexpr (std::is_same<Src, LabPlanar>::value) {
@@ -1214,6 +1223,9 @@ cudaError_t launch_em_pass(Src lab, const Geom& g, const float* gp, void* partia
     if (g.cm == kColourGray) return em_pass_wpc<float, true, Src, kColourGray>(lab, g, gp, part, wpc, s);
   }
   if (g.cm != kColourFull) return cudaErrorInvalidValue;
+  if constexpr (std::is_same<Src, LabPlanar>::value) {
+    if (diag) return em_pass_wpc<float, true, Src, kColourFull, true>(lab, g, gp, part, wpc, s);
+  }
   return em_pass_wpc<float, true, Src, kColourFull>(lab, g, gp, part, wpc, s);
 }
 
@@ -1235,9 +1247,9 @@ cudaError_t launch_label_pass(Src lab, const Geom& g, const float* gp, int32_t* 
 }
 
 template cudaError_t launch_em_pass<LabPlanar>(LabPlanar, const Geom&, const float*, void*, int, int,
-                                               cudaStream_t);
+                                               cudaStream_t, bool);
 template cudaError_t launch_em_pass<LabPitched>(LabPitched, const Geom&, const float*, void*, int, int,
-                                                cudaStream_t);
+                                                cudaStream_t, bool);
 template cudaError_t launch_label_pass<LabPlanar>(LabPlanar, const Geom&, const float*, int32_t*, double*,
                                                   cudaStream_t);
 template cudaError_t launch_label_pass<LabPitched>(LabPitched, const Geom&, const float*, int32_t*,

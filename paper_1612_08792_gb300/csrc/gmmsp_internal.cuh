@@ -243,10 +243,11 @@ cudaError_t launch_gray2l(const uint8_t* img, long long pitch, const Geom& g, fl
 template <class Src>
 cudaError_t launch_init_theta(Src lab, const Geom& g, double lambda_c, double* theta, float* gp,
                               cudaStream_t s);
-// wpc: warps per cell (1, 2 or 4); the colour model is g.cm.
+// wpc: warps per cell (1, 2 or 4); the colour model is g.cm.  diag: every
+// superpixel's covariance blocks are diagonal (see launch_em_pass_batch).
 template <class Src>
 cudaError_t launch_em_pass(Src lab, const Geom& g, const float* gp, void* partials, int precision,
-                           int wpc, cudaStream_t s);
+                           int wpc, cudaStream_t s, bool diag = false);
 // cell_ll == nullptr: labels only, no log-likelihood.
 template <class Src>
 cudaError_t launch_label_pass(Src lab, const Geom& g, const float* gp, int32_t* labels,
