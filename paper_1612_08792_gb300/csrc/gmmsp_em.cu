@@ -447,14 +447,14 @@ __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_batch(const Bat
 // diagonal (the first pass after either start).
 template <typename PT, bool SHIFT, int MINB, int CM, bool DIAG = false>
 __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_batch_flat(const BatchImage* __restrict__ imgs, int n,
-                                                                      int total_cells,
+                                                                      int first, int total_cells,
                                                                       const float* __restrict__ lab,
                                                                       const float* __restrict__ gp,
                                                                       PT* __restrict__ partials) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   EmSmem<1>& sm = *reinterpret_cast<EmSmem<1>*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cell = blockIdx.x * kEmWarps + warp;
+  const int cell = first + blockIdx.x * kEmWarps + warp;
   if (cell >= total_cells) return;  // whole warps only; a warp works alone on its cell
   const int ii = find_image(imgs, n, cell, 0);
   if (!GMMSP_IN_BOUNDS(ii, n, BND_IMAGE)) return;
@@ -641,13 +641,13 @@ __global__ void __launch_bounds__(kEmWarps * 32) k_label_pass(Src lab, Geom g, c
 // cells costs registers: 60 bytes of spill under the same bound).
 template <int CM>
 __global__ void __launch_bounds__(kEmWarps * 32, CM == kColourGray ? 8 : 5) k_label_pass_batch(const BatchImage* __restrict__ imgs, int n,
-                                                                    int total_cells,
+                                                                    int first, int total_cells,
                                                                     const float* __restrict__ lab,
                                                                     const float* __restrict__ gp,
                                                                     double* __restrict__ cell_ll) {
   __shared__ float4 sp_all[kEmWarps][kSlots * 4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cell = blockIdx.x * kEmWarps + warp;
+  const int cell = first + blockIdx.x * kEmWarps + warp;
   if (cell >= total_cells) return;
   const int ii = find_image(imgs, n, cell, 0);
   if (!GMMSP_IN_BOUNDS(ii, n, BND_IMAGE)) return;
@@ -859,14 +859,14 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(Geom g, const PT* __re
 
 template <typename PT, bool SHIFT>
 __global__ void __launch_bounds__(kFinThreads) k_finalize_batch(const BatchImage* __restrict__ imgs, int n,
-                                                                int total_k, const PT* __restrict__ partials,
+                                                                int first, int total_k, const PT* __restrict__ partials,
                                                                 double* __restrict__ theta,
                                                                 float* __restrict__ gp, double eps_s,
                                                                 double eps_c,
                                                                 unsigned long long* counters) {
   unsigned dead = 0, rs = 0, rc = 0;
   const int stride = gridDim.x * kFinThreads;
-  for (int base = blockIdx.x * kFinThreads; base < total_k; base += stride) {
+  for (int base = first + blockIdx.x * kFinThreads; base < total_k; base += stride) {
     const int k = base + threadIdx.x;
     if (k < total_k) {
       const int ii = find_image(imgs, n, k, 1);
@@ -1132,15 +1132,15 @@ __global__ void __launch_bounds__(kFin16Threads) k_finalize_l16(Geom g, const fl
 // The same over a batch: half-warp q of block b takes superpixel 4 b + q of
 // the batch, found in its image by a binary search over the offsets.
 __global__ void __launch_bounds__(kFin16Threads) k_finalize_l16_batch(const BatchImage* __restrict__ imgs, int n,
-                                                                    int total_k, const float* __restrict__ partials,
+                                                                    int first, int total_k, const float* __restrict__ partials,
                                                                     double* __restrict__ theta,
                                                                     float* __restrict__ gp, double eps_s,
                                                                     double eps_c, unsigned long long* counters) {
   __shared__ double sh[kFin16Threads / 16][48];
   __shared__ float shf[kFin16Threads / 16][8];
   const int q = threadIdx.x >> 4;
-  const int kg = blockIdx.x * (kFin16Threads / 16) + q;
-  const int ii = find_image(imgs, n, kg < total_k ? kg : 0, 1);
+  const int kg = first + blockIdx.x * (kFin16Threads / 16) + q;
+  const int ii = find_image(imgs, n, kg < total_k ? kg : first, 1);
   const bool img_ok = GMMSP_IN_BOUNDS(ii, n, BND_IMAGE);
   const BatchImage& im = imgs[img_ok ? ii : 0];
   const bool valid = kg < total_k && img_ok && GMMSP_IN_BOUNDS(kg - im.k_off, im.g.K, BND_ITEM);
@@ -1286,32 +1286,33 @@ cudaError_t launch_ll_reduce(const double* cell_ll, int n, double* out, double* 
 namespace gmmsp {
 
 template <int CM>
-static void em_pass_batch_mixed(const BatchImage* imgs, int n, int total_cells, const float* lab, const float* gp,
+static void em_pass_batch_mixed(const BatchImage* imgs, int n, int first, int total_cells, const float* lab, const float* gp,
                                 float* partials, int blocks, int minb, bool diag, cudaStream_t s) {
   constexpr int smem = em_smem_bytes<1>();
   if (minb >= 6) {  // one cell per warp over a grid sized to the work
-    const int nb = (total_cells + kEmWarps - 1) / kEmWarps;
+    const int nb = (total_cells - first + kEmWarps - 1) / kEmWarps;
     auto kernel = minb >= 7 ? (diag ? k_em_pass_batch_flat<float, true, 7, CM, true>
                                     : k_em_pass_batch_flat<float, true, 7, CM, false>)
                             : (diag ? k_em_pass_batch_flat<float, true, 6, CM, true>
                                     : k_em_pass_batch_flat<float, true, 6, CM, false>);
-    kernel<<<nb, kEmWarps * 32, smem, s>>>(imgs, n, total_cells, lab, gp, partials);
+    kernel<<<nb, kEmWarps * 32, smem, s>>>(imgs, n, first, total_cells, lab, gp, partials);
   } else {
     k_em_pass_batch<float, true, 5, CM><<<blocks, kEmWarps * 32, smem, s>>>(imgs, n, total_cells, lab, gp,
                                                                           partials);
   }
 }
 
-cudaError_t launch_em_pass_batch(const BatchImage* imgs, int n, int total_cells, const float* lab,
+cudaError_t launch_em_pass_batch(const BatchImage* imgs, int n, int first, int total_cells, const float* lab,
                                  const float* gp, void* partials, int precision, int blocks, int minb,
                                  int cm, cudaStream_t s, bool diag) {
   constexpr int smem = em_smem_bytes<1>();
+  if (minb < 6 && first != 0) return cudaErrorInvalidValue;  // the persistent kernels take the whole batch
   if (precision == 1) {  // full colour model only
     if (cm != kColourFull) return cudaErrorInvalidValue;
     if (minb >= 6) {
-      const int nb = (total_cells + kEmWarps - 1) / kEmWarps;
+      const int nb = (total_cells - first + kEmWarps - 1) / kEmWarps;
       k_em_pass_batch_flat<float, false, 6, kColourFull><<<nb, kEmWarps * 32, smem, s>>>(
-          imgs, n, total_cells, lab, gp, static_cast<float*>(partials));
+          imgs, n, first, total_cells, lab, gp, static_cast<float*>(partials));
     } else {
       k_em_pass_batch<float, false, 5, kColourFull><<<blocks, kEmWarps * 32, smem, s>>>(
           imgs, n, total_cells, lab, gp, static_cast<float*>(partials));
@@ -1320,47 +1321,50 @@ cudaError_t launch_em_pass_batch(const BatchImage* imgs, int n, int total_cells,
   }
   float* part = static_cast<float*>(partials);
   switch (cm) {
-    case kColourFull: em_pass_batch_mixed<kColourFull>(imgs, n, total_cells, lab, gp, part, blocks, minb, diag, s); break;
-    case kColourSplit: em_pass_batch_mixed<kColourSplit>(imgs, n, total_cells, lab, gp, part, blocks, minb, diag, s); break;
-    case kColourGray: em_pass_batch_mixed<kColourGray>(imgs, n, total_cells, lab, gp, part, blocks, minb, diag, s); break;
+    case kColourFull: em_pass_batch_mixed<kColourFull>(imgs, n, first, total_cells, lab, gp, part, blocks, minb, diag, s); break;
+    case kColourSplit: em_pass_batch_mixed<kColourSplit>(imgs, n, first, total_cells, lab, gp, part, blocks, minb, diag, s); break;
+    case kColourGray: em_pass_batch_mixed<kColourGray>(imgs, n, first, total_cells, lab, gp, part, blocks, minb, diag, s); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize_batch(const BatchImage* imgs, int n, int total_k, const void* partials,
+cudaError_t launch_finalize_batch(const BatchImage* imgs, int n, int first, int total_k, const void* partials,
                                   double* theta, float* gp, double eps_s, double eps_c,
-                                  unsigned long long* counters, int precision, int blocks,
+                                  unsigned long long* counters, int precision, int blocks, int priority,
                                   cudaStream_t s) {
+  const float* part = static_cast<const float*>(partials);
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributePriority;
+  attr[0].val.priority = priority;
+  cfg.attrs = attr;
+  cfg.numAttrs = priority ? 1 : 0;
   if (precision != 1 && blocks == 0) {  // 16 lanes per superpixel
-    const int nb = (total_k + kFin16Threads / 16 - 1) / (kFin16Threads / 16);
-    k_finalize_l16_batch<<<nb, kFin16Threads, 0, s>>>(imgs, n, total_k, static_cast<const float*>(partials), theta,
-                                                     gp, eps_s, eps_c, counters);
-    return cudaGetLastError();
+    cfg.gridDim = dim3((total_k - first + kFin16Threads / 16 - 1) / (kFin16Threads / 16));
+    cfg.blockDim = dim3(kFin16Threads);
+    return cudaLaunchKernelEx(&cfg, k_finalize_l16_batch, imgs, n, first, total_k, part, theta, gp, eps_s, eps_c,
+                              counters);
   }
-  if (precision == 1)
-    k_finalize_batch<float, false><<<blocks, kFinThreads, 0, s>>>(imgs, n, total_k,
-                                                                  static_cast<const float*>(partials), theta, gp,
-                                                                  eps_s, eps_c, counters);
-  else
-    k_finalize_batch<float, true><<<blocks, kFinThreads, 0, s>>>(imgs, n, total_k,
-                                                                 static_cast<const float*>(partials), theta, gp,
-                                                                 eps_s, eps_c, counters);
-  return cudaGetLastError();
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(kFinThreads);
+  return cudaLaunchKernelEx(&cfg, precision == 1 ? k_finalize_batch<float, false> : k_finalize_batch<float, true>,
+                            imgs, n, first, total_k, part, theta, gp, eps_s, eps_c, counters);
 }
 
-cudaError_t launch_label_pass_batch(const BatchImage* imgs, int n, int total_cells, const float* lab,
+cudaError_t launch_label_pass_batch(const BatchImage* imgs, int n, int first, int total_cells, const float* lab,
                                     const float* gp, double* cell_ll, int cm, cudaStream_t s) {
-  const int nb = (total_cells + kEmWarps - 1) / kEmWarps;
+  const int nb = (total_cells - first + kEmWarps - 1) / kEmWarps;
   switch (cm) {
     case kColourFull:
-      k_label_pass_batch<kColourFull><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
+      k_label_pass_batch<kColourFull><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, first, total_cells, lab, gp, cell_ll);
       break;
     case kColourSplit:
-      k_label_pass_batch<kColourSplit><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
+      k_label_pass_batch<kColourSplit><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, first, total_cells, lab, gp, cell_ll);
       break;
     case kColourGray:
-      k_label_pass_batch<kColourGray><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, total_cells, lab, gp, cell_ll);
+      k_label_pass_batch<kColourGray><<<nb, kEmWarps * 32, 0, s>>>(imgs, n, first, total_cells, lab, gp, cell_ll);
       break;
     default: return cudaErrorInvalidValue;
   }

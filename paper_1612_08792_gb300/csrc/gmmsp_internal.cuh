@@ -265,7 +265,9 @@ size_t finalize_workspace_doubles(const Geom& g);
 cudaError_t launch_pack_theta(const Geom& g, double* theta, float* gp, int* bad, cudaStream_t s);
 
 // Batches: the same steps over all images of a BatchImage table in one launch
-// each; `blocks` is the persistent grid size.
+// each; `blocks` is the persistent grid size.  The E + M (one cell per warp),
+// finalize and label launches take the cells or superpixels [first, total) of
+// the batch, so that one launch can cover some of its images.
 // Grayscale model (the images' g.cm): plane L only, as launch_rgb2lab.
 cudaError_t launch_prepare_batch(const BatchImage* imgs, int n, long long total_rows, int input_format,
                                  float* lab, unsigned long long* counters, int blocks, cudaStream_t s);
@@ -281,17 +283,17 @@ cudaError_t launch_init_batch(const BatchImage* imgs, int n, int total_k, const 
 // kernel on `blocks` blocks.  diag: every superpixel's covariance blocks are
 // diagonal (true after either start, until the first finalize); the mixed-
 // precision one-cell-per-warp kernels then skip the zero terms (same bits).
-cudaError_t launch_em_pass_batch(const BatchImage* imgs, int n, int total_cells, const float* lab,
+cudaError_t launch_em_pass_batch(const BatchImage* imgs, int n, int first, int total_cells, const float* lab,
                                  const float* gp, void* partials, int precision, int blocks, int minb,
                                  int cm, cudaStream_t s, bool diag = false);
 // blocks == 0 (mixed precision and the full colour model only): 16 lanes per
 // superpixel, one block per 4 superpixels; otherwise one thread per
 // superpixel on `blocks` blocks.
-cudaError_t launch_finalize_batch(const BatchImage* imgs, int n, int total_k, const void* partials,
+cudaError_t launch_finalize_batch(const BatchImage* imgs, int n, int first, int total_k, const void* partials,
                                   double* theta, float* gp, double eps_s, double eps_c,
-                                  unsigned long long* counters, int precision, int blocks,
+                                  unsigned long long* counters, int precision, int blocks, int priority,
                                   cudaStream_t s);
-cudaError_t launch_label_pass_batch(const BatchImage* imgs, int n, int total_cells, const float* lab,
+cudaError_t launch_label_pass_batch(const BatchImage* imgs, int n, int first, int total_cells, const float* lab,
                                     const float* gp, double* cell_ll, int cm, cudaStream_t s);
 // ll_out[i] = sum of image i's per-cell log-likelihoods (fixed order).
 cudaError_t launch_ll_per_image(const BatchImage* imgs, int n, const double* cell_ll, double* ll_out,
