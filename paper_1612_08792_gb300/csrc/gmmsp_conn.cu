@@ -183,34 +183,50 @@ __device__ __forceinline__ bool small_size(long long s, int K, long long N) { re
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncomp_; c += gridDim.x * blockDim.x)
 
 // Labels one tile of 32 x 32 pixels (x tile_rows where the call has few pixels:
-// a tile is a serial walk) per warp in shared memory: every pixel starts under
-// the first pixel of its row's run of one label (a ballot), and one union per
-// pair of vertically adjacent runs (at the leftmost pixel of their overlap)
-// is queued and then done 32 at a time.  Local indices order like pixels, so
-// a tile's root is the smallest pixel of its piece of the component.  Then
-// parent = the root's pixel.  Only the tiles' borders are left to global
-// unions: 6 % of the pixels (labelling all of them in global memory took
-// 195 + 703 us on 256 images of 481x321).
+// a tile is a serial walk) per warp.  A row's runs of one label come from a
+// ballot; a run takes the number of the leftmost run above that it touches,
+// carried down in registers, or a fresh one, and only where it touches a run
+// above of another number are the two queued for a union in shared memory, 32
+// unions at a time.  Numbers are given in the order of the pixels, so a tile's
+// root is the smallest pixel of its piece of the component.  Then parent = the
+// root's pixel.  (One union per pair of touching runs, nearly all of them
+// between runs of one piece already: 150 instructions per row of 32 pixels,
+// 308 us on 256 images of 481x321, 170 this way.)  Only the tiles' borders are left to
+// global unions: 6 % of the pixels (labelling all of them in global memory
+// took 195 + 703 us).
 __global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict__ imgs, int* __restrict__ p,
                                                           int* err, int tile_rows) {
-  __shared__ int sp[kCcWarps][kCcTile * kCcTile];
-  __shared__ uint16_t queue[kCcWarps][kCcTile * kCcTile], first[kCcWarps][kCcTile * kCcTile];
+  __shared__ int parent[kCcWarps][kCcTile * kCcTile];            // over the numbers given
+  __shared__ uint16_t first[kCcWarps][kCcTile * kCcTile];        // a number's first pixel
+  __shared__ uint16_t number[kCcWarps][kCcTile * kCcTile];       // of every pixel
+  __shared__ unsigned queue[kCcWarps][64];                       // unions to do: two numbers each
   const Img im = imgs[blockIdx.y];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tx = (im.W + kCcTile - 1) / kCcTile;
   const long long tiles = (long long)tx * ((im.H + tile_rows - 1) / tile_rows);
-  int* q = sp[warp];
-  uint16_t *Q = queue[warp], *F = first[warp];  // the unions; the runs' first pixels
+  const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
+  int* q = parent[warp];
+  uint16_t *F = first[warp], *R = number[warp];
+  unsigned* Q = queue[warp];
   for (long long t = (long long)blockIdx.x * kCcWarps + warp; t < tiles; t += (long long)gridDim.x * kCcWarps) {
     const int ty = int(t / tx), x0 = int(t - (long long)ty * tx) * kCcTile, y0 = ty * tile_rows;
     const int rows = min(tile_rows, im.H - y0);
     const bool in = x0 + lane < im.W;
     const long long g0 = (long long)y0 * im.W + x0;
     const int32_t* L = im.labels + g0 + lane;
-    int32_t next[kCcAhead], up = 0;  // the labels of the next rows, loaded ahead
+    int32_t next[kCcAhead], up = 0;  // the labels of the next rows, loaded ahead; of the row above
 #pragma unroll
     for (int j = 0; j < kCcAhead; ++j) next[j] = in && j < rows ? L[(long long)j * im.W] : 0;
-    int queued = 0, runs = 0;
+    int given = 0, queued = 0, nup = 0;  // numbers given, unions queued (below 32 between rows), the number above
+    auto work = [&](int at_least) {
+      __syncwarp();
+      while (queued >= at_least && queued > 0) {
+        const int k = min(32, queued);
+        queued -= k;
+        if (lane < k) unite(q, int(Q[queued + lane] & 0xffffu), int(Q[queued + lane] >> 16), err);
+        __syncwarp();
+      }
+    };
     for (int r0 = 0; r0 < rows; r0 += kCcAhead) {
 #pragma unroll
       for (int j = 0; j < kCcAhead; ++j) {
@@ -219,32 +235,50 @@ __global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict
         const int32_t l = next[j];
         if (in && r + kCcAhead < rows) next[j] = L[(long long)(r + kCcAhead) * im.W];
         const int32_t lprev = __shfl_up_sync(0xffffffffu, l, 1), uprev = __shfl_up_sync(0xffffffffu, up, 1);
-        const bool left_same = in && lane > 0 && lprev == l;
-        const unsigned heads = __ballot_sync(0xffffffffu, !left_same);
-        q[r * 32 + lane] = r * 32 + 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
-        const bool join = in && r > 0 && l == up && !(left_same && uprev == l);
+        const bool head = !(in && lane > 0 && lprev == l), same = in && r > 0 && l == up;
+        const unsigned heads = __ballot_sync(0xffffffffu, head), sames = __ballot_sync(0xffffffffu, same);
+        // this lane's run: lanes at .. the one before the next head
+        const int at = 31 - __clz(heads & upto);
+        const unsigned after = heads & ~upto;
+        const unsigned run = (after ? (after & (0u - after)) - 1u : 0xffffffffu) & (0xffffffffu << at);
+        const unsigned touch = sames & run;
+        const bool fresh = head && in && !touch;
+        const unsigned freshs = __ballot_sync(0xffffffffu, fresh);
+        const int mine = fresh ? given + __popc(freshs & below) : nup;
+        const int num = __shfl_sync(0xffffffffu, mine, touch ? __ffs(touch) - 1 : at);
+        if (fresh) {
+          q[num] = num;
+          F[num] = uint16_t(r * 32 + lane);
+        }
+        given += __popc(freshs);
+        R[r * 32 + lane] = uint16_t(num);
+        const bool join = same && nup != num && !(!head && uprev == l);
         const unsigned joins = __ballot_sync(0xffffffffu, join);
-        if (join) Q[queued + __popc(joins & ((1u << lane) - 1u))] = uint16_t(r * 32 + lane);
-        queued += __popc(joins);
-        if (!left_same) F[runs + __popc(heads & ((1u << lane) - 1u))] = uint16_t(r * 32 + lane);
-        runs += __popc(heads);
+        if (joins) {
+          if (join) Q[queued + __popc(joins & below)] = unsigned(num) | unsigned(nup) << 16;
+          queued += __popc(joins);
+          work(32);
+        }
         up = l;
+        nup = num;
       }
     }
-    __syncwarp();
-    for (int i = lane; i < queued; i += 32) unite(q, Q[i], Q[i] - 32, err);
-    __syncwarp();
-    // the runs' roots, from the top, each kept for the runs below (their chains
-    // are then two or three links long); then every pixel has its run's
-    for (int i = lane; i < runs; i += 32) q[F[i]] = find_root(q, F[i], err);
+    work(1);
+    // every number's root, as a pixel of the tile (F of a root stays)
+    for (int i = lane; i < given; i += 32) {
+      const int root = find_root(q, i, err);
+      q[i] = root;
+      F[i] = F[root];
+    }
     __syncwarp();
     int* P = p + im.off + g0 + lane;
     const int at0 = int(im.off + g0);
     for (int r = 0; r < rows; ++r, P += im.W) {
-      const int root = q[q[r * 32 + lane]];
-      if (in) *P = at0 + (root >> 5) * im.W + (root & 31);  // pixel numbers of a call stay below 2^30
+      if (!in) continue;
+      const int root = F[R[r * 32 + lane]];
+      *P = at0 + (root >> 5) * im.W + (root & 31);  // pixel numbers of a call stay below 2^30
     }
-    __syncwarp();  // the tile's array is refilled
+    __syncwarp();  // the tile's arrays are refilled
   }
 }
 
