@@ -83,8 +83,8 @@ struct Img {
 
 struct Scratch {
   // per pixel of the call
-  int* parent;                // union-find, then the root pixel, then the compact index
-  int* cidr;                  // at root pixels: the compact index
+  int* parent;                // union-find, then the compact index
+  int* cidr;                  // at the tiles' root pixels: the compact index
   // per component (compact index c < ncomp)
   int* size;                  // pixel count
   long long* csum;            // 3 fixed-point colour sums, then (k_comp_flags) ...
@@ -107,6 +107,11 @@ struct Scratch {
   int* next;                  // next member of its group, -1 at the end
   int* tail;                  // of a group's founder: its last member
   int* tile_sum;              // tile kernels: per tile counts, then their exclusive prefix
+  // the tiles' roots (before the per-component arrays that lie in the same memory)
+  int* roots;                 // a tile's root pixels, from its place on (tile_place)
+  int* nroots;                // at a tile's place: their number
+  unsigned* bits;             // a bit per pixel: the root of a component
+  unsigned* before;           // per 32 pixels: components of the same kScanTile pixels before them
   unsigned long long* cnt;    // counters: 0 small, 1 merged, 2 components
   int* ncomp;                 // the component count as int (read by later kernels)
   int* nbig;                  // [0] entries at the front of `big`, [1] at the back
@@ -177,10 +182,29 @@ __device__ __forceinline__ void unite(int* p, int a, int b, int* err) {
 
 __device__ __forceinline__ bool small_size(long long s, int K, long long N) { return 4LL * K * s < N; }
 
+// Loops over the roots q of image im's tiles, a warp per tile (fewer than 2^30
+// tiles: 32-bit divisions).
+#define FOR_TILE_ROOTS(q)                                                                                      \
+  const unsigned tx_ = unsigned(im.W + kCcTile - 1) / kCcTile;                                                 \
+  const unsigned tiles_ = tx_ * ((unsigned(im.H) + unsigned(tile_rows) - 1u) / unsigned(tile_rows));           \
+  for (unsigned t_ = blockIdx.x * kCcWarps + (threadIdx.x >> 5); t_ < tiles_; t_ += gridDim.x * kCcWarps)      \
+    for (int y_ = int(t_ / tx_),                                                                               \
+             at_ = int(tile_place(im, int(t_ - unsigned(y_) * tx_) * kCcTile, y_ * tile_rows,                  \
+                                  min(tile_rows, im.H - y_ * tile_rows))),                                     \
+             i_ = int(threadIdx.x & 31), n_ = S.nroots[at_];                                                   \
+         i_ < n_; i_ += 32)                                                                                    \
+      if (const int q = S.roots[at_ + i_]; true)
+
 // Per-component loops over c < *S.ncomp.
 #define FOR_COMPONENTS(c)      \
   const int ncomp_ = *S.ncomp; \
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncomp_; c += gridDim.x * blockDim.x)
+
+// Where a tile's list starts: the pixels of the tiles before it, tile row after
+// tile row (a tile has no more roots than pixels).
+__device__ __forceinline__ long long tile_place(const Img& im, int x0, int y0, int rows) {
+  return im.off + (long long)y0 * im.W + (long long)x0 * rows;
+}
 
 // Labels one tile of 32 x 32 pixels (x tile_rows where the call has few pixels:
 // a tile is a serial walk) per warp.  A row's runs of one label come from a
@@ -194,14 +218,18 @@ __device__ __forceinline__ bool small_size(long long s, int K, long long N) { re
 // 308 us on 256 images of 481x321, 170 this way.)  Only the tiles' borders are left to
 // global unions: 6 % of the pixels (labelling all of them in global memory
 // took 195 + 703 us).
-__global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict__ imgs, int* __restrict__ p,
-                                                          int* err, int tile_rows) {
+__global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict__ imgs, Scratch S, int nwords,
+                                                          int tile_rows) {
   __shared__ int parent[kCcWarps][kCcTile * kCcTile];            // over the numbers given
   __shared__ uint16_t first[kCcWarps][kCcTile * kCcTile];        // a number's first pixel
   __shared__ uint16_t number[kCcWarps][kCcTile * kCcTile];       // of every pixel
   __shared__ unsigned queue[kCcWarps][64];                       // unions to do: two numbers each
   const Img im = imgs[blockIdx.y];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int *p = S.parent, *err = S.err;
+  for (int i = int((blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x); i < nwords;
+       i += int(gridDim.x * gridDim.y * blockDim.x))
+    S.bits[i] = 0u;
   const int tx = (im.W + kCcTile - 1) / kCcTile;
   const long long tiles = (long long)tx * ((im.H + tile_rows - 1) / tile_rows);
   const unsigned below = (1u << lane) - 1u, upto = 0xffffffffu >> (31 - lane);
@@ -264,15 +292,23 @@ __global__ void __launch_bounds__(kCcWarps * 32) k_cc_tile(const Img* __restrict
       }
     }
     work(1);
-    // every number's root, as a pixel of the tile (F of a root stays)
-    for (int i = lane; i < given; i += 32) {
-      const int root = find_root(q, i, err);
-      q[i] = root;
-      F[i] = F[root];
+    // every number's root, as a pixel of the tile (F of a root stays); the roots go to the tile's list
+    const int at0 = int(im.off + g0);
+    const long long place = tile_place(im, x0, y0, rows);
+    int listed = 0;
+    for (int i = lane; i - lane < given; i += 32) {
+      const int root = i < given ? find_root(q, i, err) : -1;
+      const unsigned is_root = __ballot_sync(0xffffffffu, root == i);
+      if (root == i) S.roots[place + listed + __popc(is_root & below)] = at0 + (F[i] >> 5) * im.W + (F[i] & 31);
+      listed += __popc(is_root);
+      if (root >= 0) {
+        q[i] = root;
+        F[i] = F[root];
+      }
     }
+    if (lane == 0) S.nroots[place] = listed;
     __syncwarp();
     int* P = p + im.off + g0 + lane;
-    const int at0 = int(im.off + g0);
     for (int r = 0; r < rows; ++r, P += im.W) {
       if (!in) continue;
       const int root = F[R[r * 32 + lane]];
@@ -355,40 +391,69 @@ __device__ __forceinline__ int image_of(const Img* __restrict__ imgs, int n, lon
   return lo;
 }
 
-// After the unions: every pixel points at its root, and the roots are counted
-// per tile of kScanTile pixels.  The walks only read, so the one store per
-// pixel (its root) cannot be overwritten by another thread's walk (a halving
+// After the unions only the tiles' roots are looked at again (a few per cent
+// of the pixels; every pixel points at one): each points at its component's
+// root, and the components' roots set their bits.  The walks only read, so the
+// one store per root cannot be overwritten by another thread's walk (a halving
 // store here could leave a non-root behind).  The compact indices of the
-// components are in the order of their roots (smallest pixels): these counts,
-// a scan of them, the assignment; no counter that every block updates.
-__global__ void __launch_bounds__(1024) k_cc_flatten(long long T, Scratch S) {
-  __shared__ unsigned warp_sums[32];
-  const long long g0 = (long long)blockIdx.x * kScanTile + 4LL * threadIdx.x;
-  int c = 0;
-  if (g0 + 3 < T) {
-    int4 q = *reinterpret_cast<const int4*>(S.parent + g0);
-    c = (q.x == int(g0)) + (q.y == int(g0 + 1)) + (q.z == int(g0 + 2)) + (q.w == int(g0 + 3));
-    q.x = find_root(S.parent, q.x, S.err);
-    q.y = find_root(S.parent, q.y, S.err);
-    q.z = find_root(S.parent, q.z, S.err);
-    q.w = find_root(S.parent, q.w, S.err);
-    *reinterpret_cast<int4*>(S.parent + g0) = q;
-  } else {
-    for (int j = 0; j < 4 && g0 + j < T; ++j) {
-      const int q = S.parent[g0 + j];
-      c += q == int(g0 + j);
-      S.parent[g0 + j] = find_root(S.parent, q, S.err);
-    }
+// components are in the order of their roots (smallest pixels): bits set
+// before, counted and scanned; no counter that every block updates.  (Over all
+// pixels, which a second pass read again for the indices: 96 + 116 us on 256
+// images of 481x321.)
+__global__ void __launch_bounds__(kCcWarps * 32) k_tile_roots(const Img* __restrict__ imgs, Scratch S, int tile_rows) {
+  const Img im = imgs[blockIdx.y];
+  FOR_TILE_ROOTS(q) {
+    const int r = find_root(S.parent, q, S.err);
+    S.parent[q] = r;
+    if (r == q) atomicOr(S.bits + (q >> 5), 1u << (q & 31));
   }
-  unsigned total;
-  block_exclusive_scan(unsigned(c), warp_sums, total);
-  if (threadIdx.x == 0) S.tile_sum[blockIdx.x] = int(total);
+}
+
+// Components of tile `tile` of kScanTile pixels (the warp's result), and of
+// those the ones before each 32 pixels: four words per lane.
+__device__ __forceinline__ int count_roots(const Scratch& S, int tile, int nwords, int lane) {
+  const int w0 = tile * (kScanTile / 32) + 4 * lane;
+  int n[4], sum = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    n[j] = w0 + j < nwords ? __popc(S.bits[w0 + j]) : 0;
+    sum += n[j];
+  }
+  int x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  const int total = __shfl_sync(0xffffffffu, x, 31);
+  x -= sum;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (w0 + j < nwords) S.before[w0 + j] = unsigned(x);
+    x += n[j];
+  }
+  return total;
+}
+
+__global__ void __launch_bounds__(256) k_root_count(int ntiles, int nwords, Scratch S) {
+  const int tile = int(blockIdx.x * 8 + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  if (tile >= ntiles) return;
+  const int n = count_roots(S, tile, nwords, lane);
+  if (lane == 0) S.tile_sum[tile] = n;
 }
 
 // Exclusive scan of the ntiles tile counts in place (one block); the total
-// is the component count.
-__global__ void __launch_bounds__(1024) k_root_scan(int ntiles, Scratch S) {
+// is the component count.  COUNT: the block counts them first (few tiles).
+template <bool COUNT>
+__global__ void __launch_bounds__(1024) k_root_scan(int ntiles, int nwords, Scratch S) {
   __shared__ unsigned warp_sums[32];
+  if (COUNT) {
+    for (int tile = int(threadIdx.x >> 5); tile < ntiles; tile += 32) {
+      const int n = count_roots(S, tile, nwords, int(threadIdx.x & 31));
+      if ((threadIdx.x & 31) == 0) S.tile_sum[tile] = n;
+    }
+    __syncthreads();
+  }
   int carry = 0;
   for (int c = 0; c < ntiles; c += 1024) {
     const int i = c + threadIdx.x;
@@ -404,39 +469,26 @@ __global__ void __launch_bounds__(1024) k_root_scan(int ntiles, Scratch S) {
   }
 }
 
-__global__ void __launch_bounds__(1024) k_root_assign(const Img* __restrict__ imgs, int n, long long T, Scratch S) {
-  __shared__ unsigned warp_sums[32];
-  __shared__ uint16_t root[kScanTile];  // the tile's roots in order, so that a thread takes one
-  __shared__ int first_image;
-  const long long base = (long long)blockIdx.x * kScanTile, g0 = base + 4LL * threadIdx.x;
-  bool f[4];
-  int cnt = 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    f[j] = g0 + j < T && S.parent[g0 + j] == int(g0 + j);
-    cnt += f[j];
-  }
-  if (threadIdx.x == 0) first_image = image_of(imgs, n, base);
-  unsigned total;
-  unsigned at = block_exclusive_scan(unsigned(cnt), warp_sums, total);
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    if (f[j]) root[at++] = uint16_t(4 * threadIdx.x + j);
-  __syncthreads();
-  const int c0 = S.tile_sum[blockIdx.x];
-  for (unsigned k = threadIdx.x; k < total; k += 1024) {
-    const long long g = base + root[k];
-    const int c = c0 + int(k);
-    int i = first_image;
-    while (i + 1 < n && imgs[i + 1].off <= g) ++i;
-    S.cidr[g] = c;
-    S.cimg[c] = i;
-    S.clabel[c] = imgs[i].labels[g - imgs[i].off];
+// The compact index at every tile's root; the start of every component, what is
+// zero in the order of the components (tile after tile, each 32-byte sector
+// of these arrays is written in several pieces: 106 us on 256 images of 481x321).
+__global__ void __launch_bounds__(kCcWarps * 32) k_root_assign(const Img* __restrict__ imgs, Scratch S, int tile_rows) {
+  const Img im = imgs[blockIdx.y];
+  const int ncomp = *S.ncomp, step = int(gridDim.x * gridDim.y * blockDim.x);
+  for (int c = int((blockIdx.y * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x); c < ncomp; c += step) {
     S.size[c] = 0;
     S.deg[c] = 0;
     S.cl_count[c] = 0;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) S.csum[3LL * c + q] = 0;
+    for (int k = 0; k < 3; ++k) S.csum[c + (long long)k * ncomp] = 0;
+  }
+  FOR_TILE_ROOTS(q) {
+    const int r = S.parent[q];
+    const int c = S.tile_sum[r / kScanTile] + int(S.before[r >> 5]) + __popc(S.bits[r >> 5] & ((1u << (r & 31)) - 1u));
+    S.cidr[q] = c;
+    if (r != q) continue;
+    S.cimg[c] = int(blockIdx.y);
+    S.clabel[c] = im.labels[q - im.off];
   }
 }
 
@@ -457,7 +509,7 @@ __global__ void __launch_bounds__(128) k_comp_map(const Img* __restrict__ imgs, 
     const int cy = int(t / cx), x = int(t - (long long)cy * cx) * kChunk + 4 * lane, y0 = cy * chunk_rows;
     const int n = min(4, im.W - x), rows = min(chunk_rows, im.H - y0);
     if (n <= 0) continue;
-    int root = -1, c = 0, cnt = 0;
+    int c = -1, cnt = 0;
     long long s0 = 0, s1 = 0, s2 = 0;
     auto flush = [&] {
       if (!cnt) return;
@@ -482,21 +534,19 @@ __global__ void __launch_bounds__(128) k_comp_map(const Img* __restrict__ imgs, 
     };
     ahead(P, Z);
     for (int r = 0; r < rows; ++r, P += im.W, Z += im.W) {
-      int q[4], cq[4];
+      int cq[4];
       float z[3][4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        q[j] = qn[j];
-        cq[j] = j < n ? S.cidr[q[j]] : 0;
+        cq[j] = j < n ? S.cidr[qn[j]] : 0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) z[k][j] = zn[k][j];
       }
       if (r + 1 < rows) ahead(P + im.W, Z + im.W);
       auto add = [&](int j) {
         if (j >= n) return;
-        if (q[j] != root) {
+        if (cq[j] != c) {
           flush();
-          root = q[j];
           c = cq[j];
           cnt = 0;
           s0 = s1 = s2 = 0;
@@ -1184,6 +1234,12 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   S.nbig = reinterpret_cast<int*>(b + o[O_CNT] + 192);
   S.cl_key = reinterpret_cast<unsigned long long*>(b + o[O_KEY]);
   S.tile_sum = ia(O_TILE);
+  // before the adjacency lists, the cluster keys and the member lists are written
+  const int nwords = int((T + 31) / 32);
+  S.roots = S.adj;
+  S.bits = reinterpret_cast<unsigned*>(S.cl_key);
+  S.before = S.aoff;
+  S.nroots = S.next;
   // blocks per image: enough to fill the machine across the images
   const long long per = std::max<long long>(1, std::min<long long>((maxN + 255) / 256, (152LL * 16 + n - 1) / n));
   const dim3 gp{static_cast<unsigned>(per), static_cast<unsigned>(n)};
@@ -1216,11 +1272,16 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   int herr = 0;
   do {
     if ((e = cudaMemcpyAsync(table, up_host.data(), up_host.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
-    k_cc_tile<<<gt, kCcWarps * 32, 0, s>>>(table, S.parent, S.err, tile_rows);
+    k_cc_tile<<<gt, kCcWarps * 32, 0, s>>>(table, S, nwords, tile_rows);
     k_cc_border<<<gp, 256, 0, s>>>(table, S.parent, S.err, tile_rows);
-    k_cc_flatten<<<nt, 1024, 0, s>>>(T, S);
-    k_root_scan<<<1, 1024, 0, s>>>(int(ntiles), S);
-    k_root_assign<<<nt, 1024, 0, s>>>(table, n, T, S);
+    k_tile_roots<<<gt, kCcWarps * 32, 0, s>>>(table, S, tile_rows);
+    if (one) {
+      k_root_scan<true><<<1, 1024, 0, s>>>(int(ntiles), nwords, S);
+    } else {
+      k_root_count<<<(nt + 7) / 8, 256, 0, s>>>(int(ntiles), nwords, S);
+      k_root_scan<false><<<1, 1024, 0, s>>>(int(ntiles), nwords, S);
+    }
+    k_root_assign<<<gt, kCcWarps * 32, 0, s>>>(table, S, tile_rows);
     k_comp_map<<<gc, 128, 0, s>>>(table, S, rows);
     k_comp_flags<<<gs, 256, 0, s>>>(table, S);
     if (one) {
