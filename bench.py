@@ -78,13 +78,23 @@ FLOPS_PER_CAND_MODEL = {"full": FLOPS_PER_CAND, "split": 53, "gray": 33}
 
 # The E + M pass's other two rooflines, reported beside the binding FP32 one:
 #   HBM: DRAM bytes per launch (ncu-measured where the launch variant was captured, else the
-#        algorithmic 12 B of CIELAB per pixel plus the 544 B FP32 partial of every cell) over
+#        algorithmic 12 B of CIELAB per pixel plus the 576 B FP32 partial of every cell) over
 #        the pass time, against the measured copy bandwidth of MEASURED_PEAKS.json;
 #   MUFU (XU pipe): one ex2 per (pixel, candidate) and rcp + lg2 per pixel over the pass time,
 #        against 152 SMs x 32 results per clock (the project probe's measured ex2 rate per SM)
 #        x 2.07 GHz.
 MUFU_PEAK_TOPS = 152 * 32 * 2.070e9 / 1e12
-PARTIAL_BYTES_PER_CELL = 544
+PARTIAL_BYTES_PER_CELL = 576
+
+
+def batch_parts(bt, n):
+    """Parts in which a batch context of n images launches its EM iterations and label pass: two, beside one
+    another, from 16 cells per SM on with the one-cell-per-warp launches (6 blocks per SM or more), else one."""
+    import torch
+    t = bt.tuning()
+    sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    return 2 if (n > 1 and bt.info()[2] >= 16 * sms and
+                 min(t["blocks_per_sm"], t["first_pass_blocks_per_sm"]) >= 6) else 1
 
 
 def side_rooflines(units, pixels, cells, em_ms, traffic):
@@ -463,7 +473,7 @@ def run_other_workload(args):
                   "images": 256, "pixels": pix, "K": K, "cells": cells, "blocks_per_sm": bps,
                   "colour_model": args.colour,
                   "l2": "flushed between timed steps (256 MiB memset)"}
-        launches = 2 + 2 * ITERS + 1
+        launches = 2 + (2 * ITERS + 1) * batch_parts(bt, 256)
         extra = {"loglik_mean_per_pixel": float(np.sum(ll)) / pix, "em_pass_autotune_ms": tune}
         bt.close()
     else:
@@ -528,8 +538,8 @@ NET_FLOPS_PER_CELL = 2 * (3 * 288 * 32 + 288 * 16)
 # 96 such images (dram__bytes_read.sum + dram__bytes_write.sum), scaled per image
 # (traffic grows with the image count), per launch variant (blocks per SM); a variant
 # not captured with the current kernel reports null.
-#   7: one-cell-per-warp k_em_pass_batch_flat capped at 72 registers: 182.06 MB + 29.63 MB.
-EM_BATCH_TRAFFIC_PER_IMAGE = {7: int((182.059520e6 + 29.629184e6) / 96)}
+#   6: one-cell-per-warp k_em_pass_batch_flat capped at 80 registers: 182.05 MB + 30.31 MB.
+EM_BATCH_TRAFFIC_PER_IMAGE = {6: int((182.050304e6 + 30.305792e6) / 96)}
 
 
 def measured_peaks():
@@ -610,6 +620,7 @@ def run_learned(args):
         learned.set_init_net(net)
         tuning = {"plain": plain.tuning(), "learned": learned.tuning(),
                   "em_pass_ms_by_blocks_per_sm": {str(k): round(v_, 5) for k, v_ in tune.items()}}
+        learned_parts = batch_parts(learned, n)
     step_l = lambda: learned.segment(imgs, LEARN_T)  # noqa: E731
     step_p = lambda: plain.segment(imgs, ITERS)  # noqa: E731
     with torch.cuda.stream(stream):
@@ -803,7 +814,7 @@ def run_learned(args):
                        "step overlap the kernels of the others); each step copies its images in (one copy of the stacked "
                        "images) and its labels out (one copy of the context's label buffer)",
                 "serial": round(e2e_serial, 3), "clocks": clk_e2e.summary()},
-        "gpu_launches": (1 + 5 + 1 + 2 * LEARN_T + 1) * args.steps,
+        "gpu_launches": (1 + 5 + 1 + (2 * LEARN_T + 1) * learned_parts) * args.steps,
         "clocks": clocks, "clocks_plain": clocks_p,
         "weights": os.path.relpath(pretrained_path(LEARN_V), ROOT),
     }
@@ -907,7 +918,7 @@ def run_profile_case(args):
 # Algorithmic DRAM bytes per pixel of the connectivity post-processing: the input
 # labels (4 B) and CIELAB colour (12 B) read once, the output labels (4 B) written.
 CONN_BYTES_PER_PIXEL = 20
-CONN_LAUNCHES = 21  # kernels of one gmmsp_batch_connectivity call
+CONN_LAUNCHES = 20  # kernels of one gmmsp_batch_connectivity call
 
 
 def _conn_case(gm, torch, n, stream, keep_images=False, regions=None):
@@ -1010,7 +1021,7 @@ def run_conn_workload(args):
 # Algorithmic DRAM bytes per pixel of the accuracy metrics: the labels and the ground
 # truth read once (4 + 4 B).
 METRICS_BYTES_PER_PIXEL = 8
-METRICS_LAUNCHES = 4  # kernels of one gmmsp_segmentation_metrics_many call
+METRICS_LAUNCHES = 2  # kernels of one gmmsp_segmentation_metrics_many call
 
 
 def run_metrics_workload(args):

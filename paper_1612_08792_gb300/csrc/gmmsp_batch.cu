@@ -1,7 +1,8 @@
 // Batched segmentation (declared in include/gmmsp.h, gmmsp_batch_*): many
 // images of uneven sizes through Algorithm 1, steps 1-7, with one launch per
 // step for the whole batch, the step sequence captured once into a CUDA
-// graph, and a persistent grid whose size the autotuner picks.
+// graph, and a launch shape that the autotuner picks (a persistent grid or one
+// cell per warp).  Larger batches run as two parts on two streams.
 //
 // Device memory of a batch context is one allocation: the CIELAB planes of
 // all images, theta / packed coefficients of all superpixels, the per-cell

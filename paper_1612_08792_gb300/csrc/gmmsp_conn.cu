@@ -26,11 +26,13 @@
 //
 // Kernels (all images of a call at once; pixel kernels take blockIdx.y as the
 // image, tile loops cover all pixels of the call):
-//   k_cc_tile                       union-find labelling of 32 x 32 tiles in
-//                                   shared memory, parent = the tile's root
+//   k_cc_tile                       labelling of 32 x 32 tiles, parent = the
+//                                   tile's root; the list of the tile's roots
 //   k_cc_border                     unions across the tiles' borders
-//   k_cc_flatten / k_root_scan / k_root_assign  parent = root pixel, compact
-//                                   index per root (tile counts, scan)
+//   k_tile_roots / k_root_count / k_root_scan / k_root_assign  the tiles'
+//                                   roots point at their component's, a bit per
+//                                   component, counts and a scan, compact index
+//                                   per tile root
 //   k_comp_map                      parent := compact index; sizes and
 //                                   fixed-point colour sums (atomics)
 //   k_comp_flags                    small flag, mean colour, group state per component

@@ -148,13 +148,19 @@ __device__ __forceinline__ void e_pixel(const float4* sp, unsigned mask, const P
 // slot (posteriors), of (x, y) pairs, of (L, a) pairs and of b, the pixel of E
 // lane i at 12 (i mod 3) + i / 3.  The pixels of one M phase are then
 // consecutive and 16-byte aligned, and an M lane reads four of its pixels with
-// six loads: 18 loads per batch instead of 33, about 45 wavefronts instead of
-// 88.  Its pixels keep their order, so the sums keep their bits.
+// six loads: 18 loads per batch instead of 33 (a 16-byte load of three
+// addresses costs about 3.3 wavefronts, so the wavefronts stay about the
+// same).  256 images of 481x321: 0.986 -> 0.953 ms.  Its pixels keep their
+// order, so the sums keep their bits.
 //
-// The pass is bound by instruction issue (84 % of the cycles before the
-// following): the statistics of x and y, and of L and a, run as packed FP32
-// pairs, which takes 18 instructions per (pixel, slot) instead of 25, each
-// component rounded as before.
+// The statistics of x and y, and of L and a, run as packed FP32 pairs, which
+// takes 18 instructions per (pixel, slot) instead of 25, each component
+// rounded as before (0.953 -> 0.909 ms with the E part's pairs); the pixels
+// are walked by additions (0.893 at 6 blocks per SM).  What bounds it now, 18.6
+// warp instructions per pixel (24.0 before): issue 65 %, FMA pipe 56 % (a
+// packed operation takes it for two cycles), LSU data pipe 87 % of its
+// wavefronts, fixed-latency waits.  Taking a tenth of the wavefronts away
+// (candidates' parameters in tensor memory) did not make it faster.
 constexpr int kBatchLd = 36;
 constexpr int kBatchXY = kSlots * kBatchLd, kBatchLa = kBatchXY + 2 * kBatchLd, kBatchB = kBatchLa + 2 * kBatchLd,
               kBatchFloats = kBatchB + kBatchLd;
@@ -441,9 +447,10 @@ __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_batch(const Bat
 }
 
 // Non-persistent variant: one cell per warp over a grid sized to the work,
-// registers capped so that MINB blocks fit on an SM (6: 80 registers and 8
-// bytes of spill; 7: 72 registers and some spill); the autotuner's choice of
-// 6 or 7 blocks per SM selects it.  DIAG: every superpixel's blocks are
+// registers capped so that MINB blocks fit on an SM (6: 80 registers; 7: 72
+// registers, with more spill); 6 or 7 blocks per SM select it.  It covers the
+// cells [first, total_cells).  256 images of 481x321: 0.893 ms at 6, 0.953 at
+// 7 (first pass 0.832 and 0.844); the persistent kernel 0.986 at 5.  DIAG: every superpixel's blocks are
 // diagonal (the first pass after either start).
 template <typename PT, bool SHIFT, int MINB, int CM, bool DIAG = false>
 __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_batch_flat(const BatchImage* __restrict__ imgs, int n,
