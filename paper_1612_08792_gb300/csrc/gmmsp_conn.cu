@@ -72,7 +72,7 @@ constexpr int kCcTile = 32;            // side of the tiles labelled in shared m
 constexpr int kCcWarps = 4;            // tiles per block
 constexpr int kCcAhead = 8;            // rows of labels in flight
 constexpr int kChunk = 128;            // pixels a warp walks down at once: four per lane
-constexpr int kChunkRows = 32;         // at most; fewer where the call has few pixels
+constexpr int kMapRows = 16, kEdgeRows = 8;  // ... by k_comp_map and k_edges at most; fewer where the call has few pixels
 constexpr long long kOneBlockScan = 1 << 18;  // pixels up to which one block scans (64 steps at most)
 
 // One image of a call: pixels [off, off + W H) of the call's arrays.
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(kCcWarps * 32) k_root_assign(const Img* __rest
 }
 
 // parent := compact index of the pixel's component; component sizes and
-// fixed-point colour sums.  A warp walks a chunk of 128 pixels down 32 rows,
+// fixed-point colour sums.  A warp walks a chunk of 128 pixels down 16 rows,
 // four pixels per lane; a lane adds its pixels of one component in registers,
 // going back and forth along its four pixels, and updates the component's sums
 // when it changes: about one set of atomics per eight pixels.  (A warp-wide
@@ -620,7 +620,7 @@ __device__ __forceinline__ void add_edge(const Scratch& S, int i, int j) {
 // the previous edge along the same line already gave (the row above for the
 // edge to the right, the pixel to the left for the edge below) is skipped: the
 // lists are neighbour sets, and most repeats go.  A warp walks a chunk of 128
-// pixels down 32 rows, four pixels per lane with the rows above and below in
+// pixels down 8 rows, four pixels per lane with the rows above and below in
 // registers, so an index is loaded once; the edges found go through a queue in
 // shared memory and are worked on 32 at a time, so that their chains of random
 // accesses overlap (worked on where they were found: 684 us on 256 images of
@@ -1255,13 +1255,15 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
       most = std::max(most, ((W[i] + w - 1LL) / w) * ((H[i] + h - 1LL) / h));
     return dim3(unsigned(std::max<long long>(1, std::min<long long>((most + 3) / 4, (152LL * 64 + n - 1) / n))), unsigned(n));
   };
-  // rows a warp walks: 32, fewer where that would leave most of the machine idle (the walk over a chunk is serial)
+  // rows a warp walks: fewer where the most would leave much of the machine idle (the walk over a chunk is serial).  On
+  // 256 images of 481x321 (128-pixel chunks: 11264 warps at 32 rows, 2.3 waves) the sums take 283 / 276 / 291 us and
+  // the edges 251 / 229 / 215 us at 32 / 16 / 8 rows.
   long long chunk_cols = 0;
   for (int i = 0; i < n; ++i) chunk_cols += (W[i] + kChunk - 1LL) / kChunk * H[i];
-  int rows = kChunkRows;
+  int rows = kCcTile;
   while (rows > 4 && chunk_cols / rows < 152LL * 32) rows /= 2;
-  const int tile_rows = rows < kChunkRows ? 8 : kCcTile;
-  const dim3 gt = blocks_of(kCcTile, tile_rows), gc = blocks_of(kChunk, rows);
+  const int tile_rows = rows < kCcTile ? 8 : kCcTile, map_rows = std::min(rows, kMapRows), edge_rows = std::min(rows, kEdgeRows);
+  const dim3 gt = blocks_of(kCcTile, tile_rows), gm = blocks_of(kChunk, map_rows), ge = blocks_of(kChunk, edge_rows);
   // merging: twice as many blocks as fit on the machine for either kind of cluster, so that an SM whose clusters are
   // done early takes more (half of the resident blocks for either kind: 549 us, 2.13 ms for the call on 256 images of
   // 481x321; this many 1.93 ms, and no less with 32 to 128 per SM)
@@ -1284,7 +1286,7 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
       k_root_scan<false><<<1, 1024, 0, s>>>(int(ntiles), nwords, S);
     }
     k_root_assign<<<gt, kCcWarps * 32, 0, s>>>(table, S, tile_rows);
-    k_comp_map<<<gc, 128, 0, s>>>(table, S, rows);
+    k_comp_map<<<gm, 128, 0, s>>>(table, S, map_rows);
     k_comp_flags<<<gs, 256, 0, s>>>(table, S);
     if (one) {
       k_scan_one<kScanLists><<<1, 1024, 0, s>>>(S, S.aoff);
@@ -1293,7 +1295,7 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
       k_scan_tile_sums<<<1, 1024, 0, s>>>(S, S.aoff);
       k_scan_add<<<nt, 1024, 0, s>>>(S, S.aoff);
     }
-    k_edges<<<gc, 128, 0, s>>>(table, S, rows);
+    k_edges<<<ge, 128, 0, s>>>(table, S, edge_rows);
     k_cluster_count<<<gs, 256, 0, s>>>(S);
     if (one) {
       k_scan_one<kScanClusters><<<1, 1024, 0, s>>>(S, S.cl_off);
