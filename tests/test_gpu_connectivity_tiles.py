@@ -1,7 +1,7 @@
-"""Connectivity post-processing at the edges of its tiles (32 x 32 labelling tiles, chunks of 128 x 32 pixels)
+"""Connectivity post-processing at the edges of its tiles (32 x 32 labelling tiles, chunks of 128 pixels by 16 and 8 rows)
 against the oracle: exact.  Components that wind through many tiles, widths and heights around the tile sizes,
-one-pixel checkerboards (every pixel a component, full adjacency lists), and a call large enough for the
-multi-block scans."""
+one-pixel checkerboards (every pixel a component, full adjacency lists), a call large enough for the
+multi-block scans, and one of so many pixel rows that tiles and chunks take their full heights."""
 import numpy as np
 import pytest
 
@@ -79,3 +79,36 @@ def test_near_ties_are_decided_in_fp64(spread):
     L[m] = rng.integers(20, 24, m.sum())
     lab = (np.array([60.0, -35.0, 80.0]) + spread * rng.normal(0, 1, (H, W, 3))).astype(np.float32)
     run(gm, [(L, lab, K)])
+
+
+def test_full_tile_rows_over_many_images():
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1612_08792_gb300 as gm
+    rng = np.random.default_rng(11)
+    v, n = 15, 1620
+    sizes = [(97, 33), (98, 31), (99, 64), (100, 65), (128, 32), (96, 130), (101, 40), (33, 97)]
+    sizes = [sizes[i % 8] for i in range(n)]
+    chunk_rows = sum(-(-w // 128) * h for h, w in sizes)
+    assert chunk_rows >= 32 * 152 * 32               # the full 32 rows
+    maps, ref = [], []
+    for i, (h, w) in enumerate(sizes[:8]):
+        lab = rng.normal(40, 20, (h, w, 3)).astype(np.float32)
+        lab[rng.random((h, w)) < 0.3] = 40.0
+        L, K = winding(h, w, rng, 0.02 * (i + 1)), (w // v) * (h // v)
+        maps.append((torch.from_numpy(L).cuda(), torch.from_numpy(lab).cuda()))
+        ref.append(oc.enforce_connectivity(L, lab, K))
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        bt = gm.SuperpixelsBatch(sizes, spacing=v, lab_input=True)
+        bt.segment([maps[i % 8][1] for i in range(n)], 0)      # the CIELAB planes
+        for i, x in enumerate(bt.labels):
+            x.copy_(maps[i % 8][0])
+        st = bt.connectivity()
+        got = [x.cpu().numpy() for x in bt.labels]
+    for i in range(n):
+        np.testing.assert_array_equal(got[i], ref[i % 8][0])
+    for key in st:
+        assert st[key] == sum(ref[i % 8][1][key] for i in range(n))
+    bt.close()
