@@ -37,6 +37,7 @@
 #include "../../include/gmmsp.h"
 #include "../../include/gmmsp_cnn.h"
 #include "gmmsp_cnn_internal.cuh"
+#include "gmmsp_grid3.cuh"
 #include "gmmsp_internal.cuh"
 #include "gmmsp_lab.cuh"
 #include "gmmsp_math.cuh"
@@ -86,13 +87,7 @@ __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u <<
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
 // ------------------------------------------------- 3 x 3 layers: tiles
-// The cell grid of an image is cut into strips of at most kStripMax columns
-// (one strip up to nx = 126).  Within a strip the positions are numbered with
-// a zero border column on either side, q = y PW + x', PW = TW + 2, x' = 0 and
-// PW - 1 being the neighbouring columns (zero outside the image).  A tile is
-// 128 consecutive numbers q; its inputs are the 130 + 2 PW numbers
-// q0 - PW - 1 .. q0 + 127 + PW + 1 (rows above and below the image zero), and
-// tap (dy, dx) of row q is the input at q + dy PW + dx.
+// Tiles, their positions and inputs: gmmsp_grid3.cuh.
 //
 // In shared memory the inputs lie as channel groups of 8 (16 bytes), position
 // after position: group g of input i at g GS + 16 i.  Eight consecutive
@@ -103,50 +98,9 @@ __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 
 // times from L2 and paid one MMA round trip per tap).  The same bytes serve as
 // a K-major operand (rows = positions: 8-row groups 128 bytes apart, K groups
 // GS apart) and as an MN-major one (K = positions).
-constexpr int kStripMax = 126;
 constexpr int kWLd = 528;                     // bytes between (tap, input group) slices of the staged weights
 constexpr int kWBytes = 36 * kWLd;            // 9 taps x 4 groups x 32 output channels x 16 bytes, padded
 constexpr int kRowTile = 128 * 16 + 32;       // a group of a 128-position tile without halo (bank offset 32)
-
-struct Grid3 {
-  int B, H, W;         // images and their cell grids
-  int strips, TW, PW;  // strips per image, their columns, the bordered row length
-  int tps;             // tiles per strip
-  int tiles;           // B strips tps
-  int NP, GS;          // inputs of a tile; bytes per channel group of them
-  unsigned rPW;        // floor(2^32 / PW) + 1: q / PW = umulhi(q, rPW) for q PW < 2^32, which holds here
-                       // (PW <= 128, and H PW <= 3 * the image's < 2^31 / 9 cells for narrower strips)
-};
-inline Grid3 grid3_of(int B, int H, int W) {
-  Grid3 g{};
-  g.B = B;
-  g.H = H;
-  g.W = W;
-  g.strips = (W + kStripMax - 1) / kStripMax;
-  g.TW = (W + g.strips - 1) / g.strips;
-  g.PW = g.TW + 2;
-  g.rPW = unsigned((1ull << 32) / unsigned(g.PW)) + 1u;
-  g.tps = (H * g.PW + 127) / 128;
-  g.tiles = B * g.strips * g.tps;
-  g.NP = 130 + 2 * g.PW;
-  g.GS = (g.NP * 16 + 127) / 128 * 128 + 32;  // 32 mod 128: the four groups of a position fall into other banks
-  return g;
-}
-
-struct Tile3 {
-  int img, c0, q0;
-};
-__device__ __forceinline__ Tile3 tile3_at(const Grid3& g, int tile) {
-  const int s = tile / g.tps;
-  return {s / g.strips, (s % g.strips) * g.TW, (tile - s * g.tps) * 128};
-}
-
-// Row of position q of a tile's strip in the [B H W] arrays, or -1 where q is
-// no output (border column, below the image, past the strip or the image).
-__device__ __forceinline__ int row3(const Grid3& g, const Tile3& t, int q) {
-  const int y = int(__umulhi(unsigned(q), g.rPW)), x = q - y * g.PW, col = t.c0 + x - 1;
-  return (y < g.H && x >= 1 && x <= g.TW && col < g.W) ? (t.img * g.H + y) * g.W + col : -1;
-}
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
@@ -159,11 +113,8 @@ __device__ __forceinline__ void load_halo(const Grid3& g, const Tile3& t, const 
                                           uint32_t dst) {
   for (int i = threadIdx.x; i < g.NP * G; i += 128) {
     const int p = i / G, gr = i - p * G;
-    const int q = t.q0 + p + g.PW - 1;  // t.q0 - (PW + 1) + p + 2 PW, not negative
-    const int y = int(__umulhi(unsigned(q), g.rPW)) - 2, col = t.c0 + q - (y + 2) * g.PW - 1;
-    const bool ok = unsigned(y) < unsigned(g.H) && unsigned(col) < unsigned(g.W);
-    const int r = ok ? (t.img * g.H + y) * g.W + col : 0;
-    cp_async16(dst + gr * g.GS + p * 16, x + (long long)r * (8 * G) + gr * 8, ok);
+    const int r = in3(g, t, p);
+    cp_async16(dst + gr * g.GS + p * 16, x + (long long)max(r, 0) * (8 * G) + gr * 8, r >= 0);
   }
 }
 
@@ -264,7 +215,7 @@ __global__ void __launch_bounds__(128, 6) k_conv3(Conv3 c, int* err) {
       }
       tc::mma_commit(&mbar);
     }
-    const int row = row3(c.g, t, t.q0 + tid);
+    const int row = row3(c.g, t, tid);
     uint4 m[4] = {};
     if (DGRAD && c.mask && row >= 0) {
       const uint4* ms = reinterpret_cast<const uint4*>(c.mask + (long long)row * kC);
@@ -328,7 +279,7 @@ __device__ __forceinline__ void load_rows3(const Grid3& g, const Tile3& t, const
                                            uint32_t dst) {
   for (int i = threadIdx.x; i < 128 * G; i += 128) {
     const int p = i / G, gr = i - p * G;
-    const int r = row3(g, t, t.q0 + p);
+    const int r = row3(g, t, p);
     cp_async16(dst + gr * kRowTile + p * 16, x + (long long)max(r, 0) * (8 * G) + gr * 8, r >= 0);
   }
 }
