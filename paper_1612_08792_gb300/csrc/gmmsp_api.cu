@@ -74,6 +74,7 @@ struct gmmsp_ctx_s {
   int wpc = 1;                    // warps per cell of the E+M pass (launch shape)
   gmmsp::ConnScratch conn;        // post-processing scratch, kept between calls
   bool diag = true;               // theta as a start left it: covariance blocks diagonal
+  bool captured = false;          // a caller's graph holds steps on theta, whose replays are not seen here
   bool timing = false;            // record events between the kernels (gmmsp_set_timing)
   std::vector<cudaEvent_t> tev;   // timing events, created on demand
   int tev_used = 0;               // events recorded by the last enqueued sequence
@@ -184,6 +185,20 @@ gmmsp_status mark(gmmsp_ctx c) {
 // Smallest row pitch of a W-pixel row of the input format.
 long long row_bytes(int format, int W) {
   return (long long)W * (format == GMMSP_RGB8 ? 3 : (format == GMMSP_GRAY8 ? 1 : 12));
+}
+
+// Notes whether the caller is capturing the context's stream, at every entry
+// point that enqueues steps on theta.  From then on `diag` says nothing about
+// theta (a captured start has not run, and a replay runs without a call here),
+// so the E+M pass takes the general kernel, which gives the same bits; only a
+// segment, whose own sequence holds the start, still knows.
+void note_capture(gmmsp_ctx c) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    c->captured = true;
+  }
+  if (cs != cudaStreamCaptureStatusNone) c->captured = true;
 }
 
 // Enqueues step 1 of Algorithm 1: image -> CIELAB, theta_0; clears counters.
@@ -374,6 +389,7 @@ gmmsp_status gmmsp_reinit(gmmsp_ctx c, const void* image_dev, int pitch_bytes) {
   if (c->state == GMMSP_E_CUDA || c->state == GMMSP_E_NOMEM) return GMMSP_E_STATE;
   c->state = GMMSP_OK;
   c->err.clear();
+  note_capture(c);
   return enqueue_prepare(c, image_dev, pitch_bytes);
 }
 
@@ -382,6 +398,8 @@ gmmsp_status gmmsp_em_iters(gmmsp_ctx c, int iters, double* loglik_host) {
   gmmsp_status st = check_ready(c);
   if (st != GMMSP_OK) return st;
   if (iters < 0) return fail(c, GMMSP_E_INVALID, "iters < 0");
+  note_capture(c);
+  if (c->captured) c->diag = false;
   c->tev_used = 0;
   GM_MARK(c);
   for (int done = 0; done < iters; done += kLlkCap) {
@@ -551,6 +569,7 @@ gmmsp_status gmmsp_set_init(gmmsp_ctx c, const float* dmu_dev, const float* loge
   if (st != GMMSP_OK) return st;
   if (!dmu_dev || !logeig_dev) return fail(c, GMMSP_E_INVALID, "null array");
   if (c->g.cm == gmmsp::kColourGray) return fail(c, GMMSP_E_INVALID, "theta_0 arrays need a colour model with a, b");
+  note_capture(c);
   GM_CHECK(c, gmmsp::launch_init_from_outputs(dmu_dev, 5, logeig_dev, 5, c->lab, 1, c->g, c->p.lambda_c, c->p.eps_s,
                                               c->p.eps_c, c->theta, c->gp, c->counters, c->stream));
   c->diag = true;
@@ -572,6 +591,7 @@ gmmsp_status gmmsp_init_from_net(gmmsp_ctx c, gmmsp_net n) {
     c->err = why;  // the network's failure: the context stays usable
     return st;
   }
+  note_capture(c);
   GM_CHECK(c, gmmsp::net_enqueue_init(n, c->lab, nullptr, 1, c->g, c->p.lambda_c, c->p.eps_s, c->p.eps_c, c->theta, c->gp,
                                       c->counters, c->stream));
   c->diag = true;
