@@ -377,14 +377,15 @@ __device__ __forceinline__ void wgrad3_layer(const Wgrad3& c, int layer, int* er
     for (int c0 = 0; c0 <= 288; c0 += 16) {
       float v[16];
       tc::tmem_ld16(tmem + uint32_t(c0), v);
-      if (tid >= 8 * GC) continue;
-      if (c0 == 288) {
-        out[8 * GC * 288 + tid] = v[0];
-      } else {
-        const int j = c0 >> 5, tap = j < 4 ? j : (j < 8 ? j + 1 : 4);
-        float4* o = reinterpret_cast<float4*>(out + tid * 288 + tap * 32 + (c0 & 16));
+      if (tid < 8 * GC) {  // lanes past the channels only load
+        if (c0 == 288) {
+          out[8 * GC * 288 + tid] = v[0];
+        } else {
+          const int j = c0 >> 5, tap = j < 4 ? j : (j < 8 ? j + 1 : 4);
+          float4* o = reinterpret_cast<float4*>(out + tid * 288 + tap * 32 + (c0 & 16));
 #pragma unroll
-        for (int i = 0; i < 4; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+          for (int i = 0; i < 4; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
       }
     }
   }
