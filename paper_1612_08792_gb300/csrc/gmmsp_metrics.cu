@@ -121,7 +121,9 @@ __global__ void __launch_bounds__(kTileChunks * 32, 7) k_tiles(const MImg* __res
   const int halo = radius > 0 ? 1 : 0, rows = min(kTileRows, im.H - y0);
   unsigned bad = 0;
   for (int w = warp; w < kTileChunks + 2 * halo; w += kTileChunks) {
-    const int xw = x0 + kChunk * (w - halo), x = xw + 4 * lane;
+    // sides up to 2^31 - 1: a chunk that would start past the last int wraps to a
+    // negative column (outside), and no sum below goes past the image's sides
+    const int xw = int(unsigned(x0) + unsigned(kChunk * (w - halo))), x = xw + 4 * lane;
     const bool inner = w >= halo && w < halo + kTileChunks;
     if (xw < 0 || xw >= im.W) {  // no pixel of the chunk lies in the image
       for (int i = lane; i < (rows + 2 * radius) * 4; i += 32) sb[i >> 2][4 * w + (i & 3)] = 0;
@@ -130,7 +132,7 @@ __global__ void __launch_bounds__(kTileChunks * 32, 7) k_tiles(const MImg* __res
       continue;
     }
     const int beside = lane == 0 ? -1 : 4;
-    const bool lft = x > 0 && x < im.W, rgt = x + 4 < im.W;
+    const bool lft = x > 0 && x < im.W, rgt = im.W - x > 4;
     unsigned in = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) in |= x + j < im.W ? 1u << j : 0u;
@@ -140,8 +142,8 @@ __global__ void __launch_bounds__(kTileChunks * 32, 7) k_tiles(const MImg* __res
     Quad L;
     L.start(im.labels, at(y - 1), at(y), at(y + 1), in, beside);
     auto step = [&] {  // no step where the row below stays the first or the last
-      ++y;
-      return y >= 0 && y + 1 < im.H ? im.W : 0;
+      if (y < im.H) ++y;
+      return y >= 0 && y < im.H - 1 ? im.W : 0;
     };
     unsigned b[4];
     // the rows of the radius above and below the tile: superpixel bits only
@@ -318,7 +320,7 @@ extern "C" gmmsp_status gmmsp_segmentation_metrics_many(int n, const int32_t* co
                    cnt + size_t(C_N) * i};
   MImg* table = reinterpret_cast<MImg*>(b);
   std::vector<unsigned long long> hc(size_t(C_N) * n, 0ull);
-  const long long tx = (maxW + kTileChunks * (long long)kChunk - 1) / (kTileChunks * kChunk), ty = (maxH + kTileRows - 1LL) / kTileRows;
+  const long long tx = (maxW + (kTileChunks * kChunk - 1LL)) / (kTileChunks * kChunk), ty = (maxH + (kTileRows - 1LL)) / kTileRows;
   const unsigned perk = unsigned(std::min<long long>((maxK + 7) / 8, std::max<long long>(1, (152LL * 32 + n - 1) / n)));
   do {
     if ((e = cudaMemcpyAsync(table, host.data(), sizeof(MImg) * n, cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
