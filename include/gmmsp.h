@@ -322,6 +322,12 @@ gmmsp_status gmmsp_batch_get_lab(gmmsp_batch b, int i, float *lab_host);
 const char *gmmsp_batch_last_error(gmmsp_batch b);
 void gmmsp_batch_destroy(gmmsp_batch b);
 
+/* Gives back the device scratch that calls without a context (the accuracy
+ * metrics, gmmsp_enforce_connectivity) keep between them: at most 256 MiB per
+ * device.  Safe at any time; scratch in use stays until its call ends.
+ * Errors: GMMSP_E_CUDA. */
+gmmsp_status gmmsp_release_scratch(void);
+
 /*
  * Bounds-check status (no counterpart in the paper: a stand-in for a memory
  * checker, which is not run on this hardware).  A library built with the
@@ -352,12 +358,7 @@ void gmmsp_batch_destroy(gmmsp_batch b);
 #define GMMSP_BND_LABEL_K 8    /* a label's value: k in [0, K)                             */
 #define GMMSP_BND_CELL_LL 9    /* a cell's log-likelihood written: cell in [0, cells)      */
 #define GMMSP_BND_IMAGE 10     /* a batch item's image: in [0, n)                          */
-#define GMMSP_BND_ITEM 11      /* Gives back the device scratch that calls without a context (the accuracy
- * metrics, gmmsp_enforce_connectivity) keep between them: at most 256 MiB per
- * device.  Safe at any time; scratch in use stays until its call ends. */
-gmmsp_status gmmsp_release_scratch(void);
-
-/* a batch item in its image: cell or superpixel in range   */
+#define GMMSP_BND_ITEM 11      /* a batch item in its image: cell or superpixel in range   */
 gmmsp_status gmmsp_bounds_status(int *checked, unsigned long long *first_violation);
 
 /*
