@@ -718,7 +718,7 @@ def gmmsp_segmentation_metrics_many(labels, gts, Ks, Gs, radius: int = 2, eps: f
             or not all(t.is_contiguous() for t in gts)):
         raise ValueError("labels and gt must be contiguous (H, W) maps of one size")
     if shapes.count(shapes[0]) == n:
-        Hs, Ws = (np.full(n, d, dtype=np.int32) for d in shapes[0])
+        Hs, Ws = (np.full(n, shapes[0][i], dtype=np.int32) for i in (0, 1))
     else:
         Hs, Ws = (np.array([s[i] for s in shapes], dtype=np.int32) for i in (0, 1))
     out = np.empty(n, dtype=_METRICS_DTYPE)
