@@ -40,7 +40,7 @@ def _sources():
 def _fingerprint(extra_flags=()) -> str:
     h = hashlib.sha256()
     h.update(" ".join(extra_flags).encode())
-    files = _sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + [
+    files = _sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))) + [
         *sorted(glob.glob(os.path.join(ROOT, "include", "*.h"))),
         os.path.abspath(__file__)]
     for f in files:

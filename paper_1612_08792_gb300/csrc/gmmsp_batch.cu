@@ -22,6 +22,7 @@
 
 #include "../../include/gmmsp.h"
 #include "../../include/gmmsp_cnn.h"
+#include "gmmsp_batch_rules.h"
 #include "gmmsp_cnn_internal.cuh"
 #include "gmmsp_internal.cuh"
 
@@ -56,10 +57,10 @@ struct gmmsp_batch_s {
   gmmsp_net net = nullptr;         // learned initialiser (null: Sec. III-C start)
   bool uniform = true;             // all images of one size
   // Second stream of a batch that runs as two parts (see split_image; null: one part), its fork and join events,
-  // and the device's highest priority.
+  // and the launch priority of the parts' finalizes.
   cudaStream_t side = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
-  int high_priority = 0;
+  int fin_priority = 0;
   cudaGraphExec_t exec = nullptr;
   int g_iters = -1;
   bool g_ll = false;
@@ -184,7 +185,7 @@ gmmsp_status enqueue_part(gmmsp_batch b, int iters, bool want_ll, int c0, int c1
 // within each: while one part's finalize keeps the FP64 pipe busy (and little
 // else: issue slots 19 %, shared-memory pipe 21 %), the other's E + M pass,
 // bound by the shared-memory pipe, runs beside it, and neither pass ends with
-// a nearly empty machine.  The finalize goes first (launch priority), on 4
+// a nearly empty machine.  The finalize goes first (finalize_priority), on 4
 // warps per SM, one per FP64 unit's sub-partition: 16, as in a batch of one part,
 // push the E + M blocks out (256 uneven images 42.2 ms, 41.1 with 4, 41.3 with
 // 1; as one part 42.7).  Before / after, alone on the GPU, 10 iterations, us:
@@ -196,7 +197,7 @@ gmmsp_status enqueue_part(gmmsp_batch b, int iters, bool want_ll, int c0, int c1
 // one part.  The persistent E + M kernels (fewer than 6 blocks per SM) take the
 // whole batch.
 int split_image(gmmsp_batch b) {
-  if (!b->side || b->total_cells < 16 * b->sm_count || b->blocks_per_sm < 6 || first_bps(b) < 6) return 0;
+  if (!b->side || !gmmsp::two_parts(b->n, b->total_cells, b->sm_count, b->blocks_per_sm, first_bps(b))) return 0;
   int best = 1;
   auto off_half = [b](int i) { return llabs(2LL * b->host[i].cell_off - b->total_cells); };
   for (int i = 2; i < b->n; ++i)
@@ -216,11 +217,11 @@ gmmsp_status enqueue_batch(gmmsp_batch b, int iters, bool want_ll) {
     const int c1 = b->host[i1].cell_off, k1 = b->host[i1].k_off;
     GB_CHECK(b, cudaEventRecord(b->fork, s));
     GB_CHECK(b, cudaStreamWaitEvent(b->side, b->fork, 0));
-    st = enqueue_part(b, iters, want_ll, 0, c1, 0, k1, 4, b->high_priority, s);
+    st = enqueue_part(b, iters, want_ll, 0, c1, 0, k1, 4, b->fin_priority, s);
     // the side stream joins again whatever happened: the caller's stream then
     // orders all of the call's work
     const gmmsp_status st2 = st != GMMSP_OK ? st : enqueue_part(b, iters, want_ll, c1, b->total_cells, k1, b->total_k, 4,
-                                                                b->high_priority, b->side);
+                                                                b->fin_priority, b->side);
     GB_CHECK(b, cudaEventRecord(b->join, b->side));
     GB_CHECK(b, cudaStreamWaitEvent(s, b->join, 0));
     if (st2 != GMMSP_OK) return st2;
@@ -257,8 +258,8 @@ void drop_side(gmmsp_batch b) {
 // The second stream has the priority of the caller's; without it (the
 // creation fails) the batch runs as one part.
 void make_side(gmmsp_batch b) {
-  int least = 0, prio = 0;
-  bool ok = b->n > 1 && cudaDeviceGetStreamPriorityRange(&least, &b->high_priority) == cudaSuccess &&
+  int least = 0, most = 0, prio = 0;
+  bool ok = b->n > 1 && cudaDeviceGetStreamPriorityRange(&least, &most) == cudaSuccess &&
             cudaStreamGetPriority(b->stream, &prio) == cudaSuccess &&
             cudaStreamCreateWithPriority(&b->side, cudaStreamNonBlocking, prio) == cudaSuccess &&
             cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess &&
@@ -267,6 +268,7 @@ void make_side(gmmsp_batch b) {
     cudaGetLastError();
     drop_side(b);
   }
+  b->fin_priority = gmmsp::finalize_priority(prio, most);
 }
 
 void drop_graph(gmmsp_batch b) {
