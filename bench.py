@@ -87,16 +87,6 @@ MUFU_PEAK_TOPS = 152 * 32 * 2.070e9 / 1e12
 PARTIAL_BYTES_PER_CELL = 576
 
 
-def batch_parts(bt, n):
-    """Parts in which a batch context of n images launches its EM iterations and label pass: two, beside one
-    another, from 16 cells per SM on with the one-cell-per-warp launches (6 blocks per SM or more), else one."""
-    import torch
-    t = bt.tuning()
-    sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    return 2 if (n > 1 and bt.info()[2] >= 16 * sms and
-                 min(t["blocks_per_sm"], t["first_pass_blocks_per_sm"]) >= 6) else 1
-
-
 def side_rooflines(units, pixels, cells, em_ms, traffic):
     peaks = measured_peaks()
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
@@ -473,7 +463,7 @@ def run_other_workload(args):
                   "images": 256, "pixels": pix, "K": K, "cells": cells, "blocks_per_sm": bps,
                   "colour_model": args.colour,
                   "l2": "flushed between timed steps (256 MiB memset)"}
-        launches = 2 + (2 * ITERS + 1) * batch_parts(bt, 256)
+        launches = 2 + (2 * ITERS + 1) * bt.parts()
         extra = {"loglik_mean_per_pixel": float(np.sum(ll)) / pix, "em_pass_autotune_ms": tune}
         bt.close()
     else:
@@ -620,7 +610,7 @@ def run_learned(args):
         learned.set_init_net(net)
         tuning = {"plain": plain.tuning(), "learned": learned.tuning(),
                   "em_pass_ms_by_blocks_per_sm": {str(k): round(v_, 5) for k, v_ in tune.items()}}
-        learned_parts = batch_parts(learned, n)
+        learned_parts = learned.parts()
     step_l = lambda: learned.segment(imgs, LEARN_T)  # noqa: E731
     step_p = lambda: plain.segment(imgs, ITERS)  # noqa: E731
     with torch.cuda.stream(stream):

@@ -263,7 +263,10 @@ gmmsp_status gmmsp_autotune(gmmsp_ctx c, int reps, int *best, double *times_ms);
  *   (its covariance blocks are diagonal after either start, Sec. III-C or the
  *   learned one) gets a choice of its own: the diagonal kernels at 6 and 7
  *   are timed too, and the fastest of them and the 3-5 times is kept.
- *   Synchronises.
+ *   Where a segment can run as two parts (gmmsp_batch_parts), 2 reps EM
+ *   iterations are then timed as they run, with these choices and with the
+ *   fastest of 6 and 7, each with either finalize, and the fastest is kept.
+ *   Writes no labels.  Synchronises.
  * gmmsp_batch_set_launch: blocks per SM of the E + M pass (1..16; >= 6
  *   selects the one-cell-per-warp kernel); the first pass keeps its own
  *   choice where the autotuner or gmmsp_batch_set_first_pass made one.
@@ -314,6 +317,12 @@ gmmsp_status gmmsp_batch_get_tuning(gmmsp_batch b, int *blocks_per_sm, int *fina
  * pass follows blocks_per_sm again until gmmsp_batch_set_first_pass. */
 gmmsp_status gmmsp_batch_set_tuning(gmmsp_batch b, int blocks_per_sm, int finalize16);
 gmmsp_status gmmsp_batch_info(gmmsp_batch b, long long *total_pixels, int *total_k, int *total_cells);
+/* In how many parts (1, or 2 on two streams beside one another) b runs the EM
+ * iterations and label pass of a segment with its present launch choices: two
+ * for several images of 16 cells per SM or more with the one-cell-per-warp
+ * kernels.  Each part is 2 iterations + 1 launches.  The finalizes of two parts
+ * are launched one priority level above the caller's stream. */
+gmmsp_status gmmsp_batch_parts(gmmsp_batch b, int *parts);
 /* Copies image i's CIELAB colours (Sec. III-A, after the conversion of Sec.
  * IV) as the last gmmsp_batch_segment left them on the device to the host as
  * W H x (L, a, b) float32 (synchronises the batch's stream).

@@ -27,7 +27,7 @@ __all__ = [
     "gmmsp_profile_kernel", "gmmsp_probe_peaks", "gmmsp_probe_fp64_helpers", "gmmsp_set_timing", "gmmsp_get_timing", "gmmsp_set_launch", "gmmsp_get_launch",
     "gmmsp_autotune", "gmmsp_segment_lab_noalloc", "gmmsp_last_error", "SuperpixelsBatch", "gmmsp_bounds_status", "gmmsp_release_scratch",
     "gmmsp_batch_create", "gmmsp_batch_segment", "gmmsp_batch_get_params", "gmmsp_batch_autotune",
-    "gmmsp_batch_set_launch", "gmmsp_batch_set_tuning", "gmmsp_batch_info", "gmmsp_batch_destroy", "gmmsp_status_string", "gmmsp_destroy",
+    "gmmsp_batch_set_launch", "gmmsp_batch_set_tuning", "gmmsp_batch_info", "gmmsp_batch_parts", "gmmsp_batch_destroy", "gmmsp_status_string", "gmmsp_destroy",
     "gmmsp_batch_get_tuning", "gmmsp_batch_set_first_pass", "gmmsp_batch_get_first_pass",
     "gmmsp_batch_first_pass_partials", "gmmsp_batch_set_init_net", "gmmsp_batch_lab", "gmmsp_batch_targets", "gmmsp_batch_get_lab",
     "gmmsp_net_param_count", "gmmsp_net_create", "gmmsp_net_set_weights", "gmmsp_net_get_weights",
@@ -377,6 +377,7 @@ def _batch_lib():
             "gmmsp_batch_set_launch": (I, [P, I]),
             "gmmsp_batch_set_tuning": (I, [P, I, I]),
             "gmmsp_batch_info": (I, [P, ctypes.POINTER(ctypes.c_longlong), pint, pint]),
+            "gmmsp_batch_parts": (I, [P, pint]),
             "gmmsp_batch_get_lab": (I, [P, I, P]),
             "gmmsp_batch_get_tuning": (I, [P, pint, pint, P]),
             "gmmsp_batch_set_first_pass": (I, [P, I]),
@@ -473,6 +474,12 @@ def gmmsp_batch_info(b):
     pix, K, cells = ctypes.c_longlong(), ctypes.c_int(), ctypes.c_int()
     _bcheck(b, _batch_lib().gmmsp_batch_info(b, ctypes.byref(pix), ctypes.byref(K), ctypes.byref(cells)))
     return pix.value, K.value, cells.value
+
+
+def gmmsp_batch_parts(b) -> int:
+    parts = ctypes.c_int()
+    _bcheck(b, _batch_lib().gmmsp_batch_parts(b, ctypes.byref(parts)))
+    return parts.value
 
 
 def gmmsp_batch_get_lab(b, i, H, W):
@@ -867,6 +874,10 @@ class SuperpixelsBatch:
 
     def info(self):
         return gmmsp_batch_info(self.b)
+
+    def parts(self) -> int:
+        """Parts (1 or 2) in which a segment's EM iterations and label pass run."""
+        return gmmsp_batch_parts(self.b)
 
     def tuning(self):
         return gmmsp_batch_get_tuning(self.b)

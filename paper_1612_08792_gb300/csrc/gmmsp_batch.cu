@@ -159,11 +159,12 @@ gmmsp_status enqueue_start(gmmsp_batch b) {
   return GMMSP_OK;
 }
 
-// The EM iterations and the label pass of the cells [c0, c1) and superpixels
-// [k0, k1) of the batch (whole images) on stream s; fin_bps and priority: the
-// finalize launches' blocks (one warp each) per SM and launch priority.
-gmmsp_status enqueue_part(gmmsp_batch b, int iters, bool want_ll, int c0, int c1, int k0, int k1, int fin_bps,
-                          int priority, cudaStream_t s) {
+// The EM iterations and, unless `steps_only`, the label pass of the cells
+// [c0, c1) and superpixels [k0, k1) of the batch (whole images) on stream s;
+// fin_bps and priority: the finalize launches' blocks (one warp each) per SM
+// and launch priority.
+gmmsp_status enqueue_part(gmmsp_batch b, int iters, bool want_ll, bool steps_only, int c0, int c1, int k0, int k1,
+                          int fin_bps, int priority, cudaStream_t s) {
   const int n = b->n;
   const int fblocks = int(std::min<long long>((k1 - k0 + 31) / 32, (long long)b->sm_count * fin_bps));
   for (int t = 0; t < iters; ++t) {
@@ -176,6 +177,7 @@ gmmsp_status enqueue_part(gmmsp_batch b, int iters, bool want_ll, int c0, int c1
                                              b->p.eps_c, b->counters, b->p.precision, use_fin16(b) ? 0 : fblocks,
                                              priority, s));
   }
+  if (steps_only) return GMMSP_OK;
   GB_CHECK(b, gmmsp::launch_label_pass_batch(b->table, n, c0, c1, b->lab, b->gp, want_ll ? b->cell_ll : nullptr,
                                              b->p.colour_model, s));
   return GMMSP_OK;
@@ -205,28 +207,29 @@ int split_image(gmmsp_batch b) {
   return best;
 }
 
-gmmsp_status enqueue_batch(gmmsp_batch b, int iters, bool want_ll) {
+// The EM iterations of the whole batch, in one part or two, and the label pass.
+gmmsp_status enqueue_parts(gmmsp_batch b, int iters, bool want_ll, bool steps_only) {
   cudaStream_t s = b->stream;
-  gmmsp_status st = enqueue_start(b);
-  if (st != GMMSP_OK) return st;
   const int i1 = iters > 0 ? split_image(b) : 0;
-  if (i1 == 0) {
-    st = enqueue_part(b, iters, want_ll, 0, b->total_cells, 0, b->total_k, 16, 0, s);
-    if (st != GMMSP_OK) return st;
-  } else {
-    const int c1 = b->host[i1].cell_off, k1 = b->host[i1].k_off;
-    GB_CHECK(b, cudaEventRecord(b->fork, s));
-    GB_CHECK(b, cudaStreamWaitEvent(b->side, b->fork, 0));
-    st = enqueue_part(b, iters, want_ll, 0, c1, 0, k1, 4, b->fin_priority, s);
-    // the side stream joins again whatever happened: the caller's stream then
-    // orders all of the call's work
-    const gmmsp_status st2 = st != GMMSP_OK ? st : enqueue_part(b, iters, want_ll, c1, b->total_cells, k1, b->total_k, 4,
-                                                                b->fin_priority, b->side);
-    GB_CHECK(b, cudaEventRecord(b->join, b->side));
-    GB_CHECK(b, cudaStreamWaitEvent(s, b->join, 0));
-    if (st2 != GMMSP_OK) return st2;
-  }
-  if (want_ll) GB_CHECK(b, gmmsp::launch_ll_per_image(b->table, b->n, b->cell_ll, b->img_ll, s));
+  if (i1 == 0) return enqueue_part(b, iters, want_ll, steps_only, 0, b->total_cells, 0, b->total_k, 16, 0, s);
+  const int c1 = b->host[i1].cell_off, k1 = b->host[i1].k_off;
+  GB_CHECK(b, cudaEventRecord(b->fork, s));
+  GB_CHECK(b, cudaStreamWaitEvent(b->side, b->fork, 0));
+  gmmsp_status st = enqueue_part(b, iters, want_ll, steps_only, 0, c1, 0, k1, 4, b->fin_priority, s);
+  if (st == GMMSP_OK)
+    st = enqueue_part(b, iters, want_ll, steps_only, c1, b->total_cells, k1, b->total_k, 4, b->fin_priority, b->side);
+  // the side stream joins again whatever happened: the caller's stream then
+  // orders all of the call's work
+  GB_CHECK(b, cudaEventRecord(b->join, b->side));
+  GB_CHECK(b, cudaStreamWaitEvent(s, b->join, 0));
+  return st;
+}
+
+gmmsp_status enqueue_batch(gmmsp_batch b, int iters, bool want_ll) {
+  gmmsp_status st = enqueue_start(b);
+  if (st == GMMSP_OK) st = enqueue_parts(b, iters, want_ll, false);
+  if (st != GMMSP_OK) return st;
+  if (want_ll) GB_CHECK(b, gmmsp::launch_ll_per_image(b->table, b->n, b->cell_ll, b->img_ll, b->stream));
   return GMMSP_OK;
 }
 
@@ -269,6 +272,28 @@ void make_side(gmmsp_batch b) {
     drop_side(b);
   }
   b->fin_priority = gmmsp::finalize_priority(prio, most);
+}
+
+// What `enqueue` launches on the batch's stream (not the default one) as a graph.
+template <class F>
+gmmsp_status capture(gmmsp_batch b, F enqueue, cudaGraphExec_t* exec) {
+  *exec = nullptr;
+  GB_CHECK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+  const gmmsp_status st = enqueue();
+  cudaGraph_t graph = nullptr;
+  cudaError_t e = cudaStreamEndCapture(b->stream, &graph);
+  if (st != GMMSP_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    return st;
+  }
+  if (e != cudaSuccess) return bfail(b, GMMSP_E_CUDA, cudaGetErrorString(e));
+  e = cudaGraphInstantiate(exec, graph, cudaGraphInstantiateFlagUseNodePriority);
+  cudaGraphDestroy(graph);
+  if (e != cudaSuccess) {
+    *exec = nullptr;
+    return bfail(b, GMMSP_E_CUDA, cudaGetErrorString(e));
+  }
+  return GMMSP_OK;
 }
 
 void drop_graph(gmmsp_batch b) {
@@ -391,6 +416,12 @@ gmmsp_status gmmsp_batch_get_tuning(gmmsp_batch b, int* blocks_per_sm, int* fina
   return GMMSP_OK;
 }
 
+gmmsp_status gmmsp_batch_parts(gmmsp_batch b, int* parts) {
+  if (!b || !parts) return GMMSP_E_INVALID;
+  *parts = split_image(b) ? 2 : 1;
+  return GMMSP_OK;
+}
+
 gmmsp_status gmmsp_batch_info(gmmsp_batch b, long long* total_pixels, int* total_k, int* total_cells) {
   if (!b) return GMMSP_E_INVALID;
   if (total_pixels) *total_pixels = b->total_pix;
@@ -417,21 +448,8 @@ gmmsp_status gmmsp_batch_segment(gmmsp_batch b, const void* const* images_dev, c
     if (!(b->exec && b->g_iters == iters && b->g_ll == want_ll && b->g_bps == b->blocks_per_sm &&
           b->g_fbps == first_bps(b) && b->g_net == b->net && b->g_gen == gen)) {
       drop_graph(b);
-      GB_CHECK(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-      st = enqueue_batch(b, iters, want_ll);
-      cudaGraph_t graph = nullptr;
-      cudaError_t e = cudaStreamEndCapture(b->stream, &graph);
-      if (st != GMMSP_OK) {
-        if (graph) cudaGraphDestroy(graph);
-        return st;
-      }
-      if (e != cudaSuccess) return bfail(b, GMMSP_E_CUDA, cudaGetErrorString(e));
-      e = cudaGraphInstantiate(&b->exec, graph, cudaGraphInstantiateFlagUseNodePriority);
-      cudaGraphDestroy(graph);
-      if (e != cudaSuccess) {
-        b->exec = nullptr;
-        return bfail(b, GMMSP_E_CUDA, cudaGetErrorString(e));
-      }
+      st = capture(b, [&] { return enqueue_batch(b, iters, want_ll); }, &b->exec);
+      if (st != GMMSP_OK) return st;
       b->g_iters = iters;
       b->g_ll = want_ll;
       b->g_bps = b->blocks_per_sm;
@@ -584,13 +602,14 @@ gmmsp_status gmmsp_batch_autotune(gmmsp_batch b, const void* const* images_dev, 
     *per = double(ms) / reps;
     return GMMSP_OK;
   };
-  double best_ms = 1e30, first_best = 1e30;
+  double best_ms = 1e30, first_best = 1e30, flat_ms[2] = {0.0, 0.0};
   int best_c = b->blocks_per_sm, first_c = 0;
   for (int i = 0; i < 5; ++i) {
     double per = 0.0;
     st = time_pass(cand[i], false, &per);
     if (st != GMMSP_OK) return st;
     if (times_ms) times_ms[i] = per;
+    if (cand[i] >= 6) flat_ms[cand[i] - 6] = per;
     if (per < best_ms) { best_ms = per; best_c = cand[i]; }
     if (cand[i] < 6 && per < first_best) { first_best = per; first_c = cand[i]; }  // no diagonal variant
   }
@@ -626,6 +645,57 @@ gmmsp_status gmmsp_batch_autotune(gmmsp_batch b, const void* const* images_dev, 
     b->fin16 = fin_ms[0] <= fin_ms[1];
     b->fin_ms[0] = fin_ms[0];
     b->fin_ms[1] = fin_ms[1];
+    GB_CHECK(b, cudaMemsetAsync(b->counters, 0, sizeof(unsigned long long) * gmmsp::CNT_N, b->stream));
+  }
+  // A kernel alone on the machine says little about one beside the other part's:
+  // where the batch can run as two parts, the iterations are timed as they run,
+  // with the choices above and with the fastest one-cell-per-warp kernels, each
+  // with either finalize.  10 images of 481x321: 5 blocks per SM are the fastest
+  // alone, and a segment then takes 571 us as one part, 517 as two at 6; 8
+  // images: 16 lanes take 20.7 us alone against 19.3, and a segment 529 us
+  // against 556; 16 images: 893 against 862.
+  const int flat_c = flat_ms[0] <= flat_ms[1] ? 6 : 7, flat_first = b->first_ms[0] <= b->first_ms[1] ? 6 : 7;
+  if (b->side && gmmsp::two_parts(b->n, b->total_cells, b->sm_count, flat_c, flat_first)) {
+    const bool both_fin = b->p.precision != GMMSP_PREC_FP32 && b->p.colour_model == GMMSP_COLOUR_FULL;
+    const int as_run[2][2] = {{best_c, first_c}, {flat_c, flat_first}};
+    const bool same = best_c == flat_c && first_c == flat_first;
+    const bool fin16 = b->fin16;
+    double run_best = 1e30;
+    int run_c = 0;
+    for (int c = 0; c < 4; ++c) {
+      if ((same && (c & 1)) || (!both_fin && c >= 2)) continue;
+      b->blocks_per_sm = as_run[c & 1][0];
+      b->first_bps = as_run[c & 1][1];
+      b->fin16 = both_fin ? c >= 2 : fin16;
+      const auto steps = [&]() -> gmmsp_status {  // from theta_0, as a segment: a finalize's time depends on theta
+        GB_CHECK(b, gmmsp::launch_init_batch(b->table, b->n, b->total_k, b->lab, b->p.lambda_c, b->theta, b->gp, kblocks,
+                                             b->stream));
+        return enqueue_parts(b, 2 * reps, false, true);
+      };
+      cudaGraphExec_t exec = nullptr;
+      if (b->stream && (st = capture(b, steps, &exec)) != GMMSP_OK) return st;
+      float ms = 1e30f;
+      for (int r = 0; r < 3 && st == GMMSP_OK; ++r) {  // the first run is a warm-up
+        cudaError_t e = cudaEventRecord(e0, b->stream);
+        if (!exec) st = steps();
+        else if (e == cudaSuccess) e = cudaGraphLaunch(exec, b->stream);
+        float one = 0.f;
+        if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&one, e0, e1);
+        if (e != cudaSuccess && st == GMMSP_OK) st = bfail(b, GMMSP_E_CUDA, cudaGetErrorString(e));
+        if (r > 0) ms = std::min(ms, one);
+      }
+      if (exec) cudaGraphExecDestroy(exec);
+      if (st != GMMSP_OK) return st;
+      if (ms < run_best) {
+        run_best = ms;
+        run_c = c;
+      }
+    }
+    best_c = b->blocks_per_sm = as_run[run_c & 1][0];
+    b->first_bps = as_run[run_c & 1][1];
+    b->fin16 = both_fin ? run_c >= 2 : fin16;
     GB_CHECK(b, cudaMemsetAsync(b->counters, 0, sizeof(unsigned long long) * gmmsp::CNT_N, b->stream));
   }
   cudaEventDestroy(e0);

@@ -1,0 +1,66 @@
+"""The autotuner of a batch that can run as two parts: it keeps launch choices that make such a segment fast (a
+kernel alone on the machine says little about one beside the other part's), leaves the labels it is given alone,
+and gmmsp_batch_parts tells in how many parts a segment runs."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def batch(n):
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1612_08792_gb300 as gm
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    x = torch.randint(0, 256, (n, 321, 481, 3), generator=g, device="cuda", dtype=torch.uint8)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        bt = gm.SuperpixelsBatch([(321, 481)] * n, spacing=15, stream=stream)
+    return torch, gm, x, stream, bt
+
+
+def segment_ms(torch, bt, x, stream, finalize16, gm, bps, first):
+    gm.gmmsp_batch_set_tuning(bt.b, bps, finalize16)
+    bt.set_launch(bps, first)
+    best = 1e30
+    with torch.cuda.stream(stream):
+        bt.segment_stacked(x, 10)
+        for _ in range(8):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(5):
+                bt.segment_stacked(x, 10)
+            e1.record()
+            e1.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+    return best
+
+
+@pytest.mark.parametrize("n", [8, 10, 16, 32])
+def test_keeps_choices_that_are_fast_as_they_run(n):
+    torch, gm, x, stream, bt = batch(n)
+    with torch.cuda.stream(stream):
+        bt.labels_buffer.fill_(-7)
+        best, times = bt.autotune(list(x), reps=5)
+        assert bool((bt.labels_buffer == -7).all())
+    t = bt.tuning()
+    assert best == t["blocks_per_sm"] and sorted(times) == [3, 4, 5, 6, 7]
+    got = segment_ms(torch, bt, x, stream, t["finalize16"], gm, best, t["first_pass_blocks_per_sm"])
+    others = {(b, f): segment_ms(torch, bt, x, stream, f, gm, b, 6) for b in (5, 6) for f in (False, True)}
+    assert got <= 1.03 * min(others.values()), (t, got, others)  # 3 %: timing noise between equally good choices
+    bt.close()
+
+
+def test_parts():
+    torch, gm, x, stream, bt = batch(8)
+    assert bt.parts() == 2
+    bt.set_launch(5, 0)
+    assert bt.parts() == 1
+    bt.set_launch(7, 6)
+    assert bt.parts() == 2
+    bt.close()
+    one = gm.SuperpixelsBatch([(2000, 3000)], spacing=15)
+    assert one.parts() == 1
+    one.close()
