@@ -1,11 +1,14 @@
 // Host check of the 3 x 3 layers' index arithmetic (gmmsp_grid3.cuh) against
 // 64-bit divisions:
-//  * small grids of every kind: every cell is the output of exactly one
-//    position of one tile, and every tile's inputs are the right cells;
+//  * small grids of every kind, few and many images (stacked or not): every
+//    cell is the output of exactly one position of one tile, and every tile's
+//    inputs are the right cells;
 //  * every bordered row length at the most rows a network call accepts
 //    (2^30 cells, image sides below 2^31 at a spacing of 3): tiles at the ends,
 //    around the rows where the multiplication in place of the division starts
-//    to fail, and at random.
+//    to fail, and at random;
+//  * as many images of small grids as a call accepts;
+//  * many images of any grid take few more tiles than their positions fill.
 // Prints "ok <counts>" and exits 0, or prints the first mismatch and exits 1.
 #include <stdio.h>
 #include <stdlib.h>
@@ -26,20 +29,21 @@ static uint64_t next_u64() {  // splitmix64
   return z ^ (z >> 31);
 }
 
-// Row of number q of strip s of image img, -1 off the cells.  `halo`: the
-// neighbouring strips' columns count too.
-static ll want_row(const Grid3& g, ll img, int strip, ll q, bool halo) {
-  const ll y = q >= 0 ? q / g.PW : -((-q + g.PW - 1) / g.PW), x = q - y * g.PW;
+// Row of number q of strip `strip` of the stack that begins with image `first`,
+// -1 off the cells.  `halo`: the neighbouring strips' columns count too.
+static ll want_row(const Grid3& g, ll first, int strip, ll q, bool halo) {
+  const ll Y = q >= 0 ? q / g.PW : -((-q + g.PW - 1) / g.PW), x = q - Y * g.PW;
   const ll col = (ll)strip * g.TW + x - 1;
-  if (y < 0 || y >= g.H || col < 0 || col >= g.W) return -1;
-  if (!halo && (x < 1 || x > g.TW)) return -1;
-  return (img * g.H + y) * g.W + col;
+  if (Y < 0 || col < 0 || col >= g.W || (!halo && (x < 1 || x > g.TW))) return -1;
+  const ll i = g.per > 1 ? Y / (g.H + 1) : 0, y = Y - i * (g.H + 1);
+  if (y >= g.H || i >= g.per || first + i >= g.B) return -1;
+  return ((first + i) * g.H + y) * g.W + col;
 }
 
 static ll checked = 0;
 static bool check_tile(const Grid3& g, ll tile, std::vector<int>* seen) {
   const Tile3 t = tile3_at(g, int(tile));
-  const ll s = tile / g.tps, img = s / g.strips, q0 = (tile - s * g.tps) * 128;
+  const ll s = tile / g.tps, img = s / g.strips * g.per, q0 = (tile - s * g.tps) * 128;
   const int strip = int(s % g.strips);
   for (int p = 0; p < 128; ++p) {
     const ll r = row3(g, t, p), w = want_row(g, img, strip, q0 + p, false);
@@ -85,10 +89,14 @@ static bool check_all(int B, int H, int W) {
 }
 
 int main() {
+  ll stacked = 0;
   for (int W = 1; W <= 400; W += W < 12 ? 1 : (W < 120 ? 19 : (W < 131 ? 1 : 31)))
     for (int H : {1, 2, 3, 5, 8, 21, 64, 131})
-      for (int B : {1, 2, 3, 7})
+      for (int B : {1, 2, 3, 7, 61, 1500}) {
+        if ((ll)B * H * W > 300000) continue;
         if (!check_all(B, H, W)) return 1;
+        stacked += grid3_of(B, H, W).per > 1;
+      }
   const ll small = checked;
   for (int W = 1; W <= 300; ++W) {
     const int H = int(std::min<ll>((1ll << 30) / W, 715827882ll));
@@ -109,6 +117,25 @@ int main() {
         for (int s = 0; s < g.strips; ++s)
           if (!check_tile(g, s * n + i, nullptr)) return 1;
   }
-  printf("ok small %lld tall %lld\n", small, checked - small);
+  const ll tall = checked - small;
+  for (int H : {1, 2, 3, 5, 8, 13})
+    for (int W : {1, 2, 3, 5, 8, 14, 64, 126, 127, 260}) {
+      const Grid3 g = grid3_of(int((1ll << 30) / ((ll)H * W)), H, W);
+      for (ll c : {(ll)0, (ll)g.tps, (ll)g.tiles / 2, (ll)g.tiles - 1})
+        for (ll d = -40; d <= 40; ++d)
+          if (c + d >= 0 && c + d < g.tiles && !check_tile(g, c + d, nullptr)) return 1;
+      for (int i = 0; i < 300; ++i)
+        if (!check_tile(g, ll(next_u64() % uint64_t(g.tiles)), nullptr)) return 1;
+    }
+  for (int H = 1; H <= 40; ++H)
+    for (int W = 1; W <= 140; ++W) {
+      const Grid3 g = grid3_of(4096, H, W);
+      const ll full = (4096ll * (H + 1) * g.PW + 127) / 128 * g.strips;
+      if (7LL * g.tiles > 8 * (full + 2 * g.strips * g.stacks) && 8LL * full <= 7LL * g.tiles) {
+        printf("H %d W %d: %d tiles for %lld tiles' positions\n", H, W, g.tiles, full);
+        return 1;
+      }
+    }
+  printf("ok small %lld (%lld grids stacked) tall %lld many %lld\n", small, stacked, tall, checked - small - tall);
   return 0;
 }
