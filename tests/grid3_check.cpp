@@ -131,7 +131,7 @@ int main() {
     for (int W = 1; W <= 140; ++W) {
       const Grid3 g = grid3_of(4096, H, W);
       const ll full = (4096ll * (H + 1) * g.PW + 127) / 128 * g.strips;
-      if (7LL * g.tiles > 8 * (full + 2 * g.strips * g.stacks) && 8LL * full <= 7LL * g.tiles) {
+      if (7LL * g.tiles > 8 * (full + 4LL * g.strips * (full / 1024 + 1))) {  // an eighth, and a partly empty tile per stack
         printf("H %d W %d: %d tiles for %lld tiles' positions\n", H, W, g.tiles, full);
         return 1;
       }
