@@ -404,12 +404,7 @@ __global__ void __launch_bounds__(kEmWarps * 32) k_em_pass(Src lab, Geom g, cons
   em_pass_body<PT, SHIFT, WPC, Src, CM, DIAG>(lab, g, gp, partials);
 }
 
-// The same, registers capped for MINB blocks per SM, in the full colour model
-// (the split and grayscale kernels are faster uncapped).  One warp per cell: 6
-// (3840x2160, v = 20: 189 us, 203 us at 7).  Four warps per cell: 7, which
-// puts the 1107 cells of a 481x321 image at v = 12 into little more than one
-// wave of 1064 blocks (10 iterations and labels 162 us, 175 uncapped at 5
-// blocks, 166 at 8).  Two warps per cell run uncapped.
+// The same, registers capped for MINB blocks per SM (em_pass_impl chooses).
 template <typename PT, bool SHIFT, int WPC, class Src, int CM, bool DIAG, int MINB>
 __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_capped(Src lab, Geom g, const float* __restrict__ gp,
                                                                         PT* __restrict__ partials) {
@@ -481,17 +476,16 @@ __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_batch_flat(cons
 // Grayscale: one pixel per lane, whose kernel then fits 8 blocks on an SM
 // (64 images of 640x480: conversion, start and labels 0.208 ms against 0.218;
 // the split model is slower that way, 0.247 against 0.236 on 96 of 481x321,
-// the full model the same).
+// the full model the same), but not for one image (launch_label_pass).
 template <int CM>
 constexpr int kLabelPixels = CM == kColourGray ? 1 : 2;
 
 // LL = false: argmax only (no log-sum-exp), for callers that want no
 // log-likelihood.
-template <bool FULL, bool LL, class Src, int CM>
+template <bool FULL, bool LL, class Src, int CM, int kLabelPPL>
 __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
                                                   const Cell& c, const float4* sp, int lane,
                                                   int32_t* __restrict__ labels, float& ll) {
-  constexpr int kLabelPPL = kLabelPixels<CM>;
   const int npx_all = c.cw * c.ch;
   auto locate = [&](int p, int& rx, int& ry) {
     ry = __float2int_rz((float(p) + 0.5f) * (1.f / float(c.cw)));  // exact floor(p / cw)
@@ -608,7 +602,7 @@ __device__ __forceinline__ void label_cell_pixels(const Src& lab, const Geom& g,
 }
 
 // One cell of the label pass, run by one warp.
-template <class Src, int CM>
+template <class Src, int CM, int PPL>
 __device__ __forceinline__ void label_cell_warp(const Src& lab, const Geom& g, const float* __restrict__ gp,
                                                 int32_t* __restrict__ labels, double* __restrict__ cell_ll,
                                                 int cell, float4* sp, int lane) {
@@ -617,22 +611,22 @@ __device__ __forceinline__ void label_cell_warp(const Src& lab, const Geom& g, c
   float ll = 0.f;
   if (!cell_ll) {  // labels only
     if (c.mask == 0x1ffu)
-      label_cell_pixels<true, false, Src, CM>(lab, g, c, sp, lane, labels, ll);
+      label_cell_pixels<true, false, Src, CM, PPL>(lab, g, c, sp, lane, labels, ll);
     else
-      label_cell_pixels<false, false, Src, CM>(lab, g, c, sp, lane, labels, ll);
+      label_cell_pixels<false, false, Src, CM, PPL>(lab, g, c, sp, lane, labels, ll);
     return;
   }
   if (c.mask == 0x1ffu)
-    label_cell_pixels<true, true, Src, CM>(lab, g, c, sp, lane, labels, ll);
+    label_cell_pixels<true, true, Src, CM, PPL>(lab, g, c, sp, lane, labels, ll);
   else
-    label_cell_pixels<false, true, Src, CM>(lab, g, c, sp, lane, labels, ll);
+    label_cell_pixels<false, true, Src, CM, PPL>(lab, g, c, sp, lane, labels, ll);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
   if (lane == 0 && GMMSP_IN_BOUNDS(cell, g.ncells, BND_CELL_LL)) cell_ll[cell] = double(ll) * 0.69314718055994530942;
 }
 
-template <class Src, int CM>
-__global__ void __launch_bounds__(kEmWarps * 32) k_label_pass(Src lab, Geom g, const float* __restrict__ gp,
+template <class Src, int CM, int PPL = kLabelPixels<CM>, int MINB = CM != kColourGray ? 5 : (PPL == 1 ? 10 : 8)>
+__global__ void __launch_bounds__(kEmWarps * 32, MINB) k_label_pass(Src lab, Geom g, const float* __restrict__ gp,
                                                               int32_t* __restrict__ labels,
                                                               double* __restrict__ cell_ll) {
   __shared__ float4 sp_all[kEmWarps][kSlots * 4];
@@ -641,7 +635,7 @@ __global__ void __launch_bounds__(kEmWarps * 32) k_label_pass(Src lab, Geom g, c
   pdl_wait();
   pdl_trigger();
   if (cell >= g.ncells) return;
-  label_cell_warp<Src, CM>(lab, g, gp, labels, cell_ll, cell, sp_all[warp], lane);
+  label_cell_warp<Src, CM, PPL>(lab, g, gp, labels, cell_ll, cell, sp_all[warp], lane);
 }
 
 // One cell per warp over a grid sized to the work (a persistent loop over the
@@ -661,7 +655,7 @@ __global__ void __launch_bounds__(kEmWarps * 32, CM == kColourGray ? 8 : 5) k_la
   const BatchImage& im = imgs[ii];
   if (!GMMSP_IN_BOUNDS(cell - im.cell_off, im.g.ncells, BND_ITEM)) return;
   const LabPlanar src{lab + 3 * im.pix_off, (long long)im.g.W * im.g.H, im.g.W};
-  label_cell_warp<LabPlanar, CM>(src, im.g, gp + (long long)im.k_off * kGP, im.labels,
+  label_cell_warp<LabPlanar, CM, kLabelPixels<CM>>(src, im.g, gp + (long long)im.k_off * kGP, im.labels,
                                  cell_ll ? cell_ll + im.cell_off : nullptr, cell - im.cell_off, sp_all[warp], lane);
 }
 
@@ -1187,15 +1181,40 @@ size_t finalize_workspace_doubles(const Geom& g) {
   return (b16 > size_t(ll_blocks(g)) ? b16 : size_t(ll_blocks(g))) + 1;
 }
 
+constexpr int kSms = 152;
+// Rounds of resident blocks that a launch takes at per_sm blocks per SM.
+static int rounds(int blocks, int per_sm) { return (blocks + per_sm * kSms - 1) / (per_sm * kSms); }
+
 template <typename PT, bool SHIFT, int WPC, class Src, int CM, bool DIAG>
 static cudaError_t em_pass_impl(Src lab, const Geom& g, const float* gp, PT* partials,
                                 cudaStream_t s) {
   constexpr int smem = em_smem_bytes<WPC>();
   static_assert(smem <= 227 * 1024, "shared memory");
-  const auto kernel = [] {
-    if constexpr (WPC == 1 && CM == kColourFull) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 6>;
-    else if constexpr (WPC == 4 && CM == kColourFull) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 7>;
-    else return k_em_pass<PT, SHIFT, WPC, Src, CM, DIAG>;
+  constexpr int cpb = kEmWarps / WPC;
+  const int blocks = (g.ncells + cpb - 1) / cpb;
+  // The register bound, by how many rounds of resident blocks the launch takes.
+  // A bound costs spills or longer code and gains only where a tighter one saves
+  // a round or, with many, hides more latency.  10 iterations and labels, us,
+  // the bound taken and the other one:
+  //  full model, up to 5 blocks per SM: none (5 where that is needed to fit 5).
+  //    320x240 v = 20 (192 blocks of four warps per cell) 144, 154 at 7; 481x321
+  //    v = 30 191, 209; 1000x560 v = 14 (one warp) 298, 306 at 6
+  //  four warps, more blocks: 7.  481x321 v = 12 (1107 blocks) 164, 184 without
+  //  one warp, 6 to 7 blocks per SM: 7, one round.  800x600 v = 11 312, 317 at 6;
+  //    otherwise 6: an E+M pass at 3840x2160, v = 20 takes 189, 203 at 7
+  //  split model (86 registers) and the FP32 variant's two warps (87): 6 where
+  //    that saves a round.  1280x720 v = 16 402, 436 without; 1920x1080 v = 40
+  //    704 without, 748 at 6; grayscale: none (63 registers)
+  const auto kernel = [blocks] {
+    constexpr auto uncapped = k_em_pass<PT, SHIFT, WPC, Src, CM, DIAG>;
+    if constexpr (CM == kColourFull && WPC != 2) {
+      if (blocks <= 5 * kSms) return WPC == 1 && SHIFT ? k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 5> : uncapped;
+      if (WPC == 4 || (blocks > 6 * kSms && blocks <= 7 * kSms)) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 7>;
+      if constexpr (WPC == 1) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 6>;
+    } else if constexpr (CM == kColourSplit || (CM == kColourFull && !SHIFT)) {
+      if (rounds(blocks, 6) < rounds(blocks, 5)) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 6>;
+    }
+    return uncapped;
   }();
   static bool attr_set = false;  // per process; the attribute is per function
   if (!attr_set && smem > 48 * 1024) {
@@ -1203,8 +1222,6 @@ static cudaError_t em_pass_impl(Src lab, const Geom& g, const float* gp, PT* par
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  constexpr int cpb = kEmWarps / WPC;
-  const int blocks = (g.ncells + cpb - 1) / cpb;
   return launch_pdl(kernel, dim3(blocks), dim3(kEmWarps * 32), smem, s, lab, g, gp, partials);
 }
 
@@ -1239,18 +1256,26 @@ cudaError_t launch_em_pass(Src lab, const Geom& g, const float* gp, void* partia
 template <class Src>
 cudaError_t launch_label_pass(Src lab, const Geom& g, const float* gp, int32_t* labels,
                               double* cell_ll, cudaStream_t s) {
+  // One round of resident blocks gains nothing from more of them, and one that
+  // the ordinary bound just misses does.  Label pass alone, us, these / the
+  // ordinary variant: grayscale up to 8 blocks per SM with two pixels per lane,
+  // 481x321 v = 15 6.4 / 8.3; split model at 6 blocks, 1280x720 v = 16 12.5 /
+  // 14.3; caller's rows at 7 with one pixel, 800x600 v = 11 (10 iterations and
+  // labels) 291 / 302.
   const int blocks = (g.ncells + kEmWarps - 1) / kEmWarps;
+  auto kernel = k_label_pass<Src, kColourFull>;
   if constexpr (std::is_same<Src, LabPlanar>::value) {
     if (g.cm == kColourSplit)
-      return launch_pdl(k_label_pass<Src, kColourSplit>, dim3(blocks), dim3(kEmWarps * 32), 0, s, lab, g, gp,
-                        labels, cell_ll);
-    if (g.cm == kColourGray)
-      return launch_pdl(k_label_pass<Src, kColourGray>, dim3(blocks), dim3(kEmWarps * 32), 0, s, lab, g, gp,
-                        labels, cell_ll);
+      kernel = blocks > 5 * kSms && blocks <= 6 * kSms ? k_label_pass<Src, kColourSplit, 2, 6> : k_label_pass<Src, kColourSplit>;
+    else if (g.cm == kColourGray)
+      kernel = blocks <= 8 * kSms ? k_label_pass<Src, kColourGray, 2> : k_label_pass<Src, kColourGray>;
+    else if (g.cm != kColourFull)
+      return cudaErrorInvalidValue;
+  } else {
+    if (g.cm != kColourFull) return cudaErrorInvalidValue;
+    if (blocks > 5 * kSms) kernel = k_label_pass<Src, kColourFull, 1, 7>;
   }
-  if (g.cm != kColourFull) return cudaErrorInvalidValue;
-  return launch_pdl(k_label_pass<Src, kColourFull>, dim3(blocks), dim3(kEmWarps * 32), 0, s, lab, g, gp, labels,
-                    cell_ll);
+  return launch_pdl(kernel, dim3(blocks), dim3(kEmWarps * 32), 0, s, lab, g, gp, labels, cell_ll);
 }
 
 template cudaError_t launch_em_pass<LabPlanar>(LabPlanar, const Geom&, const float*, void*, int, int,
