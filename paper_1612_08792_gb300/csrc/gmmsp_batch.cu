@@ -34,10 +34,7 @@ struct gmmsp_batch_s {
   gmmsp_params p{};
   cudaStream_t stream = nullptr;
   int sm_count = 152;
-  // E + M pass (autotuned).  Untuned: one cell per warp at 6 blocks per SM, the fastest choice on every batch
-  // measured (256 images of 481x321: 0.895 ms against 1.007 at 4 persistent blocks; 64 grey 640x480: 0.328
-  // against 0.366; uneven sizes at v = 12: 0.826 against 0.952).
-  int blocks_per_sm = 6;
+  int blocks_per_sm = 6;           // E + M pass (default_blocks, then autotuned)
   int first_bps = 0;               // the first E + M pass (diagonal blocks); 0: as blocks_per_sm
   double first_ms[2] = {0.0, 0.0}; // autotuned first-pass times at 6 and 7 blocks per SM
   bool fin16 = false;              // finalize with 16 lanes per superpixel (autotuned)
@@ -400,6 +397,7 @@ gmmsp_status gmmsp_batch_create(gmmsp_batch* out, int n, const int* widths, cons
       return GMMSP_E_CUDA;
     }
   }
+  b->blocks_per_sm = gmmsp::default_blocks(n, cells, b->sm_count, p->colour_model == GMMSP_COLOUR_GRAY);
   make_side(b);
   *out = b;
   return GMMSP_OK;

@@ -19,4 +19,18 @@ inline bool two_parts(int n, long long cells, int sms, int bps, int first_bps) {
   return n > 1 && cells >= 16LL * sms && bps >= 6 && first_bps >= 6;
 }
 
+// Blocks per SM of the E + M pass before any tuning.  6 (one cell per warp) is
+// the fastest on every larger batch measured: 256 images of 481x321 0.895 ms a
+// pass against 1.007 at 4 persistent blocks, 64 grey 640x480 0.328 against
+// 0.366.  A launch that does not fill 5 blocks per SM gains nothing from room
+// for a sixth and pays its register bound (56 bytes of spill a thread; none in
+// the grayscale model), unless it runs as two parts, which take 6: 10 iterations
+// on 4 images of 1000x1000 at v = 100 2.95 ms at 5, 3.46 at 6, 20 of 320x240 at
+// v = 30 0.644 and 0.673, one of 1000x700 at v = 20 0.419 and 0.429; 4 of
+// 481x321 0.402 as one part at 5, 0.397 as two at 6.
+inline int default_blocks(int n, long long cells, int sms, bool gray) {
+  if (gray || two_parts(n, cells, sms, 6, 6)) return 6;
+  return cells <= 4LL * 5 * sms ? 5 : 6;
+}
+
 }  // namespace gmmsp

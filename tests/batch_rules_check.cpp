@@ -25,6 +25,18 @@ int main() {
       printf("parts of %d images, %lld cells, %d and %d blocks per SM\n", c.n, c.cells, c.bps, c.first);
       return 1;
     }
+  struct {
+    int n;
+    long long cells;
+    bool gray;
+    int blocks;
+  } untuned[] = {{4, 400, false, 5},          {4, 400, true, 6},  {1, 20 * 152, false, 5}, {1, 20 * 152 + 1, false, 6},
+                 {2, 16 * 152 - 1, false, 5}, {2, 16 * 152, false, 6}, {256, 185856, false, 6}};
+  for (const auto& u : untuned)
+    if (gmmsp::default_blocks(u.n, u.cells, 152, u.gray) != u.blocks) {
+      printf("untuned blocks per SM of %d images, %lld cells\n", u.n, u.cells);
+      return 1;
+    }
   printf("ok\n");
   return 0;
 }

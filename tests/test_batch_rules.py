@@ -1,5 +1,6 @@
 """The batch context's launch rules that are plain integer arithmetic (gmmsp_batch_rules.h), checked on the host:
-a batch's finalizes go one level before the caller's stream, never to the device's most urgent level at once."""
+a batch's finalizes go one level before the caller's stream, never to the device's most urgent level at once; a
+batch that leaves an SM part empty does not start with the tightest register bound."""
 import os
 import shutil
 import subprocess
@@ -20,4 +21,5 @@ def test_rules(tmp_path):
 
 def test_the_context_uses_them():
     text = open(os.path.join(ROOT, "paper_1612_08792_gb300", "csrc", "gmmsp_batch.cu")).read()
+    assert "default_blocks(n, cells, b->sm_count" in text
     assert "finalize_priority(prio, most)" in text and "two_parts(" in text and "high_priority" not in text
