@@ -40,6 +40,7 @@ struct gmmsp_batch_s {
   bool fin16 = false;              // finalize with 16 lanes per superpixel (autotuned)
   double fin_ms[2] = {0.0, 0.0};   // autotuned finalize times: 16 lanes, one thread per superpixel
   std::vector<BatchImage> host;    // the table as last uploaded
+  std::vector<double> back;        // host side of the counters and log-likelihoods
   long long total_pix = 0;
   int total_rows = 0, total_cells = 0, total_k = 0;
   void* slab = nullptr;
@@ -323,7 +324,13 @@ gmmsp_status gmmsp_batch_create(gmmsp_batch* out, int n, const int* widths, cons
   b->n = n;
   b->p = *p;
   b->stream = static_cast<cudaStream_t>(stream);
-  b->host.resize(n);
+  try {
+    b->host.resize(n);
+    b->back.resize(gmmsp::CNT_N + size_t(n));
+  } catch (const std::bad_alloc&) {
+    delete b;
+    return GMMSP_E_NOMEM;
+  }
   long long pix = 0, rows = 0, cells = 0, ks = 0;
   for (int i = 0; i < n; ++i) {
     Geom g;
@@ -459,7 +466,7 @@ gmmsp_status gmmsp_batch_segment(gmmsp_batch b, const void* const* images_dev, c
   }
   if (want_ll) {
     // the counters lie directly before the log-likelihoods: one copy
-    std::vector<double> buf(gmmsp::CNT_N + size_t(b->n));
+    std::vector<double>& buf = b->back;
     GB_CHECK(b, cudaMemcpyAsync(buf.data(), b->counters, sizeof(double) * buf.size(), cudaMemcpyDeviceToHost, b->stream));
     GB_CHECK(b, cudaStreamSynchronize(b->stream));
     unsigned long long cnt[gmmsp::CNT_N];
@@ -554,16 +561,15 @@ gmmsp_status gmmsp_batch_first_pass_partials(gmmsp_batch b, const void* const* i
   GB_CHECK(b, gmmsp::launch_em_pass_batch(b->table, b->n, 0, b->total_cells, b->lab, b->gp, b->partials,
                                           b->p.precision, em_blocks(b, blocks_per_sm), blocks_per_sm,
                                           b->p.colour_model, b->stream, diagonal != 0));
-  std::vector<float> rows(size_t(b->total_cells) * gmmsp::kPartStride);
-  GB_CHECK(b, cudaMemcpyAsync(rows.data(), b->partials, rows.size() * sizeof(float), cudaMemcpyDeviceToHost, b->stream));
+  // every cell's 15 statistics of a slot, slot after slot, then the log-likelihoods
+  const size_t from = gmmsp::kPartStride * sizeof(float), to = kRow * sizeof(float);
+  const float* parts = reinterpret_cast<const float*>(b->partials);
+  for (int s = 0; s < gmmsp::kSlots; ++s)
+    GB_CHECK(b, cudaMemcpy2DAsync(partials_host + s * gmmsp::kStats, to, parts + s * gmmsp::kSlotLd, from,
+                                  gmmsp::kStats * sizeof(float), size_t(b->total_cells), cudaMemcpyDeviceToHost, b->stream));
+  GB_CHECK(b, cudaMemcpy2DAsync(partials_host + kRow - 1, to, parts + gmmsp::kPartLl, from, sizeof(float),
+                                size_t(b->total_cells), cudaMemcpyDeviceToHost, b->stream));
   GB_CHECK(b, cudaStreamSynchronize(b->stream));
-  for (int c = 0; c < b->total_cells; ++c) {
-    const float* from = rows.data() + size_t(c) * gmmsp::kPartStride;
-    float* to = partials_host + size_t(c) * kRow;
-    for (int s = 0; s < gmmsp::kSlots; ++s)
-      memcpy(to + s * gmmsp::kStats, from + s * gmmsp::kSlotLd, gmmsp::kStats * sizeof(float));
-    to[kRow - 1] = from[gmmsp::kPartLl];
-  }
   return GMMSP_OK;
 }
 

@@ -30,6 +30,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -1087,7 +1088,7 @@ struct gmmsp_net_s {
   float *wpart0 = nullptr, *wpart1 = nullptr;  // weight-gradient partials per block: layers 0-1, layers 2-5
   double* lpart = nullptr;
   long long last_cells = 0;  // superpixels of the last forward pass
-  std::vector<char> back;    // host side of grad_to_host
+  std::unique_ptr<char[]> back;  // host side of grad_to_host: the gradient, the loss sums and the error word
   std::string msg;
 };
 
@@ -1315,10 +1316,9 @@ gmmsp_status check_err(gmmsp_net n) {
 gmmsp_status grad_to_host(gmmsp_net n, long long cells, float* grad_host, double* loss_host) {
   const char* from = grad_host ? reinterpret_cast<const char*>(n->grad) : reinterpret_cast<const char*>(n->lpart);
   const size_t bytes = size_t(reinterpret_cast<const char*>(n->err + 1) - from);
-  n->back.resize(bytes);
-  GN_CHECK(n, cudaMemcpyAsync(n->back.data(), from, bytes, cudaMemcpyDeviceToHost, n->stream));
+  GN_CHECK(n, cudaMemcpyAsync(n->back.get(), from, bytes, cudaMemcpyDeviceToHost, n->stream));
   GN_CHECK(n, cudaStreamSynchronize(n->stream));
-  auto at = [&](const void* dev) { return n->back.data() + (static_cast<const char*>(dev) - from); };
+  auto at = [&](const void* dev) { return n->back.get() + (static_cast<const char*>(dev) - from); };
   int e = 0;
   memcpy(&e, at(n->err), sizeof(int));
   if (grad_host) memcpy(grad_host, at(n->grad), size_t(n->pl.total) * 4);
@@ -1418,6 +1418,11 @@ gmmsp_status gmmsp_net_create(gmmsp_net* out, int spacing, void* stream) {
   const size_t o_b = off; off += up256(np * 2);
   const size_t o_s = off; off += up256(4 * kWBytes);
   const size_t o_t = off; off += 256 * 4;
+  n->back.reset(new (std::nothrow) char[o_e + sizeof(int) - o_g]);
+  if (!n->back) {
+    delete n;
+    return GMMSP_E_NOMEM;
+  }
   const char* inj = getenv("GMMSP_FAIL_ALLOC");
   cudaError_t e = (inj && inj[0] == '1') ? cudaErrorMemoryAllocation : cudaMalloc(&n->pslab, off);
   if (e != cudaSuccess) {

@@ -52,7 +52,8 @@
 #include <string.h>
 
 #include <algorithm>
-#include <vector>
+#include <memory>
+#include <new>
 
 #include "../../include/gmmsp.h"
 #include "../../include/gmmsp_conn.h"
@@ -1164,7 +1165,11 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   GMMSP_NVTX("enforce_connectivity_many");
   using namespace conn;
   if (n < 1 || n > 65535) return GMMSP_E_INVALID;
-  std::vector<Img> host(n);
+  // the image table and, behind it, the counters (zeros): uploaded in one copy
+  const size_t up_bytes = ((sizeof(Img) * n + 255) & ~size_t(255)) + 256;
+  const std::unique_ptr<char[]> up_host(new (std::nothrow) char[up_bytes]());
+  if (!up_host) return GMMSP_E_NOMEM;
+  Img* host = reinterpret_cast<Img*>(up_host.get());
   long long T = 0, maxN = 0;
   for (int i = 0; i < n; ++i) {
     if (W[i] < 1 || H[i] < 1 || K[i] < 1 || !labels[i] || !lab[i]) return GMMSP_E_INVALID;
@@ -1269,13 +1274,11 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   // 481x321; this many 1.93 ms, and no less with 32 to 128 per SM)
   const int warp_blocks = int(std::max<long long>(1, std::min<long long>(152 * 16, (T + 1023) / 1024)));
   const int thread_blocks = warp_blocks;
-  std::vector<char> up_host(o[O_CNT] + 256 - o[O_TABLE], 0);
-  memcpy(up_host.data(), host.data(), sizeof(Img) * n);
   char back[256] = {};
   unsigned long long hc[3] = {};
   int herr = 0;
   do {
-    if ((e = cudaMemcpyAsync(table, up_host.data(), up_host.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
+    if ((e = cudaMemcpyAsync(table, up_host.get(), up_bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) break;
     k_cc_tile<<<gt, kCcWarps * 32, 0, s>>>(table, S, nwords, tile_rows);
     k_cc_border<<<gp, 256, 0, s>>>(table, S.parent, S.err, tile_rows);
     k_tile_roots<<<gt, kCcWarps * 32, 0, s>>>(table, S, tile_rows);
