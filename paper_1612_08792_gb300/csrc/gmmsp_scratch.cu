@@ -49,9 +49,16 @@ cudaMemPool_t pool_of_device(int* device) {
 
 cudaError_t CallScratch::alloc(size_t bytes, cudaStream_t s) {
   stream = s;
+  // These calls synchronise, which a capture does not allow: refused before
+  // anything of them is recorded (the pool would allocate inside the graph).
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &cs);
+  if (e != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return cudaErrorStreamCaptureUnsupported;
+  }
   int dev = 0;
   cudaMemPool_t pool = pool_of_device(&dev);
-  cudaError_t e;
   if (pool) {
     pooled = true;
     e = cudaMallocFromPoolAsync(&ptr, bytes, pool, s);
