@@ -87,28 +87,26 @@ struct Img {
 struct Scratch {
   // per pixel of the call
   int* parent;                // union-find, then the compact index
-  int* cidr;                  // at the tiles' root pixels: the compact index
+  int* cidr;                  // at the tiles' root pixels: the compact index; then (k_cluster_fill) ...
+  int* big;                   // ... in the same memory, roots of clusters above kThreadCluster members: those
+                              // above kHugeCluster from the front, the others from the back
   // per component (compact index c < ncomp)
-  int* size;                  // pixel count
+  int* size;                  // pixel count; in the merge, of a small founder's group
   long long* csum;            // 3 fixed-point colour sums, then (k_comp_flags) ...
   double* mean;               // ... the 3 mean colours csum / size, in the same memory
   float4* mean32;             // the means in FP32 and the largest of their magnitudes
   int* cimg;                  // image
   int32_t* clabel;            // its label
-  int* small;                 // 1 for a small component
-  int* cpar;                  // cluster union-find over small components
+  int* cpar;                  // cluster union-find over small components, -1 for the others
   int* deg;                   // entries of its adjacency list
   unsigned* aoff;             // (ncomp + 1) offsets of the lists, each with room for the component's perimeter
   int* adj;                   // adjacency lists (compact indices of neighbouring components)
-  int* cl_count;              // members of the cluster it roots, counted down as they are filled in
+  int* cl_count;              // members of the cluster it roots, counted down as they are filled in; in the
+                              // merge, the order of a large cluster's members
   unsigned* cl_off;           // (ncomp + 1) member offsets
   unsigned long long* cl_key; // members as (size << 32 | c), grouped by cluster
-  int* big;                   // roots of clusters above kThreadCluster members: those above
-                              // kHugeCluster from the front, the others from the back
   int* gpar;                  // merge union-find (group founder)
-  int* gsize;                 // group size (kept for small founders)
-  int* next;                  // next member of its group, -1 at the end
-  int* tail;                  // of a group's founder: its last member
+  int* next;                  // the members of a group as a ring (small founders' groups)
   int* tile_sum;              // tile kernels: per tile counts, then their exclusive prefix
   // the tiles' roots (before the per-component arrays that lie in the same memory)
   int* roots;                 // a tile's root pixels, from its place on (tile_place)
@@ -182,6 +180,9 @@ __device__ __forceinline__ void unite(int* p, int a, int b, int* err) {
   }
   atomicExch(err, 1);
 }
+
+// A union or a path halving may be at work on the entry: its sign stays.
+__device__ __forceinline__ bool is_small(const Scratch& S, int c) { return S.cpar[c] >= 0; }
 
 __device__ __forceinline__ bool small_size(long long s, int K, long long N) { return 4LL * K * s < N; }
 
@@ -583,17 +584,14 @@ __global__ void __launch_bounds__(256) k_comp_flags(const Img* __restrict__ imgs
       const Img im = imgs[S.cimg[c]];
       const int sz = S.size[c];
       sm = small_size(sz, im.K, (long long)im.W * im.H);
-      S.small[c] = sm ? 1 : 0;
       double m[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k) S.mean[3LL * c + k] = m[k] = double(S.csum[3LL * c + k]) / double(sz);
       const float x = float(m[0]), y = float(m[1]), z = float(m[2]);
       S.mean32[c] = make_float4(x, y, z, fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z))));
       S.gpar[c] = c;
-      S.gsize[c] = sz;
-      S.cpar[c] = c;
-      S.next[c] = -1;
-      S.tail[c] = c;
+      S.cpar[c] = sm ? c : -1;
+      S.next[c] = c;
     }
     const int nsm = __syncthreads_count(sm);
     if (threadIdx.x == 0 && nsm) atomicAdd(S.cnt + 0, (unsigned long long)nsm);
@@ -610,7 +608,7 @@ __device__ __forceinline__ void add_neighbour(const Scratch& S, int i, int j) {
   else atomicExch(S.err, 1);
 }
 __device__ __forceinline__ void add_edge(const Scratch& S, int i, int j) {
-  const int si = S.small[i], sj = S.small[j];
+  const bool si = is_small(S, i), sj = is_small(S, j);
   if (si) add_neighbour(S, i, j);
   if (sj) add_neighbour(S, j, i);
   if (si && sj) unite(S.cpar, i, j, S.err);
@@ -704,7 +702,7 @@ enum ScanOf : int { kScanLists = 0, kScanClusters = 1 };
 template <int OF>
 __device__ __forceinline__ unsigned scan_value(const Scratch& S, int c) {
   if (OF == kScanClusters) return unsigned(S.cl_count[c]);
-  return S.small[c] ? 2u * unsigned(S.size[c]) + 2u : 0u;
+  return is_small(S, c) ? 2u * unsigned(S.size[c]) + 2u : 0u;
 }
 
 // Exclusive prefix sum over the n = *S.ncomp components into out[0..n] (out[n]
@@ -786,7 +784,7 @@ __global__ void __launch_bounds__(1024) k_scan_add(Scratch S, unsigned* __restri
 // Cluster root of every small component, member counts per cluster root.
 __global__ void k_cluster_count(Scratch S) {
   FOR_COMPONENTS(c) {
-    if (!S.small[c]) continue;
+    if (!is_small(S, c)) continue;
     atomicAdd(S.cl_count + find_root(S.cpar, c, S.err), 1);
   }
 }
@@ -802,7 +800,7 @@ __global__ void __launch_bounds__(256) k_cluster_fill(Scratch S) {
     if (threadIdx.x < 2) n_of[threadIdx.x] = 0;
     __syncthreads();
     int kind = -1, at = 0;
-    if (c < ncomp && S.small[c]) {
+    if (c < ncomp && is_small(S, c)) {
       const int r = find_root(S.cpar, c, S.err);
       const unsigned off = S.cl_off[r];
       if (r == c) {
@@ -850,12 +848,13 @@ __device__ __forceinline__ float dist2_32(float4 a, float4 b, float& off) {
 // never a source, and no decision reads its size.
 __device__ __forceinline__ void merge_into(Scratch& S, int r, int best) {
   S.gpar[r] = best;
-  if (S.small[best]) {
-    S.gsize[best] += S.gsize[r];
-    S.next[S.tail[best]] = r;
-    S.tail[best] = S.tail[r];
+  if (is_small(S, best)) {
+    S.size[best] += S.size[r];
+    const int n = S.next[best];  // two rings become one
+    S.next[best] = S.next[r];
+    S.next[r] = n;
   }
-  S.gsize[r] = 0;
+  S.size[r] = 0;
 }
 
 // Insertion sort of n keys (one thread).
@@ -877,7 +876,7 @@ __device__ __forceinline__ unsigned merge_small_clusters(const Img* __restrict__
   unsigned merged = 0;
   const int ncomp = *S.ncomp;
   for (int c = first; c < ncomp; c += step) {
-    if (!S.small[c] || S.cpar[c] != c) continue;  // not a cluster root
+    if (S.cpar[c] != c) continue;  // not a cluster root
     const int n = int(S.cl_off[c + 1] - S.cl_off[c]);
     if (n > kThreadCluster) continue;
     const Img im = imgs[S.cimg[c]];
@@ -886,13 +885,13 @@ __device__ __forceinline__ unsigned merge_small_clusters(const Img* __restrict__
     sort_keys(key, n);
     for (int a = 0; a < n; ++a) {
       const int r = int(unsigned(key[a]));
-      if (S.gpar[r] != r || !small_size(S.gsize[r], im.K, N)) continue;
+      if (S.gpar[r] != r || !small_size(S.size[r], im.K, N)) continue;
       const float4 mr = S.mean32[r];
       int best = -1;
       float low = 0.f, high = INFINITY;  // the nearest one's distance lies in [low, high]
       bool close = false;                // another group may be as near
       int hops = 0;
-      for (int m = r; m >= 0 && hops < kMaxHops; m = S.next[m], ++hops) {
+      for (int m = r; (m != r || hops == 0) && hops < kMaxHops; m = S.next[m], ++hops) {
         const unsigned q0 = S.aoff[m], q1 = q0 + unsigned(S.deg[m]);
         for (unsigned q = q0; q < q1; ++q) {
           const int g = find_group(S.gpar, S.adj[q], S.err);
@@ -916,7 +915,7 @@ __device__ __forceinline__ unsigned merge_small_clusters(const Img* __restrict__
       if (close) {
         best = -1;
         double bd = 0.0;
-        for (int m = r, h = 0; m >= 0 && h < kMaxHops; m = S.next[m], ++h) {
+        for (int m = r, h = 0; (m != r || h == 0) && h < kMaxHops; m = S.next[m], ++h) {
           const unsigned q0 = S.aoff[m], q1 = q0 + unsigned(S.deg[m]);
           for (unsigned q = q0; q < q1; ++q) {
             const int g = find_group(S.gpar, S.adj[q], S.err);
@@ -991,7 +990,7 @@ __device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, 
     for (int j = 0; j < n; ++j) rank += __shfl_sync(0xffffffffu, k, j) < k;
     if (lane < n) order[rank] = int(unsigned(k));
   } else {
-    order = S.cidr + S.cl_off[c];  // the roots' indices are not needed any more
+    order = S.cl_count + S.cl_off[c];  // the counts are done with
     for (int i = lane; i < n; i += 32) {
       const unsigned long long k = key[i];
       int rank = 0;
@@ -1023,7 +1022,7 @@ __device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, 
     }
     if (a + 3 < n) m2.list(S, member(a + 3));
     const int r = me.r;
-    if (S.gpar[r] != r || !small_size(S.gsize[r], im.K, N)) continue;  // warp-uniform
+    if (S.gpar[r] != r || !small_size(S.size[r], im.K, N)) continue;  // warp-uniform
     // this lane's neighbour groups: one that is nearest in FP32, and whether
     // another may be as near
     int best = 0x7fffffff;
@@ -1049,7 +1048,7 @@ __device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, 
       consider(g, g == me.adj ? me.ma : S.mean32[g]);
     }
     int hops = 0;
-    for (int m = r; m >= 0 && hops < kMaxHops; m = S.next[m], ++hops) {
+    for (int m = r; (m != r || hops == 0) && hops < kMaxHops; m = S.next[m], ++hops) {
       const unsigned q0 = m == r ? me.q0 : S.aoff[m], q1 = q0 + (m == r ? me.deg : unsigned(S.deg[m]));
       for (unsigned q = q0 + lane + (m == r ? 32u : 0u); q < q1; q += 32) {
         const int g = find_group(S.gpar, S.adj[q], S.err);
@@ -1067,7 +1066,7 @@ __device__ __forceinline__ unsigned merge_cluster(const Img* __restrict__ imgs, 
     if (__any_sync(0xffffffffu, in && (close || best != first))) {  // FP64 decides
       best = 0x7fffffff;
       double bd = INFINITY;
-      for (int m = r, h = 0; m >= 0 && h < kMaxHops; m = S.next[m], ++h) {
+      for (int m = r, h = 0; (m != r || h == 0) && h < kMaxHops; m = S.next[m], ++h) {
         const unsigned q0 = S.aoff[m], q1 = q0 + unsigned(S.deg[m]);
         for (unsigned q = q0 + lane; q < q1; q += 32) {
           const int g = find_group(S.gpar, S.adj[q], S.err);
@@ -1179,11 +1178,10 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   }
   if (T >= (1LL << 30)) return GMMSP_E_INVALID;
   auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
-  // every per-component array has room for T components (one per pixel at most)
+  // every per-component array has room for T components (one per pixel at most): 112 bytes per pixel in all
   const size_t nI = up(size_t(T) * 4), nI1 = up(size_t(T + 1) * 4);
   const long long ntiles = std::max<long long>(1, (T + kScanTile - 1) / kScanTile);
-  enum { A_PARENT, A_CIDR, A_SIZE, A_CIMG, A_CLABEL, A_SMALL, A_CPAR, A_DEG, A_CLCOUNT, A_BIG, A_GPAR, A_GSIZE,
-         A_NEXT, A_TAIL, kIntArrays };
+  enum { A_PARENT, A_CIDR, A_SIZE, A_CIMG, A_CLABEL, A_CPAR, A_DEG, A_CLCOUNT, A_GPAR, A_NEXT, kIntArrays };
   enum { O_AOFF = kIntArrays, O_CLOFF, O_ADJ, O_CSUM, O_MEAN32, O_TABLE, O_CNT, O_KEY, O_TILE, kRegions };
   size_t o[kRegions];
   size_t off = 0;
@@ -1225,9 +1223,9 @@ gmmsp_status enforce_connectivity_many(int n, const int* W, const int* H, const 
   auto ia = [&](int j) { return reinterpret_cast<int*>(b + o[j]); };
   Scratch S{};
   S.parent = ia(A_PARENT); S.cidr = ia(A_CIDR); S.size = ia(A_SIZE); S.cimg = ia(A_CIMG);
-  S.clabel = reinterpret_cast<int32_t*>(ia(A_CLABEL)); S.small = ia(A_SMALL); S.cpar = ia(A_CPAR);
-  S.deg = ia(A_DEG); S.cl_count = ia(A_CLCOUNT); S.big = ia(A_BIG); S.gpar = ia(A_GPAR); S.gsize = ia(A_GSIZE);
-  S.next = ia(A_NEXT); S.tail = ia(A_TAIL);
+  S.clabel = reinterpret_cast<int32_t*>(ia(A_CLABEL)); S.cpar = ia(A_CPAR);
+  S.deg = ia(A_DEG); S.cl_count = ia(A_CLCOUNT); S.gpar = ia(A_GPAR); S.next = ia(A_NEXT);
+  S.big = S.cidr;
   S.aoff = reinterpret_cast<unsigned*>(ia(O_AOFF));
   S.cl_off = reinterpret_cast<unsigned*>(ia(O_CLOFF));
   S.adj = ia(O_ADJ);
