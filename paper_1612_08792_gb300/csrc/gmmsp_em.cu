@@ -1196,10 +1196,13 @@ static cudaError_t em_pass_impl(Src lab, const Geom& g, const float* gp, PT* par
   // A bound costs spills or longer code and gains only where a tighter one saves
   // a round or, with many, hides more latency.  10 iterations and labels, us,
   // the bound taken and the other one:
-  //  full model, up to 5 blocks per SM: none (5 where that is needed to fit 5).
-  //    320x240 v = 20 (192 blocks of four warps per cell) 144, 154 at 7; 481x321
-  //    v = 30 191, 209; 1000x560 v = 14 (one warp) 298, 306 at 6
-  //  four warps, more blocks: 7.  481x321 v = 12 (1107 blocks) 164, 184 without
+  //  full model, four warps per cell, up to 3 blocks per SM: none.  320x240
+  //    v = 20 (192 blocks) 143, 152 at 7; 481x321 v = 30 191, 209.  More blocks:
+  //    7.  481x321 v = 12 (1107 blocks) 166, 185 without; at 3 to 5 none is as
+  //    fast alone, 320x240 v = 12 133 and 136, but not for two images at once on
+  //    two streams, 83.3 and 82.0 an image, 481x321 v = 15 110 and 107
+  //  one warp, up to 5 blocks per SM: none (5 where that is needed to fit 5).
+  //    1000x560 v = 14 296, 306 at 6
   //  one warp, 6 to 7 blocks per SM: 7, one round.  800x600 v = 11 312, 317 at 6;
   //    otherwise 6: an E+M pass at 3840x2160, v = 20 takes 189, 203 at 7
   //  split model (86 registers) and the FP32 variant's two warps (87): 6 where
@@ -1208,7 +1211,7 @@ static cudaError_t em_pass_impl(Src lab, const Geom& g, const float* gp, PT* par
   const auto kernel = [blocks] {
     constexpr auto uncapped = k_em_pass<PT, SHIFT, WPC, Src, CM, DIAG>;
     if constexpr (CM == kColourFull && WPC != 2) {
-      if (blocks <= 5 * kSms) return WPC == 1 && SHIFT ? k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 5> : uncapped;
+      if (blocks <= (WPC == 4 ? 3 : 5) * kSms) return WPC == 1 && SHIFT ? k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 5> : uncapped;
       if (WPC == 4 || (blocks > 6 * kSms && blocks <= 7 * kSms)) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 7>;
       if constexpr (WPC == 1) return k_em_pass_capped<PT, SHIFT, WPC, Src, CM, DIAG, 6>;
     } else if constexpr (CM == kColourSplit || (CM == kColourFull && !SHIFT)) {

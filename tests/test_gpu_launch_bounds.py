@@ -1,5 +1,5 @@
 """The register-bound variants of the single-image E+M and label kernels, which the number of blocks chooses: on
-either side of every line (5, 6, 7 and 8 blocks of four cells per SM) one warp per cell gives the bits of a batch
+either side of every line (3 blocks of one cell, 5, 6, 7 and 8 blocks of four cells per SM) one warp per cell gives the bits of a batch
 of that one image (whose kernels do not vary), for every colour model; four warps per cell agree with that to
 their summation order; and the allocation-free call gives the labels of a context."""
 import numpy as np
@@ -10,8 +10,9 @@ from synth import voronoi_image
 pytestmark = pytest.mark.gpu
 
 V = 4
-# cell grids: up to 5 blocks of four cells on each of 152 SMs, 5 to 6, 6 to 7, 7 to 8, more
-GRIDS = [(19, 40), (58, 52), (60, 55), (65, 62), (70, 66), (80, 70)]
+# cell grids: blocks of one cell (four warps per cell) up to 3 on each of 152 SMs, 3 to 5; blocks of four cells up to 5
+# on each, 5 to 6, 6 to 7, 7 to 8, more
+GRIDS = [(19, 20), (19, 40), (58, 52), (60, 55), (65, 62), (70, 66), (80, 70)]
 
 
 def setup(nx, ny):
