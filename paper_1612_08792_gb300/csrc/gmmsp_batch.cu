@@ -658,8 +658,12 @@ gmmsp_status gmmsp_batch_autotune(gmmsp_batch b, const void* const* images_dev, 
   // alone, and a segment then takes 571 us as one part, 517 as two at 6; 8
   // images: 16 lanes take 20.7 us alone against 19.3, and a segment 529 us
   // against 556; 16 images: 893 against 862.
+  // From 128 cells per SM on (17,424 cells of 24 images are fewer) the choices
+  // alone are the right ones unless they would keep it in one part, and the
+  // timing would take long (0.18 s of 0.77 for 256 uneven images).
   const int flat_c = flat_ms[0] <= flat_ms[1] ? 6 : 7, flat_first = b->first_ms[0] <= b->first_ms[1] ? 6 : 7;
-  if (b->side && gmmsp::two_parts(b->n, b->total_cells, b->sm_count, flat_c, flat_first)) {
+  if (b->side && gmmsp::two_parts(b->n, b->total_cells, b->sm_count, flat_c, flat_first) &&
+      (b->total_cells < 128 * b->sm_count || best_c < 6 || first_c < 6)) {
     const bool both_fin = b->p.precision != GMMSP_PREC_FP32 && b->p.colour_model == GMMSP_COLOUR_FULL;
     const int as_run[2][2] = {{best_c, first_c}, {flat_c, flat_first}};
     const bool same = best_c == flat_c && first_c == flat_first;
