@@ -236,7 +236,7 @@ gmmsp_status gmmsp_autotune(gmmsp_ctx c, int reps, int *best, double *times_ms);
 /*
  * Batches: many images of uneven sizes segmented together, Algorithm 1,
  * steps 1-7, for every image, with one kernel launch per step for the whole
- * batch (persistent blocks walk the batch's cells / superpixels), the step
+ * batch (one cell per warp, or persistent blocks that walk the cells), the step
  * sequence captured into one CUDA graph on the first call (per iteration
  * count) and replayed afterwards.  The paper segments one image at a time;
  * batching is this library's way of filling the GPU with small images.

@@ -1,4 +1,4 @@
-// Per-cell helpers shared by the EM kernels (gmmsp_em.cu, gmmsp_rows.cu):
+// Per-cell helpers shared by the kernels of gmmsp_em.cu:
 // the cell's extent and candidate mask, the special-function approximations
 // of the E-step, the log2 density of one candidate, and the image lookup of
 // a batch.

@@ -416,9 +416,10 @@ __global__ void __launch_bounds__(kEmWarps * 32, MINB) k_em_pass_capped(Src lab,
 // [cell_off, cell_off + ncells), the superpixels [k_off, k_off + K) and the
 // pixels [pix_off, pix_off + W H) of the batch (its CIELAB planes start at
 // lab + 3 pix_off).  Work items are found by a binary search over these
-// prefix offsets; warps (threads for per-superpixel work) loop over the
-// batch's items with the grid's stride, so the grid is sized to the machine
-// (persistent blocks) rather than to the work.
+// prefix offsets.  k_em_pass_batch is the persistent form of the E+M pass:
+// warps loop over the cells with the grid's stride, and the grid is sized to the
+// machine; the form of larger launches, one cell per warp, follows it.  The
+// finalize's threads loop likewise.
 // MINB caps the registers so that MINB blocks fit on an SM (5: at most 102
 // registers, no spills).
 template <typename PT, bool SHIFT, int MINB, int CM>
