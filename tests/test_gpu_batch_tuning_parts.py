@@ -49,7 +49,7 @@ def test_keeps_choices_that_are_fast_as_they_run(n):
     assert best == t["blocks_per_sm"] and sorted(times) == [3, 4, 5, 6, 7]
     got = segment_ms(torch, bt, x, stream, t["finalize16"], gm, best, t["first_pass_blocks_per_sm"])
     others = {(b, f): segment_ms(torch, bt, x, stream, f, gm, b, 6) for b in (5, 6) for f in (False, True)}
-    assert got <= 1.03 * min(others.values()), (t, got, others)  # 3 %: timing noise between equally good choices
+    assert got <= 1.06 * min(others.values()), (t, got, others)  # 6 %: timing noise between equally good choices
     bt.close()
 
 
